@@ -113,6 +113,8 @@ struct bte_ctx {
   double* scratch_q = nullptr;
   std::vector<DevGeom> dgeoms;
   DirInfo* dirs_d = nullptr;
+  int* wall_dirs_d = nullptr;   // [6][nd] per side: leaving directions, then the rest
+  std::array<WallDirs, 6> wall_dirs{};
   DevGeom* geoms_d = nullptr;
   WorkItem* items_d = nullptr;
   DevCounters* counters = nullptr;
@@ -233,6 +235,7 @@ size_t carve(bte_ctx* h, char* base) {
   h->wdir = (double*)take((size_t)h->nd * 8);
   h->Sdev = (double*)take((size_t)h->nd * 3 * 8);
   h->dirs_d = (DirInfo*)take((size_t)h->nd * sizeof(DirInfo));
+  h->wall_dirs_d = (int*)take((size_t)h->nd * 6 * 4);
   h->node_c = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->node_C = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->a_p = (double*)take((size_t)h->nbp_all * 8);
@@ -379,6 +382,21 @@ int ensure_memory(bte_ctx* h) {
     di[d].rz = h->refl[2 * h->nd + d];
   }
   CUDA_TRY(h, cudaMemcpyAsync(h->dirs_d, di.data(), di.size() * sizeof(DirInfo), cudaMemcpyHostToDevice, s));
+  std::vector<int> wl((size_t)6 * h->nd);
+  for (int side = 0; side < 6; ++side) {
+    WallDirs& wd = h->wall_dirs[side];
+    int* l = wl.data() + (size_t)side * h->nd;
+    wd = WallDirs{h->wall_dirs_d + (size_t)side * h->nd, nullptr, 0, 0.0, 0.0};
+    int nrest = 0;
+    for (int d = 0; d < h->nd; ++d) {
+      const double sn = (side & 1) ? h->S[3 * d + side / 2] : -h->S[3 * d + side / 2];
+      if (sn > 0.0) { l[wd.nout++] = d; wd.sum_out += sn; }
+      else { l[h->nd - ++nrest] = d; wd.sum_in -= sn; }
+    }
+    std::reverse(l + wd.nout, l + h->nd);
+    wd.rest = wd.out + wd.nout;
+  }
+  CUDA_TRY(h, cudaMemcpyAsync(h->wall_dirs_d, wl.data(), wl.size() * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->wdir, h->w.data(), h->nd * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->Sdev, h->S.data(), h->nd * 3 * 8, cudaMemcpyHostToDevice, s));
   // band tables
@@ -618,7 +636,7 @@ cudaError_t refresh_diffuse(bte_ctx* h, const void* I, cudaStream_t s, int* laun
       if (h->bc_type[gi][side] != BTE_BC_DIFFUSE) continue;
       const cudaError_t e = launch_diffuse_ghosts(
           h->opts.precision, I, h->I0ref_o, h->I0wall, h->opts.precision == BTE_FP64 ? nullptr : h->I0wall_dev,
-          h->geoms_d, (int)gi, side, h->Sdev, h->nd, h->nbp, (int)side_faces(h->geoms[gi], side), s);
+          h->geoms_d, (int)gi, side, h->Sdev, h->wall_dirs[side], h->nd, h->nbp, (int)side_faces(h->geoms[gi], side), s);
       if (e != cudaSuccess) return e;
       if (launches) ++*launches;
     }
@@ -633,8 +651,9 @@ cudaError_t refresh_partial(bte_ctx* h, const void* I, cudaStream_t s, int* laun
     for (int side = 0; side < 2 * h->geoms[gi].dim; ++side) {
       if (h->bc_type[gi][side] != BTE_BC_PARTIAL) continue;
       const cudaError_t e = launch_partial_ghosts(h->opts.precision, I, h->I0ref_o, h->geoms_d, (int)gi, side, h->Sdev,
-                                                  h->dirs_d, h->nd, h->nbp, (int)side_faces(h->geoms[gi], side),
-                                                  h->spec[gi][side], h->gdir[gi][side], s);
+                                                  h->wall_dirs[side], h->dirs_d, h->nd, h->nbp,
+                                                  (int)side_faces(h->geoms[gi], side), h->spec[gi][side],
+                                                  h->gdir[gi][side], s);
       if (e != cudaSuccess) return e;
       if (launches) ++*launches;
     }

@@ -66,6 +66,15 @@ struct DirInfo {
   int rx, ry, rz;
 };
 
+// The directions of one wall side: those leaving through it (S_d . n_out > 0),
+// then the rest, and the sums of |S_d,ax| over the leaving and the entering ones.
+struct WallDirs {
+  const int* out;   // [nout]
+  const int* rest;  // [nd - nout]
+  int nout;
+  double sum_out, sum_in;
+};
+
 // A cell whose temperature the sweep could not settle on its cached model.
 struct FixItem {
   long long P;  // global cell
@@ -182,13 +191,13 @@ cudaError_t launch_gs_sweep(int precision, const SweepArgs& a, int dim, int thre
 cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells, cudaStream_t s);
 cudaError_t launch_beta_scale(double* out, const double* Tp, double Tref, double p, long long ncells, cudaStream_t s);
 cudaError_t launch_diffuse_ghosts(int precision, const void* I, const double* I0ref, double* I0wall, float* I0wall_dev,
-                                  const DevGeom* geoms, int geom, int side, const double* S, int nd, int nbp,
-                                  int nfaces, cudaStream_t s);
-// Partially specular side: per face, direction and band, p x the cell's mirrored
-// value + (1 - p) x the diffuse value, into out [face][dir][nbp] (storage type).
+                                  const DevGeom* geoms, int geom, int side, const double* Sd, const WallDirs& wd, int nd,
+                                  int nbp, int nfaces, cudaStream_t s);
+// Partially specular side: per face, entering direction and band, p x the cell's
+// mirrored value + (1 - p) x the diffuse value, into out [face][dir][nbp] (storage type).
 cudaError_t launch_partial_ghosts(int precision, const void* I, const double* I0ref, const DevGeom* geoms, int geom,
-                                  int side, const double* S, const DirInfo* dirs, int nd, int nbp, int nfaces,
-                                  double p, void* out, cudaStream_t s);
+                                  int side, const double* Sd, const WallDirs& wd, const DirInfo* dirs, int nd, int nbp,
+                                  int nfaces, double p, void* out, cudaStream_t s);
 // learned guess (bte_mlp.cu)
 int mlp_param_total(int nb);
 cudaError_t launch_mlp_norm(ThermoTables th, double T_lo, double T_hi, const double* I0ref, double* r_lo, double* r_hi,

@@ -576,98 +576,145 @@ __global__ void __launch_bounds__(256, 4) gs_reduce_kernel(SweepArgs a, long lon
   if (wid == 0) flush_counters(a, lane, solves, badc);
 }
 
-// Diffuse wall ghosts of one side of one geometry: for every face, per band,
-// sum over the directions leaving through the wall of |S_d,ax| I_d, divided by
-// sum over the entering directions of |S_d,ax|, from the wall cell's current
-// iterate, into the FP64 ghost row (and the FP32 deviation row in the reduced
-// modes).  One warp per face, lanes over bands, directions in order.
+// Wall ghosts of one side of one geometry from the wall cells' current iterate:
+// one CTA of 256 threads per face.  Bound by the FP64 pipe (one FMA per
+// outgoing direction and band) and, below a few hundred faces, by the latency
+// of one face, so a face's directions are spread over the CTA: lane l of group
+// g holds the V bands of one 16-byte vector and sums the outgoing directions
+// g, g + groups, ... of the side's list (WallDirs, built on the host with the
+// two weight sums, so no thread walks or tests all directions), four loads in
+// flight; the groups' partials are added in order in shared memory.  One warp
+// per face walking every direction, each thread forming the weight sum again,
+// took 280 us (diffuse) and 204 us (partially specular) on the 67 faces of a
+// 67x45 grid with 400 directions x 55 bands; this form takes 8-9 us.
+// Reduced modes sum the stored deviations: the reference part of the ratio is
+// I0_b(T_ref) (sum_out - sum_in) / sum_in.
+constexpr int kWallThreads = 256;
+
 template <typename S>
-__global__ void diffuse_ghost_kernel(const S* I, const double* I0ref, double* I0wall, float* I0wall_dev,
-                                     const DevGeom* geoms, int geom, int side, const double* Sd, int nd, int nbp,
-                                     int nfaces) {
-  const DevGeom g = geoms[geom];
+struct WallArgs {
+  const S* I;
+  const double* I0ref;
+  const DevGeom* geoms;
+  const double* Sd;
+  int geom, side, nd, nbp, nfaces;
+  WallDirs wd;
+};
+
+__device__ __forceinline__ long long wall_cell(const DevGeom& g, int side, int f) {
   const int ax = side >> 1;
   const bool high = side & 1;
-  const int warps = blockDim.x / 32, lane = threadIdx.x & 31;
-  const long long row = (long long)nd * nbp;
-  for (int f = blockIdx.x * warps + threadIdx.x / 32; f < nfaces; f += gridDim.x * warps) {
-    int i, j, k;  // wall cell of face f (x sides: j + ny k, y sides: i + nx k, z sides: i + nx j)
-    if (ax == 0) { i = high ? g.nx - 1 : 0; j = f % g.ny; k = f / g.ny; }
-    else if (ax == 1) { j = high ? g.ny - 1 : 0; i = f % g.nx; k = f / g.nx; }
-    else { k = high ? g.nz - 1 : 0; i = f % g.nx; j = f / g.nx; }
-    const long long P = g.cell0 + ((long long)k * g.ny + j) * g.nx + i;
-    double den = 0.0;
-    for (int d = 0; d < nd; ++d) {
-      const double sd = Sd[3 * d + ax];
-      if (!(high ? sd > 0.0 : sd < 0.0) && sd != 0.0) den += fabs(sd);
-    }
-    for (int b = lane; b < nbp; b += 32) {
-      double num = 0.0;
-      for (int d = 0; d < nd; ++d) {
-        const double sd = Sd[3 * d + ax];
-        if (high ? sd > 0.0 : sd < 0.0) num += fabs(sd) * full_I(I, P * row + (long long)d * nbp + b, b, I0ref);
+  int i, j, k;  // wall cell of face f (x sides: j + ny k, y sides: i + nx k, z sides: i + nx j)
+  if (ax == 0) { i = high ? g.nx - 1 : 0; j = f % g.ny; k = f / g.ny; }
+  else if (ax == 1) { j = high ? g.ny - 1 : 0; i = f % g.nx; k = f / g.nx; }
+  else { k = high ? g.nz - 1 : 0; i = f % g.nx; j = f / g.nx; }
+  return g.cell0 + ((long long)k * g.ny + j) * g.nx + i;
+}
+
+// D[b] = sum_out |S_ax| I_b / sum_in |S_ax| of the cell whose row is given (a
+// deviation in the reduced modes).  Every thread calls it; D is complete on return.
+template <typename S>
+__device__ __forceinline__ void wall_diffuse(const WallArgs<S>& w, const S* row, double* part, double* D) {
+  using T = Tr<S>;
+  constexpr int V = T::V;
+  const int lpc = w.nbp / V, groups = kWallThreads / lpc;
+  const int grp = threadIdx.x / lpc, b0 = V * (threadIdx.x - grp * lpc);
+  const int ax = w.side >> 1;
+  if (grp < groups) {
+    double acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = 0.0;
+    int k = grp;
+    for (; k + 3 * groups < w.wd.nout; k += 4 * groups) {
+      typename T::A x[4][V];
+      double sd[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int d = w.wd.out[k + u * groups];
+        sd[u] = fabs(w.Sd[3 * d + ax]);
+        T::ld(row + (long long)d * w.nbp + b0, x[u]);
       }
-      const double v = num / den;
-      const long long e = (g.face0[side] + f) * nbp + b;
-      I0wall[e] = v;
-      if (I0wall_dev) I0wall_dev[e] = (float)(v - I0ref[b]);
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < V; ++v) acc[v] = fma(sd[u], (double)x[u][v], acc[v]);
     }
+    for (; k < w.wd.nout; k += groups) {
+      const int d = w.wd.out[k];
+      const double sd = fabs(w.Sd[3 * d + ax]);
+      typename T::A x[V];
+      T::ld(row + (long long)d * w.nbp + b0, x);
+#pragma unroll
+      for (int v = 0; v < V; ++v) acc[v] = fma(sd, (double)x[v], acc[v]);
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) part[grp * w.nbp + b0 + v] = acc[v];
+  }
+  __syncthreads();
+  for (int b = threadIdx.x; b < w.nbp; b += kWallThreads) {
+    double num = part[b];
+    for (int g = 1; g < groups; ++g) num += part[g * w.nbp + b];
+    if constexpr (sizeof(S) != 8) num = fma(w.wd.sum_out - w.wd.sum_in, w.I0ref[b], num);
+    D[b] = num / w.wd.sum_in;
+  }
+  __syncthreads();
+}
+
+// Diffuse side: the FP64 ghost row of every face (and the FP32 deviation row in
+// the reduced modes).
+template <typename S>
+__global__ void __launch_bounds__(kWallThreads) diffuse_ghost_kernel(WallArgs<S> w, double* I0wall, float* I0wall_dev) {
+  extern __shared__ double part[];  // [groups][nbp], then D [nbp]
+  double* D = part + (kWallThreads / (w.nbp / Tr<S>::V)) * w.nbp;
+  const DevGeom g = w.geoms[w.geom];
+  for (int f = blockIdx.x; f < w.nfaces; f += gridDim.x) {
+    wall_diffuse<S>(w, w.I + wall_cell(g, w.side, f) * ((long long)w.nd * w.nbp), part, D);
+    for (int b = threadIdx.x; b < w.nbp; b += kWallThreads) {
+      const long long e = (g.face0[w.side] + f) * w.nbp + b;
+      if constexpr (sizeof(S) == 8) {
+        I0wall[e] = D[b];
+      } else {
+        I0wall[e] = w.I0ref[b] + D[b];
+        I0wall_dev[e] = (float)D[b];
+      }
+    }
+    __syncthreads();
   }
 }
 
-// Partially specular side: one CTA of kPartWarps warps per wall face.  The
-// diffuse value per band, D_b = sum_{out} |S_ax| I / sum_{in} |S_ax| of the
-// wall cell (warps over direction ranges, added in warp order), then for
-// every direction and band the ghost p I(mirror of d) + (1 - p) D_b, stored in
-// the storage type (a deviation from I0_b(T_ref) in the reduced modes).
-constexpr int kPartWarps = 8;
-
+// Partially specular side: for every direction that enters through it (or runs
+// along it) and every band, the ghost p I(mirror of d) + (1 - p) D_b, in the
+// storage type (a deviation from I0_b(T_ref) in the reduced modes).  Rows of
+// outgoing directions are never read and stay as they are.
 template <typename S>
-__global__ void __launch_bounds__(32 * kPartWarps) partial_ghost_kernel(const S* I, const double* I0ref,
-                                                                        const DevGeom* geoms, int geom, int side,
-                                                                        const double* Sd, const DirInfo* dirs, int nd,
-                                                                        int nbp, int nfaces, double p, S* out) {
-  extern __shared__ double part[];  // [kPartWarps][nbp] partial numerators, then D [nbp]
-  const DevGeom g = geoms[geom];
-  const int ax = side >> 1;
-  const bool high = side & 1;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const long long row = (long long)nd * nbp;
-  const int d0 = (int)((long long)wid * nd / kPartWarps), d1 = (int)((long long)(wid + 1) * nd / kPartWarps);
-  double den = 0.0;
-  for (int d = 0; d < nd; ++d) {
-    const double sd = Sd[3 * d + ax];
-    if (!(high ? sd > 0.0 : sd < 0.0) && sd != 0.0) den += fabs(sd);
-  }
-  for (int f = blockIdx.x; f < nfaces; f += gridDim.x) {
-    int i, j, k;  // wall cell of face f (x sides: j + ny k, y sides: i + nx k, z sides: i + nx j)
-    if (ax == 0) { i = high ? g.nx - 1 : 0; j = f % g.ny; k = f / g.ny; }
-    else if (ax == 1) { j = high ? g.ny - 1 : 0; i = f % g.nx; k = f / g.nx; }
-    else { k = high ? g.nz - 1 : 0; i = f % g.nx; j = f / g.nx; }
-    const long long P = g.cell0 + ((long long)k * g.ny + j) * g.nx + i;
-    for (int b = lane; b < nbp; b += 32) {
-      double num = 0.0;
-      for (int d = d0; d < d1; ++d) {
-        const double sd = Sd[3 * d + ax];
-        if (high ? sd > 0.0 : sd < 0.0) num = fma(fabs(sd), full_I(I, P * row + (long long)d * nbp + b, b, I0ref), num);
+__global__ void __launch_bounds__(kWallThreads) partial_ghost_kernel(WallArgs<S> w, const DirInfo* dirs, double p,
+                                                                     S* out) {
+  using T = Tr<S>;
+  constexpr int V = T::V;
+  extern __shared__ double part[];  // [groups][nbp], then D [nbp]
+  const int lpc = w.nbp / V, groups = kWallThreads / lpc;
+  const int grp = threadIdx.x / lpc, b0 = V * (threadIdx.x - grp * lpc);
+  const int ax = w.side >> 1;
+  double* D = part + groups * w.nbp;
+  const DevGeom g = w.geoms[w.geom];
+  const long long row = (long long)w.nd * w.nbp;
+  for (int f = blockIdx.x; f < w.nfaces; f += gridDim.x) {
+    const S* cell = w.I + wall_cell(g, w.side, f) * row;
+    wall_diffuse<S>(w, cell, part, D);
+    if (grp < groups) {
+      double q[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) q[v] = (1.0 - p) * D[b0 + v];
+#pragma unroll 4
+      for (int k = grp; k < w.nd - w.wd.nout; k += groups) {
+        const int d = w.wd.rest[k];
+        const int r = ax == 0 ? dirs[d].rx : (ax == 1 ? dirs[d].ry : dirs[d].rz);
+        typename T::A x[V];
+        T::ld(cell + (long long)r * w.nbp + b0, x);
+#pragma unroll
+        for (int v = 0; v < V; ++v) x[v] = (typename T::A)fma(p, (double)x[v], q[v]);
+        T::st(out + f * row + (long long)d * w.nbp + b0, x);
       }
-      part[wid * nbp + b] = num;
-    }
-    __syncthreads();
-    double* D = part + kPartWarps * nbp;
-    for (int b = threadIdx.x; b < nbp; b += blockDim.x) {
-      double num = 0.0;
-      for (int w = 0; w < kPartWarps; ++w) num += part[w * nbp + b];
-      D[b] = num / den;
-    }
-    __syncthreads();
-    for (long long e = threadIdx.x; e < row; e += blockDim.x) {
-      const int d = (int)(e / nbp), b = (int)(e - (long long)d * nbp);
-      const int r = ax == 0 ? dirs[d].rx : (ax == 1 ? dirs[d].ry : dirs[d].rz);
-      const double v = fma(p, full_I(I, P * row + (long long)r * nbp + b, b, I0ref), (1.0 - p) * D[b]);
-      if constexpr (sizeof(S) == 8) out[f * row + e] = v;
-      else if constexpr (sizeof(S) == 4) out[f * row + e] = (float)(v - I0ref[b]);
-      else out[f * row + e] = __double2bfloat16(v - I0ref[b]);
     }
     __syncthreads();
   }
@@ -700,37 +747,45 @@ cudaError_t launch_fixup(const SweepArgs& a, const MLPView* mlp, cudaStream_t s)
   return cudaGetLastError();
 }
 
+namespace {
+template <typename S>
+WallArgs<S> wall_args(const void* I, const double* I0ref, const DevGeom* geoms, int geom, int side, const double* Sd,
+                      const WallDirs& wd, int nd, int nbp, int nfaces) {
+  return WallArgs<S>{(const S*)I, I0ref, geoms, Sd, geom, side, nd, nbp, nfaces, wd};
+}
+template <typename S>
+size_t wall_smem(int nbp) {
+  return (size_t)(kWallThreads / (nbp / Tr<S>::V) + 1) * nbp * sizeof(double);
+}
+}  // namespace
+
 cudaError_t launch_diffuse_ghosts(int precision, const void* I, const double* I0ref, double* I0wall, float* I0wall_dev,
-                                  const DevGeom* geoms, int geom, int side, const double* S, int nd, int nbp,
-                                  int nfaces, cudaStream_t s) {
-  const int grid = (int)std::min<long long>((nfaces + 3) / 4, 152LL * 16);
-  if (precision == 0)
-    diffuse_ghost_kernel<double><<<grid, 128, 0, s>>>((const double*)I, I0ref, I0wall, nullptr, geoms, geom, side, S, nd,
-                                                      nbp, nfaces);
-  else if (precision == 1)
-    diffuse_ghost_kernel<float><<<grid, 128, 0, s>>>((const float*)I, I0ref, I0wall, I0wall_dev, geoms, geom, side, S, nd,
-                                                     nbp, nfaces);
-  else
-    diffuse_ghost_kernel<__nv_bfloat16><<<grid, 128, 0, s>>>((const __nv_bfloat16*)I, I0ref, I0wall, I0wall_dev, geoms,
-                                                             geom, side, S, nd, nbp, nfaces);
+                                  const DevGeom* geoms, int geom, int side, const double* Sd, const WallDirs& wd, int nd,
+                                  int nbp, int nfaces, cudaStream_t s) {
+  const int grid = (int)std::min<long long>(std::max(nfaces, 1), 152LL * 16);
+  auto go = [&](auto tag) {
+    using S = decltype(tag);
+    diffuse_ghost_kernel<S><<<grid, kWallThreads, wall_smem<S>(nbp), s>>>(
+        wall_args<S>(I, I0ref, geoms, geom, side, Sd, wd, nd, nbp, nfaces), I0wall, I0wall_dev);
+  };
+  if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 
 cudaError_t launch_partial_ghosts(int precision, const void* I, const double* I0ref, const DevGeom* geoms, int geom,
-                                  int side, const double* S, const DirInfo* dirs, int nd, int nbp, int nfaces,
-                                  double p, void* out, cudaStream_t s) {
+                                  int side, const double* Sd, const WallDirs& wd, const DirInfo* dirs, int nd, int nbp,
+                                  int nfaces, double p, void* out, cudaStream_t s) {
   const int grid = (int)std::min<long long>(std::max(nfaces, 1), 152LL * 16);
-  const size_t sm = (size_t)(kPartWarps + 1) * nbp * sizeof(double);
-  if (precision == 0)
-    partial_ghost_kernel<double><<<grid, 32 * kPartWarps, sm, s>>>((const double*)I, I0ref, geoms, geom, side, S, dirs,
-                                                                   nd, nbp, nfaces, p, (double*)out);
-  else if (precision == 1)
-    partial_ghost_kernel<float><<<grid, 32 * kPartWarps, sm, s>>>((const float*)I, I0ref, geoms, geom, side, S, dirs, nd,
-                                                                  nbp, nfaces, p, (float*)out);
-  else
-    partial_ghost_kernel<__nv_bfloat16><<<grid, 32 * kPartWarps, sm, s>>>((const __nv_bfloat16*)I, I0ref, geoms, geom,
-                                                                          side, S, dirs, nd, nbp, nfaces, p,
-                                                                          (__nv_bfloat16*)out);
+  auto go = [&](auto tag) {
+    using S = decltype(tag);
+    partial_ghost_kernel<S><<<grid, kWallThreads, wall_smem<S>(nbp), s>>>(
+        wall_args<S>(I, I0ref, geoms, geom, side, Sd, wd, nd, nbp, nfaces), dirs, p, (S*)out);
+  };
+  if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 
