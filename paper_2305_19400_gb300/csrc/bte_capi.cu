@@ -20,6 +20,7 @@
 #include "../../include/bte.h"
 #include "bte_internal.h"
 #include "bte_mlp.cuh"
+#include "bte_solve.cuh"
 #include "bte_tables.h"
 
 using namespace bte;
@@ -95,7 +96,7 @@ struct bte_ctx {
   float* dirc_ff = nullptr;   // [cls][nd][3][2]
   float* band_ff = nullptr;   // [2][nbp] 1/(v_b dt), beta_b/v_b pairs
   double *J = nullptr, *Teval = nullptr, *I0ref = nullptr, *scratch_pack = nullptr;
-  double* Msum = nullptr;     // [cell][3] the T_p model's sums sum_b a_p,b J_k,b
+  double* Msum = nullptr;     // [cell][4] the T_p model's sums sum_b a_p,b J_k,b
   double* I0ref_o = nullptr;  // I0_b(T_ref) of the stored bands (aliases I0ref unless a band range is set)
   double* Epart = nullptr;    // band-range handles: [ncells][2] partial (E_L, E_p) for the exchange
   float *I0wall_dev = nullptr, *wdir32 = nullptr, *vb32 = nullptr, *bb32 = nullptr;
@@ -202,9 +203,9 @@ size_t carve(bte_ctx* h, char* base) {
   const size_t ibytes = (size_t)h->ncells * row * elem_bytes(h->opts.precision);
   for (int i = 0; i < 3; ++i) h->Ibuf[i] = take(ibytes);
   h->I0cell = (double*)take((size_t)h->ncells * h->nbp * 8);
-  h->J = (double*)take((size_t)h->ncells * 3 * h->nbp_all * 8);
+  h->J = (double*)take((size_t)h->ncells * 4 * h->nbp_all * 8);
   h->Teval = (double*)take((size_t)h->ncells * 8);
-  h->Msum = (double*)take((size_t)h->ncells * 3 * 8);
+  h->Msum = (double*)take((size_t)h->ncells * 4 * 8);
   h->I0ref = (double*)take((size_t)h->nbp_all * 8);
   const bool ranged = h->nb != h->nb_all;
   h->I0ref_o = ranged ? (double*)take((size_t)h->nbp * 8) : h->I0ref;
@@ -545,7 +546,7 @@ int ensure_TL(bte_ctx* h) {
   if (h->TL_valid) return BTE_OK;
   // warm start from T_p (or the previous T_L when T_p is not solved)
   CUDA_TRY(h, launch_solve_TL(h->TL, h->EL, h->solve_tp ? h->Tp : h->TL, h->J, h->Teval, h->ncells, thermo(h),
-                              std::cbrt(h->opts.newton_rtol / 4.0), h->opts.newton_maxit, h->counters, h->stream));
+                              model_trust(h->opts.newton_rtol), h->opts.newton_maxit, h->counters, h->stream));
   h->TL_valid = true;
   return BTE_OK;
 }
@@ -603,7 +604,7 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.lpc = h->lpc;
   a.dteam = h->dteam;
   a.solve_tp = h->solve_tp ? 1 : 0;
-  a.trust_rel = std::cbrt(h->opts.newton_rtol / 4.0);
+  a.trust_rel = model_trust(h->opts.newton_rtol);
   a.maxit = h->opts.newton_maxit;
   a.counters = h->counters;
   a.dry = 0;
@@ -1490,8 +1491,8 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
     }
     CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, cudaMemcpyHostToDevice, s));
   }
-  CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 3 * h->nbp_all,
-                                   h->Msum + h->cell0[geom] * 3,
+  CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
+                                   h->Msum + h->cell0[geom] * 4,
                                    h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));
   if (h->Epart) {
     h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange
@@ -1694,7 +1695,7 @@ int bte_solve_T(bte_handle h, const double* Ep, const double* T0, int n, int lea
   if (e == cudaSuccess && T0) e = cudaMemcpyAsync(dT0, T0, (size_t)n * 8, cudaMemcpyHostToDevice, s);
   const MLPView m = mlp_view(h);
   if (e == cudaSuccess)
-    e = launch_solve_batch(thermo(h), dE, T0 ? dT0 : nullptr, n, std::cbrt(h->opts.newton_rtol / 4.0),
+    e = launch_solve_batch(thermo(h), dE, T0 ? dT0 : nullptr, n, model_trust(h->opts.newton_rtol),
                            h->opts.newton_maxit, learned ? &m : nullptr, dT, dev, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(T_out, dT, (size_t)n * 8, cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess && evals) e = cudaMemcpyAsync(evals, dev, (size_t)n * 4, cudaMemcpyDeviceToHost, s);

@@ -4,7 +4,7 @@
 //   I buffers      3 x [cell][dir][nbp]      storage type per precision mode
 //                                            (FP32/BF16 store I - I0_b(T_ref))
 //   I0cell         [cell][nbp]  double        I0_b(T_p) of every cell
-//   J, Teval       [cell][3][nbp], [cell]     cached quadrature model per cell
+//   J, Teval       [cell][4][nbp], [cell]     cached quadrature model per cell
 //   Tp, TL, EL     [cell]       double        temperatures, lattice energy
 //   I0wall         [wall face][nbp] double    Eq. 6 ghost for isothermal faces
 //   coef           [class][5][dir][nbp] double  sweep coefficients (A_n, A_x, A_y, A_z, A_s)
@@ -116,8 +116,8 @@ struct SweepArgs {
   double* I0cell;           // [cell][nbp] in: I0^k, out: I0^{k+1}
   double* Tp;               // [cell] in/out
   double* Teval;            // [cell] evaluation point of the cached quadrature model
-  double* J;                // [cell][3][nbp] I0, dI0/dT, d2I0/dT2 at Teval
-  double* Msum;             // [cell][3] sum_b a_p,b J_k,b: the T_p model's sums, kept with J
+  double* J;                // [cell][4][nbp] I0 and its first three derivatives at Teval
+  double* Msum;             // [cell][4] sum_b a_p,b J_k,b: the T_p model's sums, kept with J
   double* EL;               // [cell] out
   const double* I0wall;     // [face][nbp] FP64 ghosts
   const float* I0wall_dev;  // [face][nbp] FP32 ghosts minus I0ref (reduced modes)

@@ -70,24 +70,21 @@ __global__ void __cluster_dims__(kFixCluster, 1, 1) __launch_bounds__(kFixThread
       __syncthreads();
     }
     const double T0 = net ? t0_sm[0] : it.T0;
-    const SolveResult r = exact_solve_cluster(a.th, it.Ep, T0, a.trust_rel, a.maxit, a.J + (P * 3) * nbp, solve_sm, par);
+    const SolveResult r = exact_solve_cluster(a.th, it.Ep, T0, a.trust_rel, a.maxit, a.J + (P * 4) * nbp, solve_sm, par);
     evals += r.evals;
     fb += r.fallback;
     bad += r.bad;
     __syncthreads();  // this CTA's model rows, written by the solve, before its I0 refresh reads them
     // I0 refresh of the stored bands whose model rows this CTA wrote, at r.Te
-    const double hd2 = 0.5 * r.delta * r.delta;
     const int s0 = max(own0 - a.th.band0, 0), s1 = min(own1 - a.th.band0, a.th.nbo);
     for (int b = s0 + (int)threadIdx.x; b < s1; b += blockDim.x) {
-      const long long j = (P * 3) * nbp + a.th.band0 + b;
-      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? fma(a.J[j + 2 * nbp], hd2, fma(a.J[j + nbp], r.delta, a.J[j])) : 0.0;
+      const double* Jb = a.J + (P * 4) * nbp + a.th.band0 + b;
+      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? model_I0(Jb, nbp, r.delta) : 0.0;
     }
     if (rank == 0 && threadIdx.x == 0) {
       a.Teval[P] = r.Te;
       a.Tp[P] = r.Te + r.delta;
-      a.Msum[3 * P] = r.M[0];  // the model just written to J
-      a.Msum[3 * P + 1] = r.M[1];
-      a.Msum[3 * P + 2] = r.M[2];
+      for (int k = 0; k < 4; ++k) a.Msum[4 * P + k] = r.M[k];  // the model just written to J
     }
     __syncthreads();  // t0_sm and the solve scratch are reused by the next item
   }
@@ -106,28 +103,30 @@ __global__ void __cluster_dims__(kFixCluster, 1, 1) __launch_bounds__(kFixThread
 __device__ void cell_state_at(double* I0cell, double* J, double* Msum, long long P, double T, ThermoTables th,
                               double* row) {
   const double rT = 1.0 / T;
+  double* Jrow = J + (P * 4) * th.nbp;
   for (int b = threadIdx.x; b < th.nbp; b += blockDim.x) {  // every band (the temperature model)
-    double f, d1, d2;
-    band_I0_d2(th.node_c + b * th.ng, th.node_C + b * th.ng, th.ng, rT, f, d1, d2);
-    row[b] = f;
-    J[(P * 3 + 0) * th.nbp + b] = f;
-    J[(P * 3 + 1) * th.nbp + b] = d1;
-    J[(P * 3 + 2) * th.nbp + b] = d2;
+    double f[4];
+    band_I0_d3(th.node_c + b * th.ng, th.node_C + b * th.ng, th.ng, rT, f);
+    row[b] = f[0];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) Jrow[k * th.nbp + b] = f[k];
   }
   __syncthreads();
   for (int b = threadIdx.x; b < th.nbo; b += blockDim.x)  // stored bands
     I0cell[P * th.nbo + b] = b < th.nbr ? row[th.band0 + b] : 0.0;
-  if (threadIdx.x == 0) {  // the model's sums with the T_p weights
-    double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-    for (int b = 0; b < th.nbp; ++b) {
+  if (threadIdx.x < 32) {  // the model's sums with the T_p weights
+    double m[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < th.nbp; b += 32) {
       const double ap = th.a_p[b];
-      m0 = fma(ap, J[(P * 3 + 0) * th.nbp + b], m0);
-      m1 = fma(ap, J[(P * 3 + 1) * th.nbp + b], m1);
-      m2 = fma(ap, J[(P * 3 + 2) * th.nbp + b], m2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) m[k] = fma(ap, Jrow[k * th.nbp + b], m[k]);
     }
-    Msum[3 * P] = m0;
-    Msum[3 * P + 1] = m1;
-    Msum[3 * P + 2] = m2;
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
+    }
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 4; ++k) Msum[4 * P + k] = m[k];
   }
 }
 
@@ -191,7 +190,7 @@ __global__ void wall_dev_kernel(float* out, const double* I0wall, const double* 
 }
 
 // Lattice temperature: sum_b a_L,b I0_b(T) = E_L per cell (evaluated on
-// request).  One warp per cell: the root of the cell's cached quadratic model
+// request).  One warp per cell: the root of the cell's cached cubic model
 // of I0_b(T) around T_e (the one the T_p solve keeps) when it lies inside the
 // trust radius, else Halley on the exact band quadrature from there (or from
 // the guess), bisection as the fallback.
@@ -209,22 +208,18 @@ __global__ void solve_TL_kernel(double* TL, const double* EL, const double* Tgue
       }
       continue;
     }
-    double F = 0.0, F1 = 0.0, F2 = 0.0;
+    double F[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b = lane; b < nbp; b += 32) {
       const double w = th.a_L[b];
-      F = fma(w, J[(P * 3 + 0) * nbp + b], F);
-      F1 = fma(w, J[(P * 3 + 1) * nbp + b], F1);
-      F2 = fma(w, J[(P * 3 + 2) * nbp + b], F2);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) F[k] = fma(w, J[(P * 4 + k) * nbp + b], F[k]);
     }
     for (int o = 16; o > 0; o >>= 1) {
-      F += __shfl_xor_sync(0xffffffffu, F, o);
-      F1 += __shfl_xor_sync(0xffffffffu, F1, o);
-      F2 += __shfl_xor_sync(0xffffffffu, F2, o);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) F[k] += __shfl_xor_sync(0xffffffffu, F[k], o);
     }
-    F -= E;
     const double Te = Teval[P];
-    const double disc = F1 * F1 - 2.0 * F * F2;
-    const double delta = (disc >= 0.0 && F1 > 0.0) ? -2.0 * F / (F1 + sqrt(disc)) : -F / F1;
+    const double delta = model_step(F[0] - E, F[1], F[2], F[3]);
     const double Tn = Te + delta;
     if (isfinite(Tn) && fabs(delta) <= trust_rel * Tn) {
       if (lane == 0) TL[P] = Tn;
@@ -358,7 +353,7 @@ __global__ void energy_L_kernel(const S* I, const double* I0ref, double* EL, con
 }
 
 // T_p step of one cell from its energies (E_L, E_p over every band), by one
-// warp: the T_p equation on the cell's cached quadratic model of all bands,
+// warp: the T_p equation on the cell's cached cubic model of all bands,
 // I0 refresh of the stored bands inside the trust radius, the rest to the
 // fix-up list.
 __device__ void solve_cell_warp(const SweepArgs& a, long long P, double EL, double Ep, int lane,
@@ -373,11 +368,9 @@ __device__ void solve_cell_warp(const SweepArgs& a, long long P, double EL, doub
     return;
   }
   // the model's sums, kept with J (sum_b a_p,b J_k,b)
-  double F = a.Msum[3 * P] - Ep;
-  const double F1 = a.Msum[3 * P + 1], F2 = a.Msum[3 * P + 2];
+  const double* M = a.Msum + 4 * P;
   const double Te = a.Teval[P];
-  const double disc = F1 * F1 - 2.0 * F * F2;
-  const double delta = (disc >= 0.0 && F1 > 0.0) ? -2.0 * F / (F1 + sqrt(disc)) : -F / F1;
+  const double delta = model_step(M[0] - Ep, M[1], M[2], M[3]);
   const double Tn = Te + delta;
   const bool ok = finite && isfinite(Tn) && fabs(delta) <= a.trust_rel * Tn;
   if (lane == 0) {
@@ -397,10 +390,9 @@ __device__ void solve_cell_warp(const SweepArgs& a, long long P, double EL, doub
     if (ok) a.Tp[P] = Tn;
   }
   if (ok) {
-    const double hd2 = 0.5 * delta * delta;
     for (int b = lane; b < a.th.nbo; b += 32) {
-      const long long j = (P * 3) * nbp + a.th.band0 + b;
-      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? fma(a.J[j + 2 * nbp], hd2, fma(a.J[j + nbp], delta, a.J[j])) : 0.0;
+      const double* Jb = a.J + (P * 4) * nbp + a.th.band0 + b;
+      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? model_I0(Jb, nbp, delta) : 0.0;
     }
   }
 }

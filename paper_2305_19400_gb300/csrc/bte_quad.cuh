@@ -5,8 +5,8 @@
 namespace bte {
 
 // Band quadrature.  I0_b(T) = sum_i C_i / expm1(c_i / T) (Gauss-Legendre on the
-// band).  With n = 1/(e^x - 1), x = c/T:  dn/dT = n(1+n) x/T and
-// d2n/dT2 = n(1+n) (x/T^2) ((1+2n) x - 2).
+// band).  With n = 1/(e^x - 1), x = c/T, q = n(1+n) x and u = (1+2n) x - 2:
+// dn/dT = q/T, d2n/dT2 = q u/T^2, d3n/dT3 = q (u^2 - 2u - 2 + 2 q x)/T^3.
 __device__ __forceinline__ double band_I0(const double* __restrict__ c, const double* __restrict__ C, int ng,
                                           double rT) {
   double s = 0.0;
@@ -14,21 +14,31 @@ __device__ __forceinline__ double band_I0(const double* __restrict__ c, const do
   return s;
 }
 
-__device__ __forceinline__ void band_I0_d2(const double* __restrict__ c, const double* __restrict__ C, int ng,
-                                           double rT, double& f, double& d1, double& d2) {
-  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+// One node's terms: n, q, q u and q (u^2 - 2u - 2 + 2 q x).
+__device__ __forceinline__ void node_terms(double x, double (&t)[4]) {
+  const double n = 1.0 / expm1(x);
+  const double q = fma(n, n, n) * x;
+  const double u = fma(2.0 * n, x, x) - 2.0;
+  t[0] = n;
+  t[1] = q;
+  t[2] = q * u;
+  t[3] = q * fma(2.0 * q, x, fma(u, u - 2.0, -2.0));
+}
+
+// I0_b and its first three temperature derivatives.
+__device__ __forceinline__ void band_I0_d3(const double* __restrict__ c, const double* __restrict__ C, int ng,
+                                           double rT, double (&f)[4]) {
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
   for (int i = 0; i < ng; ++i) {
-    const double x = c[i] * rT;
-    const double n = 1.0 / expm1(x);
-    const double qx = fma(n, n, n) * x;
-    const double u = fma(2.0 * n, x, x) - 2.0;
-    s0 = fma(C[i], n, s0);
-    s1 = fma(C[i], qx, s1);
-    s2 = fma(C[i] * qx, u, s2);
+    double t[4];
+    node_terms(c[i] * rT, t);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) s[k] = fma(C[i], t[k], s[k]);
   }
-  f = s0;
-  d1 = s1 * rT;
-  d2 = s2 * rT * rT;
+  f[0] = s[0];
+  f[1] = s[1] * rT;
+  f[2] = s[2] * rT * rT;
+  f[3] = s[3] * rT * rT * rT;
 }
 
 }  // namespace bte

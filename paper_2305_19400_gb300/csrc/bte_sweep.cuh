@@ -21,8 +21,8 @@
 // modes: float partials flushed to FP64).  The epilogue of an item: the band
 // owners add the dteam partials per band in a fixed order and reduce their
 // bands to E_L, E_p and the model sums; then one warp per cell adds those with
-// a shuffle tree and solves the T_p equation on the cell's cached quadratic
-// model of I0_b(T) (I0, dI0/dT, d2I0/dT2 at its last exact evaluation point
+// a shuffle tree and solves the T_p equation on the cell's cached cubic model
+// of I0_b(T) (I0 and three derivatives at its last exact evaluation point
 // T_e).  The model root is accepted inside the trust radius
 // |T - T_e| <= trust_rel T, where the Taylor remainder is below the solve
 // tolerance, and the warp refreshes the cell's I0 from it; other cells go to
@@ -38,6 +38,7 @@
 #include <type_traits>
 
 #include "bte_ff.cuh"
+#include "bte_solve.cuh"
 #include "bte_store.cuh"
 
 namespace bte {
@@ -141,30 +142,6 @@ struct ItemCtx {
 // barriers): G[v] is this lane's partial G_b = sum_d w_d I_{d,b} over its
 // directions (in the reduced modes without the W I0_b(T_ref) term of their
 // deviation storage, which is added here).
-// Root nearest 0 of F + F1 d + F2 d^2 / 2, the step of the cell's cached
-// temperature model: an FP32 estimate from the stable form
-// -2F / (F1 + sqrt(F1^2 - 2 F F2)) (-F / F1 without a real root), then one
-// Newton step in FP64 with the FP32 reciprocal of the derivative.  The
-// estimate is good to about 1e-7 and the step to about 1e-14 of d (the FP32
-// rounding squared), while an accepted d is below 3e-5 T.  The FP64 pipe of
-// GB300 takes about 76 cycles per warp instruction: this form issues five
-// FP64 operations where a square root and a division take twenty-odd, and its
-// conversions run on the integer pipe (bte_ff.cuh).
-__device__ __forceinline__ double model_step(double F, double F1, double F2) {
-  float f, f1, f2, lo;
-  ff::split(F, f, lo);
-  ff::split(F1, f1, lo);
-  ff::split(F2, f2, lo);
-  const float disc = fmaf(f1, f1, -2.0f * f * f2);
-  const float d0f = (disc >= 0.0f && f1 > 0.0f) ? -2.0f * f / (f1 + sqrtf(disc)) : -f / f1;
-  const double d0 = ff::to_double(d0f, 0.0f);
-  const double q = fma(fma(0.5 * F2, d0, F1), d0, F);
-  float qp;
-  ff::split(fma(F2, d0, F1), qp, lo);
-  const double r = ff::to_double(1.0f / qp, 0.0f);
-  return fma(-q, r, d0);
-}
-
 template <int V, bool kDev>
 __device__ __forceinline__ void item_epilogue(const SweepArgs& a, const ItemCtx& x, const WorkItem& wi,
                                               const DevGeom* gp, const double (&G)[V], unsigned long long& cnt_solves,
@@ -238,11 +215,11 @@ __device__ __forceinline__ void item_epilogue(const SweepArgs& a, const ItemCtx&
           atomicAdd(&cnt_bad, 1ULL);
         } else if (a.solve_tp) {
           atomicAdd(&cnt_solves, 1ULL);
-          // root of (F - E_p) + F1 d + F2 d^2 / 2 nearest 0; F, F1, F2: the model's
-          // sums sum_b a_p,b J_k,b, kept with J
-          const double Fs = a.Msum[3 * Pc] - Ep, F1s = a.Msum[3 * Pc + 1], F2s = a.Msum[3 * Pc + 2];
+          // root of (F - E_p) + F1 d + F2 d^2 / 2 + F3 d^3 / 6 nearest 0; F .. F3: the
+          // model's sums sum_b a_p,b J_k,b, kept with J
+          const double* M = a.Msum + 4 * Pc;
           const double Te = a.Teval[Pc];
-          const double delta = model_step(Fs, F1s, F2s);
+          const double delta = model_step(M[0] - Ep, M[1], M[2], M[3]);
           const double Tn = Te + delta;
           if (isfinite(Tn) && fabs(delta) <= a.trust_rel * Tn) {
             if (!a.dry) {
@@ -272,9 +249,8 @@ __device__ __forceinline__ void item_epilogue(const SweepArgs& a, const ItemCtx&
     const int cs = e / x.nbp, b = e - cs * x.nbp;
     if (cst[4 * cs + 3] == 0.0) continue;
     const long long Pc = gp->cell0 + wi.cell_begin + cs;
-    const double delta = cst[4 * cs + 2], hd2 = 0.5 * delta * delta;
-    const long long j = (Pc * 3) * x.nbp_all + x.band0 + b;
-    a.I0cell[Pc * x.nbp + b] = b < x.nbr ? fma(a.J[j + 2 * x.nbp_all], hd2, fma(a.J[j + x.nbp_all], delta, a.J[j])) : 0.0;
+    const double* Jb = a.J + (Pc * 4) * x.nbp_all + x.band0 + b;
+    a.I0cell[Pc * x.nbp + b] = b < x.nbr ? model_I0(Jb, x.nbp_all, cst[4 * cs + 2]) : 0.0;
   }
   }
 

@@ -28,6 +28,7 @@
 
 #include "../../include/bte_umesh.h"
 #include "bte_internal.h"
+#include "bte_solve.cuh"
 #include "bte_store.cuh"
 #include "bte_tables.h"
 
@@ -461,7 +462,7 @@ struct bte_umesh_ctx {
   double* I[3] = {nullptr, nullptr, nullptr};
   int cur = 0;
   double *I0cell = nullptr, *J = nullptr, *Teval = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr;
-  double* Msum = nullptr;  // [cell][3] the T_p model's sums, kept with J
+  double* Msum = nullptr;  // [cell][4] the T_p model's sums, kept with J
   double *ghost = nullptr, *g = nullptr, *gout = nullptr, *S_d = nullptr, *w_d = nullptr, *nA_d = nullptr;
   double *vb_d = nullptr, *bb_d = nullptr, *bfT_d = nullptr, *scratch = nullptr, *Qb = nullptr, *qbuf = nullptr;
   double* bf_spec_d = nullptr;  // [bface] specularity of partially specular faces, 0 elsewhere
@@ -547,7 +548,7 @@ SweepArgs cell_args(bte_umesh_ctx* u, double* Inew) {
   a.wdir = u->w_d;
   a.nd = u->nd;
   a.solve_tp = u->solve_tp ? 1 : 0;
-  a.trust_rel = std::cbrt(u->opts.newton_rtol / 4.0);
+  a.trust_rel = model_trust(u->opts.newton_rtol);
   a.maxit = u->opts.newton_maxit;
   a.counters = u->counters;
   a.fix = u->fix;
@@ -578,7 +579,7 @@ int ensure_mem(bte_umesh_ctx* u) {
   }
   if ((rc = dalloc(u, &u->I0ref, nbp)) || (rc = dalloc(u, &u->ghost_dev, nbf * nbp)) || (rc = dalloc(u, &u->w32_d, nd)))
     return rc;
-  if ((rc = dalloc(u, &u->I0cell, nc * nbp)) || (rc = dalloc(u, &u->J, nc * 3 * nbp)) || (rc = dalloc(u, &u->Msum, nc * 3)) ||
+  if ((rc = dalloc(u, &u->I0cell, nc * nbp)) || (rc = dalloc(u, &u->J, nc * 4 * nbp)) || (rc = dalloc(u, &u->Msum, nc * 4)) ||
       (rc = dalloc(u, &u->Teval, nc)) || (rc = dalloc(u, &u->Tp, nc)) || (rc = dalloc(u, &u->TL, nc)) ||
       (rc = dalloc(u, &u->EL, nc)) || (rc = dalloc(u, &u->ghost, nbf * nbp)) || (rc = dalloc(u, &u->bfT_d, nbf)) ||
       (rc = dalloc(u, &u->S_d, nd * 3)) || (rc = dalloc(u, &u->w_d, nd)) || (rc = dalloc(u, &u->nA_d, u->nf * 3)) ||
@@ -739,7 +740,7 @@ cudaError_t refresh_diffuse(bte_umesh_ctx* u, const void* I) {
 int ensure_TL(bte_umesh_ctx* u) {
   if (u->TL_valid) return BTE_OK;
   UTRY(u, launch_solve_TL(u->TL, u->EL, u->solve_tp ? u->Tp : u->TL, u->J, u->Teval, u->nc, uthermo(u),
-                          std::cbrt(u->opts.newton_rtol / 4.0), u->opts.newton_maxit, u->counters, u->stream));
+                          model_trust(u->opts.newton_rtol), u->opts.newton_maxit, u->counters, u->stream));
   u->TL_valid = true;
   return BTE_OK;
 }
