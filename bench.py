@@ -54,7 +54,7 @@ METRIC = "cell·dir·band updates/s and % HBM roofline at stated max|ΔT| vs FP6
 UNIT = "updates/s"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "sweep_traffic.json")
-KERNEL_SRCS = [os.path.join(ROOT, "paper_2305_19400_gb300", "csrc", f) for f in ("bte_sweep_ff.cuh", "bte_ff.cuh", "bte_sweep.cuh", "bte_store.cuh")]
+KERNEL_SRCS = [os.path.join(ROOT, "paper_2305_19400_gb300", "csrc", f) for f in ("bte_rows.cuh", "bte_ff.cuh", "bte_store.cuh")]
 # Algorithmic bytes of one implicit update: I^n (or B) read, I^k read once, I^{k+1} written.
 BYTES_PER_UPDATE_FP64 = 24
 # Work of the dominant kernel (the double-float sweep of inner iterations 2..n-1,

@@ -42,6 +42,7 @@ struct bte_ctx {
   int nd = 0;
   std::vector<double> S, w;
   std::vector<int> refl;
+  std::vector<int> perm;       // the caller's index of every internal direction
   double Wtot = 0.0;
   // bands
   int nb = 0, nbp = 0, ng = 16;           // bands stored by this handle (padded: nbp)
@@ -62,11 +63,12 @@ struct bte_ctx {
   std::vector<bool> init_set;
   bool TL_valid = false;
   // launch shape
-  int lpc = 0, dteam = 1, cpb = 0, threads = 0, grid = 0, pd = 1;
+  int lpc = 0, dteam = 1, cpb = 0, threads = 0, grid = 0, pd = 1;  // grid 0 (FP64, FP32): the resident CTAs
+  int dir_group = 8;                                               // rows per block of the internal order
   // CUDA graphs of one time step, keyed by (scheme, ninner, starting buffer)
   struct GraphEntry {
     int scheme, ninner, cur_in, cur_out;
-    bool ff_in;  // the step starts from ff pairs
+    bool ff_in;  // the state holds ff pairs
     cudaGraphExec_t exec;
   };
   std::vector<GraphEntry> graphs;
@@ -102,7 +104,8 @@ struct bte_ctx {
   float *I0wall_dev = nullptr, *wdir32 = nullptr, *vb32 = nullptr, *bb32 = nullptr;
   float4* dirc = nullptr;
   FixItem* fix = nullptr;
-  unsigned* fix_count = nullptr;
+  double* Gc = nullptr;       // [cell][team][nbp] band sums of the sweeps
+  void* I0wall_ff = nullptr;  // FP64: [face][nbp] isothermal ghosts as ff pairs
   // learned guess: parameters of nets A and B, Adam state, normalisation
   float *mlp_p = nullptr, *mlp_g = nullptr, *mlp_m = nullptr, *mlp_v = nullptr;
   double *mlp_rlo = nullptr, *mlp_rhi = nullptr, *mlp_elohi = nullptr;
@@ -110,10 +113,11 @@ struct bte_ctx {
   double mlp_Tlo = 0.0, mlp_Thi = 0.0, mlp_Elo = 0.0, mlp_Ehi = 0.0;
   long long pack_cells = 0;
   double *wdir = nullptr, *Sdev = nullptr, *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr;
-  double *inv_v = nullptr, *beta_d = nullptr, *scratch_faces = nullptr, *scratch_T = nullptr, *scratch_out = nullptr;
+  double *inv_v = nullptr, *beta_d = nullptr, *binv_d = nullptr, *scratch_faces = nullptr, *scratch_T = nullptr, *scratch_out = nullptr;
   double* scratch_q = nullptr;
   std::vector<DevGeom> dgeoms;
   DirInfo* dirs_d = nullptr;
+  int* perm_d = nullptr;
   int* wall_dirs_d = nullptr;   // [6][nd] per side: leaving directions, then the rest
   std::array<WallDirs, 6> wall_dirs{};
   DevGeom* geoms_d = nullptr;
@@ -121,7 +125,8 @@ struct bte_ctx {
   DevCounters* counters = nullptr;
   GsUnit* gs_units_d = nullptr;
   int* gs_dirs_d = nullptr;
-  double* bscale = nullptr;  // [cell] beta_b(T_p)/beta_b for the sweep-ordered pass
+  double* bscale = nullptr;  // [cell] beta_b(T_p)/beta_b, kept current by cells_kernel once valid
+  bool bscale_valid = false;
   // coefficient cache
   double coef_dt = -1.0;
   int coef_scheme = -1;
@@ -173,6 +178,7 @@ ThermoTables thermo(const bte_ctx* h) {
   t.a_L = h->a_L;
   t.inv_v = h->inv_v;
   t.beta = h->beta_d;
+  t.binv_v = h->binv_d;
   t.ng = h->ng;
   t.nbp = h->nbp_all;
   t.nb = h->nb_all;
@@ -189,6 +195,14 @@ ThermoTables thermo_all(const bte_ctx* h) {
   t.nbr = h->nb_all;
   t.band0 = 0;
   return t;
+}
+
+// Teams a cell of the FP64 and FP32 sweeps may have (bte_rows.cuh): one on in-plane
+// sets, two (FP32 also four) on polar x azimuthal ones; the BF16 sweep adds its
+// teams' sums itself.
+int max_teams(const bte_ctx* h) {
+  if (h->opts.precision == BTE_BF16 || h->dir_group == 4) return 1;
+  return h->opts.precision == BTE_FP64 ? 2 : 4;
 }
 
 // Workspace layout; with base == nullptr only the size is computed.
@@ -223,8 +237,9 @@ size_t carve(bte_ctx* h, char* base) {
   h->dirc = (float4*)take((size_t)h->cls_key.size() * h->nd * sizeof(float4));
   h->vb32 = (float*)take((size_t)h->nbp * 4);
   h->bb32 = (float*)take((size_t)h->nbp * 4);
-  h->fix = (FixItem*)take((size_t)std::max<long long>(h->ncells, 1) * sizeof(FixItem));
-  h->fix_count = (unsigned*)take(16);
+  h->fix = (FixItem*)take((size_t)cells_queue_entries(h->ncells) * sizeof(FixItem));
+  h->Gc = (double*)take((size_t)std::max(h->ncells, 1LL) * max_teams(h) * h->nbp * 8);
+  h->I0wall_ff = h->opts.precision == BTE_FP64 ? take((size_t)std::max(h->nfaces, 1LL) * h->nbp * 8) : nullptr;
   const size_t np = (size_t)mlp_param_total(h->nb_all);
   h->mlp_p = (float*)take(np * 4);
   h->mlp_g = (float*)take(np * 4);
@@ -237,25 +252,26 @@ size_t carve(bte_ctx* h, char* base) {
   h->Sdev = (double*)take((size_t)h->nd * 3 * 8);
   h->dirs_d = (DirInfo*)take((size_t)h->nd * sizeof(DirInfo));
   h->wall_dirs_d = (int*)take((size_t)h->nd * 6 * 4);
+  h->perm_d = (int*)take((size_t)h->nd * 4);
   h->node_c = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->node_C = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->a_p = (double*)take((size_t)h->nbp_all * 8);
   h->a_L = (double*)take((size_t)h->nbp_all * 8);
   h->inv_v = (double*)take((size_t)h->nbp * 8);   // stored bands
   h->beta_d = (double*)take((size_t)h->nbp * 8);
+  h->binv_d = (double*)take((size_t)h->nbp * 8);
   h->geoms_d = (DevGeom*)take(h->geoms.size() * sizeof(DevGeom));
   h->items_d = (WorkItem*)take((size_t)std::max<long long>(h->ncells, 1) * sizeof(WorkItem));  // room for 1 cell per item
   h->counters = (DevCounters*)take(sizeof(DevCounters));
   h->gs_units_d = (GsUnit*)take(std::max<size_t>(h->geoms.size() * h->nd, 1) * sizeof(GsUnit));
   h->gs_dirs_d = (int*)take((size_t)h->nd * 4);
   h->bscale = (double*)take((size_t)std::max(h->ncells, 1LL) * 8);
-  h->scratch_faces = (double*)take((size_t)std::max(h->max_side_faces, 1) * 8);
+  h->scratch_faces = (double*)take((size_t)std::max(h->max_side_faces, 1) * 6 * 8);
   h->scratch_T = (double*)take((size_t)std::max(h->max_side_faces, h->max_geom_cells) * 8);
   h->scratch_out = (double*)take(64);
   h->scratch_q = (double*)take((size_t)std::max(h->max_geom_cells, 1) * 3 * 8);
-  // host <-> FP64 staging of whole cell rows for the reduced-precision modes (64 MB at most)
-  h->pack_cells = h->opts.precision == BTE_FP64 ? 0
-                : std::max(1LL, std::min<long long>(h->max_geom_cells, (64LL << 20) / ((long long)h->nd * h->nb * 8)));
+  // host <-> device staging of whole cell rows in the caller's order (64 MB at most)
+  h->pack_cells = std::max(1LL, std::min<long long>(h->max_geom_cells, (64LL << 20) / ((long long)h->nd * h->nb * 8)));
   h->scratch_pack = (double*)take((size_t)h->pack_cells * h->nd * h->nb * 8);
   return off;
 }
@@ -270,17 +286,20 @@ size_t carve(bte_ctx* h, char* base) {
 constexpr int kStrip2D = 64;
 void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
   h->lpc = h->nbp / values_per_lane(h->opts.precision);  // one vector of bands per lane
-  // a cell team covers dteam directions per step: ~896 contiguous bytes of a row,
-  // but at least ~32 steps per lane, so the per-cell epilogue stays a small share
-  // when there are few directions
   const int rowb = h->nbp * (int)elem_bytes(h->opts.precision);
-  h->dteam = dteam > 0 ? dteam : std::max(1, std::min(std::min(896 / rowb, 256 / h->lpc), h->nd / 32));
+  if (dteam > 0) h->dteam = dteam;
+  else if (h->opts.precision == BTE_BF16)  // ~896 contiguous bytes of a row, at least ~32 steps per lane
+    h->dteam = std::max(1, std::min(std::min(896 / rowb, 256 / h->lpc), h->nd / 32));
+  else
+    h->dteam = h->dir_group == 4 ? 1 : 2;
   const int team = h->lpc * h->dteam;
   // default: the most cells whose CTA (at most 256 threads) is whole warps, else
-  // the most that fit
+  // the most that fit; small grids take fewer, so that every SM has two CTAs
   const int whole = 32 / std::gcd(team, 32);
   const int cpb_whole = (256 / team) / whole * whole;
   h->cpb = cpb > 0 ? cpb : (cpb_whole > 0 ? cpb_whole : std::max(1, 256 / team));
+  if (cpb <= 0 && h->opts.precision != BTE_BF16)
+    while (h->cpb > whole && h->ncells < 2LL * 152 * h->cpb) h->cpb -= whole;
   h->threads = h->cpb * team;
   h->items.clear();
   for (size_t gi = 0; gi < h->geoms.size(); ++gi) {
@@ -290,7 +309,7 @@ void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
       for (int i0 = 0; i0 < g.nx; i0 += bx)
         for (int j = 0; j < g.ny; ++j)
           for (int i = i0; i < std::min(g.nx, i0 + bx); i += h->cpb)
-            h->items.push_back(WorkItem{(int)gi, j * g.nx + i, std::min(h->cpb, std::min(g.nx, i0 + bx) - i), 0});
+            h->items.push_back(WorkItem{(int)gi, j * g.nx + i, std::min(h->cpb, std::min(g.nx, i0 + bx) - i), i, j, 0});
       continue;
     }
     // blocks of bx x by = 256 cells (bx a multiple of cpb, near square): the z
@@ -301,9 +320,10 @@ void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
         for (int k = 0; k < g.nz; ++k)
           for (int j = j0; j < std::min(g.ny, j0 + by); ++j)
             for (int i = i0; i < std::min(g.nx, i0 + bx); i += h->cpb)
-              h->items.push_back(WorkItem{(int)gi, (k * g.ny + j) * g.nx + i, std::min(h->cpb, std::min(g.nx, i0 + bx) - i), 0});
+              h->items.push_back(
+                  WorkItem{(int)gi, (k * g.ny + j) * g.nx + i, std::min(h->cpb, std::min(g.nx, i0 + bx) - i), i, j, k});
   }
-  h->grid = (int)std::min<size_t>(h->items.size(), 65535);
+  h->grid = h->opts.precision == BTE_BF16 ? (int)std::min<size_t>(h->items.size(), 65535) : 0;
 }
 
 // Sweep-ordered pass.  Directions whose upwind sides agree (one octant) share
@@ -397,6 +417,7 @@ int ensure_memory(bte_ctx* h) {
     std::reverse(l + wd.nout, l + h->nd);
     wd.rest = wd.out + wd.nout;
   }
+  CUDA_TRY(h, cudaMemcpyAsync(h->perm_d, h->perm.data(), h->perm.size() * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->wall_dirs_d, wl.data(), wl.size() * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->wdir, h->w.data(), h->nd * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->Sdev, h->S.data(), h->nd * 3 * 8, cudaMemcpyHostToDevice, s));
@@ -409,8 +430,13 @@ int ensure_memory(bte_ctx* h) {
   CUDA_TRY(h, cudaMemcpyAsync(h->a_p, ap.data(), ap.size() * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->a_L, aL.data(), aL.size() * 8, cudaMemcpyHostToDevice, s));
   {
-    std::vector<double> iv_o(h->nbp, 0.0), be_o(h->nbp, 0.0);  // stored bands, zero on padding
-    for (int b = 0; b < h->nb; ++b) { iv_o[b] = iv[h->band0 + b]; be_o[b] = be[h->band0 + b]; }
+    std::vector<double> iv_o(h->nbp, 0.0), be_o(h->nbp, 0.0), bi_o(h->nbp, 0.0);  // stored bands, zero on padding
+    for (int b = 0; b < h->nb; ++b) {
+      iv_o[b] = iv[h->band0 + b];
+      be_o[b] = be[h->band0 + b];
+      bi_o[b] = be_o[b] * iv_o[b];
+    }
+    CUDA_TRY(h, cudaMemcpyAsync(h->binv_d, bi_o.data(), bi_o.size() * 8, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->inv_v, iv_o.data(), iv_o.size() * 8, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->beta_d, be_o.data(), be_o.size() * 8, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
@@ -420,7 +446,6 @@ int ensure_memory(bte_ctx* h) {
     for (int b = 0; b < h->nb; ++b) { v32[b] = (float)h->vg[h->band0 + b]; b32[b] = (float)h->beta[h->band0 + b]; }
     CUDA_TRY(h, cudaMemcpyAsync(h->vb32, v32.data(), v32.size() * 4, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->bb32, b32.data(), b32.size() * 4, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(h, cudaMemsetAsync(h->fix_count, 0, 16, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
   }
   {
@@ -586,6 +611,7 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.EL = h->EL;
   a.I0wall = h->I0wall;
   a.I0wall_dev = h->I0wall_dev;
+  a.I0wall_ff = h->I0wall_ff;
   a.I0ref = h->I0ref_o;
   a.Epart = h->exchange_buf ? h->exchange_buf : h->Epart;
   a.partial = h->Epart ? 1 : 0;
@@ -603,11 +629,12 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.nd = h->nd;
   a.lpc = h->lpc;
   a.dteam = h->dteam;
+  a.dir_group = h->dir_group;
+  a.gsplit = h->opts.precision == BTE_BF16 ? 1 : h->dteam;
   a.solve_tp = h->solve_tp ? 1 : 0;
   a.trust_rel = model_trust(h->opts.newton_rtol);
   a.maxit = h->opts.newton_maxit;
   a.counters = h->counters;
-  a.dry = 0;
   a.explicit_scheme = h->coef_scheme == BTE_EXPLICIT ? 1 : 0;
   a.beta_exp = h->opts.beta_T_exp;
   a.beta_Tref = h->opts.T_ref;
@@ -617,7 +644,7 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.vb32 = h->vb32;
   a.bb32 = h->bb32;
   a.fix = h->fix;
-  a.fix_count = h->fix_count;
+  a.Gc = h->Gc;
   a.gs_units = h->gs_units_d;
   a.gs_dirs = h->gs_dirs_d;
   a.gs_nunits = (int)h->gs_units.size();
@@ -674,11 +701,19 @@ bool ff_sweep(const bte_ctx* h) {
   return true;
 }
 
-// The current intensity buffer as doubles (in place) when it holds ff pairs.
+// The current intensity buffer in the form the next step or call takes (in place):
+// doubles, or ff pairs for the double-float sweep.
 cudaError_t ensure_state_doubles(bte_ctx* h) {
   if (!h->state_ff) return cudaSuccess;
   const cudaError_t e = launch_ff_to_doubles(h->Ibuf[h->cur], (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
   if (e == cudaSuccess) h->state_ff = false;
+  return e;
+}
+cudaError_t ensure_state_ff(bte_ctx* h) {
+  if (h->state_ff) return cudaSuccess;
+  const cudaError_t e =
+      launch_doubles_to_ff(h->Ibuf[h->cur], h->Ibuf[h->cur], (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
+  if (e == cudaSuccess) h->state_ff = true;
   return e;
 }
 
@@ -695,27 +730,24 @@ cudaError_t record_timing_event(cudaEvent_t ev, cudaStream_t s) {
 // One time step: ninner sweeps rotating the three intensity buffers from *cur.
 // scheme BTE_IMPLICIT_GS runs the sweep-ordered pass and the per-cell step as
 // two kernels in place of the fused Jacobi sweep.
-cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaStream_t s, int* cur, bool* state_ff) {
+cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaStream_t s, int* cur) {
   int dim = 2;
   for (auto& g : h->geoms) dim = std::max(dim, g.dim);
   const int n = *cur;
   int k = n;
-  // FP64 implicit steps keep B = A_n I^n, the same in every inner iteration, in
-  // the third buffer: iteration 0 reads I^n and writes I^1 and B; iteration k
+  // double-float Jacobi sweeps read I^n in every inner iteration; FP64 implicit
+  // steps in IEEE arithmetic keep B = A_n I^n, the same in every inner iteration,
+  // in the third buffer: iteration 0 reads I^n and writes I^1 and B; iteration k
   // reads B and I^k and overwrites the buffer I^n (or I^{k-2}) was in.
-  const bool use_b = h->opts.precision == BTE_FP64 && !a.explicit_scheme && ninner >= 2 && !a.dry;
-  // double-float Jacobi sweeps: every iterate and B as ff pairs; the first
-  // inner iteration reads I^n in the state's format (a step of one inner
-  // iteration forms B without storing it)
-  const bool use_ff = h->opts.precision == BTE_FP64 && !a.explicit_scheme && !a.dry &&
-                      scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h);
-  if (*state_ff && !use_ff) return cudaErrorInvalidValue;  // the caller converts the state first
+  const bool use_ff = h->state_ff;  // bte_step has put the state in the form of this scheme
+  const bool use_b = h->opts.precision == BTE_FP64 && !use_ff && !a.explicit_scheme && ninner >= 2;
+  a.ff = use_ff ? 1 : 0;
+  if (scheme == BTE_IMPLICIT_GS) a.gsplit = 1;
   int z = -1;
   for (int it = 0; it < ninner; ++it) {
     int o = 0;
     a.bmode = 0;
     a.Bout = nullptr;
-    a.ff = use_ff ? (it == 0 && !*state_ff ? 2 : 3) : 0;
     if (use_b && it == 0) {
       while (o == n) ++o;
       z = 0;
@@ -733,8 +765,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
     }
     a.Ik = h->Ibuf[k];
     a.Iout = h->Ibuf[o];
-    cudaError_t e = cudaMemsetAsync(h->fix_count, 0, sizeof(unsigned), s);
-    if (e == cudaSuccess) e = refresh_diffuse(h, a.Ik, s);
+    cudaError_t e = refresh_diffuse(h, a.Ik, s);
     if (e == cudaSuccess) e = refresh_partial(h, a.Ik, s);
     const bool timed = h->time_sweeps && 2 * it + 1 < (int)h->tev.size();
     if (e == cudaSuccess && timed) e = record_timing_event(h->tev[2 * it], s);
@@ -750,26 +781,22 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
     if (e == cudaSuccess && a.partial) {
       // band-range handle: the caller sums the per-cell (E_L, E_p) partials over
       // the ranks that hold the other bands, then every rank solves every cell
+      e = launch_cells(a, h->ncells, 1, nullptr, s);
+      if (e != cudaSuccess) return e;
       const int xr = h->exchange(a.Epart, 2 * h->ncells, (void*)s, h->exchange_user);
       if (xr != 0) {
         h->exchange_rc = xr;
         return cudaErrorUnknown;
       }
-      e = launch_solve_cells(a, h->ncells, s);
     }
-    if (e == cudaSuccess && h->solve_tp) {
-      if (h->opts.learned) {
-        const MLPView m = mlp_view(h);
-        e = launch_fixup(a, &m, s);
-      } else {
-        e = launch_fixup(a, nullptr, s);
-      }
+    if (e == cudaSuccess) {
+      const MLPView m = mlp_view(h);
+      e = launch_cells(a, h->ncells, a.partial ? 2 : 0, h->opts.learned ? &m : nullptr, s);
     }
     if (e != cudaSuccess) return e;
     k = o;
   }
   *cur = k;
-  if (use_ff) *state_ff = true;
   return cudaSuccess;
 }
 
@@ -798,12 +825,9 @@ int flux_view(bte_ctx* h, int geom, FluxView* out) {
   if (rc) return rc;
   if (!h->mem_ready || !h->init_set[geom]) return fail(h, BTE_E_STATE, "geometry %d has no state", geom);
   const bte_geom& g = h->geoms[geom];
-  {
-    const cudaError_t e = ensure_state_doubles(h);
-    if (e != cudaSuccess) return fail(h, BTE_E_CUDA, "state conversion: %s", cudaGetErrorString(e));
-  }
   out->precision = h->opts.precision;
-  out->I = (const double*)h->Ibuf[h->cur];
+  out->I = h->Ibuf[h->cur];
+  out->state_ff = h->state_ff;
   {  // diffuse and partially specular wall ghosts of the current state (kernel launches, no allocation)
     cudaError_t e = refresh_diffuse(h, h->Ibuf[h->cur], h->stream);
     if (e == cudaSuccess) e = refresh_partial(h, h->Ibuf[h->cur], h->stream);
@@ -898,6 +922,8 @@ int bte_init_mesh(bte_handle* out, int n_geom, const bte_geom* geoms, const bte_
     delete h;
     return fail(nullptr, BTE_E_ARG, "bad direction set (in-plane needs n %% 4 == 0; polar x azimuthal needs even n_polar and n_azim %% 4 == 0)");
   }
+  h->dir_group = o.dir_kind == BTE_DIRS_INPLANE ? 4 : 8;
+  h->perm = internal_order(h->S, h->w, h->refl, h->dir_group);
   h->nd = (int)h->w.size();
   if (h->nd > 2048) {  // the sweep keeps the direction table in shared memory
     delete h;
@@ -1039,7 +1065,11 @@ int bte_set_bc(bte_handle h, int geom, int side, int type, const double* T_faces
   if (type == BTE_BC_ISOTHERMAL) {
     CUDA_TRY(h, cudaMemcpyAsync(h->scratch_T, T.data(), nf * 8, cudaMemcpyHostToDevice, h->stream));
     CUDA_TRY(h, launch_wall_I0(h->I0wall + h->face0[geom * 6 + side] * h->nbp, h->scratch_T, nf, thermo(h), h->stream));
-    if (h->opts.precision != BTE_FP64)
+    if (h->opts.precision == BTE_FP64)
+      CUDA_TRY(h, launch_doubles_to_ff(h->I0wall + h->face0[geom * 6 + side] * h->nbp,
+                                       (char*)h->I0wall_ff + h->face0[geom * 6 + side] * h->nbp * 8, nf * h->nbp / 2,
+                                       h->stream));
+    else
       CUDA_TRY(h, launch_wall_dev(h->I0wall_dev + h->face0[geom * 6 + side] * h->nbp,
                                   h->I0wall + h->face0[geom * 6 + side] * h->nbp, h->I0ref_o, nf, h->nbp,
                                   h->stream));
@@ -1084,12 +1114,16 @@ int bte_set_initial(bte_handle h, int geom, const double* T_cells, double T_unif
   for (double t : T)
     if (!(t >= kTmin && t <= kTmax)) return fail(h, BTE_E_ARG, "initial temperature %g outside [1, 5000] K", t);
   if ((rc = ensure_memory(h))) return rc;
-  CUDA_TRY(h, ensure_state_doubles(h));  // the other geometries keep their state
+  // the state starts in the form of the handle's default sweep; geometries set
+  // later follow the form it has by then
+  if (std::none_of(h->init_set.begin(), h->init_set.end(), [](bool x) { return x; }))
+    h->state_ff = h->opts.precision == BTE_FP64 && !h->opts.fp64_strict && h->opts.beta_T_exp == 0.0;
   CUDA_TRY(h, cudaMemcpyAsync(h->scratch_T, T.data(), nc * 8, cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->Tp, h->Teval, h->TL, h->EL,
+  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->state_ff, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->Tp, h->Teval, h->TL, h->EL,
                                 h->scratch_T, h->I0ref_o, h->cell0[geom], (int)nc, h->nd, thermo(h), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->init_set[geom] = true;
+  h->bscale_valid = false;
   h->TL_valid = false;  // T_L is recomputed from E_L on request
   return BTE_OK;
 }
@@ -1122,7 +1156,11 @@ int bte_step(bte_handle h, double dt, int nsteps, int ninner, int scheme, bte_st
   if (ranged && !h->exchange) return fail(h, BTE_E_STATE, "a band-range handle needs bte_set_exchange before stepping");
   h->exchange_rc = 0;
   const bool ff_step = h->opts.precision == BTE_FP64 && scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h);
-  if (!ff_step && nsteps > 0) CUDA_TRY(h, ensure_state_doubles(h));
+  if (nsteps > 0) CUDA_TRY(h, ff_step ? ensure_state_ff(h) : ensure_state_doubles(h));
+  if (h->opts.beta_T_exp != 0.0 && !h->bscale_valid && nsteps > 0) {  // later changes of T_p come from cells_kernel
+    CUDA_TRY(h, launch_beta_scale(h->bscale, h->Tp, h->opts.T_ref, h->opts.beta_T_exp, h->ncells, s));
+    h->bscale_valid = true;
+  }
   if (h->time_sweeps && nsteps > 0) {
     if ((int)h->tev.size() < 2 * ninner) {  // events for every sweep of a step; graphs captured before lack them
       drop_graphs(h);
@@ -1148,8 +1186,7 @@ int bte_step(bte_handle h, double dt, int nsteps, int ninner, int scheme, bte_st
         cudaGraph_t graph = nullptr;
         CUDA_TRY(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
         int cur = h->cur;
-        bool sff = h->state_ff;
-        cudaError_t e = enqueue_step(h, a, ninner, scheme, h->cap_stream, &cur, &sff);
+        cudaError_t e = enqueue_step(h, a, ninner, scheme, h->cap_stream, &cur);
         cudaError_t e2 = cudaStreamEndCapture(h->cap_stream, &graph);
         if (e != cudaSuccess || e2 != cudaSuccess) {
           if (graph) cudaGraphDestroy(graph);
@@ -1163,9 +1200,8 @@ int bte_step(bte_handle h, double dt, int nsteps, int ninner, int scheme, bte_st
       }
       CUDA_TRY(h, cudaGraphLaunch(exec, s));
       h->cur = cur_out;
-      if (ff_step) h->state_ff = true;
     } else {
-      const cudaError_t e = enqueue_step(h, a, ninner, scheme, s, &h->cur, &h->state_ff);
+      const cudaError_t e = enqueue_step(h, a, ninner, scheme, s, &h->cur);
       if (e != cudaSuccess && h->exchange_rc)
         return fail(h, BTE_E_EXCHANGE, "the exchange callback returned %d", h->exchange_rc);
       CUDA_TRY(h, e);
@@ -1173,10 +1209,10 @@ int bte_step(bte_handle h, double dt, int nsteps, int ninner, int scheme, bte_st
     int ndiff = 0;  // ghost refresh launches: diffuse and partially specular sides
     for (auto& bt : h->bc_type)
       for (int t : bt) ndiff += t == BTE_BC_DIFFUSE || t == BTE_BC_PARTIAL;
-    // sweep (sweep-ordered: pass + per-cell step, and the beta scale with tau(T)),
-    // fix-up, cell solve, diffuse wall ghosts
+    // sweep (sweep-ordered: pass + band sums, and the beta scale with tau(T)),
+    // per-cell step (two launches around a band-range exchange), diffuse wall ghosts
     const int sweep_k = scheme == BTE_IMPLICIT_GS ? 2 + (h->opts.beta_T_exp != 0.0 ? 1 : 0) : 1;
-    launches += ninner * (sweep_k + (h->solve_tp ? 1 : 0) + (ranged ? 1 : 0) + ndiff);
+    launches += ninner * (sweep_k + 1 + (ranged ? 1 : 0) + ndiff);
   }
   if (nsteps > 0) {
     h->TL_valid = false;
@@ -1276,20 +1312,27 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
     return fail(h, BTE_E_ARG, "unknown scheme %d", scheme);
   int rc = ensure_coef(h, dt, scheme == BTE_EXPLICIT ? BTE_EXPLICIT : BTE_IMPLICIT_JACOBI);
   if (rc) return rc;
-  if (scheme != BTE_IMPLICIT_JACOBI || !ff_sweep(h)) CUDA_TRY(h, ensure_state_doubles(h));  // timed reads of doubles
+  const bool ff = scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h);
+  CUDA_TRY(h, ff ? ensure_state_ff(h) : ensure_state_doubles(h));  // the form the timed sweeps read
+  if (h->opts.beta_T_exp != 0.0 && !h->bscale_valid) {
+    CUDA_TRY(h, launch_beta_scale(h->bscale, h->Tp, h->opts.T_ref, h->opts.beta_T_exp, h->ncells, h->stream));
+    h->bscale_valid = true;
+  }
   if (scheme == BTE_IMPLICIT_GS) return autotune_gs(h, report, report_len);
   cudaStream_t s = h->stream;
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
-  const int spare = (h->cur + 1) % 3;  // timing launches write here; the state is untouched (dry epilogue)
+  const int spare = (h->cur + 1) % 3;  // timing launches write here; the state is untouched
   struct Cand { int cpb, dteam, grid, pd; float ms; };
   std::vector<Cand> tried;
   // directions per team step: the default and half of it (fewer lanes per
   // cell, longer items: the per-item epilogue is spread over more updates)
   build_items(h);
+  const bool bf16 = h->opts.precision == BTE_BF16;
   std::vector<int> dteam_list = {h->dteam};
   if (h->dteam >= 2) dteam_list.push_back(h->dteam / 2);
-  const int pd_list[2] = {1, 2};
+  if (h->opts.precision == BTE_FP32 && max_teams(h) == 4 && 4 * h->lpc <= 256) dteam_list.push_back(4);
+  const std::vector<int> pd_list = bf16 ? std::vector<int>{1, 2} : std::vector<int>{1};
   int best_cpb = h->cpb, best_dteam = h->dteam, best_grid = h->grid, best_pd = h->pd;
   float best_ms = 1e30f;
   int dim = 2;
@@ -1306,12 +1349,14 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
     for (int cpb : cpb_list) {
       build_items(h, cpb, dteam);
       const int nit = (int)h->items.size();
-      const int grids[3] = {std::min(nit, 65535), std::min(nit, 2 * sms), std::min(nit, 4 * sms)};
-      for (int gi = 0; gi < 3; ++gi)
+      std::vector<int> grids = {std::min(nit, 65535)};
+      if (bf16) grids.insert(grids.end(), {std::min(nit, 2 * sms), std::min(nit, 4 * sms)});
+      else grids.push_back(0);  // the resident CTAs
+      for (int grid : grids)
         for (int pd : pd_list) {
           bool dup = false;
-          for (auto& c : tried) dup |= c.cpb == cpb && c.dteam == dteam && c.grid == grids[gi] && c.pd == pd;
-          if (!dup) tried.push_back({cpb, dteam, grids[gi], pd, 1e30f});
+          for (auto& c : tried) dup |= c.cpb == cpb && c.dteam == dteam && c.grid == grid && c.pd == pd;
+          if (!dup) tried.push_back({cpb, dteam, grid, pd, 1e30f});
         }
     }
   }
@@ -1330,14 +1375,10 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
         cur_dteam = c.dteam;
       }
       SweepArgs a = sweep_args(h);
-      a.dry = 1;
       a.counters = nullptr;
       a.In = a.Ik = h->Ibuf[h->cur];
       a.Iout = h->Ibuf[spare];
-      if (scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h)) {  // the middle inner iterations' variant
-        a.bmode = 2;
-        a.ff = 3;
-      }
+      a.ff = ff ? 1 : 0;
       CUDA_TRY(h, launch_sweep(h->opts.precision, c.pd, a, dim, h->threads, c.grid, s));
       CUDA_TRY(h, cudaEventRecord(h->ev0, s));
       for (int r = 0; r < reps; ++r) CUDA_TRY(h, launch_sweep(h->opts.precision, c.pd, a, dim, h->threads, c.grid, s));
@@ -1403,28 +1444,22 @@ int bte_get_flux(bte_handle h, int geom, double* q_cells, double* q_walls, int o
   if (!h->mem_ready || !h->init_set[geom]) return fail(h, BTE_E_STATE, "geometry %d has no state", geom);
   const bte_geom& g = h->geoms[geom];
   const int nc = g.nx * g.ny * g.nz;
-  CUDA_TRY(h, ensure_state_doubles(h));
   const void* I = h->Ibuf[h->cur];
   const int prec = h->opts.precision;
   cudaStream_t s = h->stream;
   if (q_cells) {
-    if (on_device) {
-      CUDA_TRY(h, launch_flux_cells(prec, I, h->I0ref_o, q_cells, h->Sdev, h->cell0[geom], nc, h->nd, h->nbp, g.dim, s));
-    } else {
-      CUDA_TRY(h, launch_flux_cells(prec, I, h->I0ref_o, h->scratch_q, h->Sdev, h->cell0[geom], nc, h->nd, h->nbp, g.dim, s));
-      CUDA_TRY(h, cudaMemcpyAsync(q_cells, h->scratch_q, (size_t)nc * g.dim * 8, cudaMemcpyDeviceToHost, s));
-    }
+    double* q = on_device ? q_cells : h->scratch_q;
+    CUDA_TRY(h, launch_flux_cells(prec, h->state_ff, I, q, h->Sdev, h->cell0[geom], nc, h->nd, h->nbp, g.dim, s));
+    if (!on_device) CUDA_TRY(h, cudaMemcpyAsync(q_cells, q, (size_t)nc * g.dim * 8, cudaMemcpyDeviceToHost, s));
   }
   if (q_walls) {
     double res[6] = {0, 0, 0, 0, 0, 0};
+    int nf[6] = {0, 0, 0, 0, 0, 0};
+    for (int side = 0; side < 2 * g.dim; ++side) nf[side] = (int)side_faces(g, side);
     CUDA_TRY(h, refresh_diffuse(h, I, s));  // diffuse and partially specular ghosts of the current state
     CUDA_TRY(h, refresh_partial(h, I, s));
-    for (int side = 0; side < 2 * g.dim; ++side) {
-      const int nf = (int)side_faces(g, side);
-      CUDA_TRY(h, launch_flux_faces(prec, I, h->I0ref_o, h->I0wall, h->geoms_d, geom, side, h->dirs_d, h->Sdev, h->nd,
-                                    h->nbp, h->scratch_faces, nf, s));
-      CUDA_TRY(h, launch_mean(h->scratch_faces, nf, h->scratch_out + side, s));
-    }
+    CUDA_TRY(h, launch_flux_walls(prec, h->state_ff, I, h->I0ref_o, h->I0wall, h->geoms_d, geom, h->dirs_d, h->Sdev, h->nd,
+                                  h->nbp, h->scratch_faces, h->max_side_faces, nf, 2 * g.dim, h->scratch_out, s));
     CUDA_TRY(h, cudaMemcpyAsync(res, h->scratch_out, 2 * g.dim * 8, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
     if (on_device) CUDA_TRY(h, cudaMemcpy(q_walls, res, 2 * g.dim * 8, cudaMemcpyHostToDevice));
@@ -1443,20 +1478,15 @@ int bte_get_intensity(bte_handle h, int geom, double* out, int on_device) {
   const long long nc = (long long)g.nx * g.ny * g.nz;
   const int prec = h->opts.precision;
   const size_t es = elem_bytes(prec);
-  CUDA_TRY(h, ensure_state_doubles(h));
   const char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
-  if (on_device) {
-    CUDA_TRY(h, launch_pack(prec, nullptr, out, I, nullptr, h->I0ref_o, nc, h->nd, h->nb, h->nbp, 0, h->stream));
-  } else if (prec == BTE_FP64) {
-    CUDA_TRY(h, cudaMemcpy2DAsync(out, h->nb * 8, I, h->nbp * 8, h->nb * 8, (size_t)nc * h->nd, cudaMemcpyDeviceToHost, h->stream));
-  } else {
-    for (long long c0 = 0; c0 < nc; c0 += h->pack_cells) {
-      const long long n = std::min(h->pack_cells, nc - c0);
-      CUDA_TRY(h, launch_pack(prec, nullptr, h->scratch_pack, I + (size_t)c0 * h->nd * h->nbp * es, nullptr, h->I0ref_o, n,
-                              h->nd, h->nb, h->nbp, 0, h->stream));
-      CUDA_TRY(h, cudaMemcpyAsync(out + (size_t)c0 * h->nd * h->nb, h->scratch_pack, (size_t)n * h->nd * h->nb * 8,
+  for (long long c0 = 0; c0 < nc; c0 += on_device ? nc : h->pack_cells) {
+    const long long n = on_device ? nc : std::min(h->pack_cells, nc - c0);
+    double* dst = on_device ? out : h->scratch_pack;
+    CUDA_TRY(h, launch_unpack(prec, h->state_ff, I + (size_t)c0 * h->nd * h->nbp * es, dst, h->I0ref_o, h->perm_d, n, h->nd,
+                              h->nb, h->nbp, h->stream));
+    if (!on_device)
+      CUDA_TRY(h, cudaMemcpyAsync(out + (size_t)c0 * h->nd * h->nb, dst, (size_t)n * h->nd * h->nb * 8,
                                   cudaMemcpyDeviceToHost, h->stream));
-    }
   }
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   return BTE_OK;
@@ -1471,44 +1501,44 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   const long long nc = (long long)g.nx * g.ny * g.nz;
   const int prec = h->opts.precision;
   const size_t es = elem_bytes(prec);
-  CUDA_TRY(h, ensure_state_doubles(h));  // the other geometries keep their state
   char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
   cudaStream_t s = h->stream;
-  if (on_device) {
-    CUDA_TRY(h, launch_pack(prec, in, nullptr, nullptr, I, h->I0ref_o, nc, h->nd, h->nb, h->nbp, 1, s));
-    CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, cudaMemcpyDeviceToDevice, s));
-  } else if (prec == BTE_FP64) {
-    CUDA_TRY(h, cudaMemcpy2DAsync(I, h->nbp * 8, in, h->nb * 8, h->nb * 8, (size_t)nc * h->nd, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, cudaMemcpyHostToDevice, s));
-  } else {
-    for (long long c0 = 0; c0 < nc; c0 += h->pack_cells) {
-      const long long n = std::min(h->pack_cells, nc - c0);
-      CUDA_TRY(h, cudaMemcpyAsync(h->scratch_pack, in + (size_t)c0 * h->nd * h->nb, (size_t)n * h->nd * h->nb * 8,
-                                  cudaMemcpyHostToDevice, s));
-      CUDA_TRY(h, launch_pack(prec, h->scratch_pack, nullptr, nullptr, I + (size_t)c0 * h->nd * h->nbp * es, h->I0ref_o, n,
-                              h->nd, h->nb, h->nbp, 1, s));
-      CUDA_TRY(h, cudaStreamSynchronize(s));
+  for (long long c0 = 0; c0 < nc; c0 += on_device ? nc : h->pack_cells) {
+    const long long n = on_device ? nc : std::min(h->pack_cells, nc - c0);
+    const double* src = in + (size_t)c0 * h->nd * h->nb;
+    if (!on_device) {
+      CUDA_TRY(h, cudaMemcpyAsync(h->scratch_pack, src, (size_t)n * h->nd * h->nb * 8, cudaMemcpyHostToDevice, s));
+      src = h->scratch_pack;
     }
-    CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, cudaMemcpyHostToDevice, s));
+    CUDA_TRY(h, launch_pack(prec, h->state_ff, src, I + (size_t)c0 * h->nd * h->nbp * es, h->I0ref_o, h->perm_d, n, h->nd, h->nb, h->nbp, s));
+    if (!on_device) CUDA_TRY(h, cudaStreamSynchronize(s));  // the caller's pageable memory and the staging buffer are reused
   }
+  CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
                                    h->Msum + h->cell0[geom] * 4,
                                    h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));
   if (h->Epart) {
     h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange
   } else {
-    CUDA_TRY(h, launch_energy_L(prec, I, h->I0ref_o, h->EL + h->cell0[geom], h->wdir, nc, h->nd, thermo(h), s));
+    CUDA_TRY(h, launch_energy_L(prec, h->state_ff, I, h->I0ref_o, h->EL + h->cell0[geom], h->wdir, nc, h->nd, thermo(h), s));
   }
   CUDA_TRY(h, cudaStreamSynchronize(s));
   h->TL_valid = false;
+  h->bscale_valid = false;
   return BTE_OK;
 }
 
 int bte_get_directions(bte_handle h, double* S, double* w, int* refl) {
   if (!h) return BTE_E_ARG;
-  if (S) std::memcpy(S, h->S.data(), h->S.size() * 8);
-  if (w) std::memcpy(w, h->w.data(), h->w.size() * 8);
-  if (refl) std::memcpy(refl, h->refl.data(), h->refl.size() * sizeof(int));
+  const int n = h->nd;
+  for (int p = 0; p < n; ++p) {  // the caller's order
+    const int d = h->perm[p];
+    for (int c = 0; c < 3; ++c) {
+      if (S) S[3 * d + c] = h->S[3 * p + c];
+      if (refl) refl[c * n + d] = h->perm[h->refl[c * n + p]];
+    }
+    if (w) w[d] = h->w[p];
+  }
   return h->nd;
 }
 

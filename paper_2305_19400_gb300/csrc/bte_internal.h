@@ -10,6 +10,8 @@
 //   coef           [class][5][dir][nbp] double  sweep coefficients (A_n, A_x, A_y, A_z, A_s)
 //   node_c, node_C [nbp][ng]    double        Gauss nodes: hbar*omega/kB and weights
 //   per-band / per-direction / per-geometry tables, work list, counters.
+// dir is the internal direction order (internal_order, bte_tables.h); the
+// caller's order appears only in what crosses the C ABI.
 // nbp is nb rounded up to a multiple of 8, so one (cell, dir) row is a whole
 // number of 16-byte vectors in every precision.  Padding bands carry zero
 // coefficients and stay zero.
@@ -45,9 +47,9 @@ struct DevGeom {
 // A run of consecutive cells of one geometry processed by one CTA.
 struct WorkItem {
   int geom;
-  int cell_begin;  // local cell index
-  int cell_count;
-  int pad;
+  int cell_begin;  // local cell index of (i0, j, k)
+  int cell_count;  // cells along x
+  int i0, j, k;
 };
 
 // Sweep-ordered (Gauss-Seidel) pass: one unit = the directions dir0 .. dir0+ndc-1
@@ -75,7 +77,7 @@ struct WallDirs {
   double sum_out, sum_in;
 };
 
-// A cell whose temperature the sweep could not settle on its cached model.
+// A cell whose temperature its cached model could not settle.
 struct FixItem {
   long long P;  // global cell
   double Ep;    // right-hand side of the T_p equation: sum_b beta_b G_b / v_b
@@ -99,6 +101,7 @@ struct ThermoTables {
   const double* a_L;      // [nbp] W / v_b         (T_L equation weights)
   const double* inv_v;    // [nbo] 1/v_b of the stored bands (0 on padding)
   const double* beta;     // [nbo] beta_b of the stored bands (0 on padding)
+  const double* binv_v;   // [nbo] beta_b/v_b of the stored bands (0 on padding)
   int ng;
   int nbp;    // all bands, padded: width of node tables, J, a_p and a_L
   int nb;     // all bands
@@ -120,13 +123,12 @@ struct SweepArgs {
   double* Msum;             // [cell][4] sum_b a_p,b J_k,b: the T_p model's sums, kept with J
   double* EL;               // [cell] out
   const double* I0wall;     // [face][nbp] FP64 ghosts
+  const void* I0wall_ff;    // [face][nbp] FP64 ghosts as ff pairs (bte_ff.cuh)
   const float* I0wall_dev;  // [face][nbp] FP32 ghosts minus I0ref (reduced modes)
   const double* I0ref;      // [nbp] I0_b(T_ref) (reduced modes)
-  int ff;                   // FP64: 0 DFMA arithmetic (sweep_kernel); else the double-float sweep
-                            // (sweep_ff_kernel; bit 0: In and I^k are ff pairs, bit 1: I^{k+1} and B
-                            // are written as ff; B is always ff)
-  // FP64 double-float sweep with factored coefficients (bte_sweep_ff.cuh), tables
-  // in the double-float pair layout of bte_ff.cuh (h_b, h_b+1, l_b, l_b+1 per two bands):
+  int ff;                   // FP64: 1 double-float arithmetic (every intensity buffer holds ff pairs), 0 IEEE
+  // tables of the double-float sweep in the pair layout of bte_ff.cuh
+  // (h_b, h_b+1, l_b, l_b+1 per two bands):
   const void* coef_R;       // [cls][nd][nbp] R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax,d)
   const float* band_ff;     // [2][nbp] 1/(v_b dt), beta_b/v_b of the stored bands (0 on padding)
   const float* dirc_ff;     // [cls][nd][3][2] c_ax,d as (h, l)
@@ -136,8 +138,8 @@ struct SweepArgs {
   const float4* dirc;       // reduced: [cls][nd] (c_x, c_y, c_z, sum), c_ax = |S_d,ax|/(w_d Delta_ax)
   const float* vb32;        // [nbp] v_b (reduced)
   const float* bb32;        // [nbp] beta_b (reduced)
-  FixItem* fix;             // cells handed to the fix-up kernel
-  unsigned* fix_count;
+  double* Gc;               // [cell][gsplit][nbo] band sums G_b, written by the sweeps, added by cells_kernel
+  FixItem* fix;             // cells_kernel's queue of exact solves, a part per CTA
   const DirInfo* dirs;
   const double* wdir;       // [nd]
   const float* wdir32;      // [nd]
@@ -147,13 +149,14 @@ struct SweepArgs {
   int nd;
   int lpc;                  // lanes per direction row = nbp / values per lane
   int dteam;                // directions one cell team covers per step (team = lpc * dteam lanes)
+  int dir_group;            // rows that differ only in the signs of S: 4 (in-plane sets) or 8 (internal_order)
+  int gsplit;               // partial band sums per cell in Gc (the teams of a cell)
   int solve_tp;             // 0 when every beta_b == 0 (T_p then unused)
   double trust_rel;         // cached model accepted when |T - T_e| <= trust_rel * T
   int maxit;
   double Wtot;              // sum of direction weights
-  int dry;                  // 1: timing run, the epilogue writes no solver state
-  int partial;              // 1: band-range handle; the epilogue writes per-cell partial (E_L, E_p)
-  double* Epart;            //    to Epart[cell][2] and the solve runs after the caller's all-reduce
+  int partial;              // 1: band-range handle; per-cell partial (E_L, E_p) go to Epart[cell][2]
+  double* Epart;            //    and the solve runs after the caller's all-reduce
   double beta_exp;          // beta_b(T) = beta_b (T_p / beta_Tref)^beta_exp per cell (0: fixed tau)
   double beta_Tref;
   int explicit_scheme;      // reduced modes compute P, Q on the fly from these:
@@ -165,7 +168,7 @@ struct SweepArgs {
   int gs_nunits;
   int gs_ndc;               // directions per unit (the CTA layout)
   int gs_tx, gs_ty;         // cross-section of a column tile (2-D: gs_tx cells along x)
-  const double* bscale;     // [cell] beta_b(T_p)/beta_b (beta_exp != 0), written before each pass
+  double* bscale;           // [cell] beta_b(T_p)/beta_b (beta_exp != 0), kept current by cells_kernel
   ThermoTables th;
 };
 
@@ -177,16 +180,19 @@ int values_per_lane(int precision);
 // needs, and a per-launch setting could lower another thread's limit between
 // its own setting and its launch.
 cudaError_t raise_dynamic_smem(const void* func, size_t bytes);
+// grid <= 0 (FP64, FP32): as many CTAs as are resident
 cudaError_t launch_sweep(int precision, int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
-cudaError_t launch_sweep_fp64(int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
-cudaError_t launch_sweep_fp32(int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
+cudaError_t launch_sweep_fp64(const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
+cudaError_t launch_sweep_fp32(const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
 cudaError_t launch_sweep_bf16(int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
 struct MLPView;
-cudaError_t launch_fixup(const SweepArgs& a, const MLPView* mlp, cudaStream_t s);
-cudaError_t launch_solve_cells(const SweepArgs& a, long long ncells, cudaStream_t s);
-// sweep-ordered pass (bte_gs.cu) and its per-cell step (bte_kernels.cu): the
-// pass writes Iout; the reduction writes E_L, E_p of the stored bands to Epart
-// (partial) or solves T_p and refreshes I0 at once (whole handle)
+// per-cell step (bte_cells.cu): mode 0 energies from Gc and solve, 1 energies
+// from Gc to Epart, 2 solve from Epart
+cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const MLPView* mlp, cudaStream_t s);
+int cells_grid(long long ncells);
+long long cells_queue_entries(long long ncells);  // FixItems of a.fix
+// sweep-ordered pass (bte_gs.cu) and its band sums (bte_kernels.cu): the pass
+// writes Iout, the reduction G_b of every cell to Gc
 cudaError_t launch_gs_sweep(int precision, const SweepArgs& a, int dim, int threads, cudaStream_t s);
 cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells, cudaStream_t s);
 cudaError_t launch_beta_scale(double* out, const double* Tp, double Tref, double p, long long ncells, cudaStream_t s);
@@ -210,7 +216,7 @@ cudaError_t mlp_forward_backward(const float* p, int k, const float* X, int ldx,
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s);
 cudaError_t launch_solve_batch(ThermoTables th, const double* Ep, const double* T0, int n, double trust_rel, int maxit,
                                const MLPView* mlp, double* Tout, int* evals, cudaStream_t s);
-cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J, double* Msum, double* Tp, double* Te,
+cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* Tp, double* Te,
                               double* TL, double* EL, const double* Tcells, const double* I0ref, long long cell0,
                               int ncells, int nd, ThermoTables th, cudaStream_t s);
 cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, const double* Tp, double* Te, long long ncells,
@@ -221,24 +227,32 @@ cudaError_t launch_wall_dev(float* out, const double* I0wall, const double* I0re
 cudaError_t launch_solve_TL(double* TL, const double* EL, const double* Tguess, const double* J, const double* Teval,
                             long long ncells, ThermoTables th, double trust_rel, int maxit, DevCounters* counters,
                             cudaStream_t s);
-cudaError_t launch_flux_cells(int precision, const void* I, const double* I0ref, double* q, const double* S,
-                              long long cell0, int ncells, int nd, int nbp, int dim, cudaStream_t s);
-cudaError_t launch_flux_faces(int precision, const void* I, const double* I0ref, const double* I0wall,
-                              const DevGeom* geoms, int geom, int side, const DirInfo* dirs, const double* S, int nd,
-                              int nbp, double* face_out, int nfaces, cudaStream_t s);
-cudaError_t launch_mean(const double* v, int n, double* out, cudaStream_t s);
+// state_ff: the FP64 intensities are ff pairs (bte_ff.cuh)
+cudaError_t launch_flux_cells(int precision, bool state_ff, const void* I, double* q, const double* S, long long cell0,
+                              int ncells, int nd, int nbp, int dim, cudaStream_t s);
+// every side of one geometry: face sums to face_out[side][max_faces], means to out[side]
+cudaError_t launch_flux_walls(int precision, bool state_ff, const void* I, const double* I0ref, const double* I0wall,
+                              const DevGeom* geoms, int geom, const DirInfo* dirs, const double* S, int nd, int nbp,
+                              double* face_out, int max_faces, const int (&nfaces)[6], int nsides, double* out,
+                              cudaStream_t s);
 // In place: npairs 16-byte ff pairs of two bands (bte_ff.cuh layout) -> two doubles each.
 cudaError_t launch_ff_to_doubles(void* buf, long long npairs, cudaStream_t s);
-cudaError_t launch_pack(int precision, const double* src, double* dst_out, const void* Isrc, void* Idst,
-                        const double* I0ref, long long ncells, int nd, int nb, int nbp, int to_padded, cudaStream_t s);
-cudaError_t launch_energy_L(int precision, const void* I, const double* I0ref, double* EL, const double* wdir,
+// npairs x two doubles -> ff pairs (dst may be src)
+cudaError_t launch_doubles_to_ff(const void* src, void* dst, long long npairs, cudaStream_t s);
+// FP64 [cell][caller's d][nb] <-> internal rows; perm: the caller's index of every internal direction
+cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* perm,
+                          long long ncells, int nd, int nb, int nbp, cudaStream_t s);
+cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* perm,
+                        long long ncells, int nd, int nb, int nbp, cudaStream_t s);
+cudaError_t launch_energy_L(int precision, bool state_ff, const void* I, const double* I0ref, double* EL, const double* wdir,
                             long long ncells, int nd, ThermoTables th, cudaStream_t s);
 
 // Read-only view of one geometry's device state, for entry points that live
 // outside bte_capi.cu (bte_noalloc.cu).  flux_view returns BTE_E_* codes.
 struct FluxView {
   int precision;          // storage of I (BTE_FP64 = 0, BTE_FP32 = 1, BTE_BF16 = 2)
-  const double* I;        // current intensity buffer (padded rows; FP64 only when precision == 0)
+  const void* I;          // current intensity buffer (padded rows)
+  bool state_ff;          // FP64: it holds ff pairs
   const double* I0wall;
   const DevGeom* geoms;
   const DirInfo* dirs;

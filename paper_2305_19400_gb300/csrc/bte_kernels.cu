@@ -1,22 +1,18 @@
-// bte_kernels.cu -- CUDA kernels around the sweep (sm_103a).  The sweep itself
-// (upwind update, walls, per-cell reduction, cached-model T_p solve, I0
-// refresh; Sec. 3.1, Eq. 4-6) lives in bte_sweep.cuh.  Here:
-//   fixup_kernel        exact FP64 T_p solve (Halley on the band quadrature,
-//                       bisection fallback) for the cells the model left, which
-//                       also refreshes their cached model and I0;
-//   solve_cells_kernel  the T_p step of a band-range handle after the caller's
-//                       all-reduce of the per-cell energy partials (Sec. 3.3);
-//   gs_reduce_kernel    per-cell energies (and the T_p step) after a
-//                       sweep-ordered pass (bte_gs.cu);
+// bte_kernels.cu -- CUDA kernels around the sweep (sm_103a).  The sweeps (upwind
+// update, walls, band sums; Sec. 3.1, Eq. 4-6) live in bte_sweep.cuh and
+// bte_sweep_ff.cuh, the per-cell T_p step in bte_cells.cu.  Here:
+//   gs_reduce_kernel    band sums after a sweep-ordered pass (bte_gs.cu) or an
+//                       unstructured sweep;
 //   init_cells / state_from_Tp / wall_I0 / wall_dev
 //                       equilibrium state, cached models and Eq. 6 ghosts;
 //   solve_TL_kernel     T_L on request (cached model first, exact otherwise);
-//   flux_cells / flux_faces / mean / pack / energy_L
+//   flux_cells / flux_faces / mean / pack / unpack / energy_L
 //                       heat flux, FP64 <-> storage packing, E_L after a restore.
 #include <algorithm>
+#include <type_traits>
 
 #include "bte_ff.cuh"
-#include "bte_mlp.cuh"
+#include "bte_flux.cuh"
 #include "bte_quad.cuh"
 #include "bte_solve.cuh"
 #include "bte_store.cuh"
@@ -24,77 +20,6 @@
 namespace bte {
 
 namespace {
-
-// Exact temperature solve of the cells the sweep could not settle on their
-// cached model: one thread-block cluster of kFixCluster CTAs per cell
-// (exact_solve_cluster spreads each evaluation's bands over the cluster's SMs;
-// with a handful of such cells per step the solve's latency, not its
-// throughput, is what the step waits for).  The start is the model root, or
-// when there is none the previous T_p (plain mode) or the learned guess (net
-// A, then surrogate Newton steps on net B, by warp 0 of each CTA: the same
-// value everywhere); the exact FP64 quadrature then refines it (each
-// evaluation becomes the cell's cached model) and every CTA refreshes I0 of
-// the bands whose model row it wrote.
-constexpr int kFixThreads = 128;
-constexpr int kFixCluster = 4;
-
-__global__ void __cluster_dims__(kFixCluster, 1, 1) __launch_bounds__(kFixThreads)
-    fixup_kernel(SweepArgs a, int learned, MLPView m) {
-  extern __shared__ double fsm[];  // exact_solve_cluster scratch, T0, then the learned-mode buffers
-  namespace cg = cooperative_groups;
-  cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
-  const unsigned cid = blockIdx.x / (unsigned)nr, ncl = gridDim.x / (unsigned)nr;
-  const int nbp = a.th.nbp;
-  const int own0 = rank * nbp / nr, own1 = (rank + 1) * nbp / nr;  // bands whose model row this CTA writes
-  double* solve_sm = fsm;
-  double* t0_sm = fsm + cta_solve_smem_doubles(nbp);
-  float* ybuf = reinterpret_cast<float*>(t0_sm + 2);
-  float* hbuf = ybuf + 2 * nbp;
-  const unsigned count = *a.fix_count;
-  unsigned long long evals = 0, fb = 0, bad = 0;
-  unsigned par = 0;  // evaluations of this cluster so far (the solve's buffer parity)
-  for (unsigned w = cid; w < count; w += ncl) {  // the same items, in the same order, in every CTA of the cluster
-    const FixItem it = a.fix[w];
-    const long long P = it.P;
-    // learned mode: the networks' guess starts the cells that have no usable
-    // root of their cached model (a cold or far-off start); a model root, when
-    // there is one, is the closer start (measured: twice the evaluations from
-    // the networks' guess on the learned 3-D workload)
-    const bool net = learned && !it.model;  // uniform over the cluster (one item)
-    if (net) {
-      if (threadIdx.x < 32) {
-        const double g = mlp_guess_T(m, a.th.a_p, it.Ep, 2, ybuf, hbuf);
-        if (threadIdx.x == 0) t0_sm[0] = g;
-      }
-      __syncthreads();
-    }
-    const double T0 = net ? t0_sm[0] : it.T0;
-    const SolveResult r = exact_solve_cluster(a.th, it.Ep, T0, a.trust_rel, a.maxit, a.J + (P * 4) * nbp, solve_sm, par);
-    evals += r.evals;
-    fb += r.fallback;
-    bad += r.bad;
-    __syncthreads();  // this CTA's model rows, written by the solve, before its I0 refresh reads them
-    // I0 refresh of the stored bands whose model rows this CTA wrote, at r.Te
-    const int s0 = max(own0 - a.th.band0, 0), s1 = min(own1 - a.th.band0, a.th.nbo);
-    for (int b = s0 + (int)threadIdx.x; b < s1; b += blockDim.x) {
-      const double* Jb = a.J + (P * 4) * nbp + a.th.band0 + b;
-      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? model_I0(Jb, nbp, r.delta) : 0.0;
-    }
-    if (rank == 0 && threadIdx.x == 0) {
-      a.Teval[P] = r.Te;
-      a.Tp[P] = r.Te + r.delta;
-      for (int k = 0; k < 4; ++k) a.Msum[4 * P + k] = r.M[k];  // the model just written to J
-    }
-    __syncthreads();  // t0_sm and the solve scratch are reused by the next item
-  }
-  cl.sync();  // no CTA leaves while another may still read its shared memory
-  if (rank == 0 && threadIdx.x == 0 && a.counters) {
-    if (evals) atomicAdd(&a.counters->evals, evals);
-    if (fb) atomicAdd(&a.counters->fallbacks, fb);
-    if (bad) atomicAdd(&a.counters->nonfinite, bad);
-  }
-}
 
 // ---------------------------------------------------------------------------
 // Per-cell thermodynamic state at temperature T: I0cell, cached model J at T
@@ -146,8 +71,7 @@ __global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum,
     for (long long e = threadIdx.x; e < n; e += blockDim.x) {
       const int b = (int)(e % th.nbo);  // stored band; I0ref holds the stored bands
       const double v = b < th.nbr ? (sizeof(S) == 8 ? row[th.band0 + b] : row[th.band0 + b] - I0ref[b]) : 0.0;
-      if constexpr (sizeof(S) == 2) I[P * n + e] = __double2bfloat16(v);
-      else I[P * n + e] = (S)v;
+      set_I(I, P * n + e, v);
     }
     if (threadIdx.x == 0) {
       double e = 0.0;
@@ -235,101 +159,127 @@ __global__ void solve_TL_kernel(double* TL, const double* EL, const double* Tgue
   }
 }
 
-// Deterministic block sum of one value per thread (blockDim.x a power of two <= 1024).
-__device__ double block_sum(double v, double* sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
+// Cell heat flux q(P) = sum_b sum_d S_d I_{d,b}: one CTA per cell.  A lane holds
+// the V bands of one 16-byte vector and takes every (threads / lanes)-th group of
+// four rows, (+,+), (-,+), (-,-), (+,-) of one |S|: the four values' sums and
+// differences first, then one FMA per axis, 1.5 FP64 operations per value in
+// 2-D where S_d I for every direction takes two (the FP64 pipe is the bound).
+// The reference part of the reduced modes' storage drops out: sum_d S_d = 0.
+// On 128x128 x 400 x 55: 2014 us with one 64-bit division and two FMAs per value.
+template <typename S, int V>
+__device__ __forceinline__ double vector_sum(const S* p) {  // sum of V consecutive values
+  double s = 0.0;
+  if constexpr (sizeof(S) == 8) {
+    if constexpr (std::is_same<S, FFElem>::value) {
+      double a, b;
+      ff::to_doubles(ff::ldg(p), a, b);
+      s = a + b;
+    } else {
+      double x[2];
+      Tr<double>::ld(p, x);
+      s = x[0] + x[1];
+    }
+  } else {
+    float x[V];
+    Tr<S>::ld(p, x);
+#pragma unroll
+    for (int v = 0; v < V; ++v) s += (double)x[v];
+  }
+  return s;
+}
+
+template <typename S, int V, int DIM>
+__global__ void __launch_bounds__(256) flux_cells_kernel(const S* I, double* q, const double* Sd, long long cell0,
+                                                         int ncells, int nd, int nbp) {
+  __shared__ double sh[3][8];
+  const int lpc = nbp / V, groups = 256 / lpc, grp = threadIdx.x / lpc, b0 = V * (threadIdx.x - grp * lpc);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int c = blockIdx.x; c < ncells; c += gridDim.x) {
+    const S* row = I + (cell0 + c) * (long long)nd * nbp + b0;
+    double acc[3] = {0.0, 0.0, 0.0};
+    if (grp < groups) {
+#pragma unroll 2
+      for (int r = 4 * grp; r < nd; r += 4 * groups) {
+        double v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = vector_sum<S, V>(row + (r + k) * nbp);
+        const double a = v[0] + v[3], b = v[1] + v[2];
+        acc[0] = fma(Sd[3 * r], a - b, acc[0]);
+        acc[1] = fma(Sd[3 * r + 1], (v[0] - v[3]) + (v[1] - v[2]), acc[1]);
+        if (DIM == 3) acc[2] = fma(Sd[3 * r + 2], a + b, acc[2]);
+      }
+    }
+#pragma unroll
+    for (int ax = 0; ax < DIM; ++ax) {
+      for (int o = 16; o > 0; o >>= 1) acc[ax] += __shfl_xor_sync(0xffffffffu, acc[ax], o);
+      if (lane == 0) sh[ax][wid] = acc[ax];
+    }
+    __syncthreads();
+    if (threadIdx.x < DIM) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += sh[threadIdx.x][w];
+      q[(long long)c * DIM + threadIdx.x] = t;
+    }
     __syncthreads();
   }
-  const double r = sh[0];
-  __syncthreads();
-  return r;
 }
 
-// Cell heat flux q(P) = sum_b sum_d S_d I_{d,b}: one CTA per cell.
+// Net outgoing flux through every face of every side of a geometry (blockIdx.y: side).
 template <typename S>
-__global__ void flux_cells_kernel(const S* I, const double* I0ref, double* q, const double* Sd, long long cell0,
-                                  int ncells, int nd, int nbp, int dim) {
-  extern __shared__ double sh[];
-  for (int c = blockIdx.x; c < ncells; c += gridDim.x) {
-    const long long P = cell0 + c;
-    const long long base = P * (long long)nd * nbp;
-    double acc[3] = {0.0, 0.0, 0.0};
-    for (long long e = threadIdx.x; e < (long long)nd * nbp; e += blockDim.x) {
-      const int d = (int)(e / nbp);
-      const int b = (int)(e - (long long)d * nbp);
-      const double v = full_I(I, base + e, b, I0ref);
-      acc[0] = fma(Sd[3 * d + 0], v, acc[0]);
-      acc[1] = fma(Sd[3 * d + 1], v, acc[1]);
-      acc[2] = fma(Sd[3 * d + 2], v, acc[2]);
-    }
-    for (int ax = 0; ax < dim; ++ax) {
-      const double t = block_sum(acc[ax], sh);
-      if (threadIdx.x == 0) q[(long long)c * dim + ax] = t;
-    }
-  }
-}
-
-// Net outgoing flux through each face of one wall: one CTA per face.
-template <typename S>
-__global__ void flux_faces_kernel(const S* I, const double* I0ref, const double* I0wall, const DevGeom* geoms,
-                                  int geom, int side, const DirInfo* dirs, const double* Sd, int nd, int nbp,
-                                  double* face_out, int nfaces) {
-  extern __shared__ double sh[];
+__global__ void __launch_bounds__(kFluxThreads) flux_faces_kernel(const S* I, const double* I0ref, const double* I0wall,
+                                                                  const DevGeom* geoms, int geom, const DirInfo* dirs,
+                                                                  const double* Sd, int nd, int nbp, double* face_out,
+                                                                  int max_faces) {
+  __shared__ double sh[kFluxThreads];
   const DevGeom g = geoms[geom];
-  const int ax = side / 2;
-  const double nsign = (side & 1) ? 1.0 : -1.0;
+  const int side = blockIdx.y;
+  const int nfaces = side < 2 ? g.ny * g.nz : (side < 4 ? g.nx * g.nz : g.nx * g.ny);
   for (int f = blockIdx.x; f < nfaces; f += gridDim.x) {
-    int i, j, k;
-    if (side < 2) { j = f % g.ny; k = f / g.ny; i = (side & 1) ? g.nx - 1 : 0; }
-    else if (side < 4) { i = f % g.nx; k = f / g.nx; j = (side & 1) ? g.ny - 1 : 0; }
-    else { i = f % g.nx; j = f / g.nx; k = (side & 1) ? g.nz - 1 : 0; }
-    const long long P = g.cell0 + i + (long long)g.nx * (j + (long long)g.ny * k);
-    const long long base = P * (long long)nd * nbp;
-    double acc = 0.0;
-    for (long long e = threadIdx.x; e < (long long)nd * nbp; e += blockDim.x) {
-      const int d = (int)(e / nbp);
-      const int b = (int)(e - (long long)d * nbp);
-      const double sn = Sd[3 * d + ax] * nsign;
-      double v;
-      if (sn > 0.0) v = full_I(I, base + e, b, I0ref);
-      else if (g.bc[side] == 0) v = I0wall[(g.face0[side] + f) * nbp + b];
-      else if (g.bc[side] == 3) v = full_I(reinterpret_cast<const S*>(g.gdir[side]), (long long)f * nd * nbp + e, b, I0ref);
-      else {
-        const int r = ax == 0 ? dirs[d].rx : (ax == 1 ? dirs[d].ry : dirs[d].rz);
-        v = full_I(I, base + (long long)r * nbp + b, b, I0ref);
-      }
-      acc = fma(sn, v, acc);
-    }
-    const double t = block_sum(acc, sh);
-    if (threadIdx.x == 0) face_out[f] = t;
+    const double t = face_flux(I, I0ref, I0wall, g, side, f, dirs, Sd, nd, nbp, sh);
+    if (threadIdx.x == 0) face_out[(long long)side * max_faces + f] = t;
   }
 }
 
-__global__ void mean_kernel(const double* v, int n, double* out) {
-  extern __shared__ double sh[];
+struct SideFaces {
+  int n[6];
+};
+__global__ void mean_kernel(const double* v, int max_faces, SideFaces nf, double* out) {  // a CTA per side
+  __shared__ double sh[256];
+  const int n = nf.n[blockIdx.x];
   double acc = 0.0;
-  for (int e = threadIdx.x; e < n; e += blockDim.x) acc += v[e];
+  for (int e = threadIdx.x; e < n; e += blockDim.x) acc += v[(long long)blockIdx.x * max_faces + e];
   const double t = block_sum(acc, sh);
-  if (threadIdx.x == 0) *out = t / (double)n;
+  if (threadIdx.x == 0) out[blockIdx.x] = t / (double)n;
 }
 
-// FP64 [cell][d][nb] <-> padded storage rows [cell][d][nbp] (deviation in the reduced modes).
+// FP64 [cell][caller's d][nb] <-> internal rows [cell][dir][nbp] (deviation in the
+// reduced modes): one CTA per cell, a thread per band walking every
+// (threads / nbp)-th direction, so consecutive lanes touch consecutive bands on
+// both sides and no index is divided.
 template <typename S>
-__global__ void pack_kernel(const double* src, double* dst_out, const S* Isrc, S* Idst, const double* I0ref,
-                            long long ncells, int nd, int nb, int nbp, int to_padded) {
-  const long long n = ncells * nd * (long long)nbp;
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    const long long cd = e / nbp;
-    const int b = (int)(e - cd * nbp);
-    if (to_padded) {
-      const double v = b < nb ? (sizeof(S) == 8 ? src[cd * nb + b] : src[cd * nb + b] - I0ref[b]) : 0.0;
-      if constexpr (sizeof(S) == 2) Idst[e] = __double2bfloat16(v);
-      else Idst[e] = (S)v;
-    } else if (b < nb) {
-      dst_out[cd * nb + b] = full_I(Isrc, e, b, I0ref);
+__global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, const double* I0ref, const int* perm,
+                                                     long long ncells, int nd, int nb, int nbp) {
+  const int rows = 256 / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
+  if (r >= rows || b >= nb) return;
+  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
+    double* o = out + P * nd * nb + b;
+#pragma unroll 8
+    for (int d = r; d < nd; d += rows) __stcs(o + (long long)perm[d] * nb, full_I(I, (P * nd + d) * nbp + b, b, I0ref));
+  }
+}
+
+template <typename S>
+__global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const double* I0ref, const int* perm,
+                                                   long long ncells, int nd, int nb, int nbp) {
+  const int rows = 256 / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
+  if (r >= rows) return;
+  const double ref = sizeof(S) == 8 || b >= nb ? 0.0 : I0ref[b];
+  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
+    const double* x = in + P * nd * nb + b;
+#pragma unroll 8
+    for (int d = r; d < nd; d += rows) {
+      const double v = b < nb ? __ldcs(x + (long long)perm[d] * nb) - ref : 0.0;
+      set_I(I, (P * nd + d) * nbp + b, v);
     }
   }
 }
@@ -352,75 +302,11 @@ __global__ void energy_L_kernel(const S* I, const double* I0ref, double* EL, con
   }
 }
 
-// T_p step of one cell from its energies (E_L, E_p over every band), by one
-// warp: the T_p equation on the cell's cached cubic model of all bands,
-// I0 refresh of the stored bands inside the trust radius, the rest to the
-// fix-up list.
-__device__ void solve_cell_warp(const SweepArgs& a, long long P, double EL, double Ep, int lane,
-                                unsigned long long& solves, unsigned long long& badc) {
-  const int nbp = a.th.nbp;
-  const bool finite = isfinite(EL) && isfinite(Ep);
-  if (!a.solve_tp) {  // every beta_b is zero: only E_L is kept
-    if (lane == 0) {
-      a.EL[P] = EL;
-      if (!finite) ++badc;
-    }
-    return;
-  }
-  // the model's sums, kept with J (sum_b a_p,b J_k,b)
-  const double* M = a.Msum + 4 * P;
-  const double Te = a.Teval[P];
-  const double delta = model_step(M[0] - Ep, M[1], M[2], M[3]);
-  const double Tn = Te + delta;
-  const bool ok = finite && isfinite(Tn) && fabs(delta) <= a.trust_rel * Tn;
-  if (lane == 0) {
-    a.EL[P] = EL;
-    if (!finite) ++badc;
-    else ++solves;
-    if (finite && !ok) {
-      const unsigned k = atomicAdd(a.fix_count, 1u);
-      FixItem fi;
-      fi.P = P;
-      fi.Ep = Ep;
-      fi.model = (isfinite(Tn) && Tn >= kTmin && Tn <= kTmax) ? 1 : 0;
-      fi.T0 = fi.model ? Tn : a.Tp[P];
-      fi.pad = 0;
-      a.fix[k] = fi;
-    }
-    if (ok) a.Tp[P] = Tn;
-  }
-  if (ok) {
-    for (int b = lane; b < a.th.nbo; b += 32) {
-      const double* Jb = a.J + (P * 4) * nbp + a.th.band0 + b;
-      a.I0cell[P * a.th.nbo + b] = b < a.th.nbr ? model_I0(Jb, nbp, delta) : 0.0;
-    }
-  }
-}
-
-__device__ void flush_counters(const SweepArgs& a, int lane, unsigned long long solves, unsigned long long badc) {
-  if (lane == 0 && a.counters) {
-    if (solves) atomicAdd(&a.counters->solves, solves);
-    if (badc) atomicAdd(&a.counters->nonfinite, badc);
-  }
-}
-
-// Temperature step of a band-range handle after the caller's all-reduce: one
-// warp per cell, E_L and E_p from Epart.
-__global__ void solve_cells_kernel(SweepArgs a, long long ncells) {
-  const int warps = blockDim.x / 32, lane = threadIdx.x & 31;
-  unsigned long long solves = 0, badc = 0;
-  for (long long P = blockIdx.x * (long long)warps + threadIdx.x / 32; P < ncells; P += (long long)gridDim.x * warps)
-    solve_cell_warp(a, P, a.Epart[2 * P], a.Epart[2 * P + 1], lane, solves, badc);
-  flush_counters(a, lane, solves, badc);
-}
-
-// Per-cell step after a separate sweep (the sweep-ordered pass, the
-// unstructured sweep): one CTA of 8 warps per cell.  Warp w sums the directions [w nd/8, (w+1) nd/8) for every stored
-// band (lanes over band pairs); the 8 partials are added in warp order in
-// shared memory (deterministic), then warp 0 forms
-// G_b = sum_d w_d I^{k+1}_{d,b}, E_L = sum_b G_b / v_b, E_p = sum_b beta_b G_b / v_b
-// and either writes them to Epart (band-range handle, for the caller's
-// all-reduce) or solves T_p and refreshes I0 at once (whole handle).
+// Band sums after a separate sweep (the sweep-ordered pass, the unstructured
+// sweep): one CTA of 8 warps per cell.  Warp w sums the directions
+// [w nd/8, (w+1) nd/8) for every stored band (lanes over band pairs); the 8
+// partials are added in warp order (deterministic) and
+// G_b = sum_d w_d I^{k+1}_{d,b} goes to Gc for cells_kernel.
 // Within a warp the sums over a run of equal-weight directions are exact
 // 64-bit fixed-point additions on the integer pipe (unit 2^(E-50) for the
 // cell's I0 of exponent E; a value up to 32 I0 adds at most 2^55, so a run of
@@ -469,7 +355,6 @@ __global__ void __launch_bounds__(256, 4) gs_reduce_kernel(SweepArgs a, long lon
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nbo = a.th.nbo, nd = a.nd, lpc = nbo / 2;
   const int d0 = (int)((long long)wid * nd / kRedWarps), d1 = (int)((long long)(wid + 1) * nd / kRedWarps);
-  unsigned long long solves = 0, badc = 0;
   for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
     if constexpr (sizeof(S) != 8) {
       reduce_dev_warp<S>(a, reinterpret_cast<const S*>(a.Iout) + P * (long long)nd * nbo, d0, d1, lane, gpart + wid * nbo);
@@ -540,32 +425,14 @@ __global__ void __launch_bounds__(256, 4) gs_reduce_kernel(SweepArgs a, long lon
     }
     }
     __syncthreads();
-    if (wid == 0) {
-      double el = 0.0, ep = 0.0;
-      for (int b = lane; b < nbo; b += 32) {
-        double G = gpart[b];
-        for (int w = 1; w < kRedWarps; ++w) G += gpart[w * nbo + b];
-        if constexpr (sizeof(S) != 8) G = fma(a.Wtot, a.I0ref[b], G);  // the reference part, sum_d w_d I0_b(T_ref)
-        const double e = G * a.th.inv_v[b];
-        el += e;
-        ep = fma(a.th.beta[b], e, ep);
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        el += __shfl_xor_sync(0xffffffffu, el, o);
-        ep += __shfl_xor_sync(0xffffffffu, ep, o);
-      }
-      if (a.partial) {
-        if (lane == 0) {
-          a.Epart[2 * P] = el;
-          a.Epart[2 * P + 1] = ep;
-        }
-      } else {
-        solve_cell_warp(a, P, el, ep, lane, solves, badc);
-      }
+    for (int b = threadIdx.x; b < nbo; b += blockDim.x) {
+      double G = gpart[b];
+      for (int w = 1; w < kRedWarps; ++w) G += gpart[w * nbo + b];
+      if constexpr (sizeof(S) != 8) G = fma(a.Wtot, a.I0ref[b], G);  // the reference part, sum_d w_d I0_b(T_ref)
+      a.Gc[P * nbo + b] = G;
     }
     __syncthreads();
   }
-  if (wid == 0) flush_counters(a, lane, solves, badc);
 }
 
 // Wall ghosts of one side of one geometry from the wall cells' current iterate:
@@ -725,18 +592,9 @@ inline int cell_grid(long long ncells) { return (int)(ncells < 152 * 16 ? (ncell
 int values_per_lane(int precision) { return precision == 0 ? 2 : (precision == 1 ? 4 : 8); }
 
 cudaError_t launch_sweep(int precision, int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s) {
-  if (precision == 0) return launch_sweep_fp64(pd, a, dim, threads, grid, s);
-  if (precision == 1) return launch_sweep_fp32(pd, a, dim, threads, grid, s);
+  if (precision == 0) return launch_sweep_fp64(a, dim, threads, grid, s);
+  if (precision == 1) return launch_sweep_fp32(a, dim, threads, grid, s);
   return launch_sweep_bf16(pd, a, dim, threads, grid, s);
-}
-
-cudaError_t launch_fixup(const SweepArgs& a, const MLPView* mlp, cudaStream_t s) {
-  const size_t sm = (cta_solve_smem_doubles(a.th.nbp) + 2) * sizeof(double) +
-                    (mlp ? (2 * (size_t)a.th.nbp + 4 * kHidden) * sizeof(float) : 0);
-  MLPView m{};
-  if (mlp) m = *mlp;
-  fixup_kernel<<<2 * 152, kFixThreads, sm, s>>>(a, mlp ? 1 : 0, m);  // 76 clusters of kFixCluster CTAs
-  return cudaGetLastError();
 }
 
 namespace {
@@ -781,11 +639,6 @@ cudaError_t launch_partial_ghosts(int precision, const void* I, const double* I0
   return cudaGetLastError();
 }
 
-cudaError_t launch_solve_cells(const SweepArgs& a, long long ncells, cudaStream_t s) {
-  solve_cells_kernel<<<cell_grid(ncells / 4 + 1), 128, 0, s>>>(a, ncells);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells, cudaStream_t s) {
   const int grid = (int)std::min<long long>(std::max(ncells, 1LL), 152LL * 64);
   const size_t sm = (size_t)kRedWarps * a.th.nbo * sizeof(double);
@@ -795,20 +648,18 @@ cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J, double* Msum, double* Tp, double* Te,
-                              double* TL, double* EL, const double* Tcells, const double* I0ref, long long cell0,
-                              int ncells, int nd, ThermoTables th, cudaStream_t s) {
-  const int grid = cell_grid(ncells);
-  const size_t sm = th.nbp * sizeof(double);
-  if (precision == 0)
-    init_cells_kernel<double><<<grid, 256, sm, s>>>((double*)I, I0cell, J, Msum, Tp, Te, TL, EL, Tcells, I0ref, cell0,
-                                                    ncells, nd, th);
-  else if (precision == 1)
-    init_cells_kernel<float><<<grid, 256, sm, s>>>((float*)I, I0cell, J, Msum, Tp, Te, TL, EL, Tcells, I0ref, cell0,
-                                                   ncells, nd, th);
-  else
-    init_cells_kernel<__nv_bfloat16><<<grid, 256, sm, s>>>((__nv_bfloat16*)I, I0cell, J, Msum, Tp, Te, TL, EL, Tcells,
-                                                           I0ref, cell0, ncells, nd, th);
+cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* Tp,
+                              double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
+                              long long cell0, int ncells, int nd, ThermoTables th, cudaStream_t s) {
+  auto go = [&](auto tag) {
+    using T = decltype(tag);
+    init_cells_kernel<T><<<cell_grid(ncells), 256, th.nbp * sizeof(double), s>>>((T*)I, I0cell, J, Msum, Tp, Te, TL, EL, Tcells,
+                                                                                 I0ref, cell0, ncells, nd, th);
+  };
+  if (precision == 0 && state_ff) go(FFElem{});
+  else if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 
@@ -838,28 +689,43 @@ cudaError_t launch_solve_TL(double* TL, const double* EL, const double* Tguess, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_flux_cells(int precision, const void* I, const double* I0ref, double* q, const double* S,
-                              long long cell0, int ncells, int nd, int nbp, int dim, cudaStream_t s) {
+cudaError_t launch_flux_cells(int precision, bool state_ff, const void* I, double* q, const double* S, long long cell0,
+                              int ncells, int nd, int nbp, int dim, cudaStream_t s) {
   const int grid = cell_grid(ncells);
-  const size_t sm = 256 * sizeof(double);
-  if (precision == 0) flux_cells_kernel<double><<<grid, 256, sm, s>>>((const double*)I, I0ref, q, S, cell0, ncells, nd, nbp, dim);
-  else if (precision == 1) flux_cells_kernel<float><<<grid, 256, sm, s>>>((const float*)I, I0ref, q, S, cell0, ncells, nd, nbp, dim);
-  else flux_cells_kernel<__nv_bfloat16><<<grid, 256, sm, s>>>((const __nv_bfloat16*)I, I0ref, q, S, cell0, ncells, nd, nbp, dim);
+  auto go = [&](auto tag, auto vec) {
+    using T = decltype(tag);
+    constexpr int V = decltype(vec)::value;
+    if (dim == 3) flux_cells_kernel<T, V, 3><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
+    else flux_cells_kernel<T, V, 2><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
+  };
+  if (precision == 0 && state_ff) go(FFElem{}, std::integral_constant<int, 2>{});
+  else if (precision == 0) go(double{}, std::integral_constant<int, 2>{});
+  else if (precision == 1) go(float{}, std::integral_constant<int, 4>{});
+  else go(__nv_bfloat16{}, std::integral_constant<int, 8>{});
   return cudaGetLastError();
 }
 
-cudaError_t launch_flux_faces(int precision, const void* I, const double* I0ref, const double* I0wall,
-                              const DevGeom* geoms, int geom, int side, const DirInfo* dirs, const double* S, int nd,
-                              int nbp, double* face_out, int nfaces, cudaStream_t s) {
-  const int grid = cell_grid(nfaces);
-  const size_t sm = 256 * sizeof(double);
-  if (precision == 0)
-    flux_faces_kernel<double><<<grid, 256, sm, s>>>((const double*)I, I0ref, I0wall, geoms, geom, side, dirs, S, nd, nbp, face_out, nfaces);
-  else if (precision == 1)
-    flux_faces_kernel<float><<<grid, 256, sm, s>>>((const float*)I, I0ref, I0wall, geoms, geom, side, dirs, S, nd, nbp, face_out, nfaces);
-  else
-    flux_faces_kernel<__nv_bfloat16><<<grid, 256, sm, s>>>((const __nv_bfloat16*)I, I0ref, I0wall, geoms, geom, side, dirs, S,
-                                                           nd, nbp, face_out, nfaces);
+cudaError_t launch_flux_walls(int precision, bool state_ff, const void* I, const double* I0ref, const double* I0wall,
+                              const DevGeom* geoms, int geom, const DirInfo* dirs, const double* S, int nd, int nbp,
+                              double* face_out, int max_faces, const int (&nfaces)[6], int nsides, double* out,
+                              cudaStream_t s) {
+  int most = 1;
+  SideFaces nf{};
+  for (int k = 0; k < nsides; ++k) {
+    nf.n[k] = nfaces[k];
+    most = std::max(most, nfaces[k]);
+  }
+  const dim3 grid(cell_grid(most), nsides);
+  auto go = [&](auto tag) {
+    using T = decltype(tag);
+    flux_faces_kernel<T><<<grid, kFluxThreads, 0, s>>>((const T*)I, I0ref, I0wall, geoms, geom, dirs, S, nd, nbp, face_out,
+                                                       max_faces);
+  };
+  if (precision == 0 && state_ff) go(FFElem{});
+  else if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
+  mean_kernel<<<nsides, 256, 0, s>>>(face_out, max_faces, nf, out);
   return cudaGetLastError();
 }
 
@@ -872,7 +738,21 @@ __global__ void ff_to_doubles_kernel(ulonglong2* buf, long long npairs) {
     buf[i] = make_ulonglong2((unsigned long long)__double_as_longlong(a), (unsigned long long)__double_as_longlong(b));
   }
 }
+__global__ void doubles_to_ff_kernel(const double2* src, ulonglong2* dst, long long npairs) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npairs; i += (long long)gridDim.x * blockDim.x) {
+    const double2 v = src[i];
+    const ff::P2 p = ff::from_doubles(v.x, v.y);
+    dst[i] = make_ulonglong2(p.h, p.l);
+  }
+}
 }  // namespace
+
+cudaError_t launch_doubles_to_ff(const void* src, void* dst, long long npairs, cudaStream_t s) {
+  if (npairs <= 0) return cudaSuccess;
+  doubles_to_ff_kernel<<<grid_for(npairs, 256), 256, 0, s>>>(reinterpret_cast<const double2*>(src),
+                                                             reinterpret_cast<ulonglong2*>(dst), npairs);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_ff_to_doubles(void* buf, long long npairs, cudaStream_t s) {
   if (npairs <= 0) return cudaSuccess;
@@ -880,31 +760,42 @@ cudaError_t launch_ff_to_doubles(void* buf, long long npairs, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_mean(const double* v, int n, double* out, cudaStream_t s) {
-  mean_kernel<<<1, 256, 256 * sizeof(double), s>>>(v, n, out);
+cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* perm,
+                          long long ncells, int nd, int nb, int nbp, cudaStream_t s) {
+  auto go = [&](auto tag) {
+    using T = decltype(tag);
+    unpack_kernel<T><<<cell_grid(ncells), 256, 0, s>>>((const T*)I, out, I0ref, perm, ncells, nd, nb, nbp);
+  };
+  if (precision == 0 && state_ff) go(FFElem{});
+  else if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(int precision, const double* src, double* dst_out, const void* Isrc, void* Idst,
-                        const double* I0ref, long long ncells, int nd, int nb, int nbp, int to_padded, cudaStream_t s) {
-  const int grid = grid_for(ncells * nd * (long long)nbp, 256);
-  if (precision == 0)
-    pack_kernel<double><<<grid, 256, 0, s>>>(src, dst_out, (const double*)Isrc, (double*)Idst, I0ref, ncells, nd, nb, nbp, to_padded);
-  else if (precision == 1)
-    pack_kernel<float><<<grid, 256, 0, s>>>(src, dst_out, (const float*)Isrc, (float*)Idst, I0ref, ncells, nd, nb, nbp, to_padded);
-  else
-    pack_kernel<__nv_bfloat16><<<grid, 256, 0, s>>>(src, dst_out, (const __nv_bfloat16*)Isrc, (__nv_bfloat16*)Idst, I0ref,
-                                                    ncells, nd, nb, nbp, to_padded);
+cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* perm,
+                        long long ncells, int nd, int nb, int nbp, cudaStream_t s) {
+  auto go = [&](auto tag) {
+    using T = decltype(tag);
+    pack_kernel<T><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, perm, ncells, nd, nb, nbp);
+  };
+  if (precision == 0 && state_ff) go(FFElem{});
+  else if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_L(int precision, const void* I, const double* I0ref, double* EL, const double* wdir,
+cudaError_t launch_energy_L(int precision, bool state_ff, const void* I, const double* I0ref, double* EL, const double* wdir,
                             long long ncells, int nd, ThermoTables th, cudaStream_t s) {
-  const int grid = cell_grid(ncells);
-  const size_t sm = 64 * sizeof(double);
-  if (precision == 0) energy_L_kernel<double><<<grid, 64, sm, s>>>((const double*)I, I0ref, EL, wdir, ncells, nd, th);
-  else if (precision == 1) energy_L_kernel<float><<<grid, 64, sm, s>>>((const float*)I, I0ref, EL, wdir, ncells, nd, th);
-  else energy_L_kernel<__nv_bfloat16><<<grid, 64, sm, s>>>((const __nv_bfloat16*)I, I0ref, EL, wdir, ncells, nd, th);
+  auto go = [&](auto tag) {
+    using T = decltype(tag);
+    energy_L_kernel<T><<<cell_grid(ncells), 64, 64 * sizeof(double), s>>>((const T*)I, I0ref, EL, wdir, ncells, nd, th);
+  };
+  if (precision == 0 && state_ff) go(FFElem{});
+  else if (precision == 0) go(double{});
+  else if (precision == 1) go(float{});
+  else go(__nv_bfloat16{});
   return cudaGetLastError();
 }
 

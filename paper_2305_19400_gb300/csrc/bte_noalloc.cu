@@ -16,6 +16,7 @@
 #include <mutex>
 
 #include "../../include/bte.h"
+#include "bte_flux.cuh"
 #include "bte_internal.h"
 
 namespace bte {
@@ -46,51 +47,16 @@ cudaError_t scratch_address(int dev, double** out) {
   return cudaSuccess;
 }
 
-__device__ double block_sum_static(double v, double* sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  const double r = sh[0];
-  __syncthreads();
-  return r;
-}
-
 // Net outgoing flux through each face of one wall; face sums go to scratch[f].
-__global__ void wall_faces_static_kernel(const double* I, const double* I0wall, const DevGeom* geoms, int geom,
-                                         int side, const DirInfo* dirs, const double* S, int nd, int nbp,
-                                         double* scratch, int nfaces) {
-  __shared__ double sh[256];
+template <typename S>
+__global__ void __launch_bounds__(kFluxThreads) wall_faces_static_kernel(const S* I, const double* I0wall,
+                                                                         const DevGeom* geoms, int geom, int side,
+                                                                         const DirInfo* dirs, const double* Sd, int nd,
+                                                                         int nbp, double* scratch, int nfaces) {
+  __shared__ double sh[kFluxThreads];
   const DevGeom g = geoms[geom];
-  const int ax = side / 2;
-  const double nsign = (side & 1) ? 1.0 : -1.0;
-  const int bc = g.bc[side];
-  const long long f0 = g.face0[side];
   for (int f = blockIdx.x; f < nfaces; f += gridDim.x) {
-    int i, j, k;
-    if (side < 2) { j = f % g.ny; k = f / g.ny; i = (side & 1) ? g.nx - 1 : 0; }
-    else if (side < 4) { i = f % g.nx; k = f / g.nx; j = (side & 1) ? g.ny - 1 : 0; }
-    else { i = f % g.nx; j = f / g.nx; k = (side & 1) ? g.nz - 1 : 0; }
-    const long long P = g.cell0 + i + (long long)g.nx * (j + (long long)g.ny * k);
-    const double* row = I + P * (long long)nd * nbp;
-    double acc = 0.0;
-    for (long long e = threadIdx.x; e < (long long)nd * nbp; e += blockDim.x) {
-      const int d = (int)(e / nbp);
-      const int b = (int)(e - (long long)d * nbp);
-      const double sn = S[3 * d + ax] * nsign;
-      double v;
-      if (sn > 0.0) v = row[e];
-      else if (bc == 0) v = I0wall[(f0 + f) * nbp + b];
-      else if (bc == 3) v = reinterpret_cast<const double*>(g.gdir[side])[(long long)f * nd * nbp + e];
-      else {
-        const int r = ax == 0 ? dirs[d].rx : (ax == 1 ? dirs[d].ry : dirs[d].rz);
-        v = row[(long long)r * nbp + b];
-      }
-      acc = fma(sn, v, acc);
-    }
-    const double t = block_sum_static(acc, sh);
+    const double t = face_flux(I, (const double*)nullptr, I0wall, g, side, f, dirs, Sd, nd, nbp, sh);
     if (threadIdx.x == 0) scratch[f] = t;
   }
 }
@@ -100,7 +66,7 @@ __global__ void wall_mean_static_kernel(double* scratch, int n, int side) {
   __shared__ double sh[256];
   double acc = 0.0;
   for (int e = threadIdx.x; e < n; e += blockDim.x) acc += scratch[e];
-  const double t = block_sum_static(acc, sh);
+  const double t = block_sum(acc, sh);
   if (threadIdx.x == 0) scratch[kNoAllocMaxFaces + side] = t / (double)n;
 }
 
@@ -152,8 +118,12 @@ int wall_flux_on_device(bte_handle h, const FluxView& v, int geom, double* q_wal
   for (int side = 0; side < 2 * v.dim; ++side) {
     const int nf = v.nfaces[side];
     const int grid = nf < 152 * 16 ? nf : 152 * 16;
-    wall_faces_static_kernel<<<grid, 256, 0, v.stream>>>(v.I, v.I0wall, v.geoms, geom, side, v.dirs, v.S, v.nd,
-                                                         v.nbp, scratch, nf);
+    if (v.state_ff)
+      wall_faces_static_kernel<FFElem><<<grid, kFluxThreads, 0, v.stream>>>((const FFElem*)v.I, v.I0wall, v.geoms, geom, side,
+                                                                            v.dirs, v.S, v.nd, v.nbp, scratch, nf);
+    else
+      wall_faces_static_kernel<double><<<grid, kFluxThreads, 0, v.stream>>>((const double*)v.I, v.I0wall, v.geoms, geom, side,
+                                                                            v.dirs, v.S, v.nd, v.nbp, scratch, nf);
     wall_mean_static_kernel<<<1, 256, 0, v.stream>>>(scratch, nf, side);
   }
   e = cudaGetLastError();

@@ -163,8 +163,15 @@ __device__ inline SolveResult exact_solve_warp(const ThermoTables& th, double Ep
 }
 
 // Shared memory (doubles) of exact_solve_cluster, per CTA.
-constexpr int kCtaSolvePairs = 768;  // (band, node) pairs per chunk (42 KB of scratch at most, with 256 bands)
-__host__ __device__ inline int cta_solve_smem_doubles(int nbp) { return 4 * kCtaSolvePairs + 8 * nbp + 4; }
+// (band, node) pairs per chunk of a CTA of a cluster of nr: all of its bands'
+// nodes, 768 (42 KB of scratch with 256 bands) at most.
+__host__ __device__ inline int cta_solve_pairs(int nbp, int ng, int nr) {
+  const int all = (nbp + nr - 1) / nr * ng;
+  return all < 768 ? all : 768;
+}
+__host__ __device__ inline int cta_solve_smem_doubles(int nbp, int ng, int nr) {
+  return 4 * cta_solve_pairs(nbp, ng, nr) + 8 * nbp + 4;
+}
 
 // The same solve by a thread-block cluster, bit for bit the warp form's
 // results.  CTA r of the C in the cluster evaluates the bands
@@ -179,7 +186,7 @@ __host__ __device__ inline int cta_solve_smem_doubles(int nbp) { return 4 * kCta
 // cluster's successive evaluations (par counts them across calls): evaluation
 // k writes buffer k % 2 after the barrier of evaluation k - 1, which every
 // reader of buffer (k - 2) % 2 has passed.  One cell's evaluation thus runs
-// on C SMs' FP64 units.  sm: cta_solve_smem_doubles(nbp) doubles per CTA.
+// on C SMs' FP64 units.  sm: cta_solve_smem_doubles doubles per CTA.
 // Every thread of every CTA of the cluster must call it (it synchronises the
 // cluster).
 __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double Ep, double T0, double trust_rel,
@@ -190,9 +197,9 @@ __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double
   const double* wb = th.a_p;
   const int nbp = th.nbp, ng = th.ng;
   const int own0 = rank * nbp / nr, own1 = (rank + 1) * nbp / nr;  // this CTA's bands
-  const int cb = kCtaSolvePairs / ng;  // bands per chunk (ng <= kMaxGauss)
+  const int pairs = cta_solve_pairs(nbp, ng, nr), cb = pairs / ng;  // bands per chunk (ng <= kMaxGauss)
   double* pt = sm;                        // [4][pairs] node_terms of each pair
-  double* bv2 = pt + 4 * kCtaSolvePairs;  // [2][4][nbp] per band I0 and three derivatives (own bands), two buffers
+  double* bv2 = pt + 4 * pairs;  // [2][4][nbp] per band I0 and three derivatives (own bands), two buffers
   double* sums = bv2 + 8 * nbp;           // [4] this CTA's copy of F and its derivatives
   SolveCtl c(T0);
   for (int loop = 0; loop < maxit + 224 && !c.done; ++loop) {
@@ -201,20 +208,23 @@ __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double
     for (int b0 = own0; b0 < own1; b0 += cb) {
       const int npair = min(cb, own1 - b0) * ng;
       const double* cn = th.node_c + b0 * ng;
+#pragma unroll 1
       for (int p = threadIdx.x; p < npair; p += blockDim.x) {
         double t[4];
         node_terms(cn[p] * rT, t);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) pt[q * kCtaSolvePairs + p] = t[q];
+        for (int q = 0; q < 4; ++q) pt[q * pairs + p] = t[q];
       }
       __syncthreads();
+#pragma unroll 1
       for (int k = threadIdx.x; k < npair / ng; k += blockDim.x) {
         const int b = b0 + k;
         const double* C = th.node_C + b * ng;
         double s[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 2
         for (int i = 0; i < ng; ++i)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) s[q] = fma(C[i], pt[q * kCtaSolvePairs + k * ng + i], s[q]);
+          for (int q = 0; q < 4; ++q) s[q] = fma(C[i], pt[q * pairs + k * ng + i], s[q]);
         const double f[4] = {s[0], s[1] * rT, s[2] * rT * rT, s[3] * rT * rT * rT};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {

@@ -3,6 +3,7 @@
 #pragma once
 #include <cuda_bf16.h>
 
+#include "bte_ff.cuh"
 #include "bte_internal.h"
 
 namespace bte {
@@ -108,12 +109,37 @@ __device__ __forceinline__ void ldgv(const A* p, A (&x)[V]) {
   }
 }
 
+// One 8-byte element of a buffer of ff pairs (bte_ff.cuh: per two bands the 16
+// bytes h_b, h_b+1, l_b, l_b+1), for the kernels that only read intensities.
+struct FFElem {
+  double raw;
+};
+
 // Full intensity value (FP64) of element e of a padded row set (the reduced
 // modes store the deviation from I0_b(T_ref)).
 template <typename S>
 __device__ __forceinline__ double full_I(const S* I, long long e, int b, const double* I0ref) {
   if constexpr (sizeof(S) == 8) return (double)I[e];
   else return I0ref[b] + Tr<S>::to_double(I[e]);
+}
+// Element e of a buffer set to v (a deviation in the reduced modes).
+template <typename S>
+__device__ __forceinline__ void set_I(S* I, long long e, double v) {
+  if constexpr (sizeof(S) == 2) I[e] = __double2bfloat16(v);
+  else I[e] = (S)v;
+}
+template <>
+__device__ __forceinline__ void set_I<FFElem>(FFElem* I, long long e, double v) {
+  float* p = reinterpret_cast<float*>(I) + 4 * (e >> 1) + (e & 1);
+  float h, l;
+  ff::split(v, h, l);
+  p[0] = h;
+  p[2] = l;
+}
+template <>
+__device__ __forceinline__ double full_I<FFElem>(const FFElem* I, long long e, int, const double*) {
+  const float* p = reinterpret_cast<const float*>(I) + 4 * (e >> 1) + (e & 1);
+  return ff::to_double(p[0], p[2]);
 }
 
 }  // namespace bte

@@ -4,7 +4,7 @@
 namespace bte {
 
 cudaError_t launch_sweep_bf16(int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s) {
-  return sweep::launch<__nv_bfloat16>(pd, a, dim, threads, grid, s);
+  return sweep::launch(pd, a, dim, threads, grid, s);
 }
 
 }  // namespace bte

@@ -80,6 +80,32 @@ int build_dirs_inplane(int n, std::vector<double>& S, std::vector<double>& w, st
   return 0;
 }
 
+std::vector<int> internal_order(std::vector<double>& S, std::vector<double>& w, std::vector<int>& refl, int group) {
+  const int n = (int)w.size();
+  std::vector<int> perm;
+  for (int d = 0; d < n; ++d) {
+    if (!(S[3 * d] > 0 && S[3 * d + 1] > 0 && (group == 4 || S[3 * d + 2] > 0))) continue;
+    for (int z = 0; z < group / 4; ++z) {
+      const int q0 = z ? refl[2 * n + d] : d, q1 = refl[q0];
+      for (int q : {q0, q1, refl[n + q1], refl[n + q0]}) perm.push_back(q);
+    }
+  }
+  std::vector<int> inv(n), r2(3 * (size_t)n);
+  std::vector<double> S2(3 * (size_t)n), w2(n);
+  for (int p = 0; p < n; ++p) inv[perm[p]] = p;
+  for (int p = 0; p < n; ++p) {
+    w2[p] = w[perm[p]];
+    for (int c = 0; c < 3; ++c) {
+      S2[3 * p + c] = S[3 * perm[p] + c];
+      r2[c * n + p] = inv[refl[c * n + perm[p]]];
+    }
+  }
+  S.swap(S2);
+  w.swap(w2);
+  refl.swap(r2);
+  return perm;
+}
+
 int build_dirs_polar_azim(int nt, int np, std::vector<double>& S, std::vector<double>& w, std::vector<int>& refl) {
   if (nt < 2 || nt % 2 || np < 4 || np % 4) return -1;
   const int n = nt * np;

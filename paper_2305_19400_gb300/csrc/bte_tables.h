@@ -30,4 +30,13 @@ void build_ff_factored(int dim, const double delta[3], int nd, const double* S, 
 void build_pq(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
               const double* vg, const double* beta, double dt, int explicit_scheme, float* P, float* Q, float* dirc);
 
+// Internal order of a direction set: the directions that differ only in the
+// signs of S stand together, so that one set of sweep coefficients serves
+// consecutive rows.  Groups of four (in-plane sets) by the signs of (S_x, S_y):
+// (+,+), (-,+), (-,-), (+,-); of eight (polar x azimuthal sets): the four with
+// S_z > 0, then their mirror images across z.  Row r of a group so reflects
+// across x to r ^ 1, across y to r ^ 3, across z to r ^ 4.  Returns the
+// caller's index of every internal direction and permutes S, w, refl in place.
+std::vector<int> internal_order(std::vector<double>& S, std::vector<double>& w, std::vector<int>& refl, int group);
+
 }  // namespace bte

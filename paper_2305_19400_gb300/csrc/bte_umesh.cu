@@ -1,7 +1,7 @@
 // bte_umesh.cu -- the hot path on unstructured meshes (include/bte_umesh.h):
 // the face-sum form of Eq. 5 on a face list, then the per-cell reduction,
 // T_p solve and I0 refresh shared with the sweep-ordered scheme
-// (gs_reduce_kernel) and the exact fix-up (fixup_kernel).  FP64 storage.
+// (gs_reduce_kernel, cells_kernel).
 //
 // Device layout (cudaMalloc per array):
 //   I buffers   3 x [cell][dir][nbp]
@@ -451,6 +451,7 @@ struct bte_umesh_ctx {
   int nd = 0;
   std::vector<double> S, w;
   std::vector<int> refl;  // [5][nd]: mirror across x, y, z; rotation about z by -alpha, by +alpha
+  std::vector<int> perm;  // the caller's index of every internal direction
   double Wtot = 0.0;
   // bands
   bool bands_set = false, solve_tp = false;
@@ -475,12 +476,12 @@ struct bte_umesh_ctx {
   float* ghost_dev = nullptr;  // [bface][nbp] ghost deviations (reduced storage)
   float* w32_d = nullptr;  // [nd] direction weights as float
   float* g32 = nullptr;    // [entries][nd] g as float (reduced storage)
-  double *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr, *inv_v = nullptr, *beta_d = nullptr;
-  int *cf_ptr = nullptr, *bf_mirror_d = nullptr, *bf_axis_d = nullptr, *refl_d = nullptr;
+  double *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr, *inv_v = nullptr, *beta_d = nullptr, *binv_d = nullptr;
+  int *cf_ptr = nullptr, *bf_mirror_d = nullptr, *bf_axis_d = nullptr, *refl_d = nullptr, *perm_d = nullptr;
   long long *cf_up = nullptr, *bface_d = nullptr, *owner_d = nullptr, *diff_d = nullptr;
   int ndiff = 0;
   FixItem* fix = nullptr;
-  unsigned* fix_count = nullptr;
+  double* Gc = nullptr;    // [cell][nbp] band sums
   DevCounters* counters = nullptr;
   int lpc = 0, dteam = 1;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -528,6 +529,7 @@ ThermoTables uthermo(const bte_umesh_ctx* u) {
   t.a_L = u->a_L;
   t.inv_v = u->inv_v;
   t.beta = u->beta_d;
+  t.binv_v = u->binv_d;
   t.ng = u->ng;
   t.nbp = t.nbo = u->nbp;
   t.nb = t.nbr = u->nb;
@@ -552,7 +554,8 @@ SweepArgs cell_args(bte_umesh_ctx* u, double* Inew) {
   a.maxit = u->opts.newton_maxit;
   a.counters = u->counters;
   a.fix = u->fix;
-  a.fix_count = u->fix_count;
+  a.Gc = u->Gc;
+  a.gsplit = 1;
   a.partial = 0;
   a.I0ref = u->I0ref;
   a.Wtot = u->Wtot;
@@ -585,11 +588,11 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = dalloc(u, &u->S_d, nd * 3)) || (rc = dalloc(u, &u->w_d, nd)) || (rc = dalloc(u, &u->nA_d, u->nf * 3)) ||
       (rc = dalloc(u, &u->vb_d, nbp)) || (rc = dalloc(u, &u->bb_d, nbp)) || (rc = dalloc(u, &u->scratch, nc)) ||
       (rc = dalloc(u, &u->Qb, nbf)) || (rc = dalloc(u, &u->qbuf, nc * 3)) || (rc = dalloc(u, &u->bf_mirror_d, nbf)) || (rc = dalloc(u, &u->bf_axis_d, nbf)) || (rc = dalloc(u, &u->bf_spec_d, nbf)) || (rc = dalloc(u, &u->bscale, nc)) ||
-      (rc = dalloc(u, &u->refl_d, 5 * nd)) || (rc = dalloc(u, &u->bface_d, nbf)) || (rc = dalloc(u, &u->owner_d, u->nf)) ||
-      (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, nc)) || (rc = dalloc(u, &u->fix_count, 4)) ||
+      (rc = dalloc(u, &u->refl_d, 5 * nd)) || (rc = dalloc(u, &u->perm_d, nd)) || (rc = dalloc(u, &u->bface_d, nbf)) || (rc = dalloc(u, &u->owner_d, u->nf)) ||
+      (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, cells_queue_entries(nc))) || (rc = dalloc(u, &u->Gc, nc * nbp)) ||
       (rc = dalloc(u, &u->counters, 1)) || (rc = dalloc(u, &u->node_c, nbp * u->ng)) ||
       (rc = dalloc(u, &u->node_C, nbp * u->ng)) || (rc = dalloc(u, &u->a_p, nbp)) || (rc = dalloc(u, &u->a_L, nbp)) ||
-      (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->beta_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
+      (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->beta_d, nbp)) || (rc = dalloc(u, &u->binv_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
     return rc;
   // cell -> face entries
   std::vector<int> ptr(nc + 1, 0);
@@ -628,7 +631,7 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = upload(u, ef_d, ent_face.data(), nent)) || (rc = upload(u, ec_d, ent_cell.data(), nent)) ||
       (rc = upload(u, es_d, ent_sign.data(), nent)) || (rc = upload(u, vol_d, u->vol.data(), nc)) ||
       (rc = upload(u, u->nA_d, u->nA.data(), u->nf * 3)) || (rc = upload(u, u->S_d, u->S.data(), nd * 3)) ||
-      (rc = upload(u, u->w_d, u->w.data(), nd)) || (rc = upload(u, u->refl_d, u->refl.data(), 5 * nd)) ||
+      (rc = upload(u, u->w_d, u->w.data(), nd)) || (rc = upload(u, u->perm_d, u->perm.data(), nd)) || (rc = upload(u, u->refl_d, u->refl.data(), 5 * nd)) ||
       (rc = upload(u, u->bface_d, u->bface.data(), nbf)) || (rc = upload(u, u->owner_d, u->owner.data(), u->nf)))
     return rc;
   umesh_geom_kernel<<<grid_for(nent * nd, 256), 256, 0, s>>>(ef_d, es_d, ec_d, u->nA_d, vol_d, u->S_d, u->w_d, (int)nd,
@@ -645,12 +648,13 @@ int ensure_mem(bte_umesh_ctx* u) {
   std::vector<double> nC, nCC, ap, aL, iv, be;
   build_thermo(u->nb, u->nbp, u->ng, u->wlo.data(), u->whi.data(), u->vg.data(), u->beta.data(), u->deg.data(), u->Wtot,
                nC, nCC, ap, aL, iv, be);
-  std::vector<double> vbp(nbp, 0.0), bbp(nbp, 0.0);
-  for (int b = 0; b < u->nb; ++b) { vbp[b] = u->vg[b]; bbp[b] = u->beta[b]; }
+  std::vector<double> vbp(nbp, 0.0), bbp(nbp, 0.0), biv(nbp, 0.0);
+  for (int b = 0; b < u->nb; ++b) { vbp[b] = u->vg[b]; bbp[b] = u->beta[b]; biv[b] = be[b] * iv[b]; }
   if ((rc = upload(u, u->node_c, nC.data(), nC.size())) || (rc = upload(u, u->node_C, nCC.data(), nCC.size())) ||
       (rc = upload(u, u->a_p, ap.data(), ap.size())) || (rc = upload(u, u->a_L, aL.data(), aL.size())) ||
       (rc = upload(u, u->inv_v, iv.data(), iv.size())) || (rc = upload(u, u->beta_d, be.data(), be.size())) ||
-      (rc = upload(u, u->vb_d, vbp.data(), nbp)) || (rc = upload(u, u->bb_d, bbp.data(), nbp)))
+      (rc = upload(u, u->vb_d, vbp.data(), nbp)) || (rc = upload(u, u->bb_d, bbp.data(), nbp)) ||
+      (rc = upload(u, u->binv_d, biv.data(), nbp)))
     return rc;
   for (int i = 0; i < 3; ++i) UTRY(u, cudaMemsetAsync(u->I[i], 0, (size_t)(nc * nd * nbp) * eb, s));
   UTRY(u, cudaMemsetAsync(u->ghost, 0, (size_t)std::max(nbf * nbp, 1LL) * 8, s));
@@ -664,7 +668,6 @@ int ensure_mem(bte_umesh_ctx* u) {
     UTRY(u, launch_wall_I0(u->I0ref, u->scratch, 1, uthermo(u), s));
   }
   UTRY(u, cudaMemsetAsync(u->counters, 0, sizeof(DevCounters), s));
-  UTRY(u, cudaMemsetAsync(u->fix_count, 0, 4, s));
   UTRY(u, cudaStreamSynchronize(s));
   u->lpc = u->nbp / values_per_lane(u->prec);
   u->dteam = std::max(1, std::min(256 / u->lpc, u->nd));
@@ -813,6 +816,7 @@ int bte_umesh_create(const bte_umesh_desc* m, const bte_opts* opts, bte_umesh* o
     delete u;
     return ufail(nullptr, BTE_E_ARG, "bad direction set");
   }
+  u->perm = internal_order(u->S, u->w, u->refl, o.dir_kind == BTE_DIRS_INPLANE ? 4 : 8);
   u->nd = (int)u->w.size();
   u->refl.resize(5 * (size_t)u->nd);
   for (int d = 0; d < u->nd; ++d) u->refl[3 * u->nd + d] = u->refl[4 * u->nd + d] = d;  // until a rotation is set
@@ -932,7 +936,7 @@ int bte_umesh_set_initial(bte_umesh u, const double* T_cells, double T_uniform) 
   int rc = upload(u, u->scratch, T.data(), u->nc);
   if (rc) return rc;
   u->cur = 0;
-  UTRY(u, launch_init_cells(u->prec, u->I[0], u->I0cell, u->J, u->Msum, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
+  UTRY(u, launch_init_cells(u->prec, false, u->I[0], u->I0cell, u->J, u->Msum, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
                             (int)u->nc, u->nd, uthermo(u), u->stream));
   UTRY(u, cudaStreamSynchronize(u->stream));
   u->init_done = true;
@@ -1025,7 +1029,6 @@ int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, b
       a.Ikd = a.Ik;
       a.Ioutd = a.Iout;
       a.Boutd = a.Bout;
-      UTRY(u, cudaMemsetAsync(u->fix_count, 0, 4, s));
       UTRY(u, refresh_diffuse(u, a.Ik));
       if (tt) {  // beta_b(T_p) of the current T_p, as the oracle takes it
         UTRY(u, launch_beta_scale(u->bscale, u->Tp, u->opts.T_ref, u->opts.beta_T_exp, u->nc, s));
@@ -1035,8 +1038,8 @@ int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, b
       }
       SweepArgs c = cell_args(u, a.Iout);
       UTRY(u, launch_gs_reduce(u->prec, c, u->nc, s));
-      if (u->solve_tp) UTRY(u, launch_fixup(c, nullptr, s));
-      launches += 2 + (u->solve_tp ? 1 : 0) + (u->ndiff ? 1 : 0) + (tt ? 1 : 0);
+      UTRY(u, launch_cells(c, u->nc, 0, nullptr, s));
+      launches += 3 + (u->ndiff ? 1 : 0) + (tt ? 1 : 0);
       k = o;
     }
     u->cur = k;
@@ -1086,20 +1089,21 @@ int bte_umesh_get_T(bte_umesh u, int which, double* out, int on_device) {
 int bte_umesh_get_intensity(bte_umesh u, double* out) {
   if (!u || !out) return u ? ufail(u, BTE_E_ARG, "out is NULL") : BTE_E_ARG;
   if (!u->init_done) return ufail(u, BTE_E_STATE, "no state");
-  if (u->prec == BTE_FP64) {
-    UTRY(u, cudaMemcpy2DAsync(out, (size_t)u->nb * 8, u->I[u->cur], (size_t)u->nbp * 8, (size_t)u->nb * 8,
-                              (size_t)(u->nc * u->nd), cudaMemcpyDeviceToHost, u->stream));
-    UTRY(u, cudaStreamSynchronize(u->stream));
-    return BTE_OK;
-  }
-  // reduced storage: full FP64 values (I0_b(T_ref) + deviation) through a temporary device buffer
+  // full FP64 values in the caller's direction order through a temporary device
+  // buffer of at most 64 MB (whole cells)
   double* tmp = nullptr;
-  const size_t n = (size_t)(u->nc * u->nd) * u->nb;
-  cudaError_t e = cudaMalloc(&tmp, n * 8);
-  if (e != cudaSuccess) return ufail(u, BTE_E_NOMEM, "cudaMalloc(%zu bytes): %s", n * 8, cudaGetErrorString(e));
-  e = launch_pack(u->prec, nullptr, tmp, u->I[u->cur], nullptr, u->I0ref, u->nc, u->nd, u->nb, u->nbp, 0, u->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, n * 8, cudaMemcpyDeviceToHost, u->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(u->stream);
+  const size_t cell = (size_t)u->nd * u->nb;
+  const long long chunk = std::max(1LL, std::min<long long>(u->nc, (64LL << 20) / (long long)(cell * 8)));
+  cudaError_t e = cudaMalloc(&tmp, chunk * cell * 8);
+  if (e != cudaSuccess) return ufail(u, BTE_E_NOMEM, "cudaMalloc(%zu bytes): %s", chunk * cell * 8, cudaGetErrorString(e));
+  const size_t eb = u->prec == BTE_FP64 ? 8 : (u->prec == BTE_FP32 ? 4 : 2);
+  for (long long c0 = 0; c0 < u->nc && e == cudaSuccess; c0 += chunk) {
+    const long long m = std::min(chunk, u->nc - c0);
+    e = launch_unpack(u->prec, false, (const char*)u->I[u->cur] + (size_t)c0 * u->nd * u->nbp * eb, tmp, u->I0ref, u->perm_d, m,
+                      u->nd, u->nb, u->nbp, u->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(out + c0 * cell, tmp, m * cell * 8, cudaMemcpyDeviceToHost, u->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(u->stream);
+  }
   cudaFree(tmp);
   if (e != cudaSuccess) return ufail(u, BTE_E_CUDA, "reading the intensities: %s", cudaGetErrorString(e));
   return BTE_OK;
@@ -1119,10 +1123,10 @@ int bte_umesh_set_intensity(bte_umesh u, const double* in, const double* Tp_cell
   if (e != cudaSuccess) return ufail(u, BTE_E_NOMEM, "cudaMalloc(%zu bytes): %s", n * 8, cudaGetErrorString(e));
   e = cudaMemcpyAsync(tmp, in, n * 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess)
-    e = launch_pack(u->prec, tmp, nullptr, nullptr, u->I[u->cur], u->I0ref, u->nc, u->nd, u->nb, u->nbp, 1, s);
+    e = launch_pack(u->prec, false, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(u->Tp, Tp_cells, u->nc * 8, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = launch_state_from_Tp(u->I0cell, u->J, u->Msum, u->Tp, u->Teval, u->nc, uthermo(u), s);
-  if (e == cudaSuccess) e = launch_energy_L(u->prec, u->I[u->cur], u->I0ref, u->EL, u->w_d, u->nc, u->nd, uthermo(u), s);
+  if (e == cudaSuccess) e = launch_energy_L(u->prec, false, u->I[u->cur], u->I0ref, u->EL, u->w_d, u->nc, u->nd, uthermo(u), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(tmp);
   if (e != cudaSuccess) return ufail(u, BTE_E_CUDA, "restoring the state: %s", cudaGetErrorString(e));
@@ -1136,7 +1140,7 @@ int bte_umesh_get_flux(bte_umesh u, double* q, double* Q) {
   cudaStream_t s = u->stream;
   const double* I = u->I[u->cur];
   if (q) {
-    UTRY(u, launch_flux_cells(u->prec, I, u->I0ref, u->qbuf, u->S_d, 0, (int)u->nc, u->nd, u->nbp, 3, s));
+    UTRY(u, launch_flux_cells(u->prec, false, I, u->qbuf, u->S_d, 0, (int)u->nc, u->nd, u->nbp, 3, s));
     UTRY(u, cudaMemcpyAsync(q, u->qbuf, (size_t)u->nc * 3 * 8, cudaMemcpyDeviceToHost, s));
     UTRY(u, cudaStreamSynchronize(s));
   }
