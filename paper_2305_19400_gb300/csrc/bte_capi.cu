@@ -99,12 +99,13 @@ struct bte_ctx {
   float* band_ff = nullptr;   // [2][nbp] 1/(v_b dt), beta_b/v_b pairs
   double *J = nullptr, *Teval = nullptr, *I0ref = nullptr, *scratch_pack = nullptr;
   double* Msum = nullptr;     // [cell][4] the T_p model's sums sum_b a_p,b J_k,b
+  double* MsumL = nullptr;    // [cell][4] the same with the T_L weights
   double* I0ref_o = nullptr;  // I0_b(T_ref) of the stored bands (aliases I0ref unless a band range is set)
   double* Epart = nullptr;    // band-range handles: [ncells][2] partial (E_L, E_p) for the exchange
   float *I0wall_dev = nullptr, *wdir32 = nullptr, *vb32 = nullptr, *bb32 = nullptr;
   float4* dirc = nullptr;
   FixItem* fix = nullptr;
-  double* Gc = nullptr;       // [cell][team][nbp] band sums of the sweeps
+  double2* Ec = nullptr;      // [cell][entries] partial energies of the sweeps
   void* I0wall_ff = nullptr;  // FP64: [face][nbp] isothermal ghosts as ff pairs
   // learned guess: parameters of nets A and B, Adam state, normalisation
   float *mlp_p = nullptr, *mlp_g = nullptr, *mlp_m = nullptr, *mlp_v = nullptr;
@@ -117,7 +118,7 @@ struct bte_ctx {
   double* scratch_q = nullptr;
   std::vector<DevGeom> dgeoms;
   DirInfo* dirs_d = nullptr;
-  int* perm_d = nullptr;
+  int* rows_d = nullptr;
   int* wall_dirs_d = nullptr;   // [6][nd] per side: leaving directions, then the rest
   std::array<WallDirs, 6> wall_dirs{};
   DevGeom* geoms_d = nullptr;
@@ -220,6 +221,7 @@ size_t carve(bte_ctx* h, char* base) {
   h->J = (double*)take((size_t)h->ncells * 4 * h->nbp_all * 8);
   h->Teval = (double*)take((size_t)h->ncells * 8);
   h->Msum = (double*)take((size_t)h->ncells * 4 * 8);
+  h->MsumL = (double*)take((size_t)h->ncells * 4 * 8);
   h->I0ref = (double*)take((size_t)h->nbp_all * 8);
   const bool ranged = h->nb != h->nb_all;
   h->I0ref_o = ranged ? (double*)take((size_t)h->nbp * 8) : h->I0ref;
@@ -238,7 +240,8 @@ size_t carve(bte_ctx* h, char* base) {
   h->vb32 = (float*)take((size_t)h->nbp * 4);
   h->bb32 = (float*)take((size_t)h->nbp * 4);
   h->fix = (FixItem*)take((size_t)cells_queue_entries(h->ncells) * sizeof(FixItem));
-  h->Gc = (double*)take((size_t)std::max(h->ncells, 1LL) * max_teams(h) * h->nbp * 8);
+  h->Ec = (double2*)take((size_t)std::max(h->ncells, 1LL) *
+                         std::max(kRedEntries, max_teams(h) * h->nbp / values_per_lane(h->opts.precision)) * 16);
   h->I0wall_ff = h->opts.precision == BTE_FP64 ? take((size_t)std::max(h->nfaces, 1LL) * h->nbp * 8) : nullptr;
   const size_t np = (size_t)mlp_param_total(h->nb_all);
   h->mlp_p = (float*)take(np * 4);
@@ -252,7 +255,7 @@ size_t carve(bte_ctx* h, char* base) {
   h->Sdev = (double*)take((size_t)h->nd * 3 * 8);
   h->dirs_d = (DirInfo*)take((size_t)h->nd * sizeof(DirInfo));
   h->wall_dirs_d = (int*)take((size_t)h->nd * 6 * 4);
-  h->perm_d = (int*)take((size_t)h->nd * 4);
+  h->rows_d = (int*)take((size_t)h->nd * 4);
   h->node_c = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->node_C = (double*)take((size_t)h->nbp_all * h->ng * 8);
   h->a_p = (double*)take((size_t)h->nbp_all * 8);
@@ -290,8 +293,8 @@ void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
   if (dteam > 0) h->dteam = dteam;
   else if (h->opts.precision == BTE_BF16)  // ~896 contiguous bytes of a row, at least ~32 steps per lane
     h->dteam = std::max(1, std::min(std::min(896 / rowb, 256 / h->lpc), h->nd / 32));
-  else
-    h->dteam = h->dir_group == 4 ? 1 : 2;
+  else  // IEEE sweeps share a block's coefficients over all of its rows: they wait for the FP64 pipe
+    h->dteam = h->dir_group == 4 || (h->opts.precision == BTE_FP64 && (h->opts.fp64_strict || h->opts.beta_T_exp != 0.0)) ? 1 : 2;
   const int team = h->lpc * h->dteam;
   // default: the most cells whose CTA (at most 256 threads) is whole warps, else
   // the most that fit; small grids take fewer, so that every SM has two CTAs
@@ -417,7 +420,9 @@ int ensure_memory(bte_ctx* h) {
     std::reverse(l + wd.nout, l + h->nd);
     wd.rest = wd.out + wd.nout;
   }
-  CUDA_TRY(h, cudaMemcpyAsync(h->perm_d, h->perm.data(), h->perm.size() * 4, cudaMemcpyHostToDevice, s));
+  std::vector<int> rows(h->perm.size());  // the internal row of each of the caller's directions
+  for (size_t p = 0; p < rows.size(); ++p) rows[h->perm[p]] = (int)p;
+  CUDA_TRY(h, cudaMemcpyAsync(h->rows_d, rows.data(), rows.size() * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->wall_dirs_d, wl.data(), wl.size() * 4, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->wdir, h->w.data(), h->nd * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->Sdev, h->S.data(), h->nd * 3 * 8, cudaMemcpyHostToDevice, s));
@@ -567,15 +572,6 @@ bool ready_to_step(bte_ctx* h, std::string& why) {
   return true;
 }
 
-int ensure_TL(bte_ctx* h) {
-  if (h->TL_valid) return BTE_OK;
-  // warm start from T_p (or the previous T_L when T_p is not solved)
-  CUDA_TRY(h, launch_solve_TL(h->TL, h->EL, h->solve_tp ? h->Tp : h->TL, h->J, h->Teval, h->ncells, thermo(h),
-                              model_trust(h->opts.newton_rtol), h->opts.newton_maxit, h->counters, h->stream));
-  h->TL_valid = true;
-  return BTE_OK;
-}
-
 int copy_out(bte_ctx* h, double* out, const double* src, size_t n, int on_device) {
   CUDA_TRY(h, cudaMemcpyAsync(out, src, n * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -608,6 +604,9 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.Teval = h->Teval;
   a.J = h->J;
   a.Msum = h->Msum;
+  a.MsumL = h->MsumL;
+  a.TL = h->TL;
+  a.Tguess = h->solve_tp ? h->Tp : h->TL;  // or the previous T_L when T_p is not solved
   a.EL = h->EL;
   a.I0wall = h->I0wall;
   a.I0wall_dev = h->I0wall_dev;
@@ -630,7 +629,7 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.lpc = h->lpc;
   a.dteam = h->dteam;
   a.dir_group = h->dir_group;
-  a.gsplit = h->opts.precision == BTE_BF16 ? 1 : h->dteam;
+  a.ne = h->lpc * (h->opts.precision == BTE_BF16 ? 1 : h->dteam);
   a.solve_tp = h->solve_tp ? 1 : 0;
   a.trust_rel = model_trust(h->opts.newton_rtol);
   a.maxit = h->opts.newton_maxit;
@@ -644,7 +643,7 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.vb32 = h->vb32;
   a.bb32 = h->bb32;
   a.fix = h->fix;
-  a.Gc = h->Gc;
+  a.Ec = h->Ec;
   a.gs_units = h->gs_units_d;
   a.gs_dirs = h->gs_dirs_d;
   a.gs_nunits = (int)h->gs_units.size();
@@ -654,6 +653,13 @@ SweepArgs sweep_args(bte_ctx* h) {
   a.bscale = h->bscale;
   a.th = thermo(h);
   return a;
+}
+
+int ensure_TL(bte_ctx* h) {
+  if (h->TL_valid) return BTE_OK;
+  CUDA_TRY(h, launch_cells(sweep_args(h), h->ncells, 3, nullptr, h->stream));
+  h->TL_valid = true;
+  return BTE_OK;
 }
 
 // Diffuse wall ghosts from intensity buffer I (before a sweep that reads I as
@@ -742,7 +748,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
   const bool use_ff = h->state_ff;  // bte_step has put the state in the form of this scheme
   const bool use_b = h->opts.precision == BTE_FP64 && !use_ff && !a.explicit_scheme && ninner >= 2;
   a.ff = use_ff ? 1 : 0;
-  if (scheme == BTE_IMPLICIT_GS) a.gsplit = 1;
+  if (scheme == BTE_IMPLICIT_GS) a.ne = kRedEntries;
   int z = -1;
   for (int it = 0; it < ninner; ++it) {
     int o = 0;
@@ -835,7 +841,7 @@ int flux_view(bte_ctx* h, int geom, FluxView* out) {
   }
   out->I0wall = h->I0wall;
   out->geoms = h->geoms_d;
-  out->dirs = h->dirs_d;
+  std::copy(h->wall_dirs.begin(), h->wall_dirs.end(), out->wall_dirs);
   out->S = h->Sdev;
   out->nd = h->nd;
   out->nbp = h->nbp;
@@ -1119,7 +1125,7 @@ int bte_set_initial(bte_handle h, int geom, const double* T_cells, double T_unif
   if (std::none_of(h->init_set.begin(), h->init_set.end(), [](bool x) { return x; }))
     h->state_ff = h->opts.precision == BTE_FP64 && !h->opts.fp64_strict && h->opts.beta_T_exp == 0.0;
   CUDA_TRY(h, cudaMemcpyAsync(h->scratch_T, T.data(), nc * 8, cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->state_ff, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->Tp, h->Teval, h->TL, h->EL,
+  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->state_ff, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->MsumL, h->Tp, h->Teval, h->TL, h->EL,
                                 h->scratch_T, h->I0ref_o, h->cell0[geom], (int)nc, h->nd, thermo(h), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->init_set[geom] = true;
@@ -1449,7 +1455,7 @@ int bte_get_flux(bte_handle h, int geom, double* q_cells, double* q_walls, int o
   cudaStream_t s = h->stream;
   if (q_cells) {
     double* q = on_device ? q_cells : h->scratch_q;
-    CUDA_TRY(h, launch_flux_cells(prec, h->state_ff, I, q, h->Sdev, h->cell0[geom], nc, h->nd, h->nbp, g.dim, s));
+    CUDA_TRY(h, launch_flux_cells(prec, h->state_ff, true, I, q, h->Sdev, h->cell0[geom], nc, h->nd, h->nbp, g.dim, s));
     if (!on_device) CUDA_TRY(h, cudaMemcpyAsync(q_cells, q, (size_t)nc * g.dim * 8, cudaMemcpyDeviceToHost, s));
   }
   if (q_walls) {
@@ -1458,7 +1464,7 @@ int bte_get_flux(bte_handle h, int geom, double* q_cells, double* q_walls, int o
     for (int side = 0; side < 2 * g.dim; ++side) nf[side] = (int)side_faces(g, side);
     CUDA_TRY(h, refresh_diffuse(h, I, s));  // diffuse and partially specular ghosts of the current state
     CUDA_TRY(h, refresh_partial(h, I, s));
-    CUDA_TRY(h, launch_flux_walls(prec, h->state_ff, I, h->I0ref_o, h->I0wall, h->geoms_d, geom, h->dirs_d, h->Sdev, h->nd,
+    CUDA_TRY(h, launch_flux_walls(prec, h->state_ff, I, h->I0ref_o, h->I0wall, h->geoms_d, geom, h->wall_dirs.data(), h->Sdev, h->nd,
                                   h->nbp, h->scratch_faces, h->max_side_faces, nf, 2 * g.dim, h->scratch_out, s));
     CUDA_TRY(h, cudaMemcpyAsync(res, h->scratch_out, 2 * g.dim * 8, cudaMemcpyDeviceToHost, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
@@ -1482,7 +1488,7 @@ int bte_get_intensity(bte_handle h, int geom, double* out, int on_device) {
   for (long long c0 = 0; c0 < nc; c0 += on_device ? nc : h->pack_cells) {
     const long long n = on_device ? nc : std::min(h->pack_cells, nc - c0);
     double* dst = on_device ? out : h->scratch_pack;
-    CUDA_TRY(h, launch_unpack(prec, h->state_ff, I + (size_t)c0 * h->nd * h->nbp * es, dst, h->I0ref_o, h->perm_d, n, h->nd,
+    CUDA_TRY(h, launch_unpack(prec, h->state_ff, I + (size_t)c0 * h->nd * h->nbp * es, dst, h->I0ref_o, h->rows_d, n, h->nd,
                               h->nb, h->nbp, h->stream));
     if (!on_device)
       CUDA_TRY(h, cudaMemcpyAsync(out + (size_t)c0 * h->nd * h->nb, dst, (size_t)n * h->nd * h->nb * 8,
@@ -1503,6 +1509,10 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   const size_t es = elem_bytes(prec);
   char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
   cudaStream_t s = h->stream;
+  CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+  CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
+                                   h->Msum + h->cell0[geom] * 4, h->MsumL + h->cell0[geom] * 4,
+                                   h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));
   for (long long c0 = 0; c0 < nc; c0 += on_device ? nc : h->pack_cells) {
     const long long n = on_device ? nc : std::min(h->pack_cells, nc - c0);
     const double* src = in + (size_t)c0 * h->nd * h->nb;
@@ -1510,18 +1520,16 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
       CUDA_TRY(h, cudaMemcpyAsync(h->scratch_pack, src, (size_t)n * h->nd * h->nb * 8, cudaMemcpyHostToDevice, s));
       src = h->scratch_pack;
     }
-    CUDA_TRY(h, launch_pack(prec, h->state_ff, src, I + (size_t)c0 * h->nd * h->nbp * es, h->I0ref_o, h->perm_d, n, h->nd, h->nb, h->nbp, s));
+    char* dst = I + (size_t)c0 * h->nd * h->nbp * es;
+    SweepArgs a = sweep_args(h);  // these cells' energies
+    a.Iout = dst;
+    a.I0cell = h->I0cell + (h->cell0[geom] + c0) * h->nbp;
+    a.Ec = h->Ec + (h->cell0[geom] + c0) * kRedEntries;
+    CUDA_TRY(h, launch_pack(prec, h->state_ff, src, dst, h->I0ref_o, h->rows_d, n, h->nd, h->nb, h->nbp, h->Epart ? nullptr : &a, s));
     if (!on_device) CUDA_TRY(h, cudaStreamSynchronize(s));  // the caller's pageable memory and the staging buffer are reused
   }
-  CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-  CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
-                                   h->Msum + h->cell0[geom] * 4,
-                                   h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));
-  if (h->Epart) {
-    h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange
-  } else {
-    CUDA_TRY(h, launch_energy_L(prec, h->state_ff, I, h->I0ref_o, h->EL + h->cell0[geom], h->wdir, nc, h->nd, thermo(h), s));
-  }
+  if (h->Epart) h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange
+  else CUDA_TRY(h, launch_energy_L(h->Ec + h->cell0[geom] * kRedEntries, h->EL + h->cell0[geom], nc, s));
   CUDA_TRY(h, cudaStreamSynchronize(s));
   h->TL_valid = false;
   h->bscale_valid = false;

@@ -23,38 +23,44 @@ __device__ __forceinline__ double block_sum(double v, double* sh) {
 
 // Net outgoing flux sum_b sum_d (S_d . n_out) I_face through face f of a side,
 // by a CTA of kFluxThreads threads (every thread calls it; the sum is returned
-// to all).  A thread keeps one band and walks every (threads / nbp)-th
-// direction, four loads in flight and no index division; a ghost that does not
-// depend on the direction is read once.  One thread per (direction, band)
-// element with a 64-bit division each took 58-69 us per side of the 128x128 x
-// 400 x 55 grid.
+// to all).  Lane l of group g holds two bands and sums every groups-th leaving
+// direction of the side's list, eight loads in flight; what enters is the ghost
+// row times the sum of the entering weights (isothermal, diffuse), the leaving
+// values themselves (mirror: their difference, zero unless not finite), or the
+// face's per-direction ghosts (partially specular).  Bound by one face's
+// latency.  Walking all directions and testing each took 116 us for the four
+// sides of the 128x128 x 400 x 55 grid, 385 us for the six of a 23x18x13 one.
 template <typename S>
 __device__ double face_flux(const S* I, const double* I0ref, const double* I0wall, const DevGeom& g, int side, int f,
-                            const DirInfo* dirs, const double* Sd, int nd, int nbp, double* sh) {
+                            const WallDirs& wd, const double* Sd, int nd, int nbp, double* sh) {
   const int ax = side / 2;
   const double nsign = (side & 1) ? 1.0 : -1.0;
   int i, j, k;
   if (side < 2) { j = f % g.ny; k = f / g.ny; i = (side & 1) ? g.nx - 1 : 0; }
   else if (side < 4) { i = f % g.nx; k = f / g.nx; j = (side & 1) ? g.ny - 1 : 0; }
   else { i = f % g.nx; j = f / g.nx; k = (side & 1) ? g.nz - 1 : 0; }
-  const long long base = (g.cell0 + i + (long long)g.nx * (j + (long long)g.ny * k)) * nd * nbp;
-  const int rows = kFluxThreads / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
+  const int lpc = nbp / 2, groups = kFluxThreads / lpc, grp = threadIdx.x / lpc, b = 2 * (threadIdx.x - grp * lpc);
+  const S* row = I + (g.cell0 + i + (long long)g.nx * (j + (long long)g.ny * k)) * nd * nbp + b;
   const int bc = g.bc[side];
   double acc = 0.0;
-  if (r < rows) {
-    const double gv = bc == 0 ? I0wall[(g.face0[side] + f) * nbp + b] : 0.0;
-    const S* gd = bc == 3 ? reinterpret_cast<const S*>(g.gdir[side]) : nullptr;
-#pragma unroll 4
-    for (int d = r; d < nd; d += rows) {
-      const double sn = Sd[3 * d + ax] * nsign;
-      double v = gv;
-      if (sn > 0.0 || bc == 1) {
-        const int m = sn > 0.0 ? d : (ax == 0 ? dirs[d].rx : (ax == 1 ? dirs[d].ry : dirs[d].rz));
-        v = full_I(I, base + (long long)m * nbp + b, b, I0ref);
-      } else if (bc == 3) {
-        v = full_I(gd, ((long long)f * nd + d) * nbp + b, b, I0ref);
+  if (grp < groups) {
+    auto walk = [&](const S* from, const int* list, int n, bool diff) {
+#pragma unroll 8
+      for (int q = grp; q < n; q += groups) {
+        const int d = list[q];
+        double x0, x1;
+        ld_pair(from + (long long)d * nbp, x0, x1);
+        acc = fma(Sd[3 * d + ax] * nsign, diff ? (x0 - x0) + (x1 - x1) : x0 + x1, acc);
       }
-      acc = fma(sn, v, acc);
+    };
+    walk(row, wd.out, wd.nout, bc == 1);
+    if (bc == 3) walk(reinterpret_cast<const S*>(g.gdir[side]) + (long long)f * nd * nbp + b, wd.rest, nd - wd.nout, false);
+    if (grp == 0 && bc != 1) {
+      const double* gw = I0wall + (g.face0[side] + f) * nbp + b;
+      double ref = 0.0;  // the reference part of the reduced modes' storage
+      if constexpr (sizeof(S) != 8) ref = I0ref[b] + I0ref[b + 1];
+      acc = fma(wd.sum_out, ref, acc);
+      acc = fma(-wd.sum_in, bc == 3 ? ref : gw[0] + gw[1], acc);
     }
   }
   return block_sum(acc, sh);

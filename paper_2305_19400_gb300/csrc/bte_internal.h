@@ -119,9 +119,12 @@ struct SweepArgs {
   double* I0cell;           // [cell][nbp] in: I0^k, out: I0^{k+1}
   double* Tp;               // [cell] in/out
   double* Teval;            // [cell] evaluation point of the cached quadrature model
-  double* J;                // [cell][4][nbp] I0 and its first three derivatives at Teval
+  double* J;                // [cell][4][nbp] Taylor coefficients of I0_b(T) at Teval, to third order
   double* Msum;             // [cell][4] sum_b a_p,b J_k,b: the T_p model's sums, kept with J
+  double* MsumL;            // [cell][4] the same with the T_L weights
   double* EL;               // [cell] out
+  double* TL;               // [cell] T_L (on request)
+  const double* Tguess;     // [cell] its start where the model has no root
   const double* I0wall;     // [face][nbp] FP64 ghosts
   const void* I0wall_ff;    // [face][nbp] FP64 ghosts as ff pairs (bte_ff.cuh)
   const float* I0wall_dev;  // [face][nbp] FP32 ghosts minus I0ref (reduced modes)
@@ -138,7 +141,7 @@ struct SweepArgs {
   const float4* dirc;       // reduced: [cls][nd] (c_x, c_y, c_z, sum), c_ax = |S_d,ax|/(w_d Delta_ax)
   const float* vb32;        // [nbp] v_b (reduced)
   const float* bb32;        // [nbp] beta_b (reduced)
-  double* Gc;               // [cell][gsplit][nbo] band sums G_b, written by the sweeps, added by cells_kernel
+  double2* Ec;              // [cell][ne] partial (E_L, E_p), written by the sweeps (one per lane), added by cells_kernel
   FixItem* fix;             // cells_kernel's queue of exact solves, a part per CTA
   const DirInfo* dirs;
   const double* wdir;       // [nd]
@@ -150,7 +153,7 @@ struct SweepArgs {
   int lpc;                  // lanes per direction row = nbp / values per lane
   int dteam;                // directions one cell team covers per step (team = lpc * dteam lanes)
   int dir_group;            // rows that differ only in the signs of S: 4 (in-plane sets) or 8 (internal_order)
-  int gsplit;               // partial band sums per cell in Gc (the teams of a cell)
+  int ne;                   // entries per cell in Ec
   int solve_tp;             // 0 when every beta_b == 0 (T_p then unused)
   double trust_rel;         // cached model accepted when |T - T_e| <= trust_rel * T
   int maxit;
@@ -186,13 +189,14 @@ cudaError_t launch_sweep_fp64(const SweepArgs& a, int dim, int threads, int grid
 cudaError_t launch_sweep_fp32(const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
 cudaError_t launch_sweep_bf16(int pd, const SweepArgs& a, int dim, int threads, int grid, cudaStream_t s);
 struct MLPView;
-// per-cell step (bte_cells.cu): mode 0 energies from Gc and solve, 1 energies
-// from Gc to Epart, 2 solve from Epart
+// per-cell step (bte_cells.cu): mode 0 energies from Ec and T_p, 1 energies from
+// Ec to Epart, 2 T_p from Epart, 3 T_L from E_L
 cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const MLPView* mlp, cudaStream_t s);
 int cells_grid(long long ncells);
 long long cells_queue_entries(long long ncells);  // FixItems of a.fix
-// sweep-ordered pass (bte_gs.cu) and its band sums (bte_kernels.cu): the pass
-// writes Iout, the reduction G_b of every cell to Gc
+// sweep-ordered pass (bte_gs.cu) and its sums (bte_kernels.cu): the pass writes
+// Iout, the reduction kRedEntries partial energies per cell to Ec
+constexpr int kRedEntries = 8;
 cudaError_t launch_gs_sweep(int precision, const SweepArgs& a, int dim, int threads, cudaStream_t s);
 cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells, cudaStream_t s);
 cudaError_t launch_beta_scale(double* out, const double* Tp, double Tref, double p, long long ncells, cudaStream_t s);
@@ -216,23 +220,20 @@ cudaError_t mlp_forward_backward(const float* p, int k, const float* X, int ldx,
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s);
 cudaError_t launch_solve_batch(ThermoTables th, const double* Ep, const double* T0, int n, double trust_rel, int maxit,
                                const MLPView* mlp, double* Tout, int* evals, cudaStream_t s);
-cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* Tp, double* Te,
+cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp, double* Te,
                               double* TL, double* EL, const double* Tcells, const double* I0ref, long long cell0,
                               int ncells, int nd, ThermoTables th, cudaStream_t s);
-cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, const double* Tp, double* Te, long long ncells,
+cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, double* MsumL, const double* Tp, double* Te, long long ncells,
                                  ThermoTables th, cudaStream_t s);
 cudaError_t launch_wall_I0(double* I0wall, const double* Tfaces, long long nfaces, ThermoTables th, cudaStream_t s);
 cudaError_t launch_wall_dev(float* out, const double* I0wall, const double* I0ref, long long nfaces, int nbp,
                             cudaStream_t s);
-cudaError_t launch_solve_TL(double* TL, const double* EL, const double* Tguess, const double* J, const double* Teval,
-                            long long ncells, ThermoTables th, double trust_rel, int maxit, DevCounters* counters,
-                            cudaStream_t s);
-// state_ff: the FP64 intensities are ff pairs (bte_ff.cuh)
-cudaError_t launch_flux_cells(int precision, bool state_ff, const void* I, double* q, const double* S, long long cell0,
+// state_ff: the FP64 intensities are ff pairs (bte_ff.cuh); grouped: rows in the internal order
+cudaError_t launch_flux_cells(int precision, bool state_ff, bool grouped, const void* I, double* q, const double* S, long long cell0,
                               int ncells, int nd, int nbp, int dim, cudaStream_t s);
 // every side of one geometry: face sums to face_out[side][max_faces], means to out[side]
 cudaError_t launch_flux_walls(int precision, bool state_ff, const void* I, const double* I0ref, const double* I0wall,
-                              const DevGeom* geoms, int geom, const DirInfo* dirs, const double* S, int nd, int nbp,
+                              const DevGeom* geoms, int geom, const WallDirs* wall_dirs, const double* S, int nd, int nbp,
                               double* face_out, int max_faces, const int (&nfaces)[6], int nsides, double* out,
                               cudaStream_t s);
 // In place: npairs 16-byte ff pairs of two bands (bte_ff.cuh layout) -> two doubles each.
@@ -240,12 +241,12 @@ cudaError_t launch_ff_to_doubles(void* buf, long long npairs, cudaStream_t s);
 // npairs x two doubles -> ff pairs (dst may be src)
 cudaError_t launch_doubles_to_ff(const void* src, void* dst, long long npairs, cudaStream_t s);
 // FP64 [cell][caller's d][nb] <-> internal rows; perm: the caller's index of every internal direction
-cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* perm,
+cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* rows,
                           long long ncells, int nd, int nb, int nbp, cudaStream_t s);
-cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* perm,
-                        long long ncells, int nd, int nb, int nbp, cudaStream_t s);
-cudaError_t launch_energy_L(int precision, bool state_ff, const void* I, const double* I0ref, double* EL, const double* wdir,
-                            long long ncells, int nd, ThermoTables th, cudaStream_t s);
+cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* rows,
+                        long long ncells, int nd, int nb, int nbp, const SweepArgs* energies, cudaStream_t s);
+// E_L of every cell from its partial energies (launch_gs_reduce's or launch_pack's Ec)
+cudaError_t launch_energy_L(const double2* Ec, double* EL, long long ncells, cudaStream_t s);
 
 // Read-only view of one geometry's device state, for entry points that live
 // outside bte_capi.cu (bte_noalloc.cu).  flux_view returns BTE_E_* codes.
@@ -255,7 +256,7 @@ struct FluxView {
   bool state_ff;          // FP64: it holds ff pairs
   const double* I0wall;
   const DevGeom* geoms;
-  const DirInfo* dirs;
+  WallDirs wall_dirs[6];
   const double* S;        // [nd][3]
   int nd, nbp, dim;
   int nfaces[6];          // faces per side (0 for sides beyond 2*dim)

@@ -1,11 +1,10 @@
 // bte_kernels.cu -- CUDA kernels around the sweep (sm_103a).  The sweeps (upwind
 // update, walls, band sums; Sec. 3.1, Eq. 4-6) live in bte_sweep.cuh and
 // bte_sweep_ff.cuh, the per-cell T_p step in bte_cells.cu.  Here:
-//   gs_reduce_kernel    band sums after a sweep-ordered pass (bte_gs.cu) or an
+//   gs_reduce_kernel    energies after a sweep-ordered pass (bte_gs.cu) or an
 //                       unstructured sweep;
 //   init_cells / state_from_Tp / wall_I0 / wall_dev
 //                       equilibrium state, cached models and Eq. 6 ghosts;
-//   solve_TL_kernel     T_L on request (cached model first, exact otherwise);
 //   flux_cells / flux_faces / mean / pack / unpack / energy_L
 //                       heat flux, FP64 <-> storage packing, E_L after a restore.
 #include <algorithm>
@@ -23,15 +22,15 @@ namespace {
 
 // ---------------------------------------------------------------------------
 // Per-cell thermodynamic state at temperature T: I0cell, cached model J at T
-// with its T_p sums Msum, T_e = T_p = T.  One CTA per cell (grid-stride);
-// bands over threads.
-__device__ void cell_state_at(double* I0cell, double* J, double* Msum, long long P, double T, ThermoTables th,
-                              double* row) {
-  const double rT = 1.0 / T;
+// with its T_p and T_L sums, T_e = T_p = T.  One CTA per cell (grid-stride); bands
+// over threads.
+__device__ void cell_state_at(double* I0cell, double* J, double* Msum, double* MsumL, long long P, double T,
+                              ThermoTables th, double* row) {
+  const double rT = rcp_pos(T);
   double* Jrow = J + (P * 4) * th.nbp;
   for (int b = threadIdx.x; b < th.nbp; b += blockDim.x) {  // every band (the temperature model)
     double f[4];
-    band_I0_d3(th.node_c + b * th.ng, th.node_C + b * th.ng, th.ng, rT, f);
+    band_taylor(th.node_c + b * th.ng, th.node_C + b * th.ng, th.ng, rT, f);
     row[b] = f[0];
 #pragma unroll
     for (int k = 0; k < 4; ++k) Jrow[k * th.nbp + b] = f[k];
@@ -39,10 +38,12 @@ __device__ void cell_state_at(double* I0cell, double* J, double* Msum, long long
   __syncthreads();
   for (int b = threadIdx.x; b < th.nbo; b += blockDim.x)  // stored bands
     I0cell[P * th.nbo + b] = b < th.nbr ? row[th.band0 + b] : 0.0;
-  if (threadIdx.x < 32) {  // the model's sums with the T_p weights
+  if (threadIdx.x < 64) {  // the model's sums: warp 0 with the T_p weights, warp 1 with T_L's
+    const int lane = threadIdx.x & 31;
+    const double* wt = threadIdx.x < 32 ? th.a_p : th.a_L;
     double m[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < th.nbp; b += 32) {
-      const double ap = th.a_p[b];
+    for (int b = lane; b < th.nbp; b += 32) {
+      const double ap = wt[b];
 #pragma unroll
       for (int k = 0; k < 4; ++k) m[k] = fma(ap, Jrow[k * th.nbp + b], m[k]);
     }
@@ -50,22 +51,22 @@ __device__ void cell_state_at(double* I0cell, double* J, double* Msum, long long
 #pragma unroll
       for (int k = 0; k < 4; ++k) m[k] += __shfl_xor_sync(0xffffffffu, m[k], o);
     }
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 4; ++k) Msum[4 * P + k] = m[k];
+    if (lane == 0)
+      for (int k = 0; k < 4; ++k) (threadIdx.x < 32 ? Msum : MsumL)[4 * P + k] = m[k];
   }
 }
 
 // Equilibrium initial state: I = I0_b(T_P) for every direction (stored as the
 // deviation I0_b(T_P) - I0_b(T_ref) in the reduced modes).
 template <typename S>
-__global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum, double* Tp, double* Te, double* TL,
+__global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp, double* Te, double* TL,
                                   double* EL, const double* Tcells, const double* I0ref, long long cell0, int ncells,
                                   int nd, ThermoTables th) {
   extern __shared__ double row[];  // [nbp]
   for (int c = blockIdx.x; c < ncells; c += gridDim.x) {
     const long long P = cell0 + c;
     const double T = Tcells[c];
-    cell_state_at(I0cell, J, Msum, P, T, th, row);
+    cell_state_at(I0cell, J, Msum, MsumL, P, T, th, row);
     __syncthreads();
     const long long n = (long long)nd * th.nbo;
     for (long long e = threadIdx.x; e < n; e += blockDim.x) {
@@ -86,11 +87,11 @@ __global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum,
 }
 
 // Thermodynamic state from T_p after a state restore: I0cell, J, T_e.
-__global__ void state_from_Tp_kernel(double* I0cell, double* J, double* Msum, const double* Tp, double* Te,
+__global__ void state_from_Tp_kernel(double* I0cell, double* J, double* Msum, double* MsumL, const double* Tp, double* Te,
                                      long long ncells, ThermoTables th) {
   extern __shared__ double row[];
   for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
-    cell_state_at(I0cell, J, Msum, P, Tp[P], th, row);
+    cell_state_at(I0cell, J, Msum, MsumL, P, Tp[P], th, row);
     if (threadIdx.x == 0) Te[P] = Tp[P];
     __syncthreads();
   }
@@ -113,52 +114,6 @@ __global__ void wall_dev_kernel(float* out, const double* I0wall, const double* 
     out[e] = (float)(I0wall[e] - I0ref[e % nbp]);
 }
 
-// Lattice temperature: sum_b a_L,b I0_b(T) = E_L per cell (evaluated on
-// request).  One warp per cell: the root of the cell's cached cubic model
-// of I0_b(T) around T_e (the one the T_p solve keeps) when it lies inside the
-// trust radius, else Halley on the exact band quadrature from there (or from
-// the guess), bisection as the fallback.
-__global__ void solve_TL_kernel(double* TL, const double* EL, const double* Tguess, const double* J,
-                                const double* Teval, long long ncells, ThermoTables th, double trust_rel, int maxit,
-                                DevCounters* counters) {
-  const int warps = blockDim.x / 32, lane = threadIdx.x & 31;
-  const int nbp = th.nbp;
-  for (long long P = blockIdx.x * (long long)warps + threadIdx.x / 32; P < ncells; P += (long long)gridDim.x * warps) {
-    const double E = EL[P];
-    if (!isfinite(E)) {
-      if (lane == 0) {
-        TL[P] = E;
-        if (counters) atomicAdd(&counters->nonfinite, 1ULL);
-      }
-      continue;
-    }
-    double F[4] = {0.0, 0.0, 0.0, 0.0};
-    for (int b = lane; b < nbp; b += 32) {
-      const double w = th.a_L[b];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) F[k] = fma(w, J[(P * 4 + k) * nbp + b], F[k]);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-      for (int k = 0; k < 4; ++k) F[k] += __shfl_xor_sync(0xffffffffu, F[k], o);
-    }
-    const double Te = Teval[P];
-    const double delta = model_step(F[0] - E, F[1], F[2], F[3]);
-    const double Tn = Te + delta;
-    if (isfinite(Tn) && fabs(delta) <= trust_rel * Tn) {
-      if (lane == 0) TL[P] = Tn;
-      continue;
-    }
-    const double start = (isfinite(Tn) && Tn >= kTmin && Tn <= kTmax) ? Tn : Tguess[P];
-    const SolveResult r = exact_solve_warp(th, E, start, trust_rel, maxit, nullptr, th.a_L);
-    if (lane == 0) {
-      TL[P] = r.Te + r.delta;
-      if (counters && r.fallback) atomicAdd(&counters->fallbacks, 1ULL);
-      if (counters && r.bad) atomicAdd(&counters->nonfinite, 1ULL);
-    }
-  }
-}
-
 // Cell heat flux q(P) = sum_b sum_d S_d I_{d,b}: one CTA per cell.  A lane holds
 // the V bands of one 16-byte vector and takes every (threads / lanes)-th group of
 // four rows, (+,+), (-,+), (-,-), (+,-) of one |S|: the four values' sums and
@@ -167,28 +122,25 @@ __global__ void solve_TL_kernel(double* TL, const double* EL, const double* Tgue
 // The reference part of the reduced modes' storage drops out: sum_d S_d = 0.
 // On 128x128 x 400 x 55: 2014 us with one 64-bit division and two FMAs per value.
 template <typename S, int V>
-__device__ __forceinline__ double vector_sum(const S* p) {  // sum of V consecutive values
-  double s = 0.0;
-  if constexpr (sizeof(S) == 8) {
-    if constexpr (std::is_same<S, FFElem>::value) {
-      double a, b;
-      ff::to_doubles(ff::ldg(p), a, b);
-      s = a + b;
-    } else {
-      double x[2];
-      Tr<double>::ld(p, x);
-      s = x[0] + x[1];
-    }
-  } else {
-    float x[V];
-    Tr<S>::ld(p, x);
-#pragma unroll
-    for (int v = 0; v < V; ++v) s += (double)x[v];
+struct Vec {  // V consecutive values, loaded and summed
+  typename RawPair<S>::R x[V / 2];
+  __device__ __forceinline__ void load(const S* p) {
+    const uint4 w = __ldg(reinterpret_cast<const uint4*>(p));
+    memcpy(x, &w, 16);
   }
-  return s;
-}
+  __device__ __forceinline__ double sum() const {
+    double s = 0.0;
+#pragma unroll
+    for (int v = 0; v < V / 2; ++v) {
+      double a, b;
+      raw_pair(x[v], a, b);
+      s = v ? (s + a) + b : a + b;
+    }
+    return s;
+  }
+};
 
-template <typename S, int V, int DIM>
+template <typename S, int V, int DIM, bool GROUPED>
 __global__ void __launch_bounds__(256) flux_cells_kernel(const S* I, double* q, const double* Sd, long long cell0,
                                                          int ncells, int nd, int nbp) {
   __shared__ double sh[3][8];
@@ -200,9 +152,19 @@ __global__ void __launch_bounds__(256) flux_cells_kernel(const S* I, double* q, 
     if (grp < groups) {
 #pragma unroll 2
       for (int r = 4 * grp; r < nd; r += 4 * groups) {
+        Vec<S, V> x[4];
         double v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = vector_sum<S, V>(row + (r + k) * nbp);
+        for (int k = 0; k < 4; ++k) x[k].load(row + (r + k) * nbp);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = x[k].sum();
+        if constexpr (!GROUPED) {  // any order: every row by its own S
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int ax = 0; ax < DIM; ++ax) acc[ax] = fma(Sd[3 * (r + k) + ax], v[k], acc[ax]);
+          continue;
+        }
         const double a = v[0] + v[3], b = v[1] + v[2];
         acc[0] = fma(Sd[3 * r], a - b, acc[0]);
         acc[1] = fma(Sd[3 * r + 1], (v[0] - v[3]) + (v[1] - v[2]), acc[1]);
@@ -225,9 +187,12 @@ __global__ void __launch_bounds__(256) flux_cells_kernel(const S* I, double* q, 
 }
 
 // Net outgoing flux through every face of every side of a geometry (blockIdx.y: side).
+struct SideDirs {
+  WallDirs d[6];
+};
 template <typename S>
 __global__ void __launch_bounds__(kFluxThreads) flux_faces_kernel(const S* I, const double* I0ref, const double* I0wall,
-                                                                  const DevGeom* geoms, int geom, const DirInfo* dirs,
+                                                                  const DevGeom* geoms, int geom, SideDirs wd,
                                                                   const double* Sd, int nd, int nbp, double* face_out,
                                                                   int max_faces) {
   __shared__ double sh[kFluxThreads];
@@ -235,7 +200,7 @@ __global__ void __launch_bounds__(kFluxThreads) flux_faces_kernel(const S* I, co
   const int side = blockIdx.y;
   const int nfaces = side < 2 ? g.ny * g.nz : (side < 4 ? g.nx * g.nz : g.nx * g.ny);
   for (int f = blockIdx.x; f < nfaces; f += gridDim.x) {
-    const double t = face_flux(I, I0ref, I0wall, g, side, f, dirs, Sd, nd, nbp, sh);
+    const double t = face_flux(I, I0ref, I0wall, g, side, f, wd.d[side], Sd, nd, nbp, sh);
     if (threadIdx.x == 0) face_out[(long long)side * max_faces + f] = t;
   }
 }
@@ -253,185 +218,275 @@ __global__ void mean_kernel(const double* v, int max_faces, SideFaces nf, double
 }
 
 // FP64 [cell][caller's d][nb] <-> internal rows [cell][dir][nbp] (deviation in the
-// reduced modes): one CTA per cell, a thread per band walking every
-// (threads / nbp)-th direction, so consecutive lanes touch consecutive bands on
-// both sides and no index is divided.
+// reduced modes): one CTA of 8 warps per cell, a warp per row.  On the internal
+// side a lane holds a pair of bands (16 bytes in FP64), on the caller's side the
+// warp touches 32 consecutive doubles at a time (rows of nb doubles start at any
+// multiple of 8 bytes), shuffles in between; four rows in flight.  The CTA walks
+// the caller's order (row[d]: its internal row), whose rows share 32-byte sectors;
+// internal rows are whole sectors and may be scattered.  Bound by HBM:
+// 16 bytes per FP64 value.  A thread per band with 8-byte accesses on both sides
+// took 569 (in) and 494 us (out) on 96x64 x 400 x 55 values as ff pairs; 406 and
+// 555 here, where the conversions of ff pairs issue most instructions.
 template <typename S>
-__global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, const double* I0ref, const int* perm,
+__global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, const double* I0ref, const int* rows,
                                                      long long ncells, int nd, int nb, int nbp) {
-  const int rows = 256 / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
-  if (r >= rows || b >= nb) return;
-  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
-    double* o = out + P * nd * nb + b;
-#pragma unroll 8
-    for (int d = r; d < nd; d += rows) __stcs(o + (long long)perm[d] * nb, full_I(I, (P * nd + d) * nbp + b, b, I0ref));
-  }
-}
-
-template <typename S>
-__global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const double* I0ref, const int* perm,
-                                                   long long ncells, int nd, int nb, int nbp) {
-  const int rows = 256 / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
-  if (r >= rows) return;
-  const double ref = sizeof(S) == 8 || b >= nb ? 0.0 : I0ref[b];
-  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
-    const double* x = in + P * nd * nb + b;
-#pragma unroll 8
-    for (int d = r; d < nd; d += rows) {
-      const double v = b < nb ? __ldcs(x + (long long)perm[d] * nb) - ref : 0.0;
-      set_I(I, (P * nd + d) * nbp + b, v);
-    }
-  }
-}
-
-// E_L of every cell from its intensity row (used after a state restore).
-template <typename S>
-__global__ void energy_L_kernel(const S* I, const double* I0ref, double* EL, const double* wdir, long long ncells,
-                                int nd, ThermoTables th) {
-  extern __shared__ double sh[];
-  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
-    const long long base = P * (long long)nd * th.nbo;
-    double acc = 0.0;
-    for (int b = threadIdx.x; b < th.nbo; b += blockDim.x) {
-      double G = 0.0;
-      for (int d = 0; d < nd; ++d) G = fma(wdir[d], full_I(I, base + (long long)d * th.nbo + b, b, I0ref), G);
-      acc = fma(G, th.inv_v[b], acc);
-    }
-    const double t = block_sum(acc, sh);
-    if (threadIdx.x == 0) EL[P] = t;
-  }
-}
-
-// Band sums after a separate sweep (the sweep-ordered pass, the unstructured
-// sweep): one CTA of 8 warps per cell.  Warp w sums the directions
-// [w nd/8, (w+1) nd/8) for every stored band (lanes over band pairs); the 8
-// partials are added in warp order (deterministic) and
-// G_b = sum_d w_d I^{k+1}_{d,b} goes to Gc for cells_kernel.
-// Within a warp the sums over a run of equal-weight directions are exact
-// 64-bit fixed-point additions on the integer pipe (unit 2^(E-50) for the
-// cell's I0 of exponent E; a value up to 32 I0 adds at most 2^55, so a run of
-// 256 cannot overflow), closed by one FP64 FMA (sum x w x unit).  Values
-// beyond that range (or negative, NaN) take the FP64 FMA directly.
-// Reduced storage (deviations from I0_b(T_ref)): each lane sums w_d x deviation
-// in FP32, flushed to FP64 every 16 directions, and G_b gets W I0_b(T_ref).
-constexpr int kRedWarps = 8;
-
-template <typename S>
-__device__ __forceinline__ void reduce_dev_warp(const SweepArgs& a, const S* row, int d0, int d1, int lane,
-                                                double* gpart_w) {
-  const int nbo = a.th.nbo;
-  for (int b0 = 2 * lane; b0 < nbo; b0 += 64) {  // two bands per lane
-    double G0 = 0.0, G1 = 0.0;
-    for (int d = d0; d < d1; d += 16) {  // 16 directions: loads first, then the float sums
-      const int m = min(16, d1 - d);
-      float x0[16], x1[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        x0[k] = x1[k] = 0.f;
-        if (k < m) {
-          const S* p = row + (long long)(d + k) * nbo + b0;
-          x0[k] = Tr<S>::to_float(p[0]);
-          x1[k] = Tr<S>::to_float(p[1]);
-        }
-      }
-      float acc0 = 0.f, acc1 = 0.f;
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float w = k < m ? a.wdir32[d + k] : 0.f;
-        acc0 = fmaf(w, x0[k], acc0);
-        acc1 = fmaf(w, x1[k], acc1);
-      }
-      G0 += (double)acc0;
-      G1 += (double)acc1;
-    }
-    gpart_w[b0] = G0;
-    gpart_w[b0 + 1] = G1;
-  }
-}
-
-template <typename S>
-__global__ void __launch_bounds__(256, 4) gs_reduce_kernel(SweepArgs a, long long ncells) {
-  extern __shared__ double gpart[];  // [kRedWarps][nbo]
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nbo = a.th.nbo, nd = a.nd, lpc = nbo / 2;
-  const int d0 = (int)((long long)wid * nd / kRedWarps), d1 = (int)((long long)(wid + 1) * nd / kRedWarps);
+  const int dlo = wid * nd / 8, dhi = (wid + 1) * nd / 8;
   for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
-    if constexpr (sizeof(S) != 8) {
-      reduce_dev_warp<S>(a, reinterpret_cast<const S*>(a.Iout) + P * (long long)nd * nbo, d0, d1, lane, gpart + wid * nbo);
-    } else {
-    const double* row = reinterpret_cast<const double*>(a.Iout) + P * (long long)nd * nbo;
-    for (int lp = lane; lp < lpc; lp += 32) {
-      const int b0 = 2 * lp;
-      double G[2] = {0.0, 0.0};
-      unsigned long long facc[2] = {0ull, 0ull};
-      long long fsc[2];
-      int fe0[2];
-#pragma unroll
-      for (int v = 0; v < 2; ++v) {
-        const int e0 = (int)((unsigned long long)__double_as_longlong(a.I0cell[P * nbo + b0 + v]) >> 52);
-        const bool on = e0 >= 200 && e0 <= 1900;
-        fe0[v] = on ? e0 + 4 : -1;
-        fsc[v] = on ? (long long)(e0 - 1073) * (1LL << 52) : 0;
+    const S* row = I + P * (long long)nd * nbp;
+    double* o = out + P * nd * nb;
+    for (int c = 0; c < nbp; c += 64) {  // 64 bands at a time
+      const int b = c + 2 * lane;
+      double r0 = 0.0, r1 = 0.0;
+      if (sizeof(S) != 8 && b < nbp) {
+        r0 = I0ref[b];
+        r1 = I0ref[b + 1];
       }
-      long long wrun = d0 < d1 ? __double_as_longlong(a.wdir[d0]) : 0;
-      int nrun = 0;
-      auto add = [&](double2 x, int d) {
-        const long long wb = __double_as_longlong(a.wdir[d]);
-        if (wb != wrun || nrun == 256) {  // close the run: sum x (w x unit)
+      for (int d0 = dlo; d0 < dhi; d0 += 4) {
+        typename RawPair<S>::R x[4];
 #pragma unroll
-          for (int v = 0; v < 2; ++v) {
-            if (facc[v] != 0ull) G[v] = fma(__ull2double_rn(facc[v]), __longlong_as_double(wrun + fsc[v]), G[v]);
-            facc[v] = 0ull;
-          }
-          wrun = wb;
-          nrun = 0;
-        }
-        ++nrun;
-        const double xv[2] = {x.x, x.y};
-        bool big = false;
+        for (int u = 0; u < 4; ++u)  // lanes and rows past the end repeat the last one's
+          x[u] = ld_raw(row + (long long)rows[min(d0 + u, dhi - 1)] * nbp + min(b, nbp - 2));
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
-          const unsigned long long rb = (unsigned long long)__double_as_longlong(xv[v]);
-          const int e = (int)(rb >> 52);  // sign bit included: negative values take the FP64 path
-          const unsigned long long m = ((rb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 2;
-          const int sh = e == 0 ? 63 : min(fe0[v] - e, 63);  // zero (and subnormal) adds nothing
-          facc[v] += sh >= 0 ? (m >> sh) : 0ull;
-          big |= sh < 0;
-        }
-        // rare: a value beyond the fixed-point range (a warp-uniform branch, so
-        // no FP64 instruction is issued in the common case)
-        if (__any_sync(__activemask(), big)) {
+        for (int u = 0; u < 4; ++u) {
+          if (d0 + u >= dhi) break;
+          double x0, x1;
+          raw_pair(x[u], x0, x1);
+          double* q = o + (long long)(d0 + u) * nb + c;
 #pragma unroll
-          for (int v = 0; v < 2; ++v) {
-            const int e = (int)((unsigned long long)__double_as_longlong(xv[v]) >> 52);
-            if (e != 0 && fe0[v] - e < 0) G[v] = fma(a.wdir[d], xv[v], G[v]);
+          for (int h = 0; h < 2; ++h) {  // elements 32 h + lane of the 64
+            const int src = 16 * h + (lane >> 1);
+            const double v0 = __shfl_sync(0xffffffffu, sizeof(S) != 8 ? x0 + r0 : x0, src);
+            const double v1 = __shfl_sync(0xffffffffu, sizeof(S) != 8 ? x1 + r1 : x1, src);
+            if (c + 32 * h + lane < nb) __stcs(q + 32 * h + lane, (lane & 1) ? v1 : v0);
           }
         }
-      };
-      int d = d0;
-      for (; d + 4 <= d1; d += 4) {
-        double2 x[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = __ldcs(reinterpret_cast<const double2*>(row + (long long)(d + u) * nbo + b0));
-#pragma unroll
-        for (int u = 0; u < 4; ++u) add(x[u], d + u);
       }
-      for (; d < d1; ++d) add(__ldcs(reinterpret_cast<const double2*>(row + (long long)d * nbo + b0)), d);
+    }
+  }
+}
+
+// Energies after a separate sweep (the sweep-ordered pass, the unstructured sweep) and
+// a restore in reduced storage: one CTA of 8 warps per cell.  Loads of 16 bytes, eight in
+// flight; FP64: warp w sums the directions [w nd / 8, (w + 1) nd / 8), lanes over
+// band pairs (whole warps on one direction, so the runs of the fixed-point sums
+// close together: groups of 28 lanes took 406 us where this takes 308 on 6144 cells
+// x 400 x 55); reduced storage: lanes over the V bands of a vector, 256 V / nbp
+// groups.  The partials are added in order (deterministic) to G_b = sum_d w_d I_{d,b};
+// warp 0 leaves kRedEntries partial energies in Ec for cells_kernel.  Bound by the
+// loads' latency and HBM, 8 bytes per FP64 value.
+// FP64: sums over a run of equal-weight directions are exact 64-bit fixed-point
+// additions on the integer pipe (unit 2^(E-50) for the cell's I0 of exponent E; a
+// value up to 32 I0 adds at most 2^55, so a run of 256 cannot overflow), closed by
+// one FP64 FMA (sum x w x unit).  Values beyond that range (or negative, NaN) take
+// the FP64 FMA directly.
+// Reduced storage (deviations from I0_b(T_ref)): each lane sums w_d x deviation in
+// FP32, added to a double-float sum every 16 directions (FP64 conversions and adds
+// there kept the FP64 pipe busy), and G_b gets W I0_b(T_ref).
+constexpr int kRedThreads = 256;
+
+struct FixedSum {
+  unsigned long long f[2];
+  double G[2];
+  long long fsc[2], w;
+  int fe0[2], n;
+  __device__ explicit FixedSum(const double* i0) : f{0ull, 0ull}, G{0.0, 0.0}, w(0), n(0) {
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const int e0 = (int)((unsigned long long)__double_as_longlong(i0[v]) >> 52);
+      const bool on = e0 >= 200 && e0 <= 1900;
+      fe0[v] = on ? e0 + 4 : -1;
+      fsc[v] = on ? (long long)(e0 - 1073) * (1LL << 52) : 0;
+    }
+  }
+  __device__ void close() {
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      if (f[v] != 0ull) G[v] = fma(__ull2double_rn(f[v]), __longlong_as_double(w + fsc[v]), G[v]);
+      f[v] = 0ull;
+    }
+    n = 0;
+  }
+  __device__ void add(double x0, double x1, double wd) {
+    const long long wb = __double_as_longlong(wd);
+    if (wb != w || n == 256) {
+      close();
+      w = wb;
+    }
+    ++n;
+    const double xv[2] = {x0, x1};
+    bool big = false;
+#pragma unroll
+    for (int v = 0; v < 2; ++v) {
+      const unsigned long long rb = (unsigned long long)__double_as_longlong(xv[v]);
+      const int e = (int)(rb >> 52);  // sign bit included: negative values take the FP64 path
+      const unsigned long long m = ((rb & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 2;
+      const int sh = e == 0 ? 63 : min(fe0[v] - e, 63);  // zero (and subnormal) adds nothing
+      f[v] += sh >= 0 ? (m >> sh) : 0ull;
+      big |= sh < 0;
+    }
+    // rare: a value beyond the fixed-point range (a warp-uniform branch, so no
+    // FP64 instruction is issued in the common case)
+    if (__any_sync(__activemask(), big)) {
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
-        if (facc[v] != 0ull) G[v] = fma(__ull2double_rn(facc[v]), __longlong_as_double(wrun + fsc[v]), G[v]);
-        gpart[wid * nbo + b0 + v] = G[v];
+        const int e = (int)((unsigned long long)__double_as_longlong(xv[v]) >> 52);
+        if (e != 0 && fe0[v] - e < 0) G[v] = fma(wd, xv[v], G[v]);
       }
     }
+  }
+};
+
+// Warp 0: the parts' band sums added in order, then kRedEntries partial energies of cell P.
+template <bool DEV>
+__device__ __forceinline__ void reduce_energies(const SweepArgs& a, const double* gpart, int parts, long long P) {
+  const int nbo = a.th.nbo;
+  double el = 0.0, ep = 0.0;
+  for (int b = threadIdx.x; b < nbo; b += 32) {
+    double G = gpart[b];
+    for (int w = 1; w < parts; ++w) G += gpart[w * nbo + b];
+    if constexpr (DEV) G = fma(a.Wtot, a.I0ref[b], G);  // the reference part, sum_d w_d I0_b(T_ref)
+    el = fma(G, a.th.inv_v[b], el);
+    ep = fma(G, a.th.binv_v[b], ep);
+  }
+  for (int o = 16; o >= kRedEntries; o >>= 1) {
+    el += __shfl_xor_sync(0xffffffffu, el, o);
+    ep += __shfl_xor_sync(0xffffffffu, ep, o);
+  }
+  if (threadIdx.x < kRedEntries) a.Ec[P * kRedEntries + threadIdx.x] = make_double2(el, ep);
+}
+
+template <typename S, int V>
+__global__ void __launch_bounds__(kRedThreads, 4) gs_reduce_kernel(SweepArgs a, long long ncells) {
+  extern __shared__ double gpart[];  // [parts][nbo]
+  constexpr bool kWarps = sizeof(S) == 8;
+  const int nbo = a.th.nbo, nd = a.nd, lpc = nbo / V, parts = kWarps ? kRedThreads / 32 : kRedThreads / lpc;
+  const int part = threadIdx.x / (kWarps ? 32 : lpc), first = threadIdx.x - part * (kWarps ? 32 : lpc);
+  const int d0 = (int)((long long)part * nd / parts), d1 = (int)((long long)(part + 1) * nd / parts);
+  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
+    for (int lp = first; part < parts && lp < lpc; lp += kWarps ? 32 : lpc) {
+      const int b0 = V * lp;
+      const S* row = reinterpret_cast<const S*>(a.Iout) + P * (long long)nd * nbo + b0;
+      double* g = gpart + part * nbo + b0;
+      if constexpr (kWarps) {
+        FixedSum sum(a.I0cell + P * nbo + b0);
+        auto batch = [&](auto n, int d) {
+          constexpr int N = decltype(n)::value;
+          double2 x[N];
+#pragma unroll
+          for (int u = 0; u < N; ++u) x[u] = __ldcs(reinterpret_cast<const double2*>(row + (long long)(d + u) * nbo));
+#pragma unroll
+          for (int u = 0; u < N; ++u) {
+            sum.add(x[u].x, x[u].y, a.wdir[d + u]);
+          }
+        };
+        int d = d0;
+        for (; d + 8 <= d1; d += 8) batch(std::integral_constant<int, 8>{}, d);
+        for (; d + 2 <= d1; d += 2) batch(std::integral_constant<int, 2>{}, d);
+        if (d < d1) batch(std::integral_constant<int, 1>{}, d);
+        sum.close();
+        g[0] = sum.G[0];
+        g[1] = sum.G[1];
+      } else {
+        ff::P2 G[V / 2];
+#pragma unroll
+        for (int v = 0; v < V / 2; ++v) G[v] = ff::zero();
+        for (int d = d0; d < d1; d += 16) {
+          float acc[V];
+#pragma unroll
+          for (int v = 0; v < V; ++v) acc[v] = 0.f;
+#pragma unroll
+          for (int h = 0; h < 16; h += 8) {  // eight loads in flight
+            float x[8][V];
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              if (d + h + u < d1) Tr<S>::ld_stream(row + (long long)(d + h + u) * nbo, x[u]);
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+              if (d + h + u < d1) {
+                const float w = a.wdir32[d + h + u];
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v] = fmaf(w, x[u][v], acc[v]);
+              }
+          }
+#pragma unroll
+          for (int v = 0; v < V / 2; ++v) ff::acc(G[v], ff::P2{ff::pack(acc[2 * v], acc[2 * v + 1]), 0ull});
+        }
+#pragma unroll
+        for (int v = 0; v < V / 2; ++v) ff::to_doubles(ff::norm(G[v]), g[2 * v], g[2 * v + 1]);
+      }
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbo; b += blockDim.x) {
-      double G = gpart[b];
-      for (int w = 1; w < kRedWarps; ++w) G += gpart[w * nbo + b];
-      if constexpr (sizeof(S) != 8) G = fma(a.Wtot, a.I0ref[b], G);  // the reference part, sum_d w_d I0_b(T_ref)
-      a.Gc[P * nbo + b] = G;
-    }
+    if (threadIdx.x < 32) reduce_energies<sizeof(S) != 8>(a, gpart, parts, P);
     __syncthreads();
+  }
+}
+
+// FP64 values and their energies in one pass (REDUCE: a.Ec as gs_reduce_kernel leaves
+// it, for the values as given): a warp's lanes hold band pairs of one direction, the
+// warps contiguous eighths of the caller's directions (runs of equal weights).  On 96x64 x 400 x 55 as ff pairs the
+// separate pass over the stored rows took 424 us after this kernel's 406; now 575.
+template <typename S, bool REDUCE>
+__global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const double* I0ref, const int* rows,
+                                                   long long ncells, int nd, int nb, int nbp, SweepArgs a) {
+  extern __shared__ double gpart[];  // REDUCE: [8][nbp]
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int dlo = wid * nd / 8, dhi = (wid + 1) * nd / 8;
+  for (long long P = blockIdx.x; P < ncells; P += gridDim.x) {
+    S* row = I + P * (long long)nd * nbp;
+    const double* x = in + P * nd * nb;
+    for (int c = 0; c < nbp; c += 64) {
+      const int b = c + 2 * lane;
+      double r0 = 0.0, r1 = 0.0;
+      if (sizeof(S) != 8) {
+        if (b < nb) r0 = I0ref[b];
+        if (b + 1 < nb) r1 = I0ref[b + 1];
+      }
+      const double zero2[2] = {0.0, 0.0};
+      FixedSum sum(REDUCE && b < nbp ? a.I0cell + P * nbp + b : zero2);
+      for (int d0 = dlo; d0 < dhi; d0 += 4) {
+        double v[4][2];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int e = c + 32 * h + lane;
+            v[u][h] = d0 + u < dhi && e < nb ? __ldcs(x + (long long)(d0 + u) * nb + e) : 0.0;
+          }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (d0 + u >= dhi) break;
+          // bands b, b + 1 = elements 2 lane, 2 lane + 1 of the 64: half lane >> 4, lanes 2 lane (+ 1) mod 32
+          const int s0 = (2 * lane) & 31, r = rows[d0 + u];
+          const double a0 = __shfl_sync(0xffffffffu, v[u][0], s0), a1 = __shfl_sync(0xffffffffu, v[u][0], s0 + 1);
+          const double e0 = __shfl_sync(0xffffffffu, v[u][1], s0), e1 = __shfl_sync(0xffffffffu, v[u][1], s0 + 1);
+          const double x0 = lane < 16 ? a0 : e0, x1 = lane < 16 ? a1 : e1;
+          if (b < nbp) st_pair(row + (long long)r * nbp + b, x0 - r0, x1 - r1);
+          if constexpr (REDUCE) sum.add(x0, x1, a.wdir[r]);
+        }
+      }
+      if constexpr (REDUCE) {
+        sum.close();
+        if (b < nbp) {
+          gpart[wid * nbp + b] = sum.G[0];
+          gpart[wid * nbp + b + 1] = sum.G[1];
+        }
+      }
+    }
+    if constexpr (REDUCE) {
+      __syncthreads();
+      if (threadIdx.x < 32) reduce_energies<false>(a, gpart, 8, P);
+      __syncthreads();
+    }
+  }
+}
+
+// E_L of every cell from its partial energies (after a state restore).
+__global__ void energy_L_kernel(const double2* Ec, double* EL, long long ncells) {
+  for (long long P = blockIdx.x * (long long)blockDim.x + threadIdx.x; P < ncells; P += (long long)gridDim.x * blockDim.x) {
+    double e = 0.0;
+    for (int k = 0; k < kRedEntries; ++k) e += Ec[P * kRedEntries + k].x;
+    EL[P] = e;
   }
 }
 
@@ -641,19 +696,24 @@ cudaError_t launch_partial_ghosts(int precision, const void* I, const double* I0
 
 cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells, cudaStream_t s) {
   const int grid = (int)std::min<long long>(std::max(ncells, 1LL), 152LL * 64);
-  const size_t sm = (size_t)kRedWarps * a.th.nbo * sizeof(double);
-  if (precision == 0) gs_reduce_kernel<double><<<grid, 32 * kRedWarps, sm, s>>>(a, ncells);
-  else if (precision == 1) gs_reduce_kernel<float><<<grid, 32 * kRedWarps, sm, s>>>(a, ncells);
-  else gs_reduce_kernel<__nv_bfloat16><<<grid, 32 * kRedWarps, sm, s>>>(a, ncells);
+  auto go = [&](auto tag, auto vec) {
+    using T = decltype(tag);
+    constexpr int V = decltype(vec)::value;
+    const size_t sm = (size_t)(sizeof(T) == 8 ? kRedThreads / 32 : kRedThreads / (a.th.nbo / V)) * a.th.nbo * sizeof(double);
+    gs_reduce_kernel<T, V><<<grid, kRedThreads, sm, s>>>(a, ncells);
+  };
+  if (precision == 0) go(double{}, std::integral_constant<int, 2>{});
+  else if (precision == 1) go(float{}, std::integral_constant<int, 4>{});
+  else go(__nv_bfloat16{}, std::integral_constant<int, 8>{});
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* Tp,
-                              double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
+cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* MsumL,
+                              double* Tp, double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
                               long long cell0, int ncells, int nd, ThermoTables th, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
-    init_cells_kernel<T><<<cell_grid(ncells), 256, th.nbp * sizeof(double), s>>>((T*)I, I0cell, J, Msum, Tp, Te, TL, EL, Tcells,
+    init_cells_kernel<T><<<cell_grid(ncells), 256, th.nbp * sizeof(double), s>>>((T*)I, I0cell, J, Msum, MsumL, Tp, Te, TL, EL, Tcells,
                                                                                  I0ref, cell0, ncells, nd, th);
   };
   if (precision == 0 && state_ff) go(FFElem{});
@@ -663,9 +723,9 @@ cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0c
   return cudaGetLastError();
 }
 
-cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, const double* Tp, double* Te,
+cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, double* MsumL, const double* Tp, double* Te,
                                  long long ncells, ThermoTables th, cudaStream_t s) {
-  state_from_Tp_kernel<<<cell_grid(ncells), 64, th.nbp * sizeof(double), s>>>(I0cell, J, Msum, Tp, Te, ncells,
+  state_from_Tp_kernel<<<cell_grid(ncells), 64, th.nbp * sizeof(double), s>>>(I0cell, J, Msum, MsumL, Tp, Te, ncells,
                                                                                th);  // row: all bands
   return cudaGetLastError();
 }
@@ -681,23 +741,17 @@ cudaError_t launch_wall_dev(float* out, const double* I0wall, const double* I0re
   return cudaGetLastError();
 }
 
-cudaError_t launch_solve_TL(double* TL, const double* EL, const double* Tguess, const double* J, const double* Teval,
-                            long long ncells, ThermoTables th, double trust_rel, int maxit, DevCounters* counters,
-                            cudaStream_t s) {
-  solve_TL_kernel<<<cell_grid(ncells / 4 + 1), 128, 0, s>>>(TL, EL, Tguess, J, Teval, ncells, th, trust_rel, maxit,
-                                                            counters);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_flux_cells(int precision, bool state_ff, const void* I, double* q, const double* S, long long cell0,
-                              int ncells, int nd, int nbp, int dim, cudaStream_t s) {
+cudaError_t launch_flux_cells(int precision, bool state_ff, bool grouped, const void* I, double* q, const double* S,
+                              long long cell0, int ncells, int nd, int nbp, int dim, cudaStream_t s) {
   const int grid = cell_grid(ncells);
   auto go = [&](auto tag, auto vec) {
     using T = decltype(tag);
     constexpr int V = decltype(vec)::value;
-    if (dim == 3) flux_cells_kernel<T, V, 3><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
-    else flux_cells_kernel<T, V, 2><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
+    if (!grouped) flux_cells_kernel<T, V, 3, false><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
+    else if (dim == 3) flux_cells_kernel<T, V, 3, true><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
+    else flux_cells_kernel<T, V, 2, true><<<grid, 256, 0, s>>>((const T*)I, q, S, cell0, ncells, nd, nbp);
   };
+  if (!grouped && dim != 3) return cudaErrorInvalidValue;
   if (precision == 0 && state_ff) go(FFElem{}, std::integral_constant<int, 2>{});
   else if (precision == 0) go(double{}, std::integral_constant<int, 2>{});
   else if (precision == 1) go(float{}, std::integral_constant<int, 4>{});
@@ -706,7 +760,7 @@ cudaError_t launch_flux_cells(int precision, bool state_ff, const void* I, doubl
 }
 
 cudaError_t launch_flux_walls(int precision, bool state_ff, const void* I, const double* I0ref, const double* I0wall,
-                              const DevGeom* geoms, int geom, const DirInfo* dirs, const double* S, int nd, int nbp,
+                              const DevGeom* geoms, int geom, const WallDirs* wall_dirs, const double* S, int nd, int nbp,
                               double* face_out, int max_faces, const int (&nfaces)[6], int nsides, double* out,
                               cudaStream_t s) {
   int most = 1;
@@ -716,9 +770,11 @@ cudaError_t launch_flux_walls(int precision, bool state_ff, const void* I, const
     most = std::max(most, nfaces[k]);
   }
   const dim3 grid(cell_grid(most), nsides);
+  SideDirs wd;
+  std::copy(wall_dirs, wall_dirs + 6, wd.d);
   auto go = [&](auto tag) {
     using T = decltype(tag);
-    flux_faces_kernel<T><<<grid, kFluxThreads, 0, s>>>((const T*)I, I0ref, I0wall, geoms, geom, dirs, S, nd, nbp, face_out,
+    flux_faces_kernel<T><<<grid, kFluxThreads, 0, s>>>((const T*)I, I0ref, I0wall, geoms, geom, wd, S, nd, nbp, face_out,
                                                        max_faces);
   };
   if (precision == 0 && state_ff) go(FFElem{});
@@ -760,11 +816,11 @@ cudaError_t launch_ff_to_doubles(void* buf, long long npairs, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* perm,
+cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* rows,
                           long long ncells, int nd, int nb, int nbp, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
-    unpack_kernel<T><<<cell_grid(ncells), 256, 0, s>>>((const T*)I, out, I0ref, perm, ncells, nd, nb, nbp);
+    unpack_kernel<T><<<cell_grid(ncells), 256, 0, s>>>((const T*)I, out, I0ref, rows, ncells, nd, nb, nbp);
   };
   if (precision == 0 && state_ff) go(FFElem{});
   else if (precision == 0) go(double{});
@@ -773,29 +829,32 @@ cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* o
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* perm,
-                        long long ncells, int nd, int nb, int nbp, cudaStream_t s) {
+cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* rows,
+                        long long ncells, int nd, int nb, int nbp, const SweepArgs* energies, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
-    pack_kernel<T><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, perm, ncells, nd, nb, nbp);
+    if constexpr (sizeof(T) == 8) {
+      if (energies) {
+        pack_kernel<T, true><<<cell_grid(ncells), 256, 8 * (size_t)nbp * sizeof(double), s>>>(in, (T*)I, I0ref, rows, ncells, nd,
+                                                                                            nb, nbp, *energies);
+        return;
+      }
+    }
+    pack_kernel<T, false><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, rows, ncells, nd, nb, nbp, SweepArgs{});
   };
   if (precision == 0 && state_ff) go(FFElem{});
   else if (precision == 0) go(double{});
   else if (precision == 1) go(float{});
   else go(__nv_bfloat16{});
+  if (energies && precision != 0) {  // of the stored deviations
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? launch_gs_reduce(precision, *energies, ncells, s) : e;
+  }
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_L(int precision, bool state_ff, const void* I, const double* I0ref, double* EL, const double* wdir,
-                            long long ncells, int nd, ThermoTables th, cudaStream_t s) {
-  auto go = [&](auto tag) {
-    using T = decltype(tag);
-    energy_L_kernel<T><<<cell_grid(ncells), 64, 64 * sizeof(double), s>>>((const T*)I, I0ref, EL, wdir, ncells, nd, th);
-  };
-  if (precision == 0 && state_ff) go(FFElem{});
-  else if (precision == 0) go(double{});
-  else if (precision == 1) go(float{});
-  else go(__nv_bfloat16{});
+cudaError_t launch_energy_L(const double2* Ec, double* EL, long long ncells, cudaStream_t s) {
+  energy_L_kernel<<<grid_for(ncells, 128), 128, 0, s>>>(Ec, EL, ncells);
   return cudaGetLastError();
 }
 

@@ -51,12 +51,12 @@ cudaError_t scratch_address(int dev, double** out) {
 template <typename S>
 __global__ void __launch_bounds__(kFluxThreads) wall_faces_static_kernel(const S* I, const double* I0wall,
                                                                          const DevGeom* geoms, int geom, int side,
-                                                                         const DirInfo* dirs, const double* Sd, int nd,
-                                                                         int nbp, double* scratch, int nfaces) {
+                                                                         WallDirs wd, const double* Sd, int nd, int nbp,
+                                                                         double* scratch, int nfaces) {
   __shared__ double sh[kFluxThreads];
   const DevGeom g = geoms[geom];
   for (int f = blockIdx.x; f < nfaces; f += gridDim.x) {
-    const double t = face_flux(I, (const double*)nullptr, I0wall, g, side, f, dirs, Sd, nd, nbp, sh);
+    const double t = face_flux(I, (const double*)nullptr, I0wall, g, side, f, wd, Sd, nd, nbp, sh);
     if (threadIdx.x == 0) scratch[f] = t;
   }
 }
@@ -120,10 +120,10 @@ int wall_flux_on_device(bte_handle h, const FluxView& v, int geom, double* q_wal
     const int grid = nf < 152 * 16 ? nf : 152 * 16;
     if (v.state_ff)
       wall_faces_static_kernel<FFElem><<<grid, kFluxThreads, 0, v.stream>>>((const FFElem*)v.I, v.I0wall, v.geoms, geom, side,
-                                                                            v.dirs, v.S, v.nd, v.nbp, scratch, nf);
+                                                                            v.wall_dirs[side], v.S, v.nd, v.nbp, scratch, nf);
     else
       wall_faces_static_kernel<double><<<grid, kFluxThreads, 0, v.stream>>>((const double*)v.I, v.I0wall, v.geoms, geom, side,
-                                                                            v.dirs, v.S, v.nd, v.nbp, scratch, nf);
+                                                                            v.wall_dirs[side], v.S, v.nd, v.nbp, scratch, nf);
     wall_mean_static_kernel<<<1, 256, 0, v.stream>>>(scratch, nf, side);
   }
   e = cudaGetLastError();

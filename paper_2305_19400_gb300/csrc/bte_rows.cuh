@@ -3,8 +3,9 @@
 //   I^{k+1} = [I^n/dt + beta_b I0_b^k + v_b sum_ax c_ax,d I_up,ax^k] / [1/dt + beta_b + v_b sum_ax c_ax,d],
 //   c_ax,d = |S_ax,d| / (w_d Delta_ax),
 // (implicit: point-Jacobi sweep of backward Euler) or the forward-Euler form of
-// Eq. 3, and the band sums G_b = sum_d w_d I^{k+1}_{d,b} to Gc, from which
-// cells_kernel (bte_cells.cu) solves T_p and refreshes I0.  The upwind value is
+// Eq. 3, and every lane's share of the cell's energies sum_b G_b / v_b and
+// sum_b beta_b G_b / v_b, G_b = sum_d w_d I^{k+1}_{d,b}, to Ec, from which cells_kernel
+// (bte_cells.cu) solves T_p and refreshes I0.  The upwind value is
 // the neighbour cell's on the side S_d comes from, or the Eq. 6 ghost at a wall.
 //
 // Work layout.  A lane holds 16 bytes of one row, V consecutive bands, and a
@@ -40,13 +41,12 @@ namespace bte {
 namespace rows {
 
 // MAP 1: in-plane sets (blocks of 4 rows, one team); 2 and 4: polar x azimuthal
-// sets (blocks of 8 rows, two or four teams); 3: these with one team (blocks of 4
-// rows, S_z > 0 and S_z < 0 in turn).
+// sets (blocks of 8 rows, two or four teams); 3: these with one team.
 template <int MAP>
 struct Map;
 template <>
 struct Map<3> {
-  static constexpr int DT = 1, RUN = 4;
+  static constexpr int DT = 1, RUN = 8;
 };
 template <>
 struct Map<1> {
@@ -580,11 +580,6 @@ __global__ void __launch_bounds__(256, M::kMinB) rows_kernel(SweepArgs a) {
   };
   auto next_block = [&]() {
     cu.r0 += ROWS;
-    if constexpr (MAP == 3 && DIM == 3) {
-      const Src t = cu.z[0];
-      cu.z[0] = cu.z[1];
-      cu.z[1] = t;
-    }
     if (++cu.blk == nblk) {
       if (cu.item + (int)gridDim.x < a.nitems) setup(cu.item + gridDim.x);
       else cu.on = false;
@@ -602,11 +597,12 @@ __global__ void __launch_bounds__(256, M::kMinB) rows_kernel(SweepArgs a) {
         return p;
       };
       constexpr bool one = MAP == 1 || MAP == 3;
-      constexpr int vx = one ? (k == 1 || k == 2) : (MAP == 2 ? k & 1 : 0);
-      constexpr int vy = one ? k >> 1 : (MAP == 2 ? k & 1 : 0);
-      constexpr int vz = one ? 0 : (MAP == 2 ? k >> 1 : k);
+      constexpr int q = k & 3;
+      constexpr int vx = one ? (q == 1 || q == 2) : (MAP == 2 ? k & 1 : 0);
+      constexpr int vy = one ? q >> 1 : (MAP == 2 ? k & 1 : 0);
+      constexpr int vz = MAP == 1 ? 0 : (MAP == 3 ? k >> 2 : (MAP == 2 ? k >> 1 : k));
       cp16(si + ostr, up(cu.x[vx], k & 1 ? -1 : 1));
-      cp16(si + 2 * ostr, up(cu.y[vy], 3 - 2 * k));
+      cp16(si + 2 * ostr, up(cu.y[vy], 3 - 2 * q));
       if (DIM == 3) cp16(si + 3 * ostr, up(cu.z[vz], 0));
     }
     cp_commit();
@@ -693,9 +689,14 @@ __global__ void __launch_bounds__(256, M::kMinB) rows_kernel(SweepArgs a) {
     double G[V];
     M::finish(a, cell, acc, b0, dg, G);
     if (act0) {
+      double eL = 0.0, eP = 0.0;
 #pragma unroll
-      for (int v = 0; v < V; v += 2)
-        *reinterpret_cast<double2*>(a.Gc + (P0 * DT + dg) * nbp + b0 + v) = make_double2(G[v], G[v + 1]);
+      for (int v = 0; v < V; v += 2) {
+        const double2 iv = ld2(a.th.inv_v + b0 + v), bi = ld2(a.th.binv_v + b0 + v);
+        eL = fma(G[v + 1], iv.y, fma(G[v], iv.x, eL));
+        eP = fma(G[v + 1], bi.y, fma(G[v], bi.x, eP));
+      }
+      a.Ec[P0 * team + tl] = make_double2(eL, eP);
     }
     if (!more) break;
   }

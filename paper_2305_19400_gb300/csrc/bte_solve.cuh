@@ -18,44 +18,52 @@ namespace bte {
 // wider radius ten times less often.
 inline double model_trust(double rtol) { return std::pow(rtol / 32.0, 0.25); }
 
-// Root nearest 0 of F + F1 d + F2 d^2 / 2 + F3 d^3 / 6, the step of the cell's
-// cached temperature model: an FP32 estimate from the stable form of the
-// quadratic's root, -2F / (F1 + sqrt(F1^2 - 2 F F2)) (-F / F1 without a real
-// root), then one Newton step on the cubic in FP64 with the FP32 reciprocal of
-// the derivative.  The estimate is good to about 2e-7 of d (FP32 rounding and,
-// inside the trust radius, the cubic term) and the step to about 1e-13 of d,
-// while an accepted d is below 2e-4 T.  The FP64 pipe of GB300 takes about 76
-// cycles per warp instruction: this form issues eight FP64 operations where a
-// square root and a division take twenty-odd, and its conversions run on the
-// integer pipe (bte_ff.cuh).
-__device__ __forceinline__ double model_step(double F, double F1, double F2, double F3) {
-  float f, f1, f2, lo;
-  ff::split(F, f, lo);
-  ff::split(F1, f1, lo);
-  ff::split(F2, f2, lo);
-  const float disc = fmaf(f1, f1, -2.0f * f * f2);
-  const float d0f = (disc >= 0.0f && f1 > 0.0f) ? -2.0f * f / (f1 + sqrtf(disc)) : -f / f1;
-  const double d0 = ff::to_double(d0f, 0.0f);
-  const double h = fma(F3 * (1.0 / 6.0), d0, 0.5 * F2);
-  const double q = fma(fma(h, d0, F1), d0, F);
-  float qp;
-  ff::split(fma(fma(0.5 * F3, d0, F2), d0, F1), qp, lo);
-  const double r = ff::to_double(1.0f / qp, 0.0f);
-  return fma(-q, r, d0);
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// Root nearest 0 of c0 + c1 d + c2 d^2 + c3 d^3, the step of a cell's cached
+// temperature model: an FP32 estimate from the stable form of the quadratic's
+// root, -2 c0 / (c1 + sqrt(c1^2 - 4 c0 c2)) (-c0 / c1 without a real root), then
+// one Newton step on the cubic in FP64 with the derivative and its reciprocal in
+// FP32.  The estimate is good to about 2e-7 of d (FP32 rounding and, inside the
+// trust radius, the cubic term) and the step to about 1e-13 of d, while an
+// accepted d is below 2e-4 T.  The FP64 pipe of GB300 takes about 73 cycles per
+// warp instruction: this form issues four FP64 operations where a square root
+// and a division take twenty-odd, and its conversions run on the integer pipe.
+__device__ __forceinline__ double model_step(double c0, double c1, double c2, double c3) {
+  float f0, f1, f2, f3, lo;
+  ff::split(c0, f0, lo);
+  ff::split(c1, f1, lo);
+  ff::split(c2, f2, lo);
+  ff::split(c3, f3, lo);
+  const float disc = fmaf(f1, f1, -4.0f * f0 * f2);
+  const float df = (disc >= 0.0f && f1 > 0.0f) ? -2.0f * f0 / (f1 + sqrtf(disc)) : -f0 / f1;
+  const double d = ff::to_double(df, 0.0f);
+  const double g = fma(fma(fma(c3, d, c2), d, c1), d, c0);
+  const float dg = fmaf(fmaf(3.0f * f3, df, 2.0f * f2), df, f1);
+  return fma(-g, ff::to_double(1.0f / dg, 0.0f), d);
+}
+
+// |d| <= trust T (T finite), decided in FP32: the radius is not sharp to 1e-7.
+__device__ __forceinline__ bool in_trust(double d, double T, float trust) {
+  float df, Tf, lo;
+  ff::split(d, df, lo);
+  ff::split(T, Tf, lo);
+  return finite(T) && fabsf(df) <= trust * Tf;
 }
 
 // The model's value at T_e + d from one band's column of the cell's rows ([4][ld]).
 __device__ __forceinline__ double model_I0(const double* Jb, int ld, double d) {
-  return fma(fma(fma(Jb[3 * ld] * (1.0 / 6.0), d, 0.5 * Jb[2 * ld]), d, Jb[ld]), d, Jb[0]);
+  return fma(fma(fma(Jb[3 * ld], d, Jb[2 * ld]), d, Jb[ld]), d, Jb[0]);
 }
 
 struct SolveResult {
-  double Te;     // last exact evaluation point (its I0 and three derivatives are in Jrow)
+  double Te;     // last exact evaluation point (its Taylor coefficients are in Jrow)
   double delta;  // accepted step from Te: T_p = Te + delta
   int evals;     // exact band-quadrature evaluations
   int fallback;  // 1 when bisection was needed
   int bad;       // 1 when no temperature in [1, 5000] K was found
-  double M[4];   // sum_b w_b of I0_b and its first three derivatives at Te: the cell's model sums
+  double M[4];   // sum_b w_b of the bands' Taylor coefficients at Te: the cell's model sums
+  double ML[4];  // the same with the T_L weights (exact_solve_cluster with Jrow)
 };
 
 // Control of the exact solve of sum_b w_b I0_b(T) = Ep: Halley steps from T0
@@ -74,25 +82,25 @@ struct SolveCtl {
 
   __device__ explicit SolveCtl(double T0)
       : T((T0 >= kTmin && T0 <= kTmax && isfinite(T0)) ? T0 : 300.0), lo(kTmin), hi(kTmax), delta(0.0), mode(0),
-        iters(0), done(false), r{T, 0.0, 0, 0, 0, {0.0, 0.0, 0.0, 0.0}} {}
+        iters(0), done(false), r{T, 0.0, 0, 0, 0, {0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}} {}
 
-  // One evaluation's sums at T; moves T to the next evaluation point or sets done.
-  __device__ void advance(double F, double F1, double F2, double F3, double Ep, double trust_rel, int maxit) {
-    r.M[0] = F;
-    r.M[1] = F1;
-    r.M[2] = F2;
-    r.M[3] = F3;
-    F -= Ep;
+  // One evaluation's sums at T (Taylor coefficients); moves T to the next
+  // evaluation point or sets done.
+  __device__ void advance(const double* c, double Ep, double trust_rel, int maxit) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) r.M[k] = c[k];
+    const double F = c[0] - Ep, F1 = c[1];
     ++r.evals;
     r.Te = T;
     if (mode == 0) {
       ++iters;
-      bool badstep = !(isfinite(F) && isfinite(F1) && F1 > 0.0);
+      bool badstep = !(finite(F) && finite(F1) && F1 > 0.0);
       double Tn = T;
       if (!badstep) {
-        const double newton = -F / F1;
-        const double h = F * F2 / (2.0 * F1 * F1);
-        delta = fabs(h) < 0.5 ? newton / (1.0 - h) : newton;
+        const double r1 = rcp_pos(F1);
+        const double newton = -F * r1;
+        const double h = -newton * c[2] * r1;
+        delta = fabs(h) < 0.5 ? newton * rcp_pos(1.0 - h) : newton;
         Tn = T + delta;
         badstep = !(Tn >= kTmin && Tn <= kTmax) || iters > maxit;
       }
@@ -103,8 +111,9 @@ struct SolveCtl {
         T = 0.5 * (lo + hi);
         r.fallback = 1;
       } else if (fabs(delta) <= trust_rel * Tn) {
-        const double g = fma(fma(fma(F3 * (1.0 / 6.0), delta, 0.5 * F2), delta, F1), delta, F);
-        delta -= g / fma(fma(0.5 * F3, delta, F2), delta, F1);
+        const double g = fma(fma(fma(c[3], delta, c[2]), delta, F1), delta, F);
+        const double dg = fma(fma(3.0 * c[3], delta, 2.0 * c[2]), delta, F1);
+        delta = dg > 0.0 ? fma(-g, rcp_pos(dg), delta) : delta;
         done = true;
       } else {
         T = Tn;
@@ -132,7 +141,7 @@ struct SolveCtl {
 };
 
 // Exact solve by one warp (w = a_p unless given): lanes over bands.  Each
-// evaluation's I0 and three derivatives per band are written to Jrow ([4][nbp],
+// evaluation's Taylor coefficients per band are written to Jrow ([4][nbp],
 // may be null).  All 32 lanes of the warp must call it.
 __device__ inline SolveResult exact_solve_warp(const ThermoTables& th, double Ep, double T0, double trust_rel, int maxit,
                                                double* Jrow, const double* wts = nullptr) {
@@ -141,11 +150,11 @@ __device__ inline SolveResult exact_solve_warp(const ThermoTables& th, double Ep
   const int nbp = th.nbp, ng = th.ng;
   SolveCtl c(T0);
   for (int loop = 0; loop < maxit + 224 && !c.done; ++loop) {
-    const double rT = 1.0 / c.T;
+    const double rT = rcp_pos(c.T);
     double F[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b = lane; b < nbp; b += 32) {
       double f[4];
-      band_I0_d3(th.node_c + b * ng, th.node_C + b * ng, ng, rT, f);
+      band_taylor(th.node_c + b * ng, th.node_C + b * ng, ng, rT, f);
       const double ap = wb[b];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
@@ -157,7 +166,7 @@ __device__ inline SolveResult exact_solve_warp(const ThermoTables& th, double Ep
 #pragma unroll
       for (int k = 0; k < 4; ++k) F[k] += __shfl_xor_sync(0xffffffffu, F[k], o);
     }
-    c.advance(F[0], F[1], F[2], F[3], Ep, trust_rel, maxit);
+    c.advance(F, Ep, trust_rel, maxit);
   }
   return c.finish();
 }
@@ -170,41 +179,42 @@ __host__ __device__ inline int cta_solve_pairs(int nbp, int ng, int nr) {
   return all < 768 ? all : 768;
 }
 __host__ __device__ inline int cta_solve_smem_doubles(int nbp, int ng, int nr) {
-  return 4 * cta_solve_pairs(nbp, ng, nr) + 8 * nbp + 4;
+  return 4 * cta_solve_pairs(nbp, ng, nr) + 8 * nbp + 8;
 }
 
-// The same solve by a thread-block cluster, bit for bit the warp form's
-// results.  CTA r of the C in the cluster evaluates the bands
-// [r nbp / C, (r + 1) nbp / C): the costly per-node terms (expm1, the
-// reciprocal, the derivative factors) are spread over its threads, and each
-// band's node sums run in node order on one thread, writing the four values to the
-// CTA's own shared memory (and the cell's model row Jrow).  After one cluster
-// barrier warp 0 of every CTA adds all bands through distributed shared
-// memory in the warp form's order, so every CTA holds the same sums and
-// advances the same controller, and the loop ends on the same evaluation
-// everywhere.  The band values alternate between two buffers over the
-// cluster's successive evaluations (par counts them across calls): evaluation
-// k writes buffer k % 2 after the barrier of evaluation k - 1, which every
-// reader of buffer (k - 2) % 2 has passed.  One cell's evaluation thus runs
-// on C SMs' FP64 units.  sm: cta_solve_smem_doubles doubles per CTA.
-// Every thread of every CTA of the cluster must call it (it synchronises the
-// cluster).
-__device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double Ep, double T0, double trust_rel,
-                                                  int maxit, double* Jrow, double* sm, unsigned& par) {
+// The same solve by a thread-block cluster, or (COOP false) by one CTA alone with
+// all bands and no cluster barrier.  CTA r of the C in the cluster
+// evaluates the bands [r nbp / C, (r + 1) nbp / C): the costly per-node terms
+// (expm1, the reciprocal, the derivative factors) are spread over its threads,
+// and each of a band's four node sums runs in node order on one thread, writing
+// the coefficient to the CTA's own shared memory (and the cell's model row Jrow).
+// After one cluster barrier warp 0 of every CTA adds all bands through
+// distributed shared memory in the warp form's order (warp 1 with the T_L
+// weights when a model is kept), so every CTA holds the same sums and advances
+// the same controller, and the loop ends on the same evaluation everywhere.  The
+// band values alternate between two buffers over the cluster's successive
+// evaluations (par counts them across calls): evaluation k writes buffer k % 2
+// after the barrier of evaluation k - 1, which every reader of buffer (k - 2) % 2
+// has passed.  One cell's evaluation thus runs on C SMs' FP64 units.  sm:
+// cta_solve_smem_doubles doubles per CTA.  Every thread of every CTA of the
+// cluster must call it (it synchronises the cluster).
+template <bool COOP>
+__device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, const double* wb, double Ep, double T0,
+                                                  double trust_rel, int maxit, double* Jrow, double* sm, unsigned& par) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
-  const int rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
-  const double* wb = th.a_p;
+  const int rank = COOP ? (int)cl.block_rank() : 0, nr = COOP ? (int)cl.num_blocks() : 1;
   const int nbp = th.nbp, ng = th.ng;
   const int own0 = rank * nbp / nr, own1 = (rank + 1) * nbp / nr;  // this CTA's bands
   const int pairs = cta_solve_pairs(nbp, ng, nr), cb = pairs / ng;  // bands per chunk (ng <= kMaxGauss)
-  double* pt = sm;                        // [4][pairs] node_terms of each pair
-  double* bv2 = pt + 4 * pairs;  // [2][4][nbp] per band I0 and three derivatives (own bands), two buffers
-  double* sums = bv2 + 8 * nbp;           // [4] this CTA's copy of F and its derivatives
+  double* pt = sm;                // [4][pairs] node_terms of each pair
+  double* bv2 = pt + 4 * pairs;   // [2][4][nbp] per band Taylor coefficients (own bands), two buffers
+  double* sums = bv2 + 8 * nbp;   // [8] this CTA's copy of the sums with wb, and with the T_L weights
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   SolveCtl c(T0);
   for (int loop = 0; loop < maxit + 224 && !c.done; ++loop) {
     double* bv = bv2 + (size_t)(par++ & 1u) * 4 * nbp;
-    const double rT = 1.0 / c.T;
+    const double rT = rcp_pos(c.T);
     for (int b0 = own0; b0 < own1; b0 += cb) {
       const int npair = min(cb, own1 - b0) * ng;
       const double* cn = th.node_c + b0 * ng;
@@ -217,33 +227,31 @@ __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double
       }
       __syncthreads();
 #pragma unroll 1
-      for (int k = threadIdx.x; k < npair / ng; k += blockDim.x) {
-        const int b = b0 + k;
+      for (int e = threadIdx.x; e < npair / ng * 4; e += blockDim.x) {
+        const int k = e >> 2, q = e & 3, b = b0 + k;
         const double* C = th.node_C + b * ng;
-        double s[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 2
-        for (int i = 0; i < ng; ++i)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) s[q] = fma(C[i], pt[q * pairs + k * ng + i], s[q]);
-        const double f[4] = {s[0], s[1] * rT, s[2] * rT * rT, s[3] * rT * rT * rT};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          bv[q * nbp + b] = f[q];
-          if (Jrow) Jrow[q * nbp + b] = f[q];
-        }
+        double s = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < ng; ++i) s = fma(C[i], pt[q * pairs + k * ng + i], s);
+        s *= taylor_scale(q, rT);
+        bv[q * nbp + b] = s;
+        if (Jrow) Jrow[q * nbp + b] = s;
       }
       __syncthreads();
     }
-    cl.sync();  // every CTA's bands are in its bv
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
+    if constexpr (COOP) cl.sync();  // every CTA's bands are in its bv
+    if (wid == 0 || (wid == 1 && Jrow)) {
+      const double* wt = wid == 0 ? wb : th.a_L;
       double F[4] = {0.0, 0.0, 0.0, 0.0};
       for (int b = lane; b < nbp; b += 32) {
-        int o = (int)(((long long)b * nr) / nbp);  // the CTA whose range holds b
-        while (o + 1 < nr && (o + 1) * nbp / nr <= b) ++o;
-        while (o > 0 && o * nbp / nr > b) --o;
-        const double* ob = cl.map_shared_rank(bv, (unsigned)o);
-        const double ap = wb[b];
+        const double* ob = bv;
+        if constexpr (COOP) {
+          int o = (int)(((long long)b * nr) / nbp);  // the CTA whose range holds b
+          while (o + 1 < nr && (o + 1) * nbp / nr <= b) ++o;
+          while (o > 0 && o * nbp / nr > b) --o;
+          ob = cl.map_shared_rank(bv, (unsigned)o);
+        }
+        const double ap = wt[b];
 #pragma unroll
         for (int q = 0; q < 4; ++q) F[q] = fma(ap, ob[q * nbp + b], F[q]);
       }
@@ -253,13 +261,16 @@ __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, double
       }
       if (lane == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) sums[q] = F[q];
+        for (int q = 0; q < 4; ++q) sums[4 * wid + q] = F[q];
       }
     }
     __syncthreads();
-    c.advance(sums[0], sums[1], sums[2], sums[3], Ep, trust_rel, maxit);
+    c.advance(sums, Ep, trust_rel, maxit);
   }
-  return c.finish();
+  SolveResult r = c.finish();
+#pragma unroll
+  for (int q = 0; q < 4; ++q) r.ML[q] = sums[4 + q];
+  return r;
 }
 
 }  // namespace bte

@@ -142,4 +142,42 @@ __device__ __forceinline__ double full_I<FFElem>(const FFElem* I, long long e, i
   return ff::to_double(p[0], p[2]);
 }
 
+
+// Two consecutive stored values (e even) as doubles, without the reference part of
+// the reduced modes, and the reverse.
+// (load and conversion apart: the conversion of ff pairs branches, and a load behind
+// a branch is not issued early, so callers with several loads in flight take both)
+template <typename S> struct RawPair { using R = double2; };
+template <> struct RawPair<FFElem> { using R = ulonglong2; };
+template <> struct RawPair<float> { using R = float2; };
+template <> struct RawPair<__nv_bfloat16> { using R = __nv_bfloat162; };
+template <typename S>
+__device__ __forceinline__ typename RawPair<S>::R ld_raw(const S* p) {
+  return *reinterpret_cast<const typename RawPair<S>::R*>(p);
+}
+__device__ __forceinline__ void raw_pair(const double2& v, double& a, double& b) { a = v.x; b = v.y; }
+__device__ __forceinline__ void raw_pair(const ulonglong2& v, double& a, double& b) { ff::to_doubles(ff::P2{v.x, v.y}, a, b); }
+__device__ __forceinline__ void raw_pair(const float2& v, double& a, double& b) { a = (double)v.x; b = (double)v.y; }
+__device__ __forceinline__ void raw_pair(const __nv_bfloat162& v, double& a, double& b) { raw_pair(__bfloat1622float2(v), a, b); }
+template <typename S>
+__device__ __forceinline__ void ld_pair(const S* p, double& a, double& b) {
+  raw_pair(ld_raw(p), a, b);
+}
+template <typename S>
+__device__ __forceinline__ void st_pair(S* p, double a, double b) {
+  if constexpr (sizeof(S) == 8) *reinterpret_cast<double2*>(p) = make_double2(a, b);
+  else if constexpr (sizeof(S) == 4) *reinterpret_cast<float2*>(p) = make_float2((float)a, (float)b);
+  else {
+    __nv_bfloat162 v;
+    v.x = __double2bfloat16(a);
+    v.y = __double2bfloat16(b);
+    *reinterpret_cast<__nv_bfloat162*>(p) = v;
+  }
+}
+template <>
+__device__ __forceinline__ void st_pair<FFElem>(FFElem* p, double a, double b) {
+  const ff::P2 v = ff::from_doubles(a, b);
+  *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.h, v.l);
+}
+
 }  // namespace bte

@@ -17,8 +17,8 @@
 // beside the row sweeps of bte_rows.cuh.
 // Each lane sums its part of G_b = sum_d w_d I^{k+1}_{d,b} in float partials flushed
 // to FP64; at the end of an item the band owners add the dteam partials per band
-// in a fixed order and write G_b to Gc, from which cells_kernel (bte_cells.cu)
-// solves T_p and refreshes I0.
+// in a fixed order and write their bands' energies to Ec, from which cells_kernel
+// (bte_cells.cu) solves T_p and refreshes I0.
 // Memory: I^n is read once, I^{k+1} written once, and each I^k row read from
 // DRAM once (adjacent cells, processed together, re-read it from L2).  Each
 // thread copies the operands of its next directions into shared memory with
@@ -101,12 +101,12 @@ struct Ring {
 
 // The end of an item: the lanes of a cell hold the partials G[v] of their
 // directions; the band owners (dg == 0) add them in a fixed order to the
-// W I0_b(T_ref) term of the deviation storage and write G_b to Gc.  With one
+// W I0_b(T_ref) term of the deviation storage and write their energies to Ec.  With one
 // direction per team step a lane's sums are complete and no barrier is needed;
 // otherwise every thread calls it (two CTA barriers).
 __device__ __forceinline__ void write_band_sums(const SweepArgs& a, double* gsm, bool active, int dg, int lane,
                                                 long long P, double (&G)[V]) {
-  const int lpc = a.lpc, nbp = a.th.nbo, b0 = V * lane;
+  const int lpc = a.lpc, b0 = V * lane;
   if (a.dteam > 1) {
 #pragma unroll
     for (int v = 0; v < V; ++v) gsm[(size_t)threadIdx.x * V + v] = G[v];
@@ -118,10 +118,14 @@ __device__ __forceinline__ void write_band_sums(const SweepArgs& a, double* gsm,
     __syncthreads();
   }
   if (dg == 0 && active) {
+    double eL = 0.0, eP = 0.0;
 #pragma unroll
-    for (int v = 0; v < V; v += 2)
-      *reinterpret_cast<double2*>(a.Gc + P * nbp + b0 + v) =
-          make_double2(fma(a.Wtot, a.I0ref[b0 + v], G[v]), fma(a.Wtot, a.I0ref[b0 + v + 1], G[v + 1]));
+    for (int v = 0; v < V; ++v) {
+      const double g = fma(a.Wtot, a.I0ref[b0 + v], G[v]);
+      eL = fma(g, a.th.inv_v[b0 + v], eL);
+      eP = fma(g, a.th.binv_v[b0 + v], eP);
+    }
+    a.Ec[P * lpc + lane] = make_double2(eL, eP);
   }
 }
 

@@ -23,10 +23,12 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <numeric>
 #include <string>
 #include <vector>
 
 #include "../../include/bte_umesh.h"
+#include "bte_flux.cuh"
 #include "bte_internal.h"
 #include "bte_solve.cuh"
 #include "bte_store.cuh"
@@ -316,47 +318,89 @@ __global__ void umesh_gout_kernel(const int* cf_ptr, const double* g, int nd, lo
 }
 
 // Diffuse ghosts: for each listed boundary face, per band,
-// sum_{S.n > 0} (S.n) I / sum_{S.n < 0} |S.n| of the owner cell.  One CTA of
-// kDiffWarps warps per face: warp w sums the directions [w nd/W, (w+1) nd/W)
-// (lanes over bands); the partial sums are added in warp order.  Reduced
-// storage sums the stored deviations and writes the ghost deviation (the
+// sum_{S.n > 0} (S.n) I / sum_{S.n < 0} |S.n| of the owner cell.  One CTA of 256
+// threads per face, bound by one face's latency (there are fewer faces than CTA
+// slots): the warps form S.n of all directions once and list the leaving ones in
+// order; then a lane holds the V bands of one 16-byte vector and sums every
+// groups-th listed direction, eight loads in flight; the groups' partials are
+// added in order.  (Eight warps, each forming S.n per direction and band lane:
+// 54 us for 64 faces x 400 x 55 in FP64, 106 us for 198 in FP32.)
+// Reduced storage sums the stored deviations and writes the ghost deviation (the
 // reference part passes through the ratio: the sets are point-symmetric).
 // On a partially specular face the row receives (1 - p) x the diffuse value
 // (the sweep adds p x the mirrored value).
-constexpr int kDiffWarps = 8;
+constexpr int kDiffThreads = 256, kDiffWarps = kDiffThreads / 32;
 
 template <typename St>
-__global__ void __launch_bounds__(32 * kDiffWarps) umesh_diffuse_kernel(const St* I, const long long* bfs, int nlist,
-                                                                        const long long* bface, const long long* owner,
-                                                                        const double* nA, const double* S, int nd,
-                                                                        int nbp, const double* spec, double* ghost,
-                                                                        float* ghost_dev) {
-  extern __shared__ double part[];  // [kDiffWarps][2][nbp]
+__global__ void __launch_bounds__(kDiffThreads) umesh_diffuse_kernel(const St* I, const long long* bfs, int nlist,
+                                                                     const long long* bface, const long long* owner,
+                                                                     const double* nA, const double* S, int nd, int nbp,
+                                                                     const double* spec, double* ghost,
+                                                                     float* ghost_dev) {
+  using T = Tr<St>;
+  constexpr int V = T::V;
+  extern __shared__ double part[];  // [groups][nbp], then S.n of the listed directions [nd], then the list [nd]
+  __shared__ int cnt[kDiffWarps];
+  __shared__ double den_w[kDiffWarps];
+  const int lpc = nbp / V, groups = kDiffThreads / lpc, grp = threadIdx.x / lpc, b0 = V * (threadIdx.x - grp * lpc);
+  double* sn_out = part + groups * nbp;
+  int* list = reinterpret_cast<int*>(sn_out + nd);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int d0 = (int)((long long)wid * nd / kDiffWarps), d1 = (int)((long long)(wid + 1) * nd / kDiffWarps);
   for (int k = blockIdx.x; k < nlist; k += gridDim.x) {
     const long long bf = bfs[k], f = bface[bf], P = owner[f];
-    const double* n = nA + 3 * f;
-    const St* row = I + P * (long long)nd * nbp;
-    for (int b = lane; b < nbp; b += 32) {
-      double num = 0.0, den = 0.0;
-#pragma unroll 4
-      for (int e = d0; e < d1; ++e) {
-        const double sn = S[3 * e] * n[0] + S[3 * e + 1] * n[1] + S[3 * e + 2] * n[2];
-        if (sn > 0.0) num = fma(sn, Tr<St>::to_double(row[(long long)e * nbp + b]), num);
-        else den -= sn;
-      }
-      part[(wid * 2) * nbp + b] = num;
-      part[(wid * 2 + 1) * nbp + b] = den;
+    const double n0 = nA[3 * f], n1 = nA[3 * f + 1], n2 = nA[3 * f + 2];
+    auto dot = [&](int d) { return S[3 * d] * n0 + S[3 * d + 1] * n1 + S[3 * d + 2] * n2; };
+    double den = 0.0;
+    int m = 0;
+    for (int d = d0 + lane; d - lane < d1; d += 32) {
+      const double sn = d < d1 ? dot(d) : 0.0;
+      if (!(sn > 0.0)) den -= sn;
+      m += __popc(__ballot_sync(0xffffffffu, sn > 0.0));
+    }
+    for (int o = 16; o > 0; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    if (lane == 0) {
+      cnt[wid] = m;
+      den_w[wid] = den;
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < nbp; b += blockDim.x) {
-      double num = 0.0, den = 0.0;
-      for (int w = 0; w < kDiffWarps; ++w) {
-        num += part[(w * 2) * nbp + b];
-        den += part[(w * 2 + 1) * nbp + b];
+    int at = 0, nout = 0;
+    for (int w = 0; w < kDiffWarps; ++w) {
+      if (w < wid) at += cnt[w];
+      nout += cnt[w];
+    }
+    for (int d = d0 + lane; d - lane < d1; d += 32) {
+      const double sn = d < d1 ? dot(d) : 0.0;
+      const unsigned b = __ballot_sync(0xffffffffu, sn > 0.0);
+      if (sn > 0.0) {
+        const int q = at + __popc(b & ((1u << lane) - 1u));
+        sn_out[q] = sn;
+        list[q] = d;
       }
-      const double v = (1.0 - spec[bf]) * (den > 0.0 ? num / den : 0.0);
+      at += __popc(b);
+    }
+    __syncthreads();
+    if (grp < groups) {
+      const St* row = I + P * (long long)nd * nbp + b0;
+      double num[V];
+#pragma unroll
+      for (int v = 0; v < V; ++v) num[v] = 0.0;
+#pragma unroll 8
+      for (int q = grp; q < nout; q += groups) {
+        typename T::A x[V];
+        T::ld(row + (long long)list[q] * nbp, x);
+#pragma unroll
+        for (int v = 0; v < V; ++v) num[v] = fma(sn_out[q], (double)x[v], num[v]);
+      }
+#pragma unroll
+      for (int v = 0; v < V; ++v) part[grp * nbp + b0 + v] = num[v];
+    }
+    __syncthreads();
+    for (int b = threadIdx.x; b < nbp; b += kDiffThreads) {
+      double num = part[b], dn = 0.0;
+      for (int g = 1; g < groups; ++g) num += part[g * nbp + b];
+      for (int w = 0; w < kDiffWarps; ++w) dn += den_w[w];
+      const double v = (1.0 - spec[bf]) * (dn > 0.0 ? num / dn : 0.0);
       if constexpr (sizeof(St) == 8) ghost[bf * nbp + b] = v;
       else ghost_dev[bf * nbp + b] = (float)v;
     }
@@ -364,37 +408,43 @@ __global__ void __launch_bounds__(32 * kDiffWarps) umesh_diffuse_kernel(const St
   }
 }
 
-// Net heat flow out through each boundary face: one warp per face.
+// Net heat flow out through each boundary face: one CTA of 256 threads per face,
+// a thread per band walking every (threads / nbp)-th direction with four loads in
+// flight (one warp per face in direction order took 363 us for 224 faces x 400 x 55).
 template <typename St>
-__global__ void umesh_face_flux_kernel(const St* I, const double* I0ref, const double* ghost, const float* ghost_dev,
-                                       const long long* bface, long long nbf, const long long* owner, const double* nA,
-                                       const int* bf_mirror, const int* bf_axis, const double* bf_spec,
-                                       const int* refl, const double* S, int nd, int nbp, int nb, double* Qb) {
-  const int warps = blockDim.x / 32, lane = threadIdx.x & 31;
-  for (long long bf = blockIdx.x * (long long)warps + threadIdx.x / 32; bf < nbf; bf += (long long)gridDim.x * warps) {
+__global__ void __launch_bounds__(kFluxThreads) umesh_face_flux_kernel(
+    const St* I, const double* I0ref, const double* ghost, const float* ghost_dev, const long long* bface, long long nbf,
+    const long long* owner, const double* nA, const int* bf_mirror, const int* bf_axis, const double* bf_spec,
+    const int* refl, const double* S, int nd, int nbp, int nb, double* Qb) {
+  __shared__ double sh[kFluxThreads];
+  const int rows = kFluxThreads / nbp, r = threadIdx.x / nbp, b = threadIdx.x - r * nbp;
+  for (long long bf = blockIdx.x; bf < nbf; bf += gridDim.x) {
     const long long f = bface[bf], P = owner[f];
-    const double* n = nA + 3 * f;
+    const double n0 = nA[3 * f], n1 = nA[3 * f + 1], n2 = nA[3 * f + 2];
     const long long base = P * (long long)nd * nbp;
     double s = 0.0;
-    for (int d = 0; d < nd; ++d) {
-      const double sn = S[3 * d] * n[0] + S[3 * d + 1] * n[1] + S[3 * d + 2] * n[2];
-      for (int b = lane; b < nb; b += 32) {
-        double v;
-        const int mk = bf_mirror[bf];
-        if (sn > 0.0) {
-          v = full_I(I, base + (long long)d * nbp + b, b, I0ref);
-        } else if (mk == 1) {
-          v = full_I(I, base + (long long)refl[bf_axis[bf] * nd + d] * nbp + b, b, I0ref);
-        } else {  // the ghost row, plus p x the mirrored value on a partially specular face
-          if constexpr (sizeof(St) == 8) v = ghost[bf * nbp + b];
-          else v = I0ref[b] * (mk == 2 ? 1.0 - bf_spec[bf] : 1.0) + (double)ghost_dev[bf * nbp + b];
-          if (mk == 2) v += bf_spec[bf] * full_I(I, base + (long long)refl[bf_axis[bf] * nd + d] * nbp + b, b, I0ref);
+    if (r < rows && b < nb) {
+      const int mk = bf_mirror[bf];
+      const int* map = refl + bf_axis[bf] * nd;
+      const double p = mk == 2 ? bf_spec[bf] : (mk == 1 ? 1.0 : 0.0);
+      double gv = 0.0;  // the ghost row (plus p x the mirrored value on a partially specular face)
+      if (mk != 1) {
+        if constexpr (sizeof(St) == 8) gv = ghost[bf * nbp + b];
+        else gv = I0ref[b] * (1.0 - p) + (double)ghost_dev[bf * nbp + b];
+      }
+#pragma unroll 4
+      for (int d = r; d < nd; d += rows) {
+        const double sn = S[3 * d] * n0 + S[3 * d + 1] * n1 + S[3 * d + 2] * n2;
+        double v = gv;
+        if (sn > 0.0 || mk != 0) {
+          const double x = full_I(I, base + (long long)(sn > 0.0 ? d : map[d]) * nbp + b, b, I0ref);
+          v = sn > 0.0 ? x : fma(p, x, gv);
         }
         s = fma(sn, v, s);
       }
     }
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) Qb[bf] = s;
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) Qb[bf] = s;
   }
 }
 
@@ -451,7 +501,7 @@ struct bte_umesh_ctx {
   int nd = 0;
   std::vector<double> S, w;
   std::vector<int> refl;  // [5][nd]: mirror across x, y, z; rotation about z by -alpha, by +alpha
-  std::vector<int> perm;  // the caller's index of every internal direction
+  std::vector<int> perm;  // the caller's index of every stored direction (the identity)
   double Wtot = 0.0;
   // bands
   bool bands_set = false, solve_tp = false;
@@ -481,7 +531,8 @@ struct bte_umesh_ctx {
   long long *cf_up = nullptr, *bface_d = nullptr, *owner_d = nullptr, *diff_d = nullptr;
   int ndiff = 0;
   FixItem* fix = nullptr;
-  double* Gc = nullptr;    // [cell][nbp] band sums
+  double2* Ec = nullptr;   // [cell][kRedEntries] partial energies
+  double* MsumL = nullptr; // [cell][4] the T_L model's sums
   DevCounters* counters = nullptr;
   int lpc = 0, dteam = 1;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
@@ -554,8 +605,11 @@ SweepArgs cell_args(bte_umesh_ctx* u, double* Inew) {
   a.maxit = u->opts.newton_maxit;
   a.counters = u->counters;
   a.fix = u->fix;
-  a.Gc = u->Gc;
-  a.gsplit = 1;
+  a.Ec = u->Ec;
+  a.ne = kRedEntries;
+  a.MsumL = u->MsumL;
+  a.TL = u->TL;
+  a.Tguess = u->solve_tp ? u->Tp : u->TL;
   a.partial = 0;
   a.I0ref = u->I0ref;
   a.Wtot = u->Wtot;
@@ -589,7 +643,7 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = dalloc(u, &u->vb_d, nbp)) || (rc = dalloc(u, &u->bb_d, nbp)) || (rc = dalloc(u, &u->scratch, nc)) ||
       (rc = dalloc(u, &u->Qb, nbf)) || (rc = dalloc(u, &u->qbuf, nc * 3)) || (rc = dalloc(u, &u->bf_mirror_d, nbf)) || (rc = dalloc(u, &u->bf_axis_d, nbf)) || (rc = dalloc(u, &u->bf_spec_d, nbf)) || (rc = dalloc(u, &u->bscale, nc)) ||
       (rc = dalloc(u, &u->refl_d, 5 * nd)) || (rc = dalloc(u, &u->perm_d, nd)) || (rc = dalloc(u, &u->bface_d, nbf)) || (rc = dalloc(u, &u->owner_d, u->nf)) ||
-      (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, cells_queue_entries(nc))) || (rc = dalloc(u, &u->Gc, nc * nbp)) ||
+      (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, cells_queue_entries(nc))) || (rc = dalloc(u, &u->Ec, nc * kRedEntries)) || (rc = dalloc(u, &u->MsumL, nc * 4)) ||
       (rc = dalloc(u, &u->counters, 1)) || (rc = dalloc(u, &u->node_c, nbp * u->ng)) ||
       (rc = dalloc(u, &u->node_C, nbp * u->ng)) || (rc = dalloc(u, &u->a_p, nbp)) || (rc = dalloc(u, &u->a_L, nbp)) ||
       (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->beta_d, nbp)) || (rc = dalloc(u, &u->binv_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
@@ -724,17 +778,18 @@ int upload_bc(bte_umesh_ctx* u) {
 cudaError_t refresh_diffuse(bte_umesh_ctx* u, const void* I) {
   if (u->ndiff == 0) return cudaSuccess;
   const int grid = (int)std::min<long long>(u->ndiff, 152LL * 16);
-  const size_t sm = (size_t)kDiffWarps * 2 * u->nbp * sizeof(double);
+  const int lpc = u->nbp / values_per_lane(u->prec);
+  const size_t sm = ((size_t)(kDiffThreads / lpc) * u->nbp + u->nd) * sizeof(double) + u->nd * sizeof(int);
   if (u->prec == BTE_FP64)
-    umesh_diffuse_kernel<double><<<grid, 32 * kDiffWarps, sm, u->stream>>>(
+    umesh_diffuse_kernel<double><<<grid, kDiffThreads, sm, u->stream>>>(
         (const double*)I, u->diff_d, u->ndiff, u->bface_d, u->owner_d, u->nA_d, u->S_d, u->nd, u->nbp, u->bf_spec_d,
         u->ghost, nullptr);
   else if (u->prec == BTE_FP32)
-    umesh_diffuse_kernel<float><<<grid, 32 * kDiffWarps, sm, u->stream>>>(
+    umesh_diffuse_kernel<float><<<grid, kDiffThreads, sm, u->stream>>>(
         (const float*)I, u->diff_d, u->ndiff, u->bface_d, u->owner_d, u->nA_d, u->S_d, u->nd, u->nbp, u->bf_spec_d,
         nullptr, u->ghost_dev);
   else
-    umesh_diffuse_kernel<__nv_bfloat16><<<grid, 32 * kDiffWarps, sm, u->stream>>>(
+    umesh_diffuse_kernel<__nv_bfloat16><<<grid, kDiffThreads, sm, u->stream>>>(
         (const __nv_bfloat16*)I, u->diff_d, u->ndiff, u->bface_d, u->owner_d, u->nA_d, u->S_d, u->nd, u->nbp,
         u->bf_spec_d, nullptr, u->ghost_dev);
   return cudaGetLastError();
@@ -742,8 +797,7 @@ cudaError_t refresh_diffuse(bte_umesh_ctx* u, const void* I) {
 
 int ensure_TL(bte_umesh_ctx* u) {
   if (u->TL_valid) return BTE_OK;
-  UTRY(u, launch_solve_TL(u->TL, u->EL, u->solve_tp ? u->Tp : u->TL, u->J, u->Teval, u->nc, uthermo(u),
-                          model_trust(u->opts.newton_rtol), u->opts.newton_maxit, u->counters, u->stream));
+  UTRY(u, launch_cells(cell_args(u, nullptr), u->nc, 3, nullptr, u->stream));
   u->TL_valid = true;
   return BTE_OK;
 }
@@ -816,8 +870,12 @@ int bte_umesh_create(const bte_umesh_desc* m, const bte_opts* opts, bte_umesh* o
     delete u;
     return ufail(nullptr, BTE_E_ARG, "bad direction set");
   }
-  u->perm = internal_order(u->S, u->w, u->refl, o.dir_kind == BTE_DIRS_INPLANE ? 4 : 8);
   u->nd = (int)u->w.size();
+  // rows in the caller's order: neighbouring azimuths share most inflow faces, so
+  // the lanes of a warp take the same branches (the structured handle's order cost
+  // the FP64 sweep 10 %)
+  u->perm.resize(u->nd);
+  std::iota(u->perm.begin(), u->perm.end(), 0);
   u->refl.resize(5 * (size_t)u->nd);
   for (int d = 0; d < u->nd; ++d) u->refl[3 * u->nd + d] = u->refl[4 * u->nd + d] = d;  // until a rotation is set
   if (m->fc) u->fc.assign(m->fc, m->fc + 3 * m->nfaces);
@@ -936,7 +994,7 @@ int bte_umesh_set_initial(bte_umesh u, const double* T_cells, double T_uniform) 
   int rc = upload(u, u->scratch, T.data(), u->nc);
   if (rc) return rc;
   u->cur = 0;
-  UTRY(u, launch_init_cells(u->prec, false, u->I[0], u->I0cell, u->J, u->Msum, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
+  UTRY(u, launch_init_cells(u->prec, false, u->I[0], u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
                             (int)u->nc, u->nd, uthermo(u), u->stream));
   UTRY(u, cudaStreamSynchronize(u->stream));
   u->init_done = true;
@@ -1122,11 +1180,12 @@ int bte_umesh_set_intensity(bte_umesh u, const double* in, const double* Tp_cell
   cudaError_t e = cudaMalloc(&tmp, n * 8);
   if (e != cudaSuccess) return ufail(u, BTE_E_NOMEM, "cudaMalloc(%zu bytes): %s", n * 8, cudaGetErrorString(e));
   e = cudaMemcpyAsync(tmp, in, n * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess)
-    e = launch_pack(u->prec, false, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(u->Tp, Tp_cells, u->nc * 8, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = launch_state_from_Tp(u->I0cell, u->J, u->Msum, u->Tp, u->Teval, u->nc, uthermo(u), s);
-  if (e == cudaSuccess) e = launch_energy_L(u->prec, false, u->I[u->cur], u->I0ref, u->EL, u->w_d, u->nc, u->nd, uthermo(u), s);
+  if (e == cudaSuccess) e = launch_state_from_Tp(u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->nc, uthermo(u), s);
+  const SweepArgs sums = cell_args(u, u->I[u->cur]);
+  if (e == cudaSuccess)
+    e = launch_pack(u->prec, false, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, &sums, s);
+  if (e == cudaSuccess) e = launch_energy_L(u->Ec, u->EL, u->nc, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(tmp);
   if (e != cudaSuccess) return ufail(u, BTE_E_CUDA, "restoring the state: %s", cudaGetErrorString(e));
@@ -1140,7 +1199,7 @@ int bte_umesh_get_flux(bte_umesh u, double* q, double* Q) {
   cudaStream_t s = u->stream;
   const double* I = u->I[u->cur];
   if (q) {
-    UTRY(u, launch_flux_cells(u->prec, false, I, u->qbuf, u->S_d, 0, (int)u->nc, u->nd, u->nbp, 3, s));
+    UTRY(u, launch_flux_cells(u->prec, false, false, I, u->qbuf, u->S_d, 0, (int)u->nc, u->nd, u->nbp, 3, s));
     UTRY(u, cudaMemcpyAsync(q, u->qbuf, (size_t)u->nc * 3 * 8, cudaMemcpyDeviceToHost, s));
     UTRY(u, cudaStreamSynchronize(s));
   }
@@ -1148,17 +1207,17 @@ int bte_umesh_get_flux(bte_umesh u, double* q, double* Q) {
     const long long nbf = (long long)u->bface.size();
     UTRY(u, refresh_diffuse(u, I));
     if (nbf > 0) {
-      const int gr = grid_for(nbf, 4);
+      const int gr = grid_for(nbf, 1);
       if (u->prec == BTE_FP64)
-        umesh_face_flux_kernel<double><<<gr, 128, 0, s>>>((const double*)I, u->I0ref, u->ghost, u->ghost_dev, u->bface_d,
+        umesh_face_flux_kernel<double><<<gr, kFluxThreads, 0, s>>>((const double*)I, u->I0ref, u->ghost, u->ghost_dev, u->bface_d,
                                                           nbf, u->owner_d, u->nA_d, u->bf_mirror_d, u->bf_axis_d, u->bf_spec_d,
                                                           u->refl_d, u->S_d, u->nd, u->nbp, u->nb, u->Qb);
       else if (u->prec == BTE_FP32)
-        umesh_face_flux_kernel<float><<<gr, 128, 0, s>>>((const float*)I, u->I0ref, u->ghost, u->ghost_dev, u->bface_d,
+        umesh_face_flux_kernel<float><<<gr, kFluxThreads, 0, s>>>((const float*)I, u->I0ref, u->ghost, u->ghost_dev, u->bface_d,
                                                          nbf, u->owner_d, u->nA_d, u->bf_mirror_d, u->bf_axis_d, u->bf_spec_d,
                                                          u->refl_d, u->S_d, u->nd, u->nbp, u->nb, u->Qb);
       else
-        umesh_face_flux_kernel<__nv_bfloat16><<<gr, 128, 0, s>>>((const __nv_bfloat16*)I, u->I0ref, u->ghost,
+        umesh_face_flux_kernel<__nv_bfloat16><<<gr, kFluxThreads, 0, s>>>((const __nv_bfloat16*)I, u->I0ref, u->ghost,
                                                                  u->ghost_dev, u->bface_d, nbf, u->owner_d, u->nA_d,
                                                                  u->bf_mirror_d, u->bf_axis_d, u->bf_spec_d, u->refl_d, u->S_d, u->nd,
                                                                  u->nbp, u->nb, u->Qb);
