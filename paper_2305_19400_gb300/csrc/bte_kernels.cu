@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, co
 
 // Energies after a separate sweep (the sweep-ordered pass, the unstructured sweep) and
 // a restore in reduced storage: one CTA of 8 warps per cell.  Loads of 16 bytes, eight in
-// flight; FP64: warp w sums the directions [w nd / 8, (w + 1) nd / 8), lanes over
+// flight; FP64: four, warp w sums the directions [w nd / 8, (w + 1) nd / 8), lanes over
 // band pairs (whole warps on one direction, so the runs of the fixed-point sums
 // close together: groups of 28 lanes took 406 us where this takes 308 on 6144 cells
 // x 400 x 55); reduced storage: lanes over the V bands of a vector, 256 V / nbp
@@ -381,9 +381,8 @@ __global__ void __launch_bounds__(kRedThreads, 4) gs_reduce_kernel(SweepArgs a, 
           }
         };
         int d = d0;
-        for (; d + 8 <= d1; d += 8) batch(std::integral_constant<int, 8>{}, d);
-        for (; d + 2 <= d1; d += 2) batch(std::integral_constant<int, 2>{}, d);
-        if (d < d1) batch(std::integral_constant<int, 1>{}, d);
+        for (; d + 4 <= d1; d += 4) batch(std::integral_constant<int, 4>{}, d);
+        for (; d < d1; ++d) batch(std::integral_constant<int, 1>{}, d);
         sum.close();
         g[0] = sum.G[0];
         g[1] = sum.G[1];

@@ -55,19 +55,21 @@ struct UArgs {
   const int* bf_axis;      // [bface]
   const double* bf_spec;   // [bface] specularity p of kind-2 faces
   const int* refl;         // [3][nd]
-  const double* R;         // [nc][nd][nbp] implicit: 1 / (1/dt + beta_b + v_b gout)
+  const double* R;         // [nc][nd][nbp] implicit: v_b / (1/dt + beta_b + v_b gout)
   const double* vb;        // [nbp] v_b (0 on padding)
   const double* bb;        // [nbp] beta_b (0 on padding)
   double dt, rdt;
   long long nc;
   int nd, nbp, lpc, dteam;
+  const double* inv_v;     // [nbp] 1 / v_b
+  const double* bov;       // [nbp] beta_b / v_b
   // reduced storage (deviations from I0_b(T_ref)): buffers in the storage type,
   // R and the ghost deviations as float
   const void* Ind;
   const void* Ikd;
   void* Ioutd;
   void* Boutd;
-  const float* Rf;
+  const float* Rf;         // 1 / (1/dt + beta_b + v_b gout)
   const float* ghost_dev;
   const double* I0ref;
   const float* g32;        // [entries][nd] g as float (reduced storage)
@@ -92,7 +94,9 @@ __device__ __forceinline__ void ldf(const float* p, float (&x)[V]) {
 // dev + dt [beta (I0 - I0ref - dev) - v (gout dev - sum |g| dev_up)].
 // A lane holds V bands (16 bytes of storage).  The kernel is bound by the
 // latency of the face gathers, so it is capped at 6 CTAs of 252 threads per SM
-// (more warps in flight; measured faster than 3-5 CTAs despite small spills).
+// (more warps in flight; measured faster than 3-5 and 8 CTAs despite small spills).
+// FP32: R is loaded before the faces (5940 tetrahedra x 400 x 55: 498 us after them,
+// 455 before).
 template <typename S, bool EXPL, int BM, bool TT>
 __global__ void __launch_bounds__(256, 6) umesh_sweep_dev_kernel(UArgs a) {
   using T = Tr<S>;
@@ -129,8 +133,9 @@ __global__ void __launch_bounds__(256, 6) umesh_sweep_dev_kernel(UArgs a) {
     for (int v = 0; v < V; ++v) src[v] = bs[v] * (float)(a.I0cell[P * a.nbp + b0 + v] - a.I0ref[b0 + v]);
     for (int d = dg; d < a.nd; d += a.dteam) {
       const long long off = P * row + (long long)d * a.nbp + b0;
-      float in[V], f[V];
+      float in[V], f[V], R[V];
       T::ld(In + off, in);
+      if (!EXPL && sizeof(S) == 4) ldf<V>(a.Rf + off, R);  // before the faces' loads
 #pragma unroll
       for (int v = 0; v < V; ++v) f[v] = 0.f;
       for (int e = e0; e < e1; ++e) {
@@ -172,8 +177,8 @@ __global__ void __launch_bounds__(256, 6) umesh_sweep_dev_kernel(UArgs a) {
 #pragma unroll
         for (int v = 0; v < V; ++v) r[v] = fmaf(dt, fmaf(-bs[v], in[v], src[v]) - vb[v] * fmaf(go, in[v], -f[v]), in[v]);
       } else {
-        float R[V], B[V];
-        ldf<V>(a.Rf + off, R);
+        float B[V];
+        if (sizeof(S) != 4) ldf<V>(a.Rf + off, R);
 #pragma unroll
         for (int v = 0; v < V; ++v) B[v] = BM == 2 ? in[v] : in[v] * rdt * R[v];
         if (BM == 1) T::st(Bo + off, B);
@@ -193,9 +198,15 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 
 // EXPL: explicit scheme.  BM (implicit): 0 In is I^n; 1 In is I^n and B =
 // (I^n/dt) R is stored; 2 In holds B (the same in every inner iteration of a
-// step), so the update is R (beta I0 + v sum |g| I_up) + B.  Capped at 5 CTAs
-// of 256 threads per SM (48 registers, a few bytes of spill outside the face
-// loop): uncapped it takes 58 registers and 4 CTAs, measured 7 % slower.
+// step), so the update is v R ((beta / v) I0 + sum |g| I_up) + B: v R is what is
+// kept per (cell, direction, band), and the sum starts from the cell's own term, one
+// FP64 FMA per inflow face and one more per value.  Bound by the latency of the
+// gathers and, at 0.85 of it, the FP64 pipe; HBM, 24 bytes per value.  On 6144
+// triangles x 400 x 55 with R kept (two more FMAs per value) and read after the
+// faces 1078 us, 890 here.  Capped at 5 CTAs of 256 threads per SM (48 registers, a
+// few bytes of spill outside the face loop): warps in flight count more than loads in
+// flight per warp; 4 CTAs take 7 % longer, 6 the same, and a direction's gathers all
+// issued before its FMAs (4 CTAs of 64 registers) 20 % longer.
 template <bool EXPL, int BM, bool TT>
 __global__ void __launch_bounds__(256, 5) umesh_sweep_kernel(UArgs a) {
   const int team = a.lpc * a.dteam;
@@ -205,11 +216,13 @@ __global__ void __launch_bounds__(256, 5) umesh_sweep_kernel(UArgs a) {
   const int b0 = 2 * lane;
   if (slot >= cpb) return;  // no barrier below
   const long long row = (long long)a.nd * a.nbp;
-  const double v0 = a.vb[b0], v1 = a.vb[b0 + 1], be0 = a.bb[b0], be1 = a.bb[b0 + 1];
+  // explicit: v, beta; implicit: 1/v, beta/v
+  const double v0 = (EXPL ? a.vb : a.inv_v)[b0], v1 = (EXPL ? a.vb : a.inv_v)[b0 + 1];
+  const double be0 = (EXPL ? a.bb : a.bov)[b0], be1 = (EXPL ? a.bb : a.bov)[b0 + 1];
   for (long long P = (long long)blockIdx.x * cpb + slot; P < a.nc; P += (long long)gridDim.x * cpb) {
     const int e0 = a.cf_ptr[P], e1 = a.cf_ptr[P + 1];
     const double2 i0 = ld2(a.I0cell + P * a.nbp + b0);
-    // beta_b(T_p) = beta_b s (s = 1 unless TT) and (s - 1) beta_b
+    // beta_b(T_p) = beta_b s (s = 1 unless TT) and (s - 1) beta_b (implicit: over v)
     const double sc = TT ? a.bscale[P] : 1.0;
     const double bs0 = TT ? sc * be0 : be0, bs1 = TT ? sc * be1 : be1;
     const double sm0 = TT ? (sc - 1.0) * be0 : 0.0, sm1 = TT ? (sc - 1.0) * be1 : 0.0;
@@ -217,8 +230,10 @@ __global__ void __launch_bounds__(256, 5) umesh_sweep_kernel(UArgs a) {
     for (int d = dg; d < a.nd; d += a.dteam) {
       const long long off = P * row + (long long)d * a.nbp + b0;
       const double2 in = ld2(a.In + off);
+      double2 rr;  // before the faces' loads
+      if (!EXPL) rr = ld2(a.R + off);
       const double* Isrc = EXPL ? a.In : a.Ik;
-      double f0 = 0.0, f1 = 0.0;  // sum over inflow faces of |g| I_up
+      double f0 = EXPL ? 0.0 : bi0, f1 = EXPL ? 0.0 : bi1;  // + sum over inflow faces of |g| I_up
       for (int e = e0; e < e1; ++e) {
         const double ge = a.g[(long long)e * a.nd + d];
         if (__double_as_longlong(ge) < 0) {  // inflow: the sign bit, tested on the integer pipe
@@ -252,16 +267,15 @@ __global__ void __launch_bounds__(256, 5) umesh_sweep_kernel(UArgs a) {
         const double go = a.gout[P * a.nd + d];
         r0 = fma(a.dt, fma(bs0, i0.x - in.x, -v0 * fma(go, in.x, -f0)), in.x);
         r1 = fma(a.dt, fma(bs1, i0.y - in.y, -v1 * fma(go, in.y, -f1)), in.y);
-      } else {  // R [beta I0 + v sum |g| I_up] + (I^n/dt) R, R = 1 / [1/dt + beta + v gout]
-        const double2 rr = ld2(a.R + off);
+      } else {  // vR [(beta/v) I0 + sum |g| I_up] + (I^n/(v dt)) vR, R = 1 / [1/dt + beta + v gout]
         double B0 = in.x, B1 = in.y;
         if (BM != 2) {
-          B0 = in.x * a.rdt * rr.x;
-          B1 = in.y * a.rdt * rr.y;
+          B0 = in.x * (a.rdt * v0) * rr.x;
+          B1 = in.y * (a.rdt * v1) * rr.y;
           if (BM == 1) *reinterpret_cast<double2*>(a.Bout + off) = make_double2(B0, B1);
         }
-        r0 = fma(rr.x, fma(v0, f0, bi0), B0);
-        r1 = fma(rr.y, fma(v1, f1, bi1), B1);
+        r0 = fma(rr.x, f0, B0);
+        r1 = fma(rr.y, f1, B1);
         if constexpr (TT) {  // R_s = R / (1 + (s - 1) beta R): the cached R is at s = 1
           r0 *= __drcp_rn(fma(sm0, rr.x, 1.0));
           r1 *= __drcp_rn(fma(sm1, rr.y, 1.0));
@@ -272,15 +286,15 @@ __global__ void __launch_bounds__(256, 5) umesh_sweep_kernel(UArgs a) {
   }
 }
 
-// R[P][d][b] = 1 / (1/dt + beta_b + v_b gout[P][d]): the implicit update's
-// reciprocal diagonal, fixed while dt is (one thread per element).
+// R[P][d][b] = c_b / (1/dt + beta_b + v_b gout[P][d]), c = v (FP64) or 1: the implicit
+// update's reciprocal diagonal, fixed while dt is (one thread per element).
 template <typename R_t>
 __global__ void umesh_rcp_kernel(const double* gout, const double* vb, const double* bb, double rdt, long long nc,
                                  int nd, int nbp, R_t* R) {
   const long long n = nc * nd * nbp;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const int b = (int)(i % nbp);
-    R[i] = (R_t)(1.0 / fma(vb[b], gout[i / nbp], rdt + bb[b]));
+    R[i] = (R_t)((sizeof(R_t) == 8 ? vb[b] : 1.0) / fma(vb[b], gout[i / nbp], rdt + bb[b]));
   }
 }
 
@@ -1044,6 +1058,8 @@ int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, b
   a.refl = u->refl_d;
   a.vb = u->vb_d;
   a.bb = u->bb_d;
+  a.inv_v = u->inv_v;
+  a.bov = u->binv_d;
   a.dt = dt;
   a.rdt = 1.0 / dt;
   a.nc = u->nc;
