@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "bte_ff.cuh"
+#include "bte_pdl.cuh"
 #include "bte_store.cuh"
 
 namespace bte {
@@ -519,6 +520,7 @@ __global__ void __launch_bounds__(256, M::kMinB) rows_kernel(SweepArgs a) {
   constexpr int V = M::V, DT = Map<MAP>::DT, RUN = Map<MAP>::RUN, ROWS = DT * RUN;
   constexpr int kOps = 1 + DIM, kSlots = M::template slots<DIM>, kAhead = kSlots - 1;
   extern __shared__ char sm[];
+  pdl_trigger();
   const int nbp = a.th.nbo, nblk = a.nd / ROWS, lpc = nbp / V, team = lpc * DT;
   const int slot = threadIdx.x / team, tl = threadIdx.x - slot * team;
   const int dg = tl / lpc, b0 = V * (tl - dg * lpc);
