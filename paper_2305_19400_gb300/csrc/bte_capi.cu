@@ -93,7 +93,7 @@ struct bte_ctx {
   bool state_ff = false;
   double *I0cell = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr, *I0wall = nullptr;
   void* coef = nullptr;
-  // FP64: tables of the factored double-float sweep (bte_sweep_ff.cuh)
+  // FP64: tables of the factored double-float sweep (bte_rows.cuh)
   void* coef_R = nullptr;     // [cls][nd][nbp] R pairs
   float* dirc_ff = nullptr;   // [cls][nd][3][2]
   float* band_ff = nullptr;   // [2][nbp] 1/(v_b dt), beta_b/v_b pairs

@@ -1,6 +1,6 @@
 // bte_kernels.cu -- CUDA kernels around the sweep (sm_103a).  The sweeps (upwind
 // update, walls, band sums; Sec. 3.1, Eq. 4-6) live in bte_sweep.cuh and
-// bte_sweep_ff.cuh, the per-cell T_p step in bte_cells.cu.  Here:
+// bte_rows.cuh, the per-cell T_p step in bte_cells.cu.  Here:
 //   gs_reduce_kernel    energies after a sweep-ordered pass (bte_gs.cu) or an
 //                       unstructured sweep;
 //   init_cells / state_from_Tp / wall_I0 / wall_dev
@@ -68,11 +68,18 @@ __global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum,
     const double T = Tcells[c];
     cell_state_at(I0cell, J, Msum, MsumL, P, T, th, row);
     __syncthreads();
-    const long long n = (long long)nd * th.nbo;
-    for (long long e = threadIdx.x; e < n; e += blockDim.x) {
-      const int b = (int)(e % th.nbo);  // stored band; I0ref holds the stored bands
-      const double v = b < th.nbr ? (sizeof(S) == 8 ? row[th.band0 + b] : row[th.band0 + b] - I0ref[b]) : 0.0;
-      set_I(I, P * n + e, v);
+    // a thread keeps one pair of stored bands and walks the rows (16-byte stores in FP64)
+    const int pairs = th.nbo / 2, groups = (int)blockDim.x / pairs;
+    const int grp = groups ? threadIdx.x / pairs : 0;
+    S* cell = I + P * (long long)nd * th.nbo;
+    for (int p = threadIdx.x - grp * pairs; grp < max(groups, 1) && p < pairs; p += groups ? pairs : blockDim.x) {
+      double v[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int b = 2 * p + k;  // stored band; I0ref holds the stored bands
+        v[k] = b < th.nbr ? (sizeof(S) == 8 ? row[th.band0 + b] : row[th.band0 + b] - I0ref[b]) : 0.0;
+      }
+      for (int r = grp; r < nd; r += max(groups, 1)) st_pair(cell + (long long)r * th.nbo + 2 * p, v[0], v[1]);
     }
     if (threadIdx.x == 0) {
       double e = 0.0;

@@ -122,20 +122,6 @@ __device__ __forceinline__ double full_I(const S* I, long long e, int b, const d
   if constexpr (sizeof(S) == 8) return (double)I[e];
   else return I0ref[b] + Tr<S>::to_double(I[e]);
 }
-// Element e of a buffer set to v (a deviation in the reduced modes).
-template <typename S>
-__device__ __forceinline__ void set_I(S* I, long long e, double v) {
-  if constexpr (sizeof(S) == 2) I[e] = __double2bfloat16(v);
-  else I[e] = (S)v;
-}
-template <>
-__device__ __forceinline__ void set_I<FFElem>(FFElem* I, long long e, double v) {
-  float* p = reinterpret_cast<float*>(I) + 4 * (e >> 1) + (e & 1);
-  float h, l;
-  ff::split(v, h, l);
-  p[0] = h;
-  p[2] = l;
-}
 template <>
 __device__ __forceinline__ double full_I<FFElem>(const FFElem* I, long long e, int, const double*) {
   const float* p = reinterpret_cast<const float*>(I) + 4 * (e >> 1) + (e & 1);

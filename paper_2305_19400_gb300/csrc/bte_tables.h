@@ -14,7 +14,7 @@ void build_thermo(int nb, int nbp, int ng, const double* wlo, const double* whi,
 void build_coef(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
                 const double* vg, const double* beta, double dt, int explicit_scheme, double* out);
 
-// Tables of the factored double-float sweep (bte_sweep_ff.cuh) for one class,
+// Tables of the factored double-float sweep (bte_rows.cuh) for one class,
 // the implicit update divided through by v_b (v_b > 0 on every real band):
 // I' = B + R (sum_ax c_ax,d u_ax + (beta_b / v_b) I0),  B = (1 / (v_b dt)) R I^n,
 // R = 1 / (1 / (v_b dt) + beta_b / v_b + sum_ax c_ax,d).

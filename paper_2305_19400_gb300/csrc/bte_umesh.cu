@@ -602,7 +602,7 @@ ThermoTables uthermo(const bte_umesh_ctx* u) {
   return t;
 }
 
-// SweepArgs for the per-cell step and the fix-up (the fields those kernels read).
+// SweepArgs for the reduction and the per-cell step (the fields those kernels read).
 SweepArgs cell_args(bte_umesh_ctx* u, double* Inew) {
   SweepArgs a{};
   a.Iout = Inew;
