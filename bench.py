@@ -55,15 +55,15 @@ UNIT = "updates/s"
 PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "sweep_traffic.json")
 KERNEL_SRCS = [os.path.join(ROOT, "paper_2305_19400_gb300", "csrc", f) for f in ("bte_rows.cuh", "bte_ff.cuh", "bte_store.cuh")]
-# Algorithmic bytes of one implicit update: I^n (or B) read, I^k read once, I^{k+1} written.
+# Algorithmic bytes of one implicit update: I^n read, I^k read once, I^{k+1} written.
 BYTES_PER_UPDATE_FP64 = 24
-# Work of the dominant kernel (the double-float sweep of inner iterations 2..n-1,
-# 2-D): per lane step of two bands, 3 products of 4 packed ops (c_x u_x, c_y u_y,
-# and R times the sum), 3 pair sums of 8 (the two products, the source term,
-# B), a normalisation of 3 and the direction sum's accumulation of 8 = 47
-# packed f32x2 instructions for 2 updates, i.e. 47 FP32 lane operations per
-# update; counted against the measured packed-FMA rate in lane operations.
-FP32_LANE_OPS_PER_UPDATE_FF_2D = 47
+# Work of the dominant kernel (the double-float sweep, 2-D): per lane step of two
+# bands, 4 products of 4 packed ops (I^n/(v dt), c_x u_x, c_y u_y, and R times the
+# sum), 3 pair sums of 8 (the products and the source term), a normalisation of 3
+# and the direction sum's accumulation of 8 = 51 packed f32x2 instructions for 2
+# updates, i.e. 51 FP32 lane operations per update; counted against the measured
+# packed-FMA rate in lane operations.
+FP32_LANE_OPS_PER_UPDATE_FF_2D = 51
 # The strict IEEE-FP64 sweep: 3 FMAs per update (B + A_x I_x + A_y I_y + A_s I0)
 # in inner iterations 2..n, 4 in the first (A_n I^n).
 FP64_FMAS_PER_UPDATE_2D = 3
@@ -384,7 +384,7 @@ def run_variants(peaks, fp64_peak):
         "exact_evaluations_per_step": [learned["solves_per_step"]["solve_evals"],
                                        plain["solves_per_step"]["solve_evals"]],
         "note": "steady operation solves every cell from its cached model; the network only starts the exact "
-                "solve of the fix-up cells"}
+                "solve of the cells outside their models' trust radius"}
     return out
 
 
@@ -668,7 +668,7 @@ def main():
     if world > 1:
         dist.all_reduce(t, op=dist.ReduceOp.MAX)
     ms_max = float(t.item())
-    # sweep + fix-up kernel per inner iteration (+ the cell solve after the exchange of a band range)
+    # sweep + per-cell step per inner iteration (+ the cells' second half after the exchange of a band range)
     launches = (3 if partitioned else 2) * args.steps * args.ninner
     total_updates_per_step = wl.dof * args.ninner if partitioned else world * updates_per_step
     value = total_updates_per_step * args.steps / (ms_max * 1e-3)
@@ -716,7 +716,7 @@ def main():
         return 0
     peaks, peak_src = read_peaks()
     # roofline of the dominant kernel: the middle inner iterations' sweep (the
-    # double-float variant that reads and writes ff iterates), per launch
+    # double-float variant), per launch
     mid = sweep_ms[1:-1] if len(sweep_ms) > 2 else sweep_ms
     launch_ms = float(np.mean(mid))
     upd_launch = updates_per_step / args.ninner
@@ -727,8 +727,8 @@ def main():
     roofline = {"bound": "hbm", "achieved": hbm, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": hbm / peaks["hbm_gbs"], "traffic": (tpu * upd_launch) if tpu else None,
                 "peak_source": f"hbm_gbs of {peak_src} peaks (copy bandwidth)",
-                "kernel": "sweep_ff_kernel<2, MINB, 2, 3> (double-float sweep of inner iterations 2..15: "
-                          "B and I^k read as ff pairs, I^{k+1} written as ff pairs)",
+                "kernel": "rows_kernel<2, MAP, FF> (double-float sweep of inner iterations 2..15: "
+                          "I^n and I^k read as ff pairs, I^{k+1} written as ff pairs)",
                 "launch_ms": launch_ms, "launches_averaged": len(mid), "bytes_per_update": BYTES_PER_UPDATE_FP64,
                 "sweep_ms_last_step": [round(float(x), 4) for x in sweep_ms],
                 "timing": "CUDA events recorded by the step graph around each sweep launch, last timed step",

@@ -164,7 +164,7 @@ int bte_set_bands(bte_handle h, int nb, const double* omega_lo, const double* om
  * bte_workspace_bytes, bte_set_bc, bte_set_initial), bte_set_band_range makes
  * this handle store and sweep only bands [band_lo, band_hi) of the table; the
  * temperature solve still uses every band.  Each inner iteration then runs
- * sweep -> exchange -> cell solve -> fix-up: the sweep writes this handle's
+ * sweep -> partial sums -> exchange -> cell solve: the second kernel writes this handle's
  * per-cell partial sums (E_L, E_p) over its bands, and the callback given to
  * bte_set_exchange must replace them by their sum over all ranks' band ranges
  * (an all-reduce), after which every rank solves the same T_p for every cell.

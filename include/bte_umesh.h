@@ -108,7 +108,7 @@ int bte_umesh_set_initial(bte_umesh u, const double* T_cells, double T_uniform);
 /* nsteps time steps of dt [s] of the face-sum update of Eq. 5 (with Eq. 6
  * ghosts on tagged faces); scheme BTE_IMPLICIT_JACOBI (ninner inner
  * iterations) or BTE_EXPLICIT (ninner ignored).  Each inner iteration is a
- * sweep kernel, the per-cell step and the fix-up (plus one kernel for the
+ * sweep kernel, the energies' reduction and the per-cell step (plus one kernel for the
  * diffuse and partially specular faces, and one for the per-cell relaxation
  * scale when beta_T_exp != 0).  stats: as bte_step, may be NULL. */
 int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, bte_stats* stats);

@@ -329,7 +329,7 @@ void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
   // One CTA per item, started in order: the cells in flight stay close together and
   // find their neighbours' rows in L2.  Resident CTAs that stride over the items drift
   // apart (128x128 x 400 x 55 in FP64 1374 us against 1084, 30.5 DRAM bytes an update
-  // against 25; 32^3 in FP32 1473 against 1172).  In-plane sets, whose items are short
+  // against 26.1; 32^3 in FP32 1473 against 1172).  In-plane sets, whose items are short
   // and whose ring would drain, take the resident CTAs (120x120 x 20 x 55: 68 us
   // against 72, IEEE 108 against 123).
   const bool persistent = h->opts.precision != BTE_BF16 && h->dir_group == 4;
