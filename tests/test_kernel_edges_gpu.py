@@ -131,3 +131,36 @@ def test_intensities_keep_the_callers_direction_order(dirs, precision):
     tol = {bte.BTE_FP64: 1e-14, bte.BTE_FP32: 1e-8, bte.BTE_BF16: 1e-4}[precision]   # 1 % deviations in 24 or 8 bits
     assert np.max(np.abs(s.intensity(0) - I) / I) <= tol
     s.close()
+
+
+# 1024 cells is the last grid whose cell step is launched behind the running sweep; a
+# random start queues every cell for the exact solve, a uniform one the few at the hot wall
+@pytest.mark.parametrize("uniform", [False, True])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (32, 32, 1), (41, 25, 1)])
+def test_cell_step_launches_and_queues(shape, uniform):
+    wl = workload(shape, W.Dirs("inplane", n_inplane=4), (3, 1, 60), [W.BC_ISOTHERMAL] * 4, [330.0, 300.0, 300.0, 300.0],
+                  nsteps=3)
+    T0 = None if uniform else W.random_temperatures(wl.geoms[0].ncells, 61, 280.0, 320.0)
+    s = bte.Solver(wl, **({} if uniform else {"T_init": [T0]}))
+    s.step()
+    check(wl, s, T0=T0)
+    s.close()
+
+
+# one pair of bands, a second pass of 64 bands, the most bands; runs of unequal weights
+@pytest.mark.parametrize("bands", [(1, 0, 62), (50, 15, 63), (240, 16, 64)])
+@pytest.mark.parametrize("kw", [{}, {"fp64_strict": True}])
+def test_restored_energies(bands, kw):
+    """T_L after a restore, from the sums formed while packing, against the T_L that the
+    step's own sums gave for the same state."""
+    wl = workload((3, 2, 1), W.Dirs("polar_azim", n_polar=6, n_azim=4), bands, [W.BC_ISOTHERMAL] * 4,
+                  [310.0, 300.0, 303.0, 300.0])
+    s = bte.Solver(wl, **kw)
+    s.step()
+    TL, I, Tp = s.T(0, bte.BTE_T_LATTICE), s.intensity(0), s.T(0, bte.BTE_T_PSEUDO)
+    r = bte.Solver(wl, **kw)
+    bte.bte_set_intensity(r.h, 0, I, Tp)
+    assert np.max(np.abs(r.T(0, bte.BTE_T_LATTICE) - TL) / TL) <= 1e-12
+    assert np.max(np.abs(r.intensity(0) - I) / I) <= 1e-14
+    s.close()
+    r.close()
