@@ -102,12 +102,11 @@ typedef struct {
  *             isothermal or mirror walls keeps the intensity in double-float
  *             form (two floats, 48-bit significand) and computes the update on
  *             the FP32 pipe with error-free transformations; the reduction,
- *             the temperature solve and I0 stay IEEE FP64.  Between such steps
- *             the intensity stays in that form; every call that reads or
- *             writes intensities (bte_get_intensity, bte_set_intensity,
- *             bte_get_flux, bte_get_wall_flux_noalloc, bte_set_initial) or
- *             steps another way converts it to FP64 in place first (one
- *             kernel).  The update rounds to about 2^-48 relative instead of
+ *             the temperature solve and I0 stay IEEE FP64.  The intensity stays
+ *             in that form between such steps and from bte_set_initial on;
+ *             reading calls convert what they return, bte_set_intensity keeps
+ *             FP64 until the next such step, and a step another way converts
+ *             the state first (one kernel).  The update rounds to about 2^-48 relative instead of
  *             2^-53, for |I| in [2^-74, 2^127) (smaller values keep a float's
  *             24 bits).  1: every update in IEEE FP64 arithmetic (DFMA). */
 typedef struct {

@@ -87,9 +87,9 @@ struct bte_ctx {
   char* Ibuf[3] = {nullptr, nullptr, nullptr};
   int cur = 0;
   // FP64 handles whose Jacobi steps run in double-float arithmetic keep the
-  // current intensity buffer as ff pairs between steps; every entry point that
-  // reads or writes intensities (or steps another way) first converts it to
-  // doubles in place (ensure_state_doubles)
+  // current intensity buffer as ff pairs between steps and from bte_set_initial on;
+  // steps of another arithmetic convert it (ensure_state_doubles), a restored state is
+  // kept as doubles until a double-float step (ensure_state_ff)
   bool state_ff = false;
   double *I0cell = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr, *I0wall = nullptr;
   void* coef = nullptr;
@@ -742,7 +742,7 @@ cudaError_t record_timing_event(cudaEvent_t ev, cudaStream_t s) {
 
 // One time step: ninner sweeps rotating the three intensity buffers from *cur.
 // scheme BTE_IMPLICIT_GS runs the sweep-ordered pass and the per-cell step as
-// two kernels in place of the fused Jacobi sweep.
+// two kernels and cells_kernel, the Jacobi sweep as one and cells_kernel.
 cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaStream_t s, int* cur) {
   int dim = 2;
   for (auto& g : h->geoms) dim = std::max(dim, g.dim);
@@ -1516,6 +1516,10 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   const size_t es = elem_bytes(prec);
   char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
   cudaStream_t s = h->stream;
+  // a restored state is kept as given, in doubles, until a double-float step; a lone
+  // geometry's is overwritten whole
+  if (h->geoms.size() == 1) h->state_ff = false;
+  else CUDA_TRY(h, ensure_state_doubles(h));
   CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
                                    h->Msum + h->cell0[geom] * 4, h->MsumL + h->cell0[geom] * 4,
@@ -1532,7 +1536,7 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
     a.Iout = dst;
     a.I0cell = h->I0cell + (h->cell0[geom] + c0) * h->nbp;
     a.Ec = h->Ec + (h->cell0[geom] + c0) * kRedEntries;
-    CUDA_TRY(h, launch_pack(prec, h->state_ff, src, dst, h->I0ref_o, h->rows_d, n, h->nd, h->nb, h->nbp, h->Epart ? nullptr : &a, s));
+    CUDA_TRY(h, launch_pack(prec, src, dst, h->I0ref_o, h->rows_d, n, h->nd, h->nb, h->nbp, h->Epart ? nullptr : &a, s));
     if (!on_device) CUDA_TRY(h, cudaStreamSynchronize(s));  // the caller's pageable memory and the staging buffer are reused
   }
   if (h->Epart) h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange

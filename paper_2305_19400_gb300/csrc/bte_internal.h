@@ -243,7 +243,7 @@ cudaError_t launch_doubles_to_ff(const void* src, void* dst, long long npairs, c
 // FP64 [cell][caller's d][nb] <-> internal rows; perm: the caller's index of every internal direction
 cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* out, const double* I0ref, const int* rows,
                           long long ncells, int nd, int nb, int nbp, cudaStream_t s);
-cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* rows,
+cudaError_t launch_pack(int precision, const double* in, void* I, const double* I0ref, const int* rows,
                         long long ncells, int nd, int nb, int nbp, const SweepArgs* energies, cudaStream_t s);
 // E_L of every cell from its partial energies (launch_gs_reduce's or launch_pack's Ec)
 cudaError_t launch_energy_L(const double2* Ec, double* EL, long long ncells, cudaStream_t s);

@@ -232,8 +232,8 @@ __global__ void mean_kernel(const double* v, int max_faces, SideFaces nf, double
 // the caller's order (row[d]: its internal row), whose rows share 32-byte sectors;
 // internal rows are whole sectors and may be scattered.  Bound by HBM:
 // 16 bytes per FP64 value.  A thread per band with 8-byte accesses on both sides
-// took 569 (in) and 494 us (out) on 96x64 x 400 x 55 values as ff pairs; 406 and
-// 555 here, where the conversions of ff pairs issue most instructions.
+// took 494 us (out) on 96x64 x 400 x 55 values from ff pairs; 409 here, where their
+// conversions issue most instructions, and 330 from doubles.
 template <typename S>
 __global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, const double* I0ref, const int* rows,
                                                      long long ncells, int nd, int nb, int nbp) {
@@ -430,8 +430,9 @@ __global__ void __launch_bounds__(kRedThreads, 4) gs_reduce_kernel(SweepArgs a, 
 
 // FP64 values and their energies in one pass (REDUCE: a.Ec as gs_reduce_kernel leaves
 // it, for the values as given): a warp's lanes hold band pairs of one direction, the
-// warps contiguous eighths of the caller's directions (runs of equal weights).  On 96x64 x 400 x 55 as ff pairs the
-// separate pass over the stored rows took 424 us after this kernel's 406; now 575.
+// warps contiguous eighths of the caller's directions (runs of equal weights).  96x64 x
+// 400 x 55: 464 us, where a separate pass over the stored rows took 424 after 406 for
+// packing (into ff pairs, which this took 575 us for).
 template <typename S, bool REDUCE>
 __global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const double* I0ref, const int* rows,
                                                    long long ncells, int nd, int nb, int nbp, SweepArgs a) {
@@ -835,7 +836,7 @@ cudaError_t launch_unpack(int precision, bool state_ff, const void* I, double* o
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I, const double* I0ref, const int* rows,
+cudaError_t launch_pack(int precision, const double* in, void* I, const double* I0ref, const int* rows,
                         long long ncells, int nd, int nb, int nbp, const SweepArgs* energies, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
@@ -848,8 +849,7 @@ cudaError_t launch_pack(int precision, bool state_ff, const double* in, void* I,
     }
     pack_kernel<T, false><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, rows, ncells, nd, nb, nbp, SweepArgs{});
   };
-  if (precision == 0 && state_ff) go(FFElem{});
-  else if (precision == 0) go(double{});
+  if (precision == 0) go(double{});
   else if (precision == 1) go(float{});
   else go(__nv_bfloat16{});
   if (energies && precision != 0) {  // of the stored deviations

@@ -1200,7 +1200,7 @@ int bte_umesh_set_intensity(bte_umesh u, const double* in, const double* Tp_cell
   if (e == cudaSuccess) e = launch_state_from_Tp(u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->nc, uthermo(u), s);
   const SweepArgs sums = cell_args(u, u->I[u->cur]);
   if (e == cudaSuccess)
-    e = launch_pack(u->prec, false, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, &sums, s);
+    e = launch_pack(u->prec, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, &sums, s);
   if (e == cudaSuccess) e = launch_energy_L(u->Ec, u->EL, u->nc, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(tmp);
