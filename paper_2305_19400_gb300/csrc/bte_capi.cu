@@ -730,6 +730,18 @@ cudaError_t ensure_state_ff(bte_ctx* h) {
   return e;
 }
 
+// The ghosts of the diffuse and partially specular sides from the current state,
+// before wall fluxes read them.  Their kernels read doubles, so a state that stands
+// as ff pairs (set, or stepped under other wall kinds) is converted first; callers take
+// the state's form afterwards.
+cudaError_t refresh_ghosts(bte_ctx* h) {
+  cudaError_t e = cudaSuccess;
+  if (h->state_ff && !ff_sweep(h)) e = ensure_state_doubles(h);
+  if (e == cudaSuccess) e = refresh_diffuse(h, h->Ibuf[h->cur], h->stream);
+  if (e == cudaSuccess) e = refresh_partial(h, h->Ibuf[h->cur], h->stream);
+  return e;
+}
+
 // A timing event on stream s: inside a stream capture it must become an event
 // record node of the graph (cudaEventRecordExternal), so that every replay
 // records it and the host can read it.
@@ -838,14 +850,13 @@ int flux_view(bte_ctx* h, int geom, FluxView* out) {
   if (rc) return rc;
   if (!h->mem_ready || !h->init_set[geom]) return fail(h, BTE_E_STATE, "geometry %d has no state", geom);
   const bte_geom& g = h->geoms[geom];
+  {  // kernel launches, no allocation
+    const cudaError_t e = refresh_ghosts(h);
+    if (e != cudaSuccess) return fail(h, BTE_E_CUDA, "diffuse wall ghosts: %s", cudaGetErrorString(e));
+  }
   out->precision = h->opts.precision;
   out->I = h->Ibuf[h->cur];
   out->state_ff = h->state_ff;
-  {  // diffuse and partially specular wall ghosts of the current state (kernel launches, no allocation)
-    cudaError_t e = refresh_diffuse(h, h->Ibuf[h->cur], h->stream);
-    if (e == cudaSuccess) e = refresh_partial(h, h->Ibuf[h->cur], h->stream);
-    if (e != cudaSuccess) return fail(h, BTE_E_CUDA, "diffuse wall ghosts: %s", cudaGetErrorString(e));
-  }
   out->I0wall = h->I0wall;
   out->geoms = h->geoms_d;
   std::copy(h->wall_dirs.begin(), h->wall_dirs.end(), out->wall_dirs);
@@ -1469,8 +1480,7 @@ int bte_get_flux(bte_handle h, int geom, double* q_cells, double* q_walls, int o
     double res[6] = {0, 0, 0, 0, 0, 0};
     int nf[6] = {0, 0, 0, 0, 0, 0};
     for (int side = 0; side < 2 * g.dim; ++side) nf[side] = (int)side_faces(g, side);
-    CUDA_TRY(h, refresh_diffuse(h, I, s));  // diffuse and partially specular ghosts of the current state
-    CUDA_TRY(h, refresh_partial(h, I, s));
+    CUDA_TRY(h, refresh_ghosts(h));
     CUDA_TRY(h, launch_flux_walls(prec, h->state_ff, I, h->I0ref_o, h->I0wall, h->geoms_d, geom, h->wall_dirs.data(), h->Sdev, h->nd,
                                   h->nbp, h->scratch_faces, h->max_side_faces, nf, 2 * g.dim, h->scratch_out, s));
     CUDA_TRY(h, cudaMemcpyAsync(res, h->scratch_out, 2 * g.dim * 8, cudaMemcpyDeviceToHost, s));
