@@ -36,6 +36,7 @@
 
 #include "bte_ff.cuh"
 #include "bte_pdl.cuh"
+#include "bte_quad.cuh"
 #include "bte_store.cuh"
 
 namespace bte {
@@ -186,9 +187,10 @@ struct FF {
 // operations (2-D; 4 with BM 1), the bound of this form: 0.53e12 FP64 FMAs per
 // second, measured.  TT: the relaxation rates depend on T, beta_b(T_p) = beta_b s;
 // every coefficient takes the factor y = 1/(1 + (s - 1) A_s), A_s also s (explicit
-// scheme: A_n + (1 - s) A_s and s A_s).  y is formed once per block too, from an
-// FP32 reciprocal and one third-order step (three FMAs, error 2^-66; a correctly
-// rounded reciprocal per update took 1745 us on 64x48 cells x 400 x 55).
+// scheme: A_n + (1 - s) A_s and s A_s).  y is formed once per block too, by
+// rcp_pos (an FP32 reciprocal and one third-order step inside its range, a division
+// outside it: s runs to (T_p/T_ref)^16; a correctly rounded reciprocal per update took
+// 1745 us on 64x48 cells x 400 x 55).
 // The direction sum runs on the integer pipe: over a run of directions with the
 // same weight each band adds I exactly in 64-bit fixed point, unit 2^(E - 50) for
 // the cell's I0 of exponent E, so a value up to 16 I0 adds at most 2^55 and a run
@@ -266,15 +268,6 @@ struct F64 {
     }
     s.n = 0;
   }
-  // 1/q for q > 0: FP32 estimate y0, then y0 (1 + e + e^2) with e = 1 - q y0
-  __device__ static double recip(double q) {
-    float h, l, r;
-    ff::split(q, h, l);
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(h));
-    const double y0 = ff::to_double(r, 0.0f);
-    const double e = fma(-q, y0, 1.0);
-    return fma(fma(e, e, e), y0, y0);
-  }
   __device__ static void yy(double2& x, double y0, double y1) {
     x.x *= y0;
     x.y *= y1;
@@ -300,7 +293,7 @@ struct F64 {
       if (BM == 0 && a.explicit_scheme) {
         b.An = make_double2(fma(1.0 - c.s, cf.As.x, cf.An.x), fma(1.0 - c.s, cf.As.y, cf.An.y));
       } else {
-        const double y0 = recip(fma(c.s - 1.0, cf.As.x, 1.0)), y1 = recip(fma(c.s - 1.0, cf.As.y, 1.0));
+        const double y0 = rcp_pos(fma(c.s - 1.0, cf.As.x, 1.0)), y1 = rcp_pos(fma(c.s - 1.0, cf.As.y, 1.0));
         yy(b.Ax, y0, y1);
         yy(b.Ay, y0, y1);
         if (DIM == 3) yy(b.Az, y0, y1);
