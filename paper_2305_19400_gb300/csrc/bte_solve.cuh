@@ -20,23 +20,45 @@ inline double model_trust(double rtol) { return std::pow(rtol / 32.0, 0.25); }
 
 __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
+// c x 2^-k by its exponent field, without an FP64 operation.  Values that leave the
+// range become zero or infinity; infinities and NaN stay.
+__device__ __forceinline__ double scale_down(double c, int k) {
+  const int hi = __double2hiint(c), e = (hi >> 20) & 0x7ff;
+  const int sgn = hi & (int)0x80000000;
+  if (e == 0x7ff) return c;
+  if (e == 0 || e - k <= 0) return __hiloint2double(sgn, 0);
+  if (e - k >= 0x7ff) return __hiloint2double(sgn | 0x7ff00000, 0);
+  return __hiloint2double(hi - k * (1 << 20), __double2loint(c));
+}
+
 // Root nearest 0 of c0 + c1 d + c2 d^2 + c3 d^3, the step of a cell's cached
-// temperature model: an FP32 estimate from the stable form of the quadratic's
+// temperature model (NaN without a positive slope): all coefficients scaled by the
+// power of two that brings c1 into [1, 2) -- they are proportional to the relaxation
+// rates, and unscaled c1^2 leaves the FP32 range above 1.8e19, rates of about 1e13
+// 1/s in silicon --, then an FP32 estimate from the stable form of the quadratic's
 // root, -2 c0 / (c1 + sqrt(c1^2 - 4 c0 c2)) (-c0 / c1 without a real root), then
 // one Newton step on the cubic in FP64 with the derivative and its reciprocal in
 // FP32.  The estimate is good to about 2e-7 of d (FP32 rounding and, inside the
 // trust radius, the cubic term) and the step to about 1e-13 of d, while an
 // accepted d is below 2e-4 T.  The FP64 pipe of GB300 takes about 73 cycles per
 // warp instruction: this form issues four FP64 operations where a square root
-// and a division take twenty-odd, and its conversions run on the integer pipe.
+// and a division take twenty-odd, and its scaling and conversions run on the
+// integer pipe.
 __device__ __forceinline__ double model_step(double c0, double c1, double c2, double c3) {
+  const int e1 = __double2hiint(c1) >> 20;  // sign and exponent
+  if (e1 <= 0 || e1 >= 0x7ff) return __hiloint2double(0x7ff80000, 0);  // zero, subnormal, negative, Inf, NaN
+  const int k = e1 - 1023;
+  c0 = scale_down(c0, k);
+  c1 = scale_down(c1, k);
+  c2 = scale_down(c2, k);
+  c3 = scale_down(c3, k);
   float f0, f1, f2, f3, lo;
   ff::split(c0, f0, lo);
   ff::split(c1, f1, lo);
   ff::split(c2, f2, lo);
   ff::split(c3, f3, lo);
   const float disc = fmaf(f1, f1, -4.0f * f0 * f2);
-  const float df = (disc >= 0.0f && f1 > 0.0f) ? -2.0f * f0 / (f1 + sqrtf(disc)) : -f0 / f1;
+  const float df = disc >= 0.0f ? -2.0f * f0 / (f1 + sqrtf(disc)) : -f0 / f1;
   const double d = ff::to_double(df, 0.0f);
   const double g = fma(fma(fma(c3, d, c2), d, c1), d, c0);
   const float dg = fmaf(fmaf(3.0f * f3, df, 2.0f * f2), df, f1);
