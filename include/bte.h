@@ -101,14 +101,16 @@ typedef struct {
  *             (any ninner) of a handle with fixed relaxation rates and
  *             isothermal or mirror walls keeps the intensity in double-float
  *             form (two floats, 48-bit significand) and computes the update on
- *             the FP32 pipe with error-free transformations; the reduction,
- *             the temperature solve and I0 stay IEEE FP64.  The intensity stays
- *             in that form between such steps and from bte_set_initial on;
- *             reading calls convert what they return, bte_set_intensity keeps
- *             FP64 until the next such step, and a step another way converts
- *             the state first (one kernel).  The update rounds to about 2^-48 relative instead of
- *             2^-53, for |I| in [2^-74, 2^127) (smaller values keep a float's
- *             24 bits).  1: every update in IEEE FP64 arithmetic (DFMA). */
+ *             the FP32 pipe with error-free transformations, the sums over
+ *             directions included; the sums over bands, the temperature solve
+ *             and I0 are FP64.  The intensity stays in that form between such
+ *             steps; an initial or restored state is FP64 until the next such
+ *             step, reading calls convert what they return (wall fluxes of
+ *             rough walls: the state), and a step another way converts the
+ *             state first (one kernel).  The update rounds to about 2^-48
+ *             relative instead of 2^-53, for |I| in [2^-74, 2^127) (smaller
+ *             values keep a float's 24 bits).  1: every update in IEEE FP64
+ *             arithmetic (DFMA). */
 typedef struct {
   int dir_kind;
   int n_inplane, n_polar, n_azim;

@@ -87,8 +87,8 @@ struct bte_ctx {
   char* Ibuf[3] = {nullptr, nullptr, nullptr};
   int cur = 0;
   // FP64 handles whose Jacobi steps run in double-float arithmetic keep the
-  // current intensity buffer as ff pairs between steps and from bte_set_initial on;
-  // steps of another arithmetic convert it (ensure_state_doubles), a restored state is
+  // current intensity buffer as ff pairs between such steps; steps of another
+  // arithmetic convert it (ensure_state_doubles), an initial or restored state is
   // kept as doubles until a double-float step (ensure_state_ff)
   bool state_ff = false;
   double *I0cell = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr, *I0wall = nullptr;
@@ -1138,12 +1138,11 @@ int bte_set_initial(bte_handle h, int geom, const double* T_cells, double T_unif
   for (double t : T)
     if (!(t >= kTmin && t <= kTmax)) return fail(h, BTE_E_ARG, "initial temperature %g outside [1, 5000] K", t);
   if ((rc = ensure_memory(h))) return rc;
-  // the state starts in the form of the handle's default sweep; geometries set
-  // later follow the form it has by then
-  if (std::none_of(h->init_set.begin(), h->init_set.end(), [](bool x) { return x; }))
-    h->state_ff = h->opts.precision == BTE_FP64 && !h->opts.fp64_strict && h->opts.beta_T_exp == 0.0;
+  // an initial state is kept in doubles until a double-float step, whatever form the
+  // other geometries' state has by now
+  CUDA_TRY(h, ensure_state_doubles(h));
   CUDA_TRY(h, cudaMemcpyAsync(h->scratch_T, T.data(), nc * 8, cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->state_ff, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->MsumL, h->Tp, h->Teval, h->TL, h->EL,
+  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->MsumL, h->Tp, h->Teval, h->TL, h->EL,
                                 h->scratch_T, h->I0ref_o, h->cell0[geom], (int)nc, h->nd, thermo(h), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->init_set[geom] = true;

@@ -715,16 +715,15 @@ cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_cells(int precision, bool state_ff, void* I, double* I0cell, double* J, double* Msum, double* MsumL,
-                              double* Tp, double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
+cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp,
+                              double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
                               long long cell0, int ncells, int nd, ThermoTables th, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
     init_cells_kernel<T><<<cell_grid(ncells), 256, th.nbp * sizeof(double), s>>>((T*)I, I0cell, J, Msum, MsumL, Tp, Te, TL, EL, Tcells,
                                                                                  I0ref, cell0, ncells, nd, th);
   };
-  if (precision == 0 && state_ff) go(FFElem{});
-  else if (precision == 0) go(double{});
+  if (precision == 0) go(double{});
   else if (precision == 1) go(float{});
   else go(__nv_bfloat16{});
   return cudaGetLastError();
