@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, co
   }
 }
 
-// Energies after a separate sweep (the sweep-ordered pass, the unstructured sweep) and
-// a restore in reduced storage: one CTA of 8 warps per cell.  Loads of 16 bytes, eight in
+// Energies after a separate sweep (the sweep-ordered pass, the unstructured sweep):
+// one CTA of 8 warps per cell.  Loads of 16 bytes, eight in
 // flight; FP64: four, warp w sums the directions [w nd / 8, (w + 1) nd / 8), lanes over
 // band pairs (whole warps on one direction, so the runs of the fixed-point sums
 // close together: groups of 28 lanes took 406 us where this takes 308 on 6144 cells
@@ -429,10 +429,12 @@ __global__ void __launch_bounds__(kRedThreads, 4) gs_reduce_kernel(SweepArgs a, 
 }
 
 // FP64 values and their energies in one pass (REDUCE: a.Ec as gs_reduce_kernel leaves
-// it, for the values as given): a warp's lanes hold band pairs of one direction, the
-// warps contiguous eighths of the caller's directions (runs of equal weights).  96x64 x
-// 400 x 55: 464 us, where a separate pass over the stored rows took 424 after 406 for
-// packing (into ff pairs, which this took 575 us for).
+// it, for the values as stored): a warp's lanes hold band pairs of one direction, the
+// warps contiguous eighths of the caller's directions.  The sums are FP64 additions:
+// the values need not be near I0(T_p), which the fixed-point sums of a step count on, and a
+// reduced mode's deviations keep all their bits.  Bound by HBM, 16 bytes per FP64 value: the
+// sums' two FMAs per lane and row hide behind the copies.  96x64 x 400 x 55, restore,
+// T_L and read-out: 1459 us, 1540 with fixed-point sums here.
 template <typename S, bool REDUCE>
 __global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const double* I0ref, const int* rows,
                                                    long long ncells, int nd, int nb, int nbp, SweepArgs a) {
@@ -444,13 +446,11 @@ __global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const
     const double* x = in + P * nd * nb;
     for (int c = 0; c < nbp; c += 64) {
       const int b = c + 2 * lane;
-      double r0 = 0.0, r1 = 0.0;
+      double r0 = 0.0, r1 = 0.0, g0 = 0.0, g1 = 0.0;
       if (sizeof(S) != 8) {
         if (b < nb) r0 = I0ref[b];
         if (b + 1 < nb) r1 = I0ref[b + 1];
       }
-      const double zero2[2] = {0.0, 0.0};
-      FixedSum sum(REDUCE && b < nbp ? a.I0cell + P * nbp + b : zero2);
       for (int d0 = dlo; d0 < dhi; d0 += 4) {
         double v[4][2];
 #pragma unroll
@@ -468,21 +468,27 @@ __global__ void __launch_bounds__(256) pack_kernel(const double* in, S* I, const
           const double a0 = __shfl_sync(0xffffffffu, v[u][0], s0), a1 = __shfl_sync(0xffffffffu, v[u][0], s0 + 1);
           const double e0 = __shfl_sync(0xffffffffu, v[u][1], s0), e1 = __shfl_sync(0xffffffffu, v[u][1], s0 + 1);
           const double x0 = lane < 16 ? a0 : e0, x1 = lane < 16 ? a1 : e1;
-          if (b < nbp) st_pair(row + (long long)r * nbp + b, x0 - r0, x1 - r1);
-          if constexpr (REDUCE) sum.add(x0, x1, a.wdir[r]);
+          S* to = row + (long long)r * nbp + b;
+          if (b < nbp) st_pair(to, x0 - r0, x1 - r1);
+          if constexpr (REDUCE) {
+            const double w = a.wdir[r];
+            double y0 = x0, y1 = x1;
+            if constexpr (sizeof(S) != 8) stored_pair<S>(x0 - r0, x1 - r1, y0, y1);
+            g0 = fma(w, y0, g0);
+            g1 = fma(w, y1, g1);
+          }
         }
       }
       if constexpr (REDUCE) {
-        sum.close();
         if (b < nbp) {
-          gpart[wid * nbp + b] = sum.G[0];
-          gpart[wid * nbp + b + 1] = sum.G[1];
+          gpart[wid * nbp + b] = g0;
+          gpart[wid * nbp + b + 1] = g1;
         }
       }
     }
     if constexpr (REDUCE) {
       __syncthreads();
-      if (threadIdx.x < 32) reduce_energies<false>(a, gpart, 8, P);
+      if (threadIdx.x < 32) reduce_energies<sizeof(S) != 8>(a, gpart, 8, P);
       __syncthreads();
     }
   }
@@ -839,22 +845,15 @@ cudaError_t launch_pack(int precision, const double* in, void* I, const double* 
                         long long ncells, int nd, int nb, int nbp, const SweepArgs* energies, cudaStream_t s) {
   auto go = [&](auto tag) {
     using T = decltype(tag);
-    if constexpr (sizeof(T) == 8) {
-      if (energies) {
-        pack_kernel<T, true><<<cell_grid(ncells), 256, 8 * (size_t)nbp * sizeof(double), s>>>(in, (T*)I, I0ref, rows, ncells, nd,
-                                                                                            nb, nbp, *energies);
-        return;
-      }
-    }
-    pack_kernel<T, false><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, rows, ncells, nd, nb, nbp, SweepArgs{});
+    if (energies)
+      pack_kernel<T, true><<<cell_grid(ncells), 256, 8 * (size_t)nbp * sizeof(double), s>>>(in, (T*)I, I0ref, rows, ncells, nd, nb,
+                                                                                          nbp, *energies);
+    else
+      pack_kernel<T, false><<<cell_grid(ncells), 256, 0, s>>>(in, (T*)I, I0ref, rows, ncells, nd, nb, nbp, SweepArgs{});
   };
   if (precision == 0) go(double{});
   else if (precision == 1) go(float{});
   else go(__nv_bfloat16{});
-  if (energies && precision != 0) {  // of the stored deviations
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? launch_gs_reduce(precision, *energies, ncells, s) : e;
-  }
   return cudaGetLastError();
 }
 

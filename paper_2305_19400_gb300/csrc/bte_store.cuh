@@ -160,4 +160,12 @@ __device__ __forceinline__ void st_pair(S* p, double a, double b) {
     *reinterpret_cast<__nv_bfloat162*>(p) = v;
   }
 }
+// The values that st_pair keeps of a and b.
+template <typename S>
+__device__ __forceinline__ void stored_pair(double a, double b, double& x, double& y) {
+  typename RawPair<S>::R r;
+  st_pair(reinterpret_cast<S*>(&r), a, b);
+  raw_pair(r, x, y);
+}
+
 }  // namespace bte
