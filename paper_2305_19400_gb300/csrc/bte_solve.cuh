@@ -20,49 +20,33 @@ inline double model_trust(double rtol) { return std::pow(rtol / 32.0, 0.25); }
 
 __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
-// c x 2^-k by its exponent field, without an FP64 operation.  Values that leave the
-// range become zero or infinity; infinities and NaN stay.
-__device__ __forceinline__ double scale_down(double c, int k) {
-  const int hi = __double2hiint(c), e = (hi >> 20) & 0x7ff;
-  const int sgn = hi & (int)0x80000000;
-  if (e == 0x7ff) return c;
-  if (e == 0 || e - k <= 0) return __hiloint2double(sgn, 0);
-  if (e - k >= 0x7ff) return __hiloint2double(sgn | 0x7ff00000, 0);
-  return __hiloint2double(hi - k * (1 << 20), __double2loint(c));
-}
-
 // Root nearest 0 of c0 + c1 d + c2 d^2 + c3 d^3, the step of a cell's cached
-// temperature model (NaN without a positive slope): all coefficients scaled by the
-// power of two that brings c1 into [1, 2) -- they are proportional to the relaxation
-// rates, and unscaled c1^2 leaves the FP32 range above 1.8e19, rates of about 1e13
-// 1/s in silicon --, then an FP32 estimate from the stable form of the quadratic's
-// root, -2 c0 / (c1 + sqrt(c1^2 - 4 c0 c2)) (-c0 / c1 without a real root), then
+// temperature model (NaN where c1 is not positive or leaves 2^-100 .. 2^101).  The
+// coefficients are proportional to the relaxation rates, and c1^2 alone leaves the FP32
+// range above 1.8e19 (rates of about 1e13 1/s in silicon), so they are divided by c1
+// first: with a, b, c = c0, c2, c3 over c1 an FP32 estimate from the stable form of the
+// quadratic's root, -2 a / (1 + sqrt(1 - 4 a b)) (-a without a real root), then
 // one Newton step on the cubic in FP64 with the derivative and its reciprocal in
-// FP32.  The estimate is good to about 2e-7 of d (FP32 rounding and, inside the
-// trust radius, the cubic term) and the step to about 1e-13 of d, while an
+// FP32.  The estimate is good to about 3e-7 of d (FP32 rounding and, inside the
+// trust radius, the cubic term) and the step to about 2e-13 of d, while an
 // accepted d is below 2e-4 T.  The FP64 pipe of GB300 takes about 73 cycles per
 // warp instruction: this form issues four FP64 operations where a square root
-// and a division take twenty-odd, and its scaling and conversions run on the
-// integer pipe.
+// and a division take twenty-odd, and its conversions run on the integer pipe.
 __device__ __forceinline__ double model_step(double c0, double c1, double c2, double c3) {
-  const int e1 = __double2hiint(c1) >> 20;  // sign and exponent
-  if (e1 <= 0 || e1 >= 0x7ff) return __hiloint2double(0x7ff80000, 0);  // zero, subnormal, negative, Inf, NaN
-  const int k = e1 - 1023;
-  c0 = scale_down(c0, k);
-  c1 = scale_down(c1, k);
-  c2 = scale_down(c2, k);
-  c3 = scale_down(c3, k);
   float f0, f1, f2, f3, lo;
-  ff::split(c0, f0, lo);
   ff::split(c1, f1, lo);
   ff::split(c2, f2, lo);
   ff::split(c3, f3, lo);
-  const float disc = fmaf(f1, f1, -4.0f * f0 * f2);
-  const float df = disc >= 0.0f ? -2.0f * f0 / (f1 + sqrtf(disc)) : -f0 / f1;
+  const float r = 1.0f / f1, b = f2 * r, c = f3 * r;  // not behind the energies
+  ff::split(c0, f0, lo);
+  const float a = f0 * r, disc = fmaf(-4.0f * a, b, 1.0f);
+  const float df = disc >= 0.0f ? -2.0f * a / (1.0f + sqrtf(disc)) : -a;
   const double d = ff::to_double(df, 0.0f);
   const double g = fma(fma(fma(c3, d, c2), d, c1), d, c0);
-  const float dg = fmaf(fmaf(3.0f * f3, df, 2.0f * f2), df, f1);
-  return fma(-g, ff::to_double(1.0f / dg, 0.0f), d);
+  const float dg = fmaf(fmaf(3.0f * c, df, 2.0f * b), df, 1.0f);
+  const double step = fma(-g, ff::to_double(r / dg, 0.0f), d);
+  const int e1 = __double2hiint(c1) >> 20;  // sign and exponent
+  return (unsigned)(e1 - 923) <= 200u ? step : __hiloint2double(0x7ff80000, 0);
 }
 
 // |d| <= trust T (T finite), decided in FP32: the radius is not sharp to 1e-7.
