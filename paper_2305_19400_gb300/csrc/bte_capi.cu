@@ -44,6 +44,7 @@ struct bte_ctx {
   std::vector<int> refl;
   std::vector<int> perm;       // the caller's index of every internal direction
   double Wtot = 0.0;
+  double T_knee = 0.0;         // ThermoTables::T_knee
   // bands
   int nb = 0, nbp = 0, ng = 16;           // bands stored by this handle (padded: nbp)
   int nb_all = 0, nbp_all = 0, band0 = 0; // every band of the table; first stored band
@@ -180,6 +181,7 @@ ThermoTables thermo(const bte_ctx* h) {
   t.inv_v = h->inv_v;
   t.beta = h->beta_d;
   t.binv_v = h->binv_d;
+  t.T_knee = h->T_knee;
   t.ng = h->ng;
   t.nbp = h->nbp_all;
   t.nb = h->nb_all;
@@ -437,6 +439,7 @@ int ensure_memory(bte_ctx* h) {
   std::vector<double> nc, nC, ap, aL, iv, be;
   build_thermo(h->nb_all, h->nbp_all, h->ng, h->wlo.data(), h->whi.data(), h->vg.data(), h->beta.data(),
                h->deg.data(), h->Wtot, nc, nC, ap, aL, iv, be);
+  h->T_knee = model_knee(nc, h->nb_all, h->ng);
   CUDA_TRY(h, cudaMemcpyAsync(h->node_c, nc.data(), nc.size() * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->node_C, nC.data(), nC.size() * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->a_p, ap.data(), ap.size() * 8, cudaMemcpyHostToDevice, s));

@@ -60,7 +60,7 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
   const int nbo = a.th.nbo, nbp = a.th.nbp;
   const int slot = threadIdx.x / kCellLanes, sub = threadIdx.x % kCellLanes;
   const bool lattice = mode == kLattice;
-  const float trust = (float)a.trust_rel;
+  const float trust = (float)a.trust_rel, T_knee = (float)a.th.T_knee;
   const bool solves = mode != kPartial && (lattice || a.solve_tp);
   if (solves) asm volatile("barrier.cluster.arrive;" ::: "memory");  // awaited before the first remote access
   if (threadIdx.x == 0) { queued = 0; nsolve = 0; nbad = 0; }
@@ -129,7 +129,7 @@ __global__ void __cluster_dims__(kCellCluster, 1, 1) __launch_bounds__(kCellThre
     // root of M_0 - E + M_1 d + M_2 d^2 + M_3 d^3 nearest 0
     const double delta = model_step(M[0] - Ep, M[1], M[2], M[3]);
     const double Tn = Te + delta;
-    if (in_trust(delta, Tn, trust)) {
+    if (in_trust(delta, Tn, trust, T_knee)) {
       if (lattice) {
         if (sub == 0) a.TL[P] = Tn;
         continue;

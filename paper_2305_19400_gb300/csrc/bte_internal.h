@@ -102,6 +102,7 @@ struct ThermoTables {
   const double* inv_v;    // [nbo] 1/v_b of the stored bands (0 on padding)
   const double* beta;     // [nbo] beta_b of the stored bands (0 on padding)
   const double* binv_v;   // [nbo] beta_b/v_b of the stored bands (0 on padding)
+  double T_knee;          // hbar omega_max / (32 k_B): the trust radius shrinks below (model_trust)
   int ng;
   int nbp;    // all bands, padded: width of node tables, J, a_p and a_L
   int nb;     // all bands
@@ -155,7 +156,7 @@ struct SweepArgs {
   int dir_group;            // rows that differ only in the signs of S: 4 (in-plane sets) or 8 (internal_order)
   int ne;                   // entries per cell in Ec
   int solve_tp;             // 0 when every beta_b == 0 (T_p then unused)
-  double trust_rel;         // cached model accepted when |T - T_e| <= trust_rel * T
+  double trust_rel;         // cached model accepted when |T - T_e| <= trust_rel * T (model_trust)
   int maxit;
   double Wtot;              // sum of direction weights
   int partial;              // 1: band-range handle; per-cell partial (E_L, E_p) go to Epart[cell][2]

@@ -10,12 +10,13 @@
 namespace bte {
 
 // Relative trust radius of a cell's third-order Taylor model of I0_b(T) for a
-// solve tolerance rtol.  For the bands up to 1e14 rad/s the remainder is at most
-// 0.4 (d/T)^4 I0_b at 300 K and 5.7 (d/T)^4 I0_b at 100 K: at the radius
-// (rtol/32)^(1/4), 1.33e-4 for 1e-14, that is 1.2e-16 and 1.8e-15.  The
-// second-order model took (rtol/4)^(1/3) = 1.36e-5 (2.1e-15 and 6.0e-14 there,
-// and no less than this one's down to 26 K); cells drift out of the ten times
-// wider radius ten times less often.
+// solve tolerance rtol, (rtol/32)^(1/4) = 1.33e-4 for 1e-14, and (rtol/x)^(1/4)
+// where x = hbar omega_max / (k_B T) is above 32: below T_knee (ThermoTables), 24 K for
+// bands up to 1e14 rad/s.  A second-order model at (rtol/4)^(1/3) = 1.36e-5 leaves a
+// remainder of 2.1e-15 I0_b at 300 K (x = 2.5) and 5.6e-14 at 100 K, this one 1.2e-16
+// and 1.8e-15, and at no x more (where x is large they are x^3 rtol/24 and
+// x^4/24 times the fourth power of the radius); cells drift out of the ten
+// times wider radius ten times less often.
 inline double model_trust(double rtol) { return std::pow(rtol / 32.0, 0.25); }
 
 __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
@@ -49,12 +50,21 @@ __device__ __forceinline__ double model_step(double c0, double c1, double c2, do
   return (unsigned)(e1 - 923) <= 200u ? step : __hiloint2double(0x7ff80000, 0);
 }
 
-// |d| <= trust T (T finite), decided in FP32: the radius is not sharp to 1e-7.
-__device__ __forceinline__ bool in_trust(double d, double T, float trust) {
+// Whether a step d to T > 0 stays inside the trust radius (R float or double).
+template <typename R>
+__device__ __forceinline__ bool in_radius(R d, R T, R trust, R T_knee) {
+  const R a = d < R(0) ? -d : d, r = trust * T;
+  if (!(a <= r)) return false;
+  if (T >= T_knee) return true;
+  const R a2 = a * a, r2 = r * r;
+  return a2 * a2 * T_knee <= r2 * r2 * T;
+}
+// The same for T finite, decided in FP32: the radius is not sharp to 1e-7.
+__device__ __forceinline__ bool in_trust(double d, double T, float trust, float T_knee) {
   float df, Tf, lo;
   ff::split(d, df, lo);
   ff::split(T, Tf, lo);
-  return finite(T) && fabsf(df) <= trust * Tf;
+  return finite(T) && in_radius(df, Tf, trust, T_knee);
 }
 
 // The model's value at T_e + d from one band's column of the cell's rows ([4][ld]).
@@ -74,8 +84,8 @@ struct SolveResult {
 
 // Control of the exact solve of sum_b w_b I0_b(T) = Ep: Halley steps from T0
 // on the exact band quadrature (F and three derivatives from one evaluation),
-// bisection on [1, 5000] K as the fallback.  A step delta is accepted when
-// |delta| <= trust_rel * T, where the third-order Taylor model at the
+// bisection on [1, 5000] K as the fallback.  A step delta is accepted inside
+// the trust radius, where the third-order Taylor model at the
 // evaluation point is accurate to the solve tolerance; an accepted step takes
 // one Newton step on that model's cubic (the Halley step itself leaves an
 // error of third order in delta).  Shared by the warp and the CTA forms
@@ -92,7 +102,7 @@ struct SolveCtl {
 
   // One evaluation's sums at T (Taylor coefficients); moves T to the next
   // evaluation point or sets done.
-  __device__ void advance(const double* c, double Ep, double trust_rel, int maxit) {
+  __device__ void advance(const double* c, double Ep, double trust_rel, double T_knee, int maxit) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) r.M[k] = c[k];
     const double F = c[0] - Ep, F1 = c[1];
@@ -116,7 +126,7 @@ struct SolveCtl {
         hi = kTmax;
         T = 0.5 * (lo + hi);
         r.fallback = 1;
-      } else if (fabs(delta) <= trust_rel * Tn) {
+      } else if (in_radius(delta, Tn, trust_rel, T_knee)) {
         const double g = fma(fma(fma(c[3], delta, c[2]), delta, F1), delta, F);
         const double dg = fma(fma(3.0 * c[3], delta, 2.0 * c[2]), delta, F1);
         delta = dg > 0.0 ? fma(-g, rcp_pos(dg), delta) : delta;
@@ -172,7 +182,7 @@ __device__ inline SolveResult exact_solve_warp(const ThermoTables& th, double Ep
 #pragma unroll
       for (int k = 0; k < 4; ++k) F[k] += __shfl_xor_sync(0xffffffffu, F[k], o);
     }
-    c.advance(F, Ep, trust_rel, maxit);
+    c.advance(F, Ep, trust_rel, th.T_knee, maxit);
   }
   return c.finish();
 }
@@ -271,7 +281,7 @@ __device__ inline SolveResult exact_solve_cluster(const ThermoTables& th, const 
       }
     }
     __syncthreads();
-    c.advance(sums, Ep, trust_rel, maxit);
+    c.advance(sums, Ep, trust_rel, th.T_knee, maxit);
   }
   SolveResult r = c.finish();
 #pragma unroll

@@ -173,6 +173,10 @@ void build_thermo(int nb, int nbp, int ng, const double* wlo, const double* whi,
   }
 }
 
+double model_knee(const std::vector<double>& node_c, int nb, int ng) {
+  return *std::max_element(node_c.begin(), node_c.begin() + (size_t)nb * ng) / 32.0;
+}
+
 // Sweep coefficients for one cell-size class: [5][nd][nbp] = A_n, A_x, A_y, A_z, A_s.
 void build_coef(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
                 const double* vg, const double* beta, double dt, int explicit_scheme, double* out) {

@@ -11,6 +11,9 @@ void build_thermo(int nb, int nbp, int ng, const double* wlo, const double* whi,
                   const double* deg, double Wtot, std::vector<double>& node_c, std::vector<double>& node_C,
                   std::vector<double>& a_p, std::vector<double>& a_L, std::vector<double>& inv_v,
                   std::vector<double>& beta_p);
+// hbar omega_max / (32 k_B) of the nb bands, omega_max the highest node's.
+double model_knee(const std::vector<double>& node_c, int nb, int ng);
+
 void build_coef(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
                 const double* vg, const double* beta, double dt, int explicit_scheme, double* out);
 

@@ -516,7 +516,7 @@ struct bte_umesh_ctx {
   std::vector<double> S, w;
   std::vector<int> refl;  // [5][nd]: mirror across x, y, z; rotation about z by -alpha, by +alpha
   std::vector<int> perm;  // the caller's index of every stored direction (the identity)
-  double Wtot = 0.0;
+  double Wtot = 0.0, T_knee = 0.0;
   // bands
   bool bands_set = false, solve_tp = false;
   int nb = 0, nbp = 0, ng = 16;
@@ -595,6 +595,7 @@ ThermoTables uthermo(const bte_umesh_ctx* u) {
   t.inv_v = u->inv_v;
   t.beta = u->beta_d;
   t.binv_v = u->binv_d;
+  t.T_knee = u->T_knee;
   t.ng = u->ng;
   t.nbp = t.nbo = u->nbp;
   t.nb = t.nbr = u->nb;
@@ -716,6 +717,7 @@ int ensure_mem(bte_umesh_ctx* u) {
   std::vector<double> nC, nCC, ap, aL, iv, be;
   build_thermo(u->nb, u->nbp, u->ng, u->wlo.data(), u->whi.data(), u->vg.data(), u->beta.data(), u->deg.data(), u->Wtot,
                nC, nCC, ap, aL, iv, be);
+  u->T_knee = model_knee(nC, u->nb, u->ng);
   std::vector<double> vbp(nbp, 0.0), bbp(nbp, 0.0), biv(nbp, 0.0);
   for (int b = 0; b < u->nb; ++b) { vbp[b] = u->vg[b]; bbp[b] = u->beta[b]; biv[b] = be[b] * iv[b]; }
   if ((rc = upload(u, u->node_c, nC.data(), nC.size())) || (rc = upload(u, u->node_C, nCC.data(), nCC.size())) ||
