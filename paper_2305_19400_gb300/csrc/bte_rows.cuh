@@ -113,7 +113,7 @@ struct FF {
     ff::P2 src;
   };
   struct Acc {
-    ff::P2 S, G, w;
+    ff::P2 B, S, G, w;  // sums of a block, of the run, of the closed runs; the run's weight
     unsigned key;
   };
   template <int DIM>
@@ -141,7 +141,7 @@ struct FF {
   __device__ static Cell cell(const SweepArgs&, const Lane& l, const double (&i0)[V], int, long long) {
     return Cell{ff::norm(ff::mul(l.betav, ff::from_doubles(i0[0], i0[1])))};
   }
-  __device__ static Acc acc(const SweepArgs&, const Cell&) { return Acc{ff::zero(), ff::zero(), ff::zero(), 0xffffffffu}; }
+  __device__ static Acc acc(const SweepArgs&, const Cell&) { return Acc{ff::zero(), ff::zero(), ff::zero(), ff::zero(), 0xffffffffu}; }
   template <int DIM>
   struct Block {
     ff::P2 c[DIM], R;
@@ -149,6 +149,7 @@ struct FF {
   template <int DIM, int RUN>
   __device__ static Block<DIM> block(const SweepArgs&, const Lane&, const Cell&, const Coef<DIM>& cf, const Tab<DIM>& t,
                                      Acc& s) {
+    ff::acc(s.S, s.B);
     if (t.key != s.key) {
       ff::acc(s.G, ff::mul(s.w, s.S));
       s.S = ff::zero();
@@ -161,7 +162,7 @@ struct FF {
     for (int k = 0; k < DIM; ++k) b.c[k] = ff::P2{t.ch[k], t.cl[k]};
     return b;
   }
-  template <int DIM>
+  template <int DIM, bool FIRST>
   __device__ static void step(const SweepArgs&, const Lane& l, const Cell& c, const Block<DIM>& b, unsigned sb, unsigned ostr,
                               char* out, char*, bool on, Acc& s) {
     ff::P2 t = ff::mul(b.c[0], ff::lds(sb + ostr));
@@ -171,9 +172,11 @@ struct FF {
     t = ff::add(t, ff::mul(l.rdtv, ff::lds(sb)));
     const ff::P2 r = ff::norm(ff::mul(b.R, t));
     if (on) ff::st_stream(out, r);
-    ff::acc(s.S, r);
+    if (FIRST) s.B = r;
+    else ff::acc(s.B, r);
   }
   __device__ static void finish(const SweepArgs&, const Cell&, Acc& s, int, int, double (&G)[V]) {
+    ff::acc(s.S, s.B);
     ff::acc(s.G, ff::mul(s.w, s.S));
     ff::to_doubles(ff::norm(s.G), G[0], G[1]);
   }
@@ -309,7 +312,7 @@ struct F64 {
     asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(x.x), "=d"(x.y) : "r"(sa));
     return x;
   }
-  template <int DIM>
+  template <int DIM, bool FIRST>
   __device__ static void step(const SweepArgs&, const Lane&, const Cell& c, const Block<DIM>& b, unsigned sb, unsigned ostr,
                               char* out, char* bout, bool on, Acc& s) {
     const double2 in = lds2(sb), ux = lds2(sb + ostr), uy = lds2(sb + 2 * ostr);
@@ -463,7 +466,7 @@ struct F32 {
     }
     return b;
   }
-  template <int DIM>
+  template <int DIM, bool FIRST>
   __device__ static void step(const SweepArgs&, const Lane& l, const Cell& c, const Block<DIM>& b, unsigned sb, unsigned ostr,
                               char* out, char*, bool on, Acc& s) {
     const ff::P2 in = ff::lds(sb);  // floats 0, 1 and 2, 3
@@ -679,7 +682,7 @@ __global__ void __launch_bounds__(256, M::kMinB) rows_kernel(SweepArgs a) {
           issue(std::integral_constant<int, ck>{}, si);
           bump(si);
           cp_wait<kAhead>();
-          M::template step<DIM>(a, ln, cell, bk, sb, ostr, out, bout, act0, acc);
+          M::template step<DIM, k == 0>(a, ln, cell, bk, sb, ostr, out, bout, act0, acc);
           out += DT * rowB;
           if (M::kStoreB) bout += DT * rowB;
           bump(sb);
