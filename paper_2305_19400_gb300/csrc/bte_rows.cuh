@@ -76,14 +76,21 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 // ------------------------------------------------------------------- modes
 // FP64 storage in double-float arithmetic (bte_ff.cuh), implicit: divided
 // through by v_b,
-//   I' = R (sum_ax c_ax u_ax + (beta_b/v_b) I0 + I^n/(v_b dt)),  R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax),
+//   I' = B + R (sum_ax c_ax u_ax + (beta_b/v_b) I0),  B = (1/(v_b dt)) R I^n,
+//   R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax),
 // 1/(v_b dt), beta_b/v_b and (beta_b/v_b) I0 in registers, c_ax of the block from
-// shared memory, R of the block from its table one block ahead.  Forming I^n/(v_b
-// dt) in every iteration costs four packed operations more than reading a stored
-// B = R I^n/(v_b dt), and saves the first iteration's write of B and its third
-// buffer's traffic.  The tables come from the host in double-float form with R
-// chosen so that R (1/(v_b dt) + beta_b/v_b + sum c_ax) = 1 holds for the table
-// values to double-double accuracy, which keeps a uniform equilibrium in place.
+// shared memory, R of the block from its table one block ahead.  Forming B in every
+// iteration costs eight packed operations more than reading a stored one, and saves
+// the first iteration's write of B and its third buffer's traffic.  R I^n comes first:
+// I^n/(v_b dt) would save four of them, but rounds alike in all directions of a cell
+// near equilibrium (1.5e-15 of a uniform state's band where this leaves 0.7e-15; 120x120 x 20
+// x 55, ten steps, 1100 us against 1109).  The tables come from the host in double-float
+// form with R chosen so that R (1/(v_b dt) + beta_b/v_b + sum c_ax) = 1 holds for the
+// table values to double-double accuracy, which keeps a uniform equilibrium in place.
+// The direction sum adds a block's rows first, then the block to its run of equal
+// weights, then the run times its weight to G: the rows of a block are close to equal, and
+// adding equal pairs twenty in a row without renormalising leaves 1.5e-14 rms where blocks
+// of four leave 2e-15, at the same number of operations.
 // Bound by HBM (24 bytes an update) and L2 to SM traffic; of few directions by
 // issue (0.51 of the slots at 16 warps per SM).  With coefficients read per
 // direction and the cells' step in the same kernel: 128x128 x 400 x 55 1535 us an
@@ -168,9 +175,8 @@ struct FF {
     ff::P2 t = ff::mul(b.c[0], ff::lds(sb + ostr));
 #pragma unroll
     for (int k = 1; k < DIM; ++k) t = ff::add(t, ff::mul(b.c[k], ff::lds(sb + (1 + k) * ostr)));
-    t = ff::add(t, c.src);
-    t = ff::add(t, ff::mul(l.rdtv, ff::lds(sb)));
-    const ff::P2 r = ff::norm(ff::mul(b.R, t));
+    const ff::P2 B = ff::mul(l.rdtv, ff::mul(b.R, ff::lds(sb)));
+    const ff::P2 r = ff::norm(ff::add(B, ff::mul(b.R, ff::add(t, c.src))));
     if (on) ff::st_stream(out, r);
     if (FIRST) s.B = r;
     else ff::acc(s.B, r);
