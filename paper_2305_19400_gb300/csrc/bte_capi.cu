@@ -419,12 +419,17 @@ int ensure_memory(bte_ctx* h) {
   for (int side = 0; side < 6; ++side) {
     WallDirs& wd = h->wall_dirs[side];
     int* l = wl.data() + (size_t)side * h->nd;
-    wd = WallDirs{h->wall_dirs_d + (size_t)side * h->nd, nullptr, 0, 0.0, 0.0};
+    wd = WallDirs{h->wall_dirs_d + (size_t)side * h->nd, nullptr, 0, 0.0, 0.0, 0.0, 0.0};
+    const auto add = [](double& s, double& lo, double x) {  // TwoSum
+      const double t = s + x, v = t - s;
+      lo += (s - (t - v)) + (x - v);
+      s = t;
+    };
     int nrest = 0;
     for (int d = 0; d < h->nd; ++d) {
       const double sn = (side & 1) ? h->S[3 * d + side / 2] : -h->S[3 * d + side / 2];
-      if (sn > 0.0) { l[wd.nout++] = d; wd.sum_out += sn; }
-      else { l[h->nd - ++nrest] = d; wd.sum_in -= sn; }
+      if (sn > 0.0) { l[wd.nout++] = d; add(wd.sum_out, wd.sum_out_lo, sn); }
+      else { l[h->nd - ++nrest] = d; add(wd.sum_in, wd.sum_in_lo, -sn); }
     }
     std::reverse(l + wd.nout, l + h->nd);
     wd.rest = wd.out + wd.nout;

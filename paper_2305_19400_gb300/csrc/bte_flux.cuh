@@ -59,8 +59,9 @@ __device__ double face_flux(const S* I, const double* I0ref, const double* I0wal
       const double* gw = I0wall + (g.face0[side] + f) * nbp + b;
       double ref = 0.0;  // the reference part of the reduced modes' storage
       if constexpr (sizeof(S) != 8) ref = I0ref[b] + I0ref[b + 1];
-      acc = fma(wd.sum_out, ref, acc);
-      acc = fma(-wd.sum_in, bc == 3 ? ref : gw[0] + gw[1], acc);
+      const double in = bc == 3 ? ref : gw[0] + gw[1];
+      acc = fma(wd.sum_out, ref, fma(-wd.sum_in, in, acc));
+      acc = fma(wd.sum_out_lo, ref, fma(-wd.sum_in_lo, in, acc));
     }
   }
   return block_sum(acc, sh);

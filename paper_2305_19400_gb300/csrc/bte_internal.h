@@ -69,12 +69,14 @@ struct DirInfo {
 };
 
 // The directions of one wall side: those leaving through it (S_d . n_out > 0),
-// then the rest, and the sums of |S_d,ax| over the leaving and the entering ones.
+// then the rest, and the sums of |S_d,ax| over the leaving and the entering ones, each
+// with the rounding error of its double: a wall's net flux is a small difference of
+// these sums' multiples.
 struct WallDirs {
   const int* out;   // [nout]
   const int* rest;  // [nd - nout]
   int nout;
-  double sum_out, sum_in;
+  double sum_out, sum_in, sum_out_lo, sum_in_lo;
 };
 
 // A cell whose temperature its cached model could not settle.

@@ -581,7 +581,7 @@ __device__ __forceinline__ void wall_diffuse(const WallArgs<S>& w, const S* row,
   for (int b = threadIdx.x; b < w.nbp; b += kWallThreads) {
     double num = part[b];
     for (int g = 1; g < groups; ++g) num += part[g * w.nbp + b];
-    if constexpr (sizeof(S) != 8) num = fma(w.wd.sum_out - w.wd.sum_in, w.I0ref[b], num);
+    if constexpr (sizeof(S) != 8) num = fma((w.wd.sum_out - w.wd.sum_in) + (w.wd.sum_out_lo - w.wd.sum_in_lo), w.I0ref[b], num);
     D[b] = num / w.wd.sum_in;
   }
   __syncthreads();

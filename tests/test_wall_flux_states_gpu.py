@@ -64,3 +64,18 @@ def test_after_a_change_of_wall_kind(dim, kind, p):
     O.Problem(rough.geoms[0], O.dirs_for(wl.dirs), wl.bands).run(ost, wl.dt, 1, wl.ninner)
     assert np.max(np.abs(s.T(0) - ost["TL"]) / ost["TL"]) <= 1e-12
     s.close()
+
+
+# No heat crosses a wall at the temperature of a uniform state.  What is left is rounding: of the
+# 252 partial sums 2e-17 of the one-sided flux, where one rounding error of the direction weights' sum,
+# common to all bands, would leave 2.8e-16 on the x sides.  Bar: half of that.
+def test_no_flux_at_equilibrium():
+    g = W.Geometry(2, 3, 3, 1, 10e-9, 10e-9, 10e-9)
+    W.uniform_walls(g, [W.BC_ISOTHERMAL] * 4, [300.0] * 4)
+    wl = W.Workload("equilibrium", [g], W.Dirs("polar_azim", n_polar=20, n_azim=20), W.make_bands(40, 15, 72), 1e-12, 1, 1)
+    s = bte.Solver(wl)
+    S = bte.bte_get_directions(s.h)[0]
+    one_sided = np.sum(s.intensity(0)[0] * np.maximum(S[:, :1], 0.0))
+    q, qw = s.flux(0)
+    assert np.max(np.abs(qw)) <= 1.4e-16 * one_sided
+    s.close()
