@@ -1533,11 +1533,11 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   const size_t es = elem_bytes(prec);
   char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
   cudaStream_t s = h->stream;
-  // a restored state is kept as given, in doubles, until a double-float step; a lone
-  // geometry's is overwritten whole
-  if (h->geoms.size() == 1) h->state_ff = false;
-  else CUDA_TRY(h, ensure_state_doubles(h));
   CUDA_TRY(h, cudaMemcpyAsync(h->Tp + h->cell0[geom], Tp_cells, nc * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+  // a restored state is kept as given, in doubles, until a double-float step; a lone
+  // geometry's is overwritten whole, and has no state when a call below fails half-way
+  if (h->geoms.size() > 1) CUDA_TRY(h, ensure_state_doubles(h));
+  else if (h->state_ff) h->init_set[geom] = h->state_ff = false;
   CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
                                    h->Msum + h->cell0[geom] * 4, h->MsumL + h->cell0[geom] * 4,
                                    h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));
@@ -1559,6 +1559,7 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   if (h->Epart) h->EL_partial = true;  // this handle holds only its bands' share of E_L until the next step's exchange
   else CUDA_TRY(h, launch_energy_L(h->Ec + h->cell0[geom] * kRedEntries, h->EL + h->cell0[geom], nc, s));
   CUDA_TRY(h, cudaStreamSynchronize(s));
+  h->init_set[geom] = true;
   h->TL_valid = false;
   h->bscale_valid = false;
   return BTE_OK;
