@@ -515,7 +515,6 @@ struct bte_umesh_ctx {
   int nd = 0;
   std::vector<double> S, w;
   std::vector<int> refl;  // [5][nd]: mirror across x, y, z; rotation about z by -alpha, by +alpha
-  std::vector<int> perm;  // the caller's index of every stored direction (the identity)
   double Wtot = 0.0, T_knee = 0.0;
   // bands
   bool bands_set = false, solve_tp = false;
@@ -541,7 +540,8 @@ struct bte_umesh_ctx {
   float* w32_d = nullptr;  // [nd] direction weights as float
   float* g32 = nullptr;    // [entries][nd] g as float (reduced storage)
   double *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr, *inv_v = nullptr, *beta_d = nullptr, *binv_d = nullptr;
-  int *cf_ptr = nullptr, *bf_mirror_d = nullptr, *bf_axis_d = nullptr, *refl_d = nullptr, *perm_d = nullptr;
+  int *cf_ptr = nullptr, *bf_mirror_d = nullptr, *bf_axis_d = nullptr, *refl_d = nullptr;
+  int* rows_d = nullptr;   // [nd] the packing kernels' row of every direction (here its own)
   long long *cf_up = nullptr, *bface_d = nullptr, *owner_d = nullptr, *diff_d = nullptr;
   int ndiff = 0;
   FixItem* fix = nullptr;
@@ -657,12 +657,14 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = dalloc(u, &u->S_d, nd * 3)) || (rc = dalloc(u, &u->w_d, nd)) || (rc = dalloc(u, &u->nA_d, u->nf * 3)) ||
       (rc = dalloc(u, &u->vb_d, nbp)) || (rc = dalloc(u, &u->bb_d, nbp)) || (rc = dalloc(u, &u->scratch, nc)) ||
       (rc = dalloc(u, &u->Qb, nbf)) || (rc = dalloc(u, &u->qbuf, nc * 3)) || (rc = dalloc(u, &u->bf_mirror_d, nbf)) || (rc = dalloc(u, &u->bf_axis_d, nbf)) || (rc = dalloc(u, &u->bf_spec_d, nbf)) || (rc = dalloc(u, &u->bscale, nc)) ||
-      (rc = dalloc(u, &u->refl_d, 5 * nd)) || (rc = dalloc(u, &u->perm_d, nd)) || (rc = dalloc(u, &u->bface_d, nbf)) || (rc = dalloc(u, &u->owner_d, u->nf)) ||
+      (rc = dalloc(u, &u->refl_d, 5 * nd)) || (rc = dalloc(u, &u->rows_d, nd)) || (rc = dalloc(u, &u->bface_d, nbf)) || (rc = dalloc(u, &u->owner_d, u->nf)) ||
       (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, cells_queue_entries(nc))) || (rc = dalloc(u, &u->Ec, nc * kRedEntries)) || (rc = dalloc(u, &u->MsumL, nc * 4)) ||
       (rc = dalloc(u, &u->counters, 1)) || (rc = dalloc(u, &u->node_c, nbp * u->ng)) ||
       (rc = dalloc(u, &u->node_C, nbp * u->ng)) || (rc = dalloc(u, &u->a_p, nbp)) || (rc = dalloc(u, &u->a_L, nbp)) ||
       (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->beta_d, nbp)) || (rc = dalloc(u, &u->binv_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
     return rc;
+  std::vector<int> rows(nd);
+  std::iota(rows.begin(), rows.end(), 0);
   // cell -> face entries
   std::vector<int> ptr(nc + 1, 0);
   for (long long f = 0; f < u->nf; ++f) {
@@ -700,7 +702,7 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = upload(u, ef_d, ent_face.data(), nent)) || (rc = upload(u, ec_d, ent_cell.data(), nent)) ||
       (rc = upload(u, es_d, ent_sign.data(), nent)) || (rc = upload(u, vol_d, u->vol.data(), nc)) ||
       (rc = upload(u, u->nA_d, u->nA.data(), u->nf * 3)) || (rc = upload(u, u->S_d, u->S.data(), nd * 3)) ||
-      (rc = upload(u, u->w_d, u->w.data(), nd)) || (rc = upload(u, u->perm_d, u->perm.data(), nd)) || (rc = upload(u, u->refl_d, u->refl.data(), 5 * nd)) ||
+      (rc = upload(u, u->w_d, u->w.data(), nd)) || (rc = upload(u, u->rows_d, rows.data(), nd)) || (rc = upload(u, u->refl_d, u->refl.data(), 5 * nd)) ||
       (rc = upload(u, u->bface_d, u->bface.data(), nbf)) || (rc = upload(u, u->owner_d, u->owner.data(), u->nf)))
     return rc;
   umesh_geom_kernel<<<grid_for(nent * nd, 256), 256, 0, s>>>(ef_d, es_d, ec_d, u->nA_d, vol_d, u->S_d, u->w_d, (int)nd,
@@ -887,11 +889,9 @@ int bte_umesh_create(const bte_umesh_desc* m, const bte_opts* opts, bte_umesh* o
     return ufail(nullptr, BTE_E_ARG, "bad direction set");
   }
   u->nd = (int)u->w.size();
-  // rows in the caller's order: neighbouring azimuths share most inflow faces, so
+  // rows stay in the caller's order: neighbouring azimuths share most inflow faces, so
   // the lanes of a warp take the same branches (the structured handle's order cost
   // the FP64 sweep 10 %)
-  u->perm.resize(u->nd);
-  std::iota(u->perm.begin(), u->perm.end(), 0);
   u->refl.resize(5 * (size_t)u->nd);
   for (int d = 0; d < u->nd; ++d) u->refl[3 * u->nd + d] = u->refl[4 * u->nd + d] = d;  // until a rotation is set
   if (m->fc) u->fc.assign(m->fc, m->fc + 3 * m->nfaces);
@@ -1165,17 +1165,23 @@ int bte_umesh_get_T(bte_umesh u, int which, double* out, int on_device) {
 int bte_umesh_get_intensity(bte_umesh u, double* out) {
   if (!u || !out) return u ? ufail(u, BTE_E_ARG, "out is NULL") : BTE_E_ARG;
   if (!u->init_done) return ufail(u, BTE_E_STATE, "no state");
-  // full FP64 values in the caller's direction order through a temporary device
+  if (u->prec == BTE_FP64) {  // no device memory beyond the state's
+    UTRY(u, cudaMemcpy2DAsync(out, (size_t)u->nb * 8, u->I[u->cur], (size_t)u->nbp * 8, (size_t)u->nb * 8,
+                              (size_t)(u->nc * u->nd), cudaMemcpyDeviceToHost, u->stream));
+    UTRY(u, cudaStreamSynchronize(u->stream));
+    return BTE_OK;
+  }
+  // reduced storage: full FP64 values (I0_b(T_ref) + deviation) through a temporary device
   // buffer of at most 64 MB (whole cells)
   double* tmp = nullptr;
   const size_t cell = (size_t)u->nd * u->nb;
   const long long chunk = std::max(1LL, std::min<long long>(u->nc, (64LL << 20) / (long long)(cell * 8)));
   cudaError_t e = cudaMalloc(&tmp, chunk * cell * 8);
   if (e != cudaSuccess) return ufail(u, BTE_E_NOMEM, "cudaMalloc(%zu bytes): %s", chunk * cell * 8, cudaGetErrorString(e));
-  const size_t eb = u->prec == BTE_FP64 ? 8 : (u->prec == BTE_FP32 ? 4 : 2);
+  const size_t eb = u->prec == BTE_FP32 ? 4 : 2;
   for (long long c0 = 0; c0 < u->nc && e == cudaSuccess; c0 += chunk) {
     const long long m = std::min(chunk, u->nc - c0);
-    e = launch_unpack(u->prec, false, (const char*)u->I[u->cur] + (size_t)c0 * u->nd * u->nbp * eb, tmp, u->I0ref, u->perm_d, m,
+    e = launch_unpack(u->prec, false, (const char*)u->I[u->cur] + (size_t)c0 * u->nd * u->nbp * eb, tmp, u->I0ref, u->rows_d, m,
                       u->nd, u->nb, u->nbp, u->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out + c0 * cell, tmp, m * cell * 8, cudaMemcpyDeviceToHost, u->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(u->stream);
@@ -1202,7 +1208,7 @@ int bte_umesh_set_intensity(bte_umesh u, const double* in, const double* Tp_cell
   if (e == cudaSuccess) e = launch_state_from_Tp(u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->nc, uthermo(u), s);
   const SweepArgs sums = cell_args(u, u->I[u->cur]);
   if (e == cudaSuccess)
-    e = launch_pack(u->prec, tmp, u->I[u->cur], u->I0ref, u->perm_d, u->nc, u->nd, u->nb, u->nbp, &sums, s);
+    e = launch_pack(u->prec, tmp, u->I[u->cur], u->I0ref, u->rows_d, u->nc, u->nd, u->nb, u->nbp, &sums, s);
   if (e == cudaSuccess) e = launch_energy_L(u->Ec, u->EL, u->nc, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(tmp);
