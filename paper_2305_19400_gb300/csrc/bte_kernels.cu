@@ -277,8 +277,10 @@ __global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, co
 // one CTA of 8 warps per cell.  Loads of 16 bytes, eight in
 // flight; FP64: four, warp w sums the directions [w nd / 8, (w + 1) nd / 8), lanes over
 // band pairs (whole warps on one direction, so the runs of the fixed-point sums
-// close together: groups of 28 lanes took 406 us where this takes 308 on 6144 cells
-// x 400 x 55); reduced storage: lanes over the V bands of a vector, 256 V / nbp
+// close together: groups of 28 lanes took 406 us where this took 308 on 6144 cells
+// x 400 x 55), their weights loaded with them: loaded behind them, each value's sum
+// waited for its own (ten sweep-ordered iterations of 128x128 x 400 x 55 31.6 ms, 30.1
+// so; of 6144 triangles 12.6 and 12.0); reduced storage: lanes over the V bands of a vector, 256 V / nbp
 // groups.  The partials are added in order (deterministic) to G_b = sum_d w_d I_{d,b};
 // warp 0 leaves kRedEntries partial energies in Ec for cells_kernel.  Bound by the
 // loads' latency and HBM, 8 bytes per FP64 value.
@@ -380,12 +382,13 @@ __global__ void __launch_bounds__(kRedThreads, 4) gs_reduce_kernel(SweepArgs a, 
         auto batch = [&](auto n, int d) {
           constexpr int N = decltype(n)::value;
           double2 x[N];
+          double w[N];
 #pragma unroll
           for (int u = 0; u < N; ++u) x[u] = __ldcs(reinterpret_cast<const double2*>(row + (long long)(d + u) * nbo));
 #pragma unroll
-          for (int u = 0; u < N; ++u) {
-            sum.add(x[u].x, x[u].y, a.wdir[d + u]);
-          }
+          for (int u = 0; u < N; ++u) w[u] = __ldg(a.wdir + d + u);
+#pragma unroll
+          for (int u = 0; u < N; ++u) sum.add(x[u].x, x[u].y, w[u]);
         };
         int d = d0;
         for (; d + 4 <= d1; d += 4) batch(std::integral_constant<int, 4>{}, d);
