@@ -672,7 +672,7 @@ SweepArgs sweep_args(bte_ctx* h) {
 
 int ensure_TL(bte_ctx* h) {
   if (h->TL_valid) return BTE_OK;
-  CUDA_TRY(h, launch_cells(sweep_args(h), h->ncells, 3, nullptr, h->stream));
+  CUDA_TRY(h, launch_cells(sweep_args(h), h->ncells, 3, nullptr, 0, h->stream));
   h->TL_valid = true;
   return BTE_OK;
 }
@@ -776,6 +776,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
   const bool use_b = h->opts.precision == BTE_FP64 && !use_ff && !a.explicit_scheme && ninner >= 2;
   a.ff = use_ff ? 1 : 0;
   if (scheme == BTE_IMPLICIT_GS) a.ne = kRedEntries;
+  const long long before = scheme == BTE_IMPLICIT_GS ? h->ncells : a.nitems;  // CTAs of gs_reduce_kernel or the sweep
   int z = -1;
   for (int it = 0; it < ninner; ++it) {
     int o = 0;
@@ -814,7 +815,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
     if (e == cudaSuccess && a.partial) {
       // band-range handle: the caller sums the per-cell (E_L, E_p) partials over
       // the ranks that hold the other bands, then every rank solves every cell
-      e = launch_cells(a, h->ncells, 1, nullptr, s);
+      e = launch_cells(a, h->ncells, 1, nullptr, before, s);
       if (e != cudaSuccess) return e;
       const int xr = h->exchange(a.Epart, 2 * h->ncells, (void*)s, h->exchange_user);
       if (xr != 0) {
@@ -824,7 +825,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
     }
     if (e == cudaSuccess) {
       const MLPView m = mlp_view(h);
-      e = launch_cells(a, h->ncells, a.partial ? 2 : 0, h->opts.learned ? &m : nullptr, s);
+      e = launch_cells(a, h->ncells, a.partial ? 2 : 0, h->opts.learned ? &m : nullptr, a.partial ? h->ncells : before, s);
     }
     if (e != cudaSuccess) return e;
     k = o;

@@ -259,17 +259,19 @@ int cells_grid(long long ncells) {
   return 113 * kCellCluster;
 }
 
-cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const MLPView* mlp, cudaStream_t s) {
+cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const MLPView* mlp, long long before,
+                         cudaStream_t s) {
   const size_t sm = mode == kPartial ? 0
                               : (cta_solve_smem_doubles(a.th.nbp, a.th.ng, 1) + 2) * sizeof(double) +
                                     (mlp ? (2 * (size_t)a.th.nbp + 4 * kHidden) * sizeof(float) : 0);
   MLPView m{};
   if (mlp) m = *mlp;
-  // Of few cells, where the sweep before leaves most SMs free, launched early: the
-  // launch and the prologue are then hidden (a step of 11 sweeps of 400 cells 221 -> 199
-  // us).  Behind a sweep that fills the chip the early CTAs crowd into the slots that are
-  // left on some SMs (3015 cells: 2 % slower, 14400: 2.5 %).
-  const bool early = ncells <= 1024;
+  // Launched early behind a sweep of at most one CTA per SM: the launch and the prologue
+  // are then hidden (11 sweeps of 400 cells x 16 x 4 in 60 CTAs 221 -> 199 us a step; 992
+  // cells x 20 x 55 in 124 CTAs 227 -> 224).  Behind more of them the early CTAs crowd into the
+  // slots that are left on some SMs (992 cells x 400 x 55 in 248 CTAs 1133 -> 1142 us,
+  // 3015 cells 2 % and 14400 cells 2.5 % slower).
+  const bool early = before <= 152;
   return launch_pdl(early, mlp ? cells_kernel<true> : cells_kernel<false>, cells_grid(ncells), kCellThreads, sm, s, a, ncells,
                     mode, m);
 }

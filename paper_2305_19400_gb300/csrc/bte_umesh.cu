@@ -815,7 +815,7 @@ cudaError_t refresh_diffuse(bte_umesh_ctx* u, const void* I) {
 
 int ensure_TL(bte_umesh_ctx* u) {
   if (u->TL_valid) return BTE_OK;
-  UTRY(u, launch_cells(cell_args(u, nullptr), u->nc, 3, nullptr, u->stream));
+  UTRY(u, launch_cells(cell_args(u, nullptr), u->nc, 3, nullptr, 0, u->stream));
   u->TL_valid = true;
   return BTE_OK;
 }
@@ -1114,7 +1114,7 @@ int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, b
       }
       SweepArgs c = cell_args(u, a.Iout);
       UTRY(u, launch_gs_reduce(u->prec, c, u->nc, s));
-      UTRY(u, launch_cells(c, u->nc, 0, nullptr, s));
+      UTRY(u, launch_cells(c, u->nc, 0, nullptr, u->nc, s));
       launches += 3 + (u->ndiff ? 1 : 0) + (tt ? 1 : 0);
       k = o;
     }
