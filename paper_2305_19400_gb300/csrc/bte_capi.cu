@@ -115,7 +115,7 @@ struct bte_ctx {
   double mlp_Tlo = 0.0, mlp_Thi = 0.0, mlp_Elo = 0.0, mlp_Ehi = 0.0;
   long long pack_cells = 0;
   double *wdir = nullptr, *Sdev = nullptr, *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr;
-  double *inv_v = nullptr, *beta_d = nullptr, *binv_d = nullptr, *scratch_faces = nullptr, *scratch_T = nullptr, *scratch_out = nullptr;
+  double *inv_v = nullptr, *binv_d = nullptr, *scratch_faces = nullptr, *scratch_T = nullptr, *scratch_out = nullptr;
   double* scratch_q = nullptr;
   std::vector<DevGeom> dgeoms;
   DirInfo* dirs_d = nullptr;
@@ -179,7 +179,6 @@ ThermoTables thermo(const bte_ctx* h) {
   t.a_p = h->a_p;
   t.a_L = h->a_L;
   t.inv_v = h->inv_v;
-  t.beta = h->beta_d;
   t.binv_v = h->binv_d;
   t.T_knee = h->T_knee;
   t.ng = h->ng;
@@ -263,7 +262,6 @@ size_t carve(bte_ctx* h, char* base) {
   h->a_p = (double*)take((size_t)h->nbp_all * 8);
   h->a_L = (double*)take((size_t)h->nbp_all * 8);
   h->inv_v = (double*)take((size_t)h->nbp * 8);   // stored bands
-  h->beta_d = (double*)take((size_t)h->nbp * 8);
   h->binv_d = (double*)take((size_t)h->nbp * 8);
   h->geoms_d = (DevGeom*)take(h->geoms.size() * sizeof(DevGeom));
   h->items_d = (WorkItem*)take((size_t)std::max<long long>(h->ncells, 1) * sizeof(WorkItem));  // room for 1 cell per item
@@ -450,15 +448,13 @@ int ensure_memory(bte_ctx* h) {
   CUDA_TRY(h, cudaMemcpyAsync(h->a_p, ap.data(), ap.size() * 8, cudaMemcpyHostToDevice, s));
   CUDA_TRY(h, cudaMemcpyAsync(h->a_L, aL.data(), aL.size() * 8, cudaMemcpyHostToDevice, s));
   {
-    std::vector<double> iv_o(h->nbp, 0.0), be_o(h->nbp, 0.0), bi_o(h->nbp, 0.0);  // stored bands, zero on padding
+    std::vector<double> iv_o(h->nbp, 0.0), bi_o(h->nbp, 0.0);  // stored bands, zero on padding
     for (int b = 0; b < h->nb; ++b) {
       iv_o[b] = iv[h->band0 + b];
-      be_o[b] = be[h->band0 + b];
-      bi_o[b] = be_o[b] * iv_o[b];
+      bi_o[b] = be[h->band0 + b] * iv_o[b];
     }
     CUDA_TRY(h, cudaMemcpyAsync(h->binv_d, bi_o.data(), bi_o.size() * 8, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaMemcpyAsync(h->inv_v, iv_o.data(), iv_o.size() * 8, cudaMemcpyHostToDevice, s));
-    CUDA_TRY(h, cudaMemcpyAsync(h->beta_d, be_o.data(), be_o.size() * 8, cudaMemcpyHostToDevice, s));
     CUDA_TRY(h, cudaStreamSynchronize(s));
   }
   {

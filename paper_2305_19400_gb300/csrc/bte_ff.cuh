@@ -195,23 +195,12 @@ __device__ __forceinline__ P2 lds(unsigned sa) {
   asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(p.h), "=l"(p.l) : "r"(sa));
   return p;
 }
-// two doubles from a 32-bit shared-memory address, as an ff pair
-__device__ __forceinline__ P2 lds_doubles(unsigned sa) {
-  double a, b;
-  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(a), "=d"(b) : "r"(sa));
-  return from_doubles(a, b);
-}
 __device__ __forceinline__ P2 ldg(const void* p) {
   const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2*>(p));
   return P2{v.x, v.y};
 }
 __device__ __forceinline__ void st_stream(void* p, const P2& v) {
   __stcs(reinterpret_cast<ulonglong2*>(p), make_ulonglong2(v.h, v.l));
-}
-__device__ __forceinline__ void st_stream_doubles(void* p, const P2& v) {
-  double a, b;
-  to_doubles(v, a, b);
-  __stcs(reinterpret_cast<double2*>(p), make_double2(a, b));
 }
 
 }  // namespace ff

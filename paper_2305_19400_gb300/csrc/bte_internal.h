@@ -102,7 +102,6 @@ struct ThermoTables {
   const double* a_p;      // [nbp] W beta_b / v_b  (T_p equation weights)
   const double* a_L;      // [nbp] W / v_b         (T_L equation weights)
   const double* inv_v;    // [nbo] 1/v_b of the stored bands (0 on padding)
-  const double* beta;     // [nbo] beta_b of the stored bands (0 on padding)
   const double* binv_v;   // [nbo] beta_b/v_b of the stored bands (0 on padding)
   double T_knee;          // hbar omega_max / (32 k_B): the trust radius shrinks below (model_trust)
   int ng;

@@ -122,12 +122,6 @@ __device__ __forceinline__ double full_I(const S* I, long long e, int b, const d
   if constexpr (sizeof(S) == 8) return (double)I[e];
   else return I0ref[b] + Tr<S>::to_double(I[e]);
 }
-template <>
-__device__ __forceinline__ double full_I<FFElem>(const FFElem* I, long long e, int, const double*) {
-  const float* p = reinterpret_cast<const float*>(I) + 4 * (e >> 1) + (e & 1);
-  return ff::to_double(p[0], p[2]);
-}
-
 
 // Two consecutive stored values (e even) as doubles, without the reference part of
 // the reduced modes, and the reverse.

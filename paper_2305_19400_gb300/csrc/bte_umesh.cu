@@ -539,7 +539,7 @@ struct bte_umesh_ctx {
   float* ghost_dev = nullptr;  // [bface][nbp] ghost deviations (reduced storage)
   float* w32_d = nullptr;  // [nd] direction weights as float
   float* g32 = nullptr;    // [entries][nd] g as float (reduced storage)
-  double *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr, *inv_v = nullptr, *beta_d = nullptr, *binv_d = nullptr;
+  double *node_c = nullptr, *node_C = nullptr, *a_p = nullptr, *a_L = nullptr, *inv_v = nullptr, *binv_d = nullptr;
   int *cf_ptr = nullptr, *bf_mirror_d = nullptr, *bf_axis_d = nullptr, *refl_d = nullptr;
   int* rows_d = nullptr;   // [nd] the packing kernels' row of every direction (here its own)
   long long *cf_up = nullptr, *bface_d = nullptr, *owner_d = nullptr, *diff_d = nullptr;
@@ -593,7 +593,6 @@ ThermoTables uthermo(const bte_umesh_ctx* u) {
   t.a_p = u->a_p;
   t.a_L = u->a_L;
   t.inv_v = u->inv_v;
-  t.beta = u->beta_d;
   t.binv_v = u->binv_d;
   t.T_knee = u->T_knee;
   t.ng = u->ng;
@@ -661,7 +660,7 @@ int ensure_mem(bte_umesh_ctx* u) {
       (rc = dalloc(u, &u->diff_d, nbf)) || (rc = dalloc(u, &u->fix, cells_queue_entries(nc))) || (rc = dalloc(u, &u->Ec, nc * kRedEntries)) || (rc = dalloc(u, &u->MsumL, nc * 4)) ||
       (rc = dalloc(u, &u->counters, 1)) || (rc = dalloc(u, &u->node_c, nbp * u->ng)) ||
       (rc = dalloc(u, &u->node_C, nbp * u->ng)) || (rc = dalloc(u, &u->a_p, nbp)) || (rc = dalloc(u, &u->a_L, nbp)) ||
-      (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->beta_d, nbp)) || (rc = dalloc(u, &u->binv_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
+      (rc = dalloc(u, &u->inv_v, nbp)) || (rc = dalloc(u, &u->binv_d, nbp)) || (rc = dalloc(u, &u->cf_ptr, nc + 1)))
     return rc;
   std::vector<int> rows(nd);
   std::iota(rows.begin(), rows.end(), 0);
@@ -724,7 +723,7 @@ int ensure_mem(bte_umesh_ctx* u) {
   for (int b = 0; b < u->nb; ++b) { vbp[b] = u->vg[b]; bbp[b] = u->beta[b]; biv[b] = be[b] * iv[b]; }
   if ((rc = upload(u, u->node_c, nC.data(), nC.size())) || (rc = upload(u, u->node_C, nCC.data(), nCC.size())) ||
       (rc = upload(u, u->a_p, ap.data(), ap.size())) || (rc = upload(u, u->a_L, aL.data(), aL.size())) ||
-      (rc = upload(u, u->inv_v, iv.data(), iv.size())) || (rc = upload(u, u->beta_d, be.data(), be.size())) ||
+      (rc = upload(u, u->inv_v, iv.data(), iv.size())) ||
       (rc = upload(u, u->vb_d, vbp.data(), nbp)) || (rc = upload(u, u->bb_d, bbp.data(), nbp)) ||
       (rc = upload(u, u->binv_d, biv.data(), nbp)))
     return rc;
