@@ -1341,7 +1341,7 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
   int rc = ensure_coef(h, dt, scheme == BTE_EXPLICIT ? BTE_EXPLICIT : BTE_IMPLICIT_JACOBI);
   if (rc) return rc;
   const bool ff = scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h);
-  CUDA_TRY(h, ff ? ensure_state_ff(h) : ensure_state_doubles(h));  // the form the timed sweeps read
+  if (!ff) CUDA_TRY(h, ensure_state_doubles(h));  // the form the timed sweeps read
   if (h->opts.beta_T_exp != 0.0 && !h->bscale_valid) {
     CUDA_TRY(h, launch_beta_scale(h->bscale, h->Tp, h->opts.T_ref, h->opts.beta_T_exp, h->ncells, h->stream));
     h->bscale_valid = true;
@@ -1351,6 +1351,11 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
   int sms = 152;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->dev);
   const int spare = (h->cur + 1) % 3;  // timing launches write here; the state is untouched
+  int src = h->cur;                    // and read it, or a copy as ff pairs of one held in doubles
+  if (ff && !h->state_ff) {
+    src = (h->cur + 2) % 3;
+    CUDA_TRY(h, launch_doubles_to_ff(h->Ibuf[h->cur], h->Ibuf[src], (long long)h->ncells * h->nd * h->nbp / 2, s));
+  }
   struct Cand { int cpb, dteam, grid, pd; float ms; };
   std::vector<Cand> tried;
   // directions per team step: the default and half of it (fewer lanes per
@@ -1404,7 +1409,7 @@ int bte_autotune(bte_handle h, double dt, int scheme, char* report, size_t repor
       }
       SweepArgs a = sweep_args(h);
       a.counters = nullptr;
-      a.In = a.Ik = h->Ibuf[h->cur];
+      a.In = a.Ik = h->Ibuf[src];
       a.Iout = h->Ibuf[spare];
       a.ff = ff ? 1 : 0;
       CUDA_TRY(h, launch_sweep(h->opts.precision, c.pd, a, dim, h->threads, c.grid, s));

@@ -41,3 +41,12 @@ def test_one_geometry_set_again_after_a_step():
     assert np.array_equal(s.intensity(1), other)
     s.close()
     ref.close()
+
+
+@pytest.mark.parametrize("scheme", [bte.BTE_IMPLICIT_JACOBI, bte.BTE_EXPLICIT, bte.BTE_IMPLICIT_GS])
+def test_tuning_leaves_the_state(scheme):
+    s = bte.Solver(workload())
+    I = s.intensity(0)
+    bte.bte_autotune(s.h, 1e-13, scheme)
+    assert np.array_equal(s.intensity(0), I)
+    s.close()
