@@ -328,10 +328,12 @@ void build_items(bte_ctx* h, int cpb = 0, int dteam = 0) {
   }
   // One CTA per item, started in order: the cells in flight stay close together and
   // find their neighbours' rows in L2.  Resident CTAs that stride over the items drift
-  // apart (128x128 x 400 x 55 in FP64 1374 us against 1084, 30.5 DRAM bytes an update
-  // against 26.1; 32^3 in FP32 1473 against 1172).  In-plane sets, whose items are short
-  // and whose ring would drain, take the resident CTAs (120x120 x 20 x 55: 68 us
-  // against 72, IEEE 108 against 123).
+  // apart: 128x128 x 400 x 55 in FP64, a step's first iteration (I^n = I^k) 1372 us and 23.0
+  // DRAM bytes an update against 1102 and 17.5, the others 1782 and 30.9 against 1430 and
+  // 26.4; 32^3 in FP32 1450 and 2203 us against 1171 and 1584.  In-plane sets, whose items are
+  // short and whose ring would drain, take the resident CTAs (120x120 x 20 x 55, first
+  // and others: IEEE 146 and 115 us against 163 and 131, double-float 73 and 86 against 77
+  // and 84).
   const bool persistent = h->opts.precision != BTE_BF16 && h->dir_group == 4;
   h->grid = persistent ? 0 : (int)std::min<size_t>(h->items.size(), 65535);
 }

@@ -284,10 +284,10 @@ __global__ void __launch_bounds__(256) unpack_kernel(const S* I, double* out, co
 // groups.  The partials are added in order (deterministic) to G_b = sum_d w_d I_{d,b};
 // warp 0 leaves kRedEntries partial energies in Ec for cells_kernel.  Bound by the
 // loads' latency and HBM, 8 bytes per FP64 value.
-// FP64: sums over a run of equal-weight directions are exact 64-bit fixed-point
-// additions on the integer pipe (unit 2^(E-50) for the cell's I0 of exponent E; a
-// value up to 32 I0 adds at most 2^55, so a run of 256 cannot overflow), closed by
-// one FP64 FMA (sum x w x unit).  Values beyond that range (or negative, NaN) take
+// FP64: sums over a run of equal-weight directions are 64-bit fixed-point additions
+// on the integer pipe (unit 2^(E-50) for the cell's I0 of exponent E; terms are cut
+// to whole units, less than one each; a value up to 32 I0 adds at most 2^55, so a run of
+// 256 cannot overflow), closed by one FP64 FMA (sum x w x unit).  Values beyond that range (or negative, NaN) take
 // the FP64 FMA directly.
 // Reduced storage (deviations from I0_b(T_ref)): each lane sums w_d x deviation in
 // FP32, added to a double-float sum every 16 directions (FP64 conversions and adds
@@ -516,7 +516,7 @@ __global__ void energy_L_kernel(const double2* Ec, double* EL, long long ncells)
 // flight; the groups' partials are added in order in shared memory.  One warp
 // per face walking every direction, each thread forming the weight sum again,
 // took 280 us (diffuse) and 204 us (partially specular) on the 67 faces of a
-// 67x45 grid with 400 directions x 55 bands; this form takes 8-9 us.
+// 67x45 grid with 400 directions x 55 bands; this form takes 15 and 23 us.
 // Reduced modes sum the stored deviations: the reference part of the ratio is
 // I0_b(T_ref) (sum_out - sum_in) / sum_in.
 constexpr int kWallThreads = 256;

@@ -94,7 +94,7 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 // Bound by HBM (24 bytes an update) and L2 to SM traffic; of few directions by
 // issue (0.51 of the slots at 16 warps per SM).  With coefficients read per
 // direction and the cells' step in the same kernel: 128x128 x 400 x 55 1535 us an
-// iteration, 23x18x13 867, 120x120 x 20 x 55 124; now 1420, 600 and 67, and 43, 30
+// iteration, 23x18x13 867, 120x120 x 20 x 55 124; now 1440, 530 and 70, and 43, 30
 // and 30 for the cells.
 struct FF {
   using S = double;
@@ -201,11 +201,13 @@ struct FF {
 // outside it: s runs to (T_p/T_ref)^16; a correctly rounded reciprocal per update took
 // 1745 us on 64x48 cells x 400 x 55).
 // The direction sum runs on the integer pipe: over a run of directions with the
-// same weight each band adds I exactly in 64-bit fixed point, unit 2^(E - 50) for
-// the cell's I0 of exponent E, so a value up to 16 I0 adds at most 2^55 and a run
-// of 256 cannot overflow; the run then enters G with one FP64 FMA (sum x w x
-// unit).  Values with a larger exponent (or negative, NaN) take the FP64 FMA
-// directly.  Terms below 2^-10 units are dropped (at most 1/4 unit per run).
+// same weight each band adds I in 64-bit fixed point, unit 2^(E - 50) for the
+// cell's I0 of exponent E, so a value up to 16 I0 adds at most 2^55 and a run of
+// 256 cannot overflow; the run then enters G with one FP64 FMA (sum x w x unit).
+// The additions are exact, the terms are cut to whole units: a value of I0's exponent
+// loses two bits (3/4 unit at most, 2.2e-16 of it on average, always downwards), any other
+// below 16 I0 less than one unit.  Values with a larger exponent (or negative, NaN)
+// take the FP64 FMA directly.
 // 64x48 x 400 x 55 with tau(T): 1745 -> 601 us; 120x120 x 20 x 55 explicit: 203 -> 107.
 template <int BM, bool TT>
 struct F64 {
