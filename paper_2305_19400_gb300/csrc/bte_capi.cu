@@ -89,9 +89,11 @@ struct bte_ctx {
   int cur = 0;
   // FP64 handles whose Jacobi steps run in double-float arithmetic keep the
   // current intensity buffer as ff pairs between such steps; steps of another
-  // arithmetic convert it (ensure_state_doubles), an initial or restored state is
-  // kept as doubles until a double-float step (ensure_state_ff)
-  bool state_ff = false;
+  // arithmetic convert it (ensure_state_doubles), a restored state is kept as doubles
+  // until a double-float step (ensure_state_ff).  An initial state (initial: no geometry has
+  // been stepped or restored since bte_set_initial) is I0cell in every direction and
+  // written again from there, in either form: no rounding of one shows in the other
+  bool state_ff = false, initial = false;
   double *I0cell = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr, *I0wall = nullptr;
   void* coef = nullptr;
   // FP64: tables of the factored double-float sweep (bte_rows.cuh)
@@ -722,19 +724,33 @@ bool ff_sweep(const bte_ctx* h) {
 
 // The current intensity buffer in the form the next step or call takes (in place):
 // doubles, or ff pairs for the double-float sweep.
+cudaError_t refill(bte_ctx* h, bool ff) {
+  cudaError_t e = cudaSuccess;
+  for (size_t gi = 0; gi < h->geoms.size() && e == cudaSuccess; ++gi) {
+    if (!h->init_set[gi]) continue;
+    const bte_geom& g = h->geoms[gi];
+    e = launch_refill(ff, h->Ibuf[h->cur] + (size_t)h->cell0[gi] * h->nd * h->nbp * 8, h->I0cell + h->cell0[gi] * h->nbp,
+                      (long long)g.nx * g.ny * g.nz, h->nd, h->nbp, h->stream);
+  }
+  return e;
+}
 cudaError_t ensure_state_doubles(bte_ctx* h) {
   if (!h->state_ff) return cudaSuccess;
-  const cudaError_t e = launch_ff_to_doubles(h->Ibuf[h->cur], (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
+  const cudaError_t e = h->initial ? refill(h, false)
+                                   : launch_ff_to_doubles(h->Ibuf[h->cur], (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
   if (e == cudaSuccess) h->state_ff = false;
   return e;
 }
 cudaError_t ensure_state_ff(bte_ctx* h) {
   if (h->state_ff) return cudaSuccess;
-  const cudaError_t e =
-      launch_doubles_to_ff(h->Ibuf[h->cur], h->Ibuf[h->cur], (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
+  const cudaError_t e = h->initial ? refill(h, true)
+                                   : launch_doubles_to_ff(h->Ibuf[h->cur], h->Ibuf[h->cur],
+                                                          (long long)h->ncells * h->nd * h->nbp / 2, h->stream);
   if (e == cudaSuccess) h->state_ff = true;
   return e;
 }
+// Reading calls return an initial state in full precision.
+cudaError_t ensure_initial_doubles(bte_ctx* h) { return h->initial ? ensure_state_doubles(h) : cudaSuccess; }
 
 // The ghosts of the diffuse and partially specular sides from the current state,
 // before wall fluxes read them.  Their kernels read doubles, so a state that stands
@@ -743,6 +759,7 @@ cudaError_t ensure_state_ff(bte_ctx* h) {
 cudaError_t refresh_ghosts(bte_ctx* h) {
   cudaError_t e = cudaSuccess;
   if (h->state_ff && !ff_sweep(h)) e = ensure_state_doubles(h);
+  else e = ensure_initial_doubles(h);
   if (e == cudaSuccess) e = refresh_diffuse(h, h->Ibuf[h->cur], h->stream);
   if (e == cudaSuccess) e = refresh_partial(h, h->Ibuf[h->cur], h->stream);
   return e;
@@ -1145,11 +1162,18 @@ int bte_set_initial(bte_handle h, int geom, const double* T_cells, double T_unif
   for (double t : T)
     if (!(t >= kTmin && t <= kTmax)) return fail(h, BTE_E_ARG, "initial temperature %g outside [1, 5000] K", t);
   if ((rc = ensure_memory(h))) return rc;
-  // an initial state is kept in doubles until a double-float step, whatever form the
-  // other geometries' state has by now
-  CUDA_TRY(h, ensure_state_doubles(h));
+  // the first geometry set, or a lone one set again, starts in the form of the handle's
+  // default sweep (as far as its walls are known); beside geometries that have been
+  // stepped or restored an initial state is written in doubles
+  bool others = false;
+  for (size_t gi = 0; gi < h->geoms.size(); ++gi) others |= (int)gi != geom && h->init_set[gi];
+  if (!others) {
+    h->initial = true;
+    h->state_ff = ff_sweep(h);
+  }
+  if (!h->initial) CUDA_TRY(h, ensure_state_doubles(h));
   CUDA_TRY(h, cudaMemcpyAsync(h->scratch_T, T.data(), nc * 8, cudaMemcpyHostToDevice, h->stream));
-  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->MsumL, h->Tp, h->Teval, h->TL, h->EL,
+  CUDA_TRY(h, launch_init_cells(h->opts.precision, h->state_ff, h->Ibuf[h->cur], h->I0cell, h->J, h->Msum, h->MsumL, h->Tp, h->Teval, h->TL, h->EL,
                                 h->scratch_T, h->I0ref_o, h->cell0[geom], (int)nc, h->nd, thermo(h), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
   h->init_set[geom] = true;
@@ -1186,7 +1210,10 @@ int bte_step(bte_handle h, double dt, int nsteps, int ninner, int scheme, bte_st
   if (ranged && !h->exchange) return fail(h, BTE_E_STATE, "a band-range handle needs bte_set_exchange before stepping");
   h->exchange_rc = 0;
   const bool ff_step = h->opts.precision == BTE_FP64 && scheme == BTE_IMPLICIT_JACOBI && ff_sweep(h);
-  if (nsteps > 0) CUDA_TRY(h, ff_step ? ensure_state_ff(h) : ensure_state_doubles(h));
+  if (nsteps > 0) {
+    CUDA_TRY(h, ff_step ? ensure_state_ff(h) : ensure_state_doubles(h));
+    h->initial = false;
+  }
   if (h->opts.beta_T_exp != 0.0 && !h->bscale_valid && nsteps > 0) {  // later changes of T_p come from cells_kernel
     CUDA_TRY(h, launch_beta_scale(h->bscale, h->Tp, h->opts.T_ref, h->opts.beta_T_exp, h->ncells, s));
     h->bscale_valid = true;
@@ -1479,6 +1506,7 @@ int bte_get_flux(bte_handle h, int geom, double* q_cells, double* q_walls, int o
   if (!h->mem_ready || !h->init_set[geom]) return fail(h, BTE_E_STATE, "geometry %d has no state", geom);
   const bte_geom& g = h->geoms[geom];
   const int nc = g.nx * g.ny * g.nz;
+  CUDA_TRY(h, ensure_initial_doubles(h));
   const void* I = h->Ibuf[h->cur];
   const int prec = h->opts.precision;
   cudaStream_t s = h->stream;
@@ -1512,6 +1540,7 @@ int bte_get_intensity(bte_handle h, int geom, double* out, int on_device) {
   const long long nc = (long long)g.nx * g.ny * g.nz;
   const int prec = h->opts.precision;
   const size_t es = elem_bytes(prec);
+  CUDA_TRY(h, ensure_initial_doubles(h));
   const char* I = h->Ibuf[h->cur] + (size_t)h->cell0[geom] * h->nd * h->nbp * es;
   for (long long c0 = 0; c0 < nc; c0 += on_device ? nc : h->pack_cells) {
     const long long n = on_device ? nc : std::min(h->pack_cells, nc - c0);
@@ -1542,6 +1571,7 @@ int bte_set_intensity(bte_handle h, int geom, const double* in, const double* Tp
   // geometry's is overwritten whole, and has no state when a call below fails half-way
   if (h->geoms.size() > 1) CUDA_TRY(h, ensure_state_doubles(h));
   else if (h->state_ff) h->init_set[geom] = h->state_ff = false;
+  h->initial = false;
   CUDA_TRY(h, launch_state_from_Tp(h->I0cell + h->cell0[geom] * h->nbp, h->J + h->cell0[geom] * 4 * h->nbp_all,
                                    h->Msum + h->cell0[geom] * 4, h->MsumL + h->cell0[geom] * 4,
                                    h->Tp + h->cell0[geom], h->Teval + h->cell0[geom], nc, thermo(h), s));

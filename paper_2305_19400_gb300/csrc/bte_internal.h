@@ -224,9 +224,11 @@ cudaError_t mlp_forward_backward(const float* p, int k, const float* X, int ldx,
 cudaError_t launch_adam(float* p, const float* g, float* m, float* v, int n, float lr, int step, cudaStream_t s);
 cudaError_t launch_solve_batch(ThermoTables th, const double* Ep, const double* T0, int n, double trust_rel, int maxit,
                                const MLPView* mlp, double* Tout, int* evals, cudaStream_t s);
-cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp, double* Te,
+// ff: FP64 intensities as ff pairs
+cudaError_t launch_init_cells(int precision, bool ff, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp, double* Te,
                               double* TL, double* EL, const double* Tcells, const double* I0ref, long long cell0,
                               int ncells, int nd, ThermoTables th, cudaStream_t s);
+cudaError_t launch_refill(bool ff, void* I, const double* I0cell, long long ncells, int nd, int nbo, cudaStream_t s);
 cudaError_t launch_state_from_Tp(double* I0cell, double* J, double* Msum, double* MsumL, const double* Tp, double* Te, long long ncells,
                                  ThermoTables th, cudaStream_t s);
 cudaError_t launch_wall_I0(double* I0wall, const double* Tfaces, long long nfaces, ThermoTables th, cudaStream_t s);

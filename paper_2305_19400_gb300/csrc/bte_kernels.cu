@@ -56,6 +56,23 @@ __device__ void cell_state_at(double* I0cell, double* J, double* Msum, double* M
   }
 }
 
+// One row of stored bands (less ref in the reduced modes) into every direction of a cell: a
+// thread keeps one pair of bands and walks the rows (16-byte stores in FP64).
+template <typename S>
+__device__ __forceinline__ void fill_cell(S* cell, const double* row, const double* ref, int nd, int nbo, int nbr) {
+  const int pairs = nbo / 2, groups = (int)blockDim.x / pairs;
+  const int grp = groups ? threadIdx.x / pairs : 0;
+  for (int p = threadIdx.x - grp * pairs; grp < max(groups, 1) && p < pairs; p += groups ? pairs : blockDim.x) {
+    double v[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int b = 2 * p + k;
+      v[k] = b < nbr ? (sizeof(S) == 8 ? row[b] : row[b] - ref[b]) : 0.0;
+    }
+    for (int r = grp; r < nd; r += max(groups, 1)) st_pair(cell + (long long)r * nbo + 2 * p, v[0], v[1]);
+  }
+}
+
 // Equilibrium initial state: I = I0_b(T_P) for every direction (stored as the
 // deviation I0_b(T_P) - I0_b(T_ref) in the reduced modes).
 template <typename S>
@@ -68,19 +85,7 @@ __global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum,
     const double T = Tcells[c];
     cell_state_at(I0cell, J, Msum, MsumL, P, T, th, row);
     __syncthreads();
-    // a thread keeps one pair of stored bands and walks the rows (16-byte stores in FP64)
-    const int pairs = th.nbo / 2, groups = (int)blockDim.x / pairs;
-    const int grp = groups ? threadIdx.x / pairs : 0;
-    S* cell = I + P * (long long)nd * th.nbo;
-    for (int p = threadIdx.x - grp * pairs; grp < max(groups, 1) && p < pairs; p += groups ? pairs : blockDim.x) {
-      double v[2];
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int b = 2 * p + k;  // stored band; I0ref holds the stored bands
-        v[k] = b < th.nbr ? (sizeof(S) == 8 ? row[th.band0 + b] : row[th.band0 + b] - I0ref[b]) : 0.0;
-      }
-      for (int r = grp; r < nd; r += max(groups, 1)) st_pair(cell + (long long)r * th.nbo + 2 * p, v[0], v[1]);
-    }
+    fill_cell(I + P * (long long)nd * th.nbo, row + th.band0, I0ref, nd, th.nbo, th.nbr);  // I0ref: the stored bands
     if (threadIdx.x == 0) {
       double e = 0.0;
       for (int b = 0; b < th.nbp; ++b) e = fma(th.a_L[b], row[b], e);
@@ -91,6 +96,13 @@ __global__ void init_cells_kernel(S* I, double* I0cell, double* J, double* Msum,
     }
     __syncthreads();
   }
+}
+
+// The intensities of an FP64 initial state again, from I0cell, in another form.
+template <typename S>
+__global__ void __launch_bounds__(256) refill_kernel(S* I, const double* I0cell, long long ncells, int nd, int nbo) {
+  for (long long P = blockIdx.x; P < ncells; P += gridDim.x)
+    fill_cell(I + P * (long long)nd * nbo, I0cell + P * nbo, nullptr, nd, nbo, nbo);
 }
 
 // Thermodynamic state from T_p after a state restore: I0cell, J, T_e.
@@ -724,7 +736,13 @@ cudaError_t launch_gs_reduce(int precision, const SweepArgs& a, long long ncells
   return cudaGetLastError();
 }
 
-cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp,
+cudaError_t launch_refill(bool ff, void* I, const double* I0cell, long long ncells, int nd, int nbo, cudaStream_t s) {
+  if (ff) refill_kernel<FFElem><<<cell_grid(ncells), 256, 0, s>>>((FFElem*)I, I0cell, ncells, nd, nbo);
+  else refill_kernel<double><<<cell_grid(ncells), 256, 0, s>>>((double*)I, I0cell, ncells, nd, nbo);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_init_cells(int precision, bool ff, void* I, double* I0cell, double* J, double* Msum, double* MsumL, double* Tp,
                               double* Te, double* TL, double* EL, const double* Tcells, const double* I0ref,
                               long long cell0, int ncells, int nd, ThermoTables th, cudaStream_t s) {
   auto go = [&](auto tag) {
@@ -732,7 +750,8 @@ cudaError_t launch_init_cells(int precision, void* I, double* I0cell, double* J,
     init_cells_kernel<T><<<cell_grid(ncells), 256, th.nbp * sizeof(double), s>>>((T*)I, I0cell, J, Msum, MsumL, Tp, Te, TL, EL, Tcells,
                                                                                  I0ref, cell0, ncells, nd, th);
   };
-  if (precision == 0) go(double{});
+  if (precision == 0 && ff) go(FFElem{});
+  else if (precision == 0) go(double{});
   else if (precision == 1) go(float{});
   else go(__nv_bfloat16{});
   return cudaGetLastError();

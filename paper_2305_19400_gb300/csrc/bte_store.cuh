@@ -154,6 +154,11 @@ __device__ __forceinline__ void st_pair(S* p, double a, double b) {
     *reinterpret_cast<__nv_bfloat162*>(p) = v;
   }
 }
+template <>
+__device__ __forceinline__ void st_pair<FFElem>(FFElem* p, double a, double b) {
+  const ff::P2 v = ff::from_doubles(a, b);
+  *reinterpret_cast<ulonglong2*>(p) = make_ulonglong2(v.h, v.l);
+}
 // The values that st_pair keeps of a and b.
 template <typename S>
 __device__ __forceinline__ void stored_pair(double a, double b, double& x, double& y) {

@@ -1009,7 +1009,7 @@ int bte_umesh_set_initial(bte_umesh u, const double* T_cells, double T_uniform) 
   int rc = upload(u, u->scratch, T.data(), u->nc);
   if (rc) return rc;
   u->cur = 0;
-  UTRY(u, launch_init_cells(u->prec, u->I[0], u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
+  UTRY(u, launch_init_cells(u->prec, false, u->I[0], u->I0cell, u->J, u->Msum, u->MsumL, u->Tp, u->Teval, u->TL, u->EL, u->scratch, u->I0ref, 0,
                             (int)u->nc, u->nd, uthermo(u), u->stream));
   UTRY(u, cudaStreamSynchronize(u->stream));
   u->init_done = true;

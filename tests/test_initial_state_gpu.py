@@ -50,3 +50,41 @@ def test_tuning_leaves_the_state(scheme):
     bte.bte_autotune(s.h, 1e-13, scheme)
     assert np.array_equal(s.intensity(0), I)
     s.close()
+
+
+def test_beside_a_restored_geometry():
+    """A restore of one geometry leaves the other's initial state in full precision."""
+    wl = workload(2)
+    s, ref = bte.Solver(wl), bte.Solver(wl, fp64_strict=True)
+    I0, I1 = ref.intensity(0), ref.intensity(1)
+    bte.bte_set_intensity(s.h, 0, I0 * 1.01, np.full(30, 301.0))
+    assert np.array_equal(s.intensity(1), I1)
+    assert np.array_equal(s.intensity(0), I0 * 1.01)
+    s.close()
+    ref.close()
+
+
+@pytest.mark.parametrize("scheme", [bte.BTE_EXPLICIT, bte.BTE_IMPLICIT_GS])
+def test_an_ieee_step_starts_from_doubles(scheme):
+    """Bit for bit the step of a handle whose state was read, and so written in doubles, before."""
+    a, b = bte.Solver(workload()), bte.Solver(workload())
+    b.intensity(0)
+    for s in (a, b):
+        s.step(dt=1e-13, scheme=scheme)
+    assert np.array_equal(a.intensity(0), b.intensity(0))
+    a.close()
+    b.close()
+
+
+def test_a_lone_geometry_set_again():
+    wl = workload()
+    a, b = bte.Solver(wl), bte.Solver(wl)
+    a.step()
+    bte.bte_set_initial(a.h, 0, np.full(30, 310.0))
+    bte.bte_set_initial(b.h, 0, np.full(30, 310.0))
+    b.intensity(0)  # b from doubles: the double-float step converts them
+    for s in (a, b):
+        s.step()
+    assert np.array_equal(a.intensity(0), b.intensity(0))
+    a.close()
+    b.close()
