@@ -791,7 +791,10 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
   const bool use_b = h->opts.precision == BTE_FP64 && !use_ff && !a.explicit_scheme && ninner >= 2;
   a.ff = use_ff ? 1 : 0;
   if (scheme == BTE_IMPLICIT_GS) a.ne = kRedEntries;
-  const long long before = scheme == BTE_IMPLICIT_GS ? h->ncells : a.nitems;  // CTAs of gs_reduce_kernel or the sweep
+  // threads behind which cells_kernel may start: those of the row sweep (gs_reduce_kernel
+  // and the BF16 sweep let nothing start before their end)
+  const long long before =
+      scheme == BTE_IMPLICIT_GS || h->opts.precision == BTE_BF16 ? 0 : (long long)a.nitems * h->threads;
   int z = -1;
   for (int it = 0; it < ninner; ++it) {
     int o = 0;
@@ -840,7 +843,7 @@ cudaError_t enqueue_step(bte_ctx* h, SweepArgs a, int ninner, int scheme, cudaSt
     }
     if (e == cudaSuccess) {
       const MLPView m = mlp_view(h);
-      e = launch_cells(a, h->ncells, a.partial ? 2 : 0, h->opts.learned ? &m : nullptr, a.partial ? h->ncells : before, s);
+      e = launch_cells(a, h->ncells, a.partial ? 2 : 0, h->opts.learned ? &m : nullptr, a.partial ? 256 * h->ncells : before, s);
     }
     if (e != cudaSuccess) return e;
     k = o;

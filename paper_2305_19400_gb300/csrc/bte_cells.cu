@@ -266,12 +266,13 @@ cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const M
                                     (mlp ? (2 * (size_t)a.th.nbp + 4 * kHidden) * sizeof(float) : 0);
   MLPView m{};
   if (mlp) m = *mlp;
-  // Launched early behind a sweep of at most one CTA per SM: the launch and the prologue
-  // are then hidden (11 sweeps of 400 cells x 16 x 4 in 60 CTAs 221 -> 199 us a step; 992
-  // cells x 20 x 55 in 124 CTAs 227 -> 224).  Behind more of them the early CTAs crowd into the
-  // slots that are left on some SMs (992 cells x 400 x 55 in 248 CTAs 1133 -> 1142 us,
-  // 3015 cells 2 % and 14400 cells 2.5 % slower).
-  const bool early = before <= 152;
+  // Launched early behind a sweep of at most eight warps per SM: the launch and the
+  // prologue are then hidden (ten inner iterations of 400 cells x 16 x 4, 60 CTAs of a warp, 221
+  // -> 199 us; of 992 cells x 20 x 55, 124 CTAs of seven warps, 227 -> 224; six of 960 cells x
+  // 120 x 27 in FP32, 480 CTAs of a warp, 235 -> 224).  Behind more of them the early CTAs crowd
+  // into the slots that are left on some SMs (992 cells x 400 x 55, 248 CTAs of seven
+  // warps, 1133 -> 1142 us, 3015 cells 2 % and 14400 cells 2.5 % slower).
+  const bool early = before <= 152 * 256;
   return launch_pdl(early, mlp ? cells_kernel<true> : cells_kernel<false>, cells_grid(ncells), kCellThreads, sm, s, a, ncells,
                     mode, m);
 }

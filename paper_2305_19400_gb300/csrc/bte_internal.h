@@ -193,7 +193,7 @@ cudaError_t launch_sweep_bf16(int pd, const SweepArgs& a, int dim, int threads, 
 struct MLPView;
 // per-cell step (bte_cells.cu): mode 0 energies from Ec and T_p, 1 energies from
 // Ec to Epart, 2 T_p from Epart, 3 T_L from E_L
-// before: CTAs of the kernel that runs before it, 0 where that lets nothing start before its end
+// before: threads of the kernel that runs before it, 0 where that one lets nothing start before its end
 cudaError_t launch_cells(const SweepArgs& a, long long ncells, int mode, const MLPView* mlp, long long before,
                          cudaStream_t s);
 int cells_grid(long long ncells);

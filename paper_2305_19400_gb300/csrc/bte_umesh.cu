@@ -1113,7 +1113,7 @@ int bte_umesh_step(bte_umesh u, double dt, int nsteps, int ninner, int scheme, b
       }
       SweepArgs c = cell_args(u, a.Iout);
       UTRY(u, launch_gs_reduce(u->prec, c, u->nc, s));
-      UTRY(u, launch_cells(c, u->nc, 0, nullptr, u->nc, s));
+      UTRY(u, launch_cells(c, u->nc, 0, nullptr, 0, s));
       launches += 3 + (u->ndiff ? 1 : 0) + (tt ? 1 : 0);
       k = o;
     }
