@@ -58,12 +58,12 @@ KERNEL_SRCS = [os.path.join(ROOT, "paper_2305_19400_gb300", "csrc", f) for f in 
 # Algorithmic bytes of one implicit update: I^n read, I^k read once, I^{k+1} written.
 BYTES_PER_UPDATE_FP64 = 24
 # Work of the dominant kernel (the double-float sweep, 2-D): per lane step of two
-# bands, 5 products of 4 packed ops (R I^n, that over v dt, c_x u_x, c_y u_y, and R
-# times the sum), 3 pair sums of 8 (the products and the source term), a normalisation
-# of 3 and the direction sum's accumulation of 8 = 55 packed f32x2 instructions for 2
-# updates, i.e. 55 FP32 lane operations per update; counted against the measured
+# bands, 4 products of 4 packed ops (W I^n, c_x u_x, c_y u_y, and R times the
+# sum), 3 pair sums of 8 (the products and the source term), a normalisation of 3
+# and the direction sum's accumulation of 8 = 51 packed f32x2 instructions for 2
+# updates, i.e. 51 FP32 lane operations per update; counted against the measured
 # packed-FMA rate in lane operations.
-FP32_LANE_OPS_PER_UPDATE_FF_2D = 55
+FP32_LANE_OPS_PER_UPDATE_FF_2D = 51
 # The strict IEEE-FP64 sweep: 3 FMAs per update (B + A_x I_x + A_y I_y + A_s I0)
 # in inner iterations 2..n, 4 in the first (A_n I^n).
 FP64_FMAS_PER_UPDATE_2D = 3

@@ -97,9 +97,9 @@ struct bte_ctx {
   double *I0cell = nullptr, *Tp = nullptr, *TL = nullptr, *EL = nullptr, *I0wall = nullptr;
   void* coef = nullptr;
   // FP64: tables of the factored double-float sweep (bte_rows.cuh)
-  void* coef_R = nullptr;     // [cls][nd][nbp] R pairs
+  void* coef_R = nullptr;     // [cls][nd][nbp] R and W pairs
   float* dirc_ff = nullptr;   // [cls][nd][3][2]
-  float* band_ff = nullptr;   // [2][nbp] 1/(v_b dt), beta_b/v_b pairs
+  float* band_ff = nullptr;   // [nbp] beta_b/v_b pairs
   double *J = nullptr, *Teval = nullptr, *I0ref = nullptr, *scratch_pack = nullptr;
   double* Msum = nullptr;     // [cell][4] the T_p model's sums sum_b a_p,b J_k,b
   double* MsumL = nullptr;    // [cell][4] the same with the T_L weights
@@ -236,9 +236,9 @@ size_t carve(bte_ctx* h, char* base) {
   h->EL = (double*)take((size_t)h->ncells * 8);
   h->I0wall = (double*)take((size_t)std::max(h->nfaces, 1LL) * h->nbp * 8);
   h->coef = take((size_t)h->cls_key.size() * row * (h->opts.precision == BTE_FP64 ? 5 * 8 : 2 * 4));
-  h->coef_R = h->opts.precision == BTE_FP64 ? take((size_t)h->cls_key.size() * row * 8) : nullptr;
+  h->coef_R = h->opts.precision == BTE_FP64 ? take((size_t)h->cls_key.size() * row * 16) : nullptr;
   h->dirc_ff = h->opts.precision == BTE_FP64 ? (float*)take((size_t)h->cls_key.size() * h->nd * 6 * 4) : nullptr;
-  h->band_ff = h->opts.precision == BTE_FP64 ? (float*)take((size_t)h->nbp * 4 * 4) : nullptr;
+  h->band_ff = h->opts.precision == BTE_FP64 ? (float*)take((size_t)h->nbp * 2 * 4) : nullptr;
   h->dirc = (float4*)take((size_t)h->cls_key.size() * h->nd * sizeof(float4));
   h->vb32 = (float*)take((size_t)h->nbp * 4);
   h->bb32 = (float*)take((size_t)h->nbp * 4);
@@ -541,14 +541,14 @@ int ensure_coef(bte_ctx* h, double dt, int scheme) {
     }
     CUDA_TRY(h, cudaMemcpyAsync(h->coef, h->coef_host.data(), h->coef_host.size() * 8, cudaMemcpyHostToDevice, h->stream));
     // the factored double-float tables (implicit update only)
-    h->R_host.assign(2 * plane * ncls, 0.0f);
+    h->R_host.assign(4 * plane * ncls, 0.0f);
     h->dirc_host.assign(6 * (size_t)h->nd * ncls, 0.0f);
-    h->band_host.assign(4 * (size_t)h->nbp, 0.0f);
+    h->band_host.assign(2 * (size_t)h->nbp, 0.0f);
     if (scheme != BTE_EXPLICIT)
       for (size_t c = 0; c < ncls; ++c) {
         const double delta[3] = {std::get<1>(h->cls_key[c]), std::get<2>(h->cls_key[c]), std::get<3>(h->cls_key[c])};
-        build_ff_factored(std::get<0>(h->cls_key[c]), delta, h->nd, h->S.data(), h->w.data(), h->nb, h->nbp,
-                          h->vg.data() + h->band0, h->beta.data() + h->band0, dt, h->R_host.data() + c * 2 * plane,
+        build_ff_factored(std::get<0>(h->cls_key[c]), delta, h->nd, h->dir_group, h->S.data(), h->w.data(), h->nb, h->nbp,
+                          h->vg.data() + h->band0, h->beta.data() + h->band0, dt, h->R_host.data() + c * 4 * plane,
                           h->dirc_host.data() + c * 6 * (size_t)h->nd, h->band_host.data());
       }
     CUDA_TRY(h, cudaMemcpyAsync(h->coef_R, h->R_host.data(), h->R_host.size() * 4, cudaMemcpyHostToDevice, h->stream));

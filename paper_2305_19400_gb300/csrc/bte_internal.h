@@ -134,8 +134,8 @@ struct SweepArgs {
   int ff;                   // FP64: 1 double-float arithmetic (every intensity buffer holds ff pairs), 0 IEEE
   // tables of the double-float sweep in the pair layout of bte_ff.cuh
   // (h_b, h_b+1, l_b, l_b+1 per two bands):
-  const void* coef_R;       // [cls][nd][nbp] R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax,d)
-  const float* band_ff;     // [2][nbp] 1/(v_b dt), beta_b/v_b of the stored bands (0 on padding)
+  const void* coef_R;       // [cls][nd][nbp] R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax,d), then W = R/(v_b dt), per two bands
+  const float* band_ff;     // [nbp] beta_b/v_b of the stored bands (0 on padding)
   const float* dirc_ff;     // [cls][nd][3][2] c_ax,d as (h, l)
   const void* coef;         // FP64: [cls][5][nd][nbp] A_n, A_x, A_y, A_z, A_s;
                             // reduced: [cls][2][nd][nbp] float P, Q with

@@ -76,17 +76,19 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 // ------------------------------------------------------------------- modes
 // FP64 storage in double-float arithmetic (bte_ff.cuh), implicit: divided
 // through by v_b,
-//   I' = B + R (sum_ax c_ax u_ax + (beta_b/v_b) I0),  B = (1/(v_b dt)) R I^n,
-//   R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax),
-// 1/(v_b dt), beta_b/v_b and (beta_b/v_b) I0 in registers, c_ax of the block from
-// shared memory, R of the block from its table one block ahead.  Forming B in every
-// iteration costs eight packed operations more than reading a stored one, and saves
-// the first iteration's write of B and its third buffer's traffic.  R I^n comes first:
-// I^n/(v_b dt) would save four of them, but rounds alike in all directions of a cell
-// near equilibrium (1.5e-15 of a uniform state's band where this leaves 0.7e-15; 120x120 x 20
-// x 55, ten steps, 1100 us against 1109).  The tables come from the host in double-float
-// form with R chosen so that R (1/(v_b dt) + beta_b/v_b + sum c_ax) = 1 holds for the
-// table values to double-double accuracy, which keeps a uniform equilibrium in place.
+//   I' = W I^n + R (sum_ax c_ax u_ax + (beta_b/v_b) I0),
+//   R = 1/(1/(v_b dt) + beta_b/v_b + sum_ax c_ax),  W = R/(v_b dt),
+// beta_b/v_b and (beta_b/v_b) I0 in registers, c_ax of the block from shared memory, R
+// and W of the block from their table one block ahead.  Forming W I^n in every iteration
+// costs four packed operations more than reading a stored B, and saves the first
+// iteration's write of B and its third buffer's traffic.  The tables come from the host
+// in double-float form: R the pair nearest its value, and W = 1 - R (beta_b/v_b + sum c_ax)
+// of that pair, formed in double-double, so that W + R (beta_b/v_b + sum c_ax) = 1 holds to
+// 2^-49 W and a uniform equilibrium stays in place: after 4000 iterations at dt = 0.2
+// ps 1e-14 rms from it, where R I^n/(v_b dt) from two products drifted by 1.2e-13 and W
+// formed on the device by 1.1e-12.  I^n/(v_b dt), added to the upwind sum before one
+// product with R, rounds alike in all directions of a cell near equilibrium (1.5e-15 of a
+// uniform state's band in one update, here 0.4e-15).
 // The direction sum adds a block's rows first, then the block to its run of equal
 // weights, then the run times its weight to G: the rows of a block are close to equal, and
 // adding equal pairs twenty in a row without renormalising leaves 1.5e-14 rms where blocks
@@ -94,7 +96,7 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 // Bound by HBM (24 bytes an update) and L2 to SM traffic; of few directions by
 // issue (0.51 of the slots at 16 warps per SM).  With coefficients read per
 // direction and the cells' step in the same kernel: 128x128 x 400 x 55 1535 us an
-// iteration, 23x18x13 867, 120x120 x 20 x 55 124; now 1440, 530 and 70, and 43, 30
+// iteration, 23x18x13 867, 120x120 x 20 x 55 124; now 1410, 520 and 69, and 43, 30
 // and 30 for the cells.
 struct FF {
   using S = double;
@@ -110,11 +112,11 @@ struct FF {
     unsigned pad;
   };
   struct Lane {
-    ff::P2 rdtv, betav;
+    ff::P2 betav;
   };
   template <int DIM>
   struct Coef {
-    ff::P2 R;
+    ff::P2 R, W;
   };
   struct Cell {
     ff::P2 src;
@@ -139,11 +141,12 @@ struct FF {
     return e;
   }
   __device__ static Lane lane(const SweepArgs& a, int b0) {
-    return Lane{ff::ldg(a.band_ff + 2 * b0), ff::ldg(a.band_ff + 2 * (a.th.nbo + b0))};
+    return Lane{ff::ldg(a.band_ff + 2 * b0)};
   }
   template <int DIM>
   __device__ static Coef<DIM> coef(const SweepArgs& a, int cls, int d, int b0) {
-    return Coef<DIM>{ff::ldg(reinterpret_cast<const double*>(a.coef_R) + ((size_t)cls * a.nd + d) * a.th.nbo + b0)};
+    const double* p = reinterpret_cast<const double*>(a.coef_R) + 2 * (((size_t)cls * a.nd + d) * a.th.nbo + b0);
+    return Coef<DIM>{ff::ldg(p), ff::ldg(p + 2)};
   }
   __device__ static Cell cell(const SweepArgs&, const Lane& l, const double (&i0)[V], int, long long) {
     return Cell{ff::norm(ff::mul(l.betav, ff::from_doubles(i0[0], i0[1])))};
@@ -151,7 +154,7 @@ struct FF {
   __device__ static Acc acc(const SweepArgs&, const Cell&) { return Acc{ff::zero(), ff::zero(), ff::zero(), ff::zero(), 0xffffffffu}; }
   template <int DIM>
   struct Block {
-    ff::P2 c[DIM], R;
+    ff::P2 c[DIM], R, W;
   };
   template <int DIM, int RUN>
   __device__ static Block<DIM> block(const SweepArgs&, const Lane&, const Cell&, const Coef<DIM>& cf, const Tab<DIM>& t,
@@ -165,18 +168,18 @@ struct FF {
     }
     Block<DIM> b;
     b.R = cf.R;
+    b.W = cf.W;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) b.c[k] = ff::P2{t.ch[k], t.cl[k]};
     return b;
   }
   template <int DIM, bool FIRST>
-  __device__ static void step(const SweepArgs&, const Lane& l, const Cell& c, const Block<DIM>& b, unsigned sb, unsigned ostr,
+  __device__ static void step(const SweepArgs&, const Lane&, const Cell& c, const Block<DIM>& b, unsigned sb, unsigned ostr,
                               char* out, char*, bool on, Acc& s) {
     ff::P2 t = ff::mul(b.c[0], ff::lds(sb + ostr));
 #pragma unroll
     for (int k = 1; k < DIM; ++k) t = ff::add(t, ff::mul(b.c[k], ff::lds(sb + (1 + k) * ostr)));
-    const ff::P2 B = ff::mul(l.rdtv, ff::mul(b.R, ff::lds(sb)));
-    const ff::P2 r = ff::norm(ff::add(B, ff::mul(b.R, ff::add(t, c.src))));
+    const ff::P2 r = ff::norm(ff::add(ff::mul(b.W, ff::lds(sb)), ff::mul(b.R, ff::add(t, c.src))));
     if (on) ff::st_stream(out, r);
     if (FIRST) s.B = r;
     else ff::acc(s.B, r);

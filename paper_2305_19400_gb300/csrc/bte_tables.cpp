@@ -242,24 +242,22 @@ void ff_of_dd(DD x, float& h, float& l) {
 }
 }  // namespace
 
-void build_ff_factored(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
-                       const double* vg, const double* beta, double dt, float* R, float* dirc, float* band) {
-  for (size_t e = 0; e < 4 * (size_t)nbp; ++e) band[e] = 0.0f;
+void build_ff_factored(int dim, const double delta[3], int nd, int group, const double* S, const double* w, int nb, int nbp,
+                       const double* vg, const double* beta, double dt, float* RW, float* dirc, float* band) {
+  for (size_t e = 0; e < 2 * (size_t)nbp; ++e) band[e] = 0.0f;
   std::vector<DD> rv_dd(nb), bv_dd(nb);
   for (int b = 0; b < nb; ++b) {  // pair layout: element b of an [nbp] array at float (b - b%2)*2 + b%2 (+2 for l)
     float h, l;
     const size_t o = (size_t)(b - (b & 1)) * 2 + (b & 1);
     ff_of(1.0 / (vg[b] * dt), h, l);  // 1 / (v_b dt)
-    band[o] = h;
-    band[o + 2] = l;
     rv_dd[b] = dd_of(h, l);
     ff_of(beta[b] / vg[b], h, l);  // beta_b / v_b
-    band[2 * (size_t)nbp + o] = h;
-    band[2 * (size_t)nbp + o + 2] = l;
+    band[o] = h;
+    band[o + 2] = l;
     bv_dd[b] = dd_of(h, l);
   }
-  for (size_t e = 0; e < 2 * (size_t)nd * nbp; ++e) R[e] = 0.0f;
-  for (int d = 0; d < nd; ++d) {
+  for (size_t e = 0; e < 4 * (size_t)nd * nbp; ++e) RW[e] = 0.0f;
+  for (int d = 0; d < nd; d += group) {
     DD csum{0.0, 0.0};
     for (int ax = 0; ax < 3; ++ax) {
       const double c = ax < dim ? std::fabs(S[3 * d + ax]) / (w[d] * delta[ax]) : 0.0;
@@ -270,12 +268,16 @@ void build_ff_factored(int dim, const double delta[3], int nd, const double* S, 
       csum = dd_add(csum, dd_of(h, l));
     }
     for (int b = 0; b < nb; ++b) {
-      const DD D = dd_add(dd_add(rv_dd[b], bv_dd[b]), csum);
+      const DD in = dd_add(bv_dd[b], csum);
       float h, l;
-      ff_of_dd(dd_recip(D), h, l);
-      const size_t o = ((size_t)d * nbp + b - (b & 1)) * 2 + (b & 1);
-      R[o] = h;
-      R[o + 2] = l;
+      ff_of_dd(dd_recip(dd_add(rv_dd[b], in)), h, l);
+      const size_t o = ((size_t)d * nbp + b - (b & 1)) * 4 + (b & 1);
+      RW[o] = h;
+      RW[o + 2] = l;
+      const DD p = dd_mul(dd_of(h, l), in);  // W = 1 - R (beta_b/v_b + sum c)
+      ff_of_dd(dd_add(DD{1.0, 0.0}, DD{-p.hi, -p.lo}), h, l);
+      RW[o + 4] = h;
+      RW[o + 6] = l;
     }
   }
 }

@@ -19,16 +19,18 @@ void build_coef(int dim, const double delta[3], int nd, const double* S, const d
 
 // Tables of the factored double-float sweep (bte_rows.cuh) for one class,
 // the implicit update divided through by v_b (v_b > 0 on every real band):
-// I' = B + R (sum_ax c_ax,d u_ax + (beta_b / v_b) I0),  B = (1 / (v_b dt)) R I^n,
-// R = 1 / (1 / (v_b dt) + beta_b / v_b + sum_ax c_ax,d).
+// I' = W I^n + R (sum_ax c_ax,d u_ax + (beta_b / v_b) I0),
+// R = 1 / (1 / (v_b dt) + beta_b / v_b + sum_ax c_ax,d),  W = R / (v_b dt).
 // dirc[nd][3][2] c_ax,d = |S_d,ax|/(w_d Delta_ax) as double-float pairs (h, l);
-// band[2][nbp] 1/(v_b dt) and beta_b/v_b and R[nd][nbp] in the pair layout of
-// bte_ff.cuh (per two bands h_b, h_b+1, l_b, l_b+1; padding bands 0).  R is the
-// double-float pair nearest the reciprocal of a denominator formed exactly
-// (double-double) from the stored pairs themselves, so that a uniform field is
-// a fixed point of the update to the pairs' resolution.
-void build_ff_factored(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
-                       const double* vg, const double* beta, double dt, float* R, float* dirc, float* band);
+// band[nbp] beta_b/v_b in the pair layout of bte_ff.cuh (per two bands h_b, h_b+1,
+// l_b, l_b+1; padding bands 0); RW[nd][nbp] the same, per two bands R's pairs, then W's.
+// R is the double-float pair nearest the reciprocal of a denominator formed exactly
+// (double-double) from the stored pairs themselves, W the pair nearest
+// 1 - R (beta_b / v_b + sum c) of the stored R, so that a uniform field is a fixed point
+// of the update to the pairs' resolution.  Only the first of each group of directions
+// (internal_order) is formed: its rows serve the group.
+void build_ff_factored(int dim, const double delta[3], int nd, int group, const double* S, const double* w, int nb, int nbp,
+                       const double* vg, const double* beta, double dt, float* RW, float* dirc, float* band);
 
 void build_pq(int dim, const double delta[3], int nd, const double* S, const double* w, int nb, int nbp,
               const double* vg, const double* beta, double dt, int explicit_scheme, float* P, float* Q, float* dirc);

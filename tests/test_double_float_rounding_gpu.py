@@ -45,3 +45,18 @@ def test_update_of_an_equilibrium():
         means.append(((s.intensity(0) - I) / I).mean(axis=1)[4])
         s.close()
     assert np.sqrt(np.mean(np.square(means))) <= 1.03e-15
+
+
+# 1000 steps of 4 iterations of the same: the coefficients add up to one closely enough for the
+# state to settle (1e-14 rms); with rounding errors of 2^-48 in their sum it drifts on (1.2e-13
+# and more).  Bar: 3.5e-14, half-way in the logarithm.
+def test_equilibrium_stays():
+    g = W.Geometry(2, 4, 4, 1, 10e-9, 10e-9, 10e-9)
+    W.uniform_walls(g, [W.BC_SPECULAR] * 4, [0.0] * 4)
+    wl = W.Workload("equilibrium", [g], W.Dirs("polar_azim", n_polar=20, n_azim=20),
+                    W.make_bands(40, 15, 85, log10_tau_range=(-6.0, -5.9)), 2e-13, 1, 1)
+    s = bte.Solver(wl, use_graph=True)
+    I0 = s.intensity(0)
+    s.step(nsteps=1000, ninner=4)
+    assert np.sqrt(np.mean(((s.intensity(0) - I0) / I0) ** 2)) <= 3.5e-14
+    s.close()
