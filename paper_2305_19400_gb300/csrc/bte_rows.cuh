@@ -83,8 +83,8 @@ __device__ __forceinline__ double2 ld2(const double* p) { return __ldg(reinterpr
 // costs four packed operations more than reading a stored B, and saves the first
 // iteration's write of B and its third buffer's traffic.  The tables come from the host
 // in double-float form: R the pair nearest its value, and W = 1 - R (beta_b/v_b + sum c_ax)
-// of that pair, formed in double-double, so that W + R (beta_b/v_b + sum c_ax) = 1 holds to
-// 2^-49 W and a uniform equilibrium stays in place: after 4000 iterations at dt = 0.2
+// of that pair, formed in double-double (below 1/4 the pair nearest R/(v_b dt)), so that W +
+// R (beta_b/v_b + sum c_ax) = 1 holds to 2^-49 W and a uniform equilibrium stays in place: after 4000 iterations at dt = 0.2
 // ps 1e-14 rms from it, where R I^n/(v_b dt) from two products drifted by 1.2e-13 and W
 // formed on the device by 1.1e-12.  I^n/(v_b dt), added to the upwind sum before one
 // product with R, rounds alike in all directions of a cell near equilibrium (1.5e-15 of a

@@ -274,8 +274,10 @@ void build_ff_factored(int dim, const double delta[3], int nd, int group, const 
       const size_t o = ((size_t)d * nbp + b - (b & 1)) * 4 + (b & 1);
       RW[o] = h;
       RW[o + 2] = l;
-      const DD p = dd_mul(dd_of(h, l), in);  // W = 1 - R (beta_b/v_b + sum c)
-      ff_of_dd(dd_add(DD{1.0, 0.0}, DD{-p.hi, -p.lo}), h, l);
+      const DD R = dd_of(h, l), p = dd_mul(R, in);
+      DD W = dd_mul(R, rv_dd[b]);
+      if (W.hi >= 0.25) W = dd_add(DD{1.0, 0.0}, DD{-p.hi, -p.lo});  // at most 2^-47 W away
+      ff_of_dd(W, h, l);
       RW[o + 4] = h;
       RW[o + 6] = l;
     }

@@ -27,7 +27,8 @@ void build_coef(int dim, const double delta[3], int nd, const double* S, const d
 // R is the double-float pair nearest the reciprocal of a denominator formed exactly
 // (double-double) from the stored pairs themselves, W the pair nearest
 // 1 - R (beta_b / v_b + sum c) of the stored R, so that a uniform field is a fixed point
-// of the update to the pairs' resolution.  Only the first of each group of directions
+// of the update to the pairs' resolution; below 1/4, where that difference would lose
+// relative accuracy, the pair nearest R / (v_b dt).  Only the first of each group of directions
 // (internal_order) is formed: its rows serve the group.
 void build_ff_factored(int dim, const double delta[3], int nd, int group, const double* S, const double* w, int nb, int nbp,
                        const double* vg, const double* beta, double dt, float* RW, float* dirc, float* band);

@@ -2,6 +2,7 @@
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_2305_19400_gb300 import bte, workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -60,3 +61,26 @@ def test_equilibrium_stays():
     s.step(nsteps=1000, ninner=4)
     assert np.sqrt(np.mean(((s.intensity(0) - I0) / I0) ** 2)) <= 3.5e-14
     s.close()
+
+
+# Steps so long that the coefficient W of I^n is 1e-6 to 1e-5, one cell at 300 K among cells and
+# walls at 2 K, no scattering to speak of: where every upwind value is cold, the hot cell is left
+# with W I^n alone.  W as 1 - R (...) would be off by 2^-49 / W, 3e-10 of it.  Bar: the FP64 parity bar
+# on I.
+def test_small_invariant_coefficient():
+    g = W.Geometry(2, 2, 2, 1, 10e-9, 10e-9, 10e-9)
+    W.uniform_walls(g, [W.BC_ISOTHERMAL] * 4, [2.0] * 4)
+    bands = W.make_bands(8, 0, 86, log10_tau_range=(-3.0, -2.9))
+    T0 = np.array([300.0, 2.0, 2.0, 2.0])
+    for dt in (1e-6, 1e-7):
+        wl = W.Workload("long step", [g], W.Dirs("polar_azim", n_polar=2, n_azim=4), bands, dt, 1, 1)
+        s = bte.Solver(wl, T_init=[T0])
+        s.step()
+        p = O.Problem(g, O.dirs_for(wl.dirs), bands)
+        ost = p.init_state(T0)
+        p.run(ost, dt, 1, 1)
+        I, ref = s.intensity(0), ost["I"]
+        ok = ref > 1e-20  # below 2^-74 a pair keeps a float's bits
+        assert ok.mean() > 0.3
+        assert np.max(np.abs(I[ok] - ref[ok]) / ref[ok]) <= 1e-11
+        s.close()
